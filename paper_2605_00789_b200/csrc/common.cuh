@@ -161,6 +161,17 @@ __device__ inline uint32_t orderable(float f) {
   return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
 }
 
+// pair score from the inner product g and the norms of the two rows: the norms themselves for FD = 1 - cosine,
+// the squared norms for the Euclidean scores |a|^2 + |b|^2 - 2 g
+__device__ __forceinline__ float pair_score(int metric, float g, float na, float nb) {
+  if (metric == LIGHTKV_FD_COSINE) {
+    const float den = na * nb;
+    return 1.0f - (den > 0.f ? g / den : 0.f);
+  }
+  const float sq = fmaxf(fmaf(-2.0f, g, na + nb), 0.f);
+  return metric == LIGHTKV_FD_L2 ? sqrtf(sq) : sq;
+}
+
 // Programmatic dependent launch.  Every kernel of the library is launched with programmatic stream
 // serialization and begins with this call: it lets the next kernel of the stream become resident, then
 // waits until the kernel before this one has completed and its writes are visible.  So a kernel's launch

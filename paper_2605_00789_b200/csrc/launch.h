@@ -35,6 +35,7 @@ struct LayerLaunch {
   int batch, hidden, n_q_heads, n_kv_heads, head_dim;
   int dtype, xi_mode, divergence;
   double keep;
+  int fd_side;                       // estimate of the larger side (A or B nodes) of a window: picks the FD kernel
   int fd_tiles;                      // estimate of FdTiling::n_tiles per sample (launch shape of the tensor-core FD kernel)
   Geometry geo;
   Workspace ws;
@@ -71,6 +72,9 @@ inline cudaError_t ensure_dynamic_smem(void (*kernel)(P...), int bytes) {
 cudaError_t launch_window_build(const LayerLaunch& L);
 // FD + best partner per A node (Step 2), fp32 FMA path
 cudaError_t launch_fd_simt(const LayerLaunch& L);
+// FD for bf16 windows of at most 40 nodes a side, rows straight from global memory into mma.sync fragments
+bool fd_stream_supported(int fd_side);
+cudaError_t launch_fd_stream(const LayerLaunch& L);
 // xi per head (Eq. "attention-factor"), fp32 FMA path; handles ATTN_FULL and ATTN_LSE
 cudaError_t launch_xi_simt(const LayerLaunch& L);
 // head sum of xi, ranking, merge map, weights (Steps 2-5)

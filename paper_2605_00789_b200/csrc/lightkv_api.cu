@@ -17,6 +17,7 @@ struct StagePlan {
   bool exact;      // cap_in is the exact count (schedule so far is data independent)
   bool exact_out;  // cap_out too
   bool use_tc;
+  int fd_side;     // larger side (A or B nodes) of a typical window: picks the FD kernel
   int fd_tiles;    // estimate of the tiles per sample of the tensor-core FD kernel (sizes its launch)
   Geometry geo;
   size_t ws_bytes;
@@ -188,6 +189,7 @@ int lightkv_plan(const lightkv_config_t* c, lightkv_plan_t** out) {
       }
       sp.cap_a = cap_a; sp.cap_b = cap_b;
       sp.fd_tiles = fd_tile_count(g.n_windows, max_a, c->batch);
+      sp.fd_side = max_a;
       if (still) {
         std::sort(next.begin(), next.end());
         alive.swap(next);
@@ -206,6 +208,8 @@ int lightkv_plan(const lightkv_config_t* c, lightkv_plan_t** out) {
       for (int t = 0; t < c->n_tiles; ++t)
         cell = std::max(cell, ((g.rows[t] + sp.w - 1) / sp.w) * ((g.cols[t] + sp.w - 1) / sp.w));
       sp.fd_tiles = fd_tile_count(g.n_windows, (std::min(cell, sp.cap_in) + 1) / 2, c->batch);
+      // the tokens still alive are spread over the cells about evenly (the kernels walk larger windows in blocks)
+      sp.fd_side = (int)(((long long)cell * sp.cap_in / p->n_vis0 + 2) / 2);
     }
     if (!exact) {   // data-dependent from here on: every window keeps at most ceil(keep n_w) tokens
       long long bound = (long long)ceil(sp.keep * sp.cap_in) + sp.n_windows;
@@ -311,13 +315,19 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
   L.batch = c.batch; L.hidden = c.hidden; L.n_q_heads = c.n_q_heads; L.n_kv_heads = c.n_kv_heads;
   L.head_dim = c.head_dim; L.dtype = c.dtype; L.xi_mode = c.xi_mode; L.divergence = c.divergence;
   L.keep = s.keep; L.geo = s.geo;
-  L.fd_tiles = s.fd_tiles;
+  L.fd_tiles = s.fd_tiles; L.fd_side = s.fd_side;
   L.ws = bind_workspace(s, a->workspace); L.text = text; L.a = a; L.stream = static_cast<cudaStream_t>(a->stream);
 
   cudaEvent_t* ev = reinterpret_cast<cudaEvent_t*>(a->trace_events);
   auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], L.stream) : cudaSuccess; };
   const bool tc_xi = s.use_tc && attn && tc_xi_supported(c.head_dim);
   const bool tc_fd = s.use_tc && tc_fd_supported(c.hidden);
+  auto launch_fd = [&](const LayerLaunch& l) {
+    if (!tc_fd) return launch_fd_simt(l);
+    // the streaming kernel addresses a sample's rows by 32-bit offsets of 16-byte units
+    const bool near = (long long)s.cap_in * a->hidden_row_stride / 8 < 0xffffffffll;
+    return near && fd_stream_supported(s.fd_side) ? launch_fd_stream(l) : launch_fd_tc(l);
+  };
   cudaStream_t aux = (a->aux_stream && attn && !ev) ? static_cast<cudaStream_t>(a->aux_stream) : nullptr;
   if (aux) {
     // fork: window build + FD (HBM bound) on the second stream, xi (bound by the exponentials) on the first.
@@ -328,7 +338,7 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
     if (cudaEventRecord(fork, L.stream) != cudaSuccess) return LIGHTKV_ERR_CUDA;
     bool ok = cudaStreamWaitEvent(aux, fork, 0) == cudaSuccess;
     ok = ok && launch_window_build(La) == cudaSuccess;
-    ok = ok && (tc_fd ? launch_fd_tc(La) : launch_fd_simt(La)) == cudaSuccess;
+    ok = ok && launch_fd(La) == cudaSuccess;
     const bool joined = cudaEventRecord(join, aux) == cudaSuccess;
     ok = ok && (tc_xi ? launch_xi_tc(L) : launch_xi_simt(L)) == cudaSuccess;
     const bool waited = joined && cudaStreamWaitEvent(L.stream, join, 0) == cudaSuccess;
@@ -338,7 +348,7 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
     if (launch_window_build(L) != cudaSuccess || mark(1) != cudaSuccess) return LIGHTKV_ERR_CUDA;
     if (attn && (tc_xi ? launch_xi_tc(L) : launch_xi_simt(L)) != cudaSuccess) return LIGHTKV_ERR_CUDA;
     if (mark(2) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-    if ((tc_fd ? launch_fd_tc(L) : launch_fd_simt(L)) != cudaSuccess || mark(3) != cudaSuccess)
+    if (launch_fd(L) != cudaSuccess || mark(3) != cudaSuccess)
       return LIGHTKV_ERR_CUDA;
   }
   if (launch_select_map(L) != cudaSuccess || mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;

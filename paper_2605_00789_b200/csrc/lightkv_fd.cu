@@ -1,0 +1,245 @@
+// liblightkv kernels, part 3: FD + best partner for small windows (bf16), one pass over the hidden states.
+#include <algorithm>
+
+#include "launch.h"
+#include "tc_common.cuh"
+
+namespace lkv {
+
+// ======================================================================================================
+// FD + best partner for windows of up to 8 * O source and 8 * O destination nodes (Eq. "similarity", Step 2).
+//
+// With windows this small the contraction has a few flops per byte and the kernel is bound by reading the vision
+// rows once from HBM.  So the rows go straight from global memory into the fragments of mma.sync m16n8k16: no
+// shared-memory staging, no swizzle, no barrier per chunk.  One CTA takes one window; its warps split the hidden
+// dimension (contiguous column ranges, about 1 KB of every row per warp at eight warps).  Lane (g, t) of a warp
+// loads 16 bytes of row g of every group of eight rows: four lanes cover 64 contiguous bytes.  The k order inside
+// an MMA is free as long as both operands agree, so the eight bf16 of a 16-byte piece serve as the lane's k
+// elements of two MMA steps, for the row's role as an A operand and as a B operand alike.  The squared norms
+// accumulate from the same registers (exact products, fp32 sums).  Partial inner products of the warps meet in
+// shared memory in warp order, then a warp per source row takes the minimum over the destinations (ties: lowest
+// index).  A window with more nodes than the template holds is walked in blocks of 8 * O by 8 * O.
+// A lane's pieces wait in shared memory (cp.async, a ring of S chunks per warp that only this lane writes and reads,
+// so no barrier): loads in flight then cost no registers.  Against the tcgen05 kernel with its gathered 128-row tiles:
+// 8 samples x 2880 tokens x 4096 in windows of 16: 59 -> 37 us between events (189 MB: 5.1 TB/s), windows of 18:
+// 41 -> 27, of 36: 39 -> 23; 32 x 576 x 5120 in windows of 36: 76 -> 45, of 72: 59 -> 29.
+// ======================================================================================================
+struct FdStreamArgs {
+  const __nv_bfloat16* x;              // first vision row of sample 0
+  const int* seq_start;                // first row of each sample (packed batches) or nullptr
+  int64_t batch_stride, row_stride;    // elements
+  int d, metric;
+  Workspace ws;
+};
+
+__device__ __forceinline__ void mma_m16n8k16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                             uint32_t b0, uint32_t b1) {
+  asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+               : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
+               : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+
+__device__ __forceinline__ void st_shared16(uint32_t addr, const uint4& v) {
+  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+// the quad of lanes takes 64 bytes of a row: ask L2 for the whole 128-byte line at once
+__device__ __forceinline__ void cp_async16_l2(uint32_t smem_dst, const void* gmem_src, uint32_t src_bytes) {
+  asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(gmem_src), "r"(src_bytes) : "memory");
+}
+// acc += lo^2 + hi^2 over the four bf16 pairs of v; every product is exact in fp32
+__device__ __forceinline__ float sumsq16(const uint4& v, float acc) {
+  const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %1;\n\t"
+        "fma.rn.f32.bf16 %0, lo, lo, %0;\n\tfma.rn.f32.bf16 %0, hi, hi, %0;\n\t}" : "+f"(acc) : "r"(u[j]));
+  return acc;
+}
+
+// O: groups of eight rows a side; S: 32-column chunks in flight per warp; WARPS: warps of a CTA
+template <int O, int S, int WARPS>
+struct FdStreamSmem {
+  static constexpr int R = 8 * O, PITCH = R + 2;
+  static constexpr int RING = WARPS * S * 2 * O * 512;                              // bytes
+  static constexpr int PART = (WARPS * R * PITCH + WARPS * 2 * R) * 4;              // over the drained ring
+  static constexpr int BYTES = (RING > PART ? RING : PART) + 2 * R * 4;
+};
+
+template <int O, int S, int WARPS>
+__global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(FdStreamArgs a) {
+  grid_dependency_sync();
+  using M = FdStreamSmem<O, S, WARPS>;
+  constexpr int R = M::R, MT = (O + 1) / 2, PITCH = M::PITCH;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = WARPS;
+  float* part = reinterpret_cast<float*>(smem_raw);      // [WARPS][R][PITCH] partial inner products
+  float* nrm = part + WARPS * R * PITCH;                 // [WARPS][2 R] partial squared norms, row 0: the norms
+  float* best_f = reinterpret_cast<float*>(smem_raw + M::BYTES - 2 * R * 4);   // [R] running minimum over blocks of destinations
+  int* best_e = reinterpret_cast<int*>(best_f + R);      // [R]
+  const int w = blockIdx.x, b = blockIdx.y, nW = a.ws.n_windows;
+  const int* win_off = a.ws.win_off + size_t(b) * (nW + 1) + w;
+  const int* a_off = a.ws.a_off + size_t(b) * (nW + 1) + w;
+  const int a_lo = a_off[0], a_hi = a_off[1], b_lo = win_off[0] - a_lo, b_hi = win_off[1] - a_hi;
+  if (a_lo >= a_hi || b_lo >= b_hi) return;
+  const int* a_tok = a.ws.a_tok + size_t(b) * a.ws.cap_a;
+  const int* b_tok = a.ws.b_tok + size_t(b) * a.ws.cap_b;
+  const int g = lane >> 2, t = lane & 3;
+  const int nc = (a.d + 31) >> 5, c_lo = warp * nc / WARPS, nk = (warp + 1) * nc / WARPS - c_lo;
+  const __nv_bfloat16* base = a.x + size_t(b) * a.batch_stride + size_t(a.seq_start ? a.seq_start[b] : 0) * a.row_stride +
+                              c_lo * 32 + t * 8;
+  const uint32_t row16 = uint32_t(a.row_stride >> 3);    // row pitch in 16-byte units
+  const uint32_t ring = tc::smem_u32(smem_raw) + (warp * S * 2 * O * 32 + lane) * 16;
+
+  for (int a0 = a_lo; a0 < a_hi; a0 += R) {
+    const int na = min(R, a_hi - a0);
+    for (int b0 = b_lo; b0 < b_hi; b0 += R) {
+      const int nb = min(R, b_hi - b0);
+      uint32_t off[2 * O];                               // row offsets in 16-byte units, A rows first; all ones: no such row
+#pragma unroll
+      for (int i = 0; i < O; ++i) {
+        off[i] = 8 * i + g < na ? uint32_t(a_tok[a0 + 8 * i + g]) * row16 : 0xffffffffu;
+        off[O + i] = 8 * i + g < nb ? uint32_t(b_tok[b0 + 8 * i + g]) * row16 : 0xffffffffu;
+      }
+      // rows the block does not have stay zero in every stage
+#pragma unroll
+      for (int i = 0; i < 2 * O; ++i)
+        if (off[i] == 0xffffffffu)
+#pragma unroll
+          for (int st = 0; st < S; ++st) st_shared16(ring + (st * 2 * O + i) * 512, make_uint4(0, 0, 0, 0));
+      auto issue = [&](int k, int st) {
+        if (k < nk) {
+          const uint32_t bytes = (c_lo + k) * 32 + t * 8 < a.d ? 16u : 0u;    // d is a multiple of 8
+          const __nv_bfloat16* p = base + (bytes ? k * 32 : 0);
+#pragma unroll
+          for (int i = 0; i < 2 * O; ++i)
+            if (off[i] != 0xffffffffu) cp_async16_l2(ring + (st * 2 * O + i) * 512, p + size_t(off[i]) * 8, bytes);
+        }
+        tc::cp_async_commit();
+      };
+      float acc[MT][O][4];
+      float ss[2 * O];
+#pragma unroll
+      for (int i = 0; i < 2 * O; ++i) ss[i] = 0.f;
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int j = 0; j < O; ++j)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
+
+#pragma unroll
+      for (int st = 0; st < S; ++st) issue(st, st);
+      for (int k = 0, st = 0; k < nk; ++k) {
+        tc::cp_async_wait<S - 1>();                      // this lane's pieces of chunk k: nobody else reads them
+        uint4 v[2 * O];
+#pragma unroll
+        for (int i = 0; i < 2 * O; ++i) v[i] = tc::ld_shared16(ring + (st * 2 * O + i) * 512);
+#pragma unroll
+        for (int i = 0; i < 2 * O; ++i) ss[i] = sumsq16(v[i], ss[i]);
+#pragma unroll
+        for (int i = 0; i < MT; ++i) {
+          const uint4 lo = v[2 * i], hi = 2 * i + 1 < O ? v[2 * i + 1] : make_uint4(0, 0, 0, 0);
+#pragma unroll
+          for (int j = 0; j < O; ++j) {
+            mma_m16n8k16(acc[i][j], lo.x, hi.x, lo.y, hi.y, v[O + j].x, v[O + j].y);
+            mma_m16n8k16(acc[i][j], lo.z, hi.z, lo.w, hi.w, v[O + j].z, v[O + j].w);
+          }
+        }
+        issue(k + S, st);
+        st = st + 1 == S ? 0 : st + 1;
+      }
+      tc::cp_async_wait<0>();
+      __syncthreads();                                   // every warp's ring is drained: the partial results go over it
+      // ---- partial results of this warp
+      float* pw = part + warp * R * PITCH;
+#pragma unroll
+      for (int i = 0; i < MT; ++i)
+#pragma unroll
+        for (int j = 0; j < O; ++j) {
+          const int r = 16 * i + g, col = 8 * j + 2 * t;
+          *reinterpret_cast<float2*>(pw + r * PITCH + col) = make_float2(acc[i][j][0], acc[i][j][1]);
+          if (2 * i + 1 < O) *reinterpret_cast<float2*>(pw + (r + 8) * PITCH + col) = make_float2(acc[i][j][2], acc[i][j][3]);
+        }
+#pragma unroll
+      for (int i = 0; i < 2 * O; ++i) {
+#pragma unroll
+        for (int o = 1; o < 4; o <<= 1) ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], o);
+        if (t == 0) nrm[warp * 2 * R + 8 * i + g] = ss[i];
+      }
+      __syncthreads();
+      // ---- norms and inner products over the warps, in warp order
+      for (int i = tid; i < 2 * R; i += blockDim.x) {
+        float s = nrm[i];
+        for (int k = 1; k < nwarps; ++k) s += nrm[k * 2 * R + i];
+        nrm[i] = a.metric == LIGHTKV_FD_COSINE ? sqrtf(s) : s;
+      }
+      __syncthreads();
+      // ---- a warp per source row, lanes over the destinations
+      for (int r = warp; r < na; r += nwarps) {
+        float best = 3.0e38f;
+        int best_c = -1;
+        for (int col = lane; col < nb; col += 32) {
+          float s = part[r * PITCH + col];
+          for (int k = 1; k < nwarps; ++k) s += part[(k * R + r) * PITCH + col];
+          const float fd = pair_score(a.metric, s, nrm[r], nrm[R + col]);
+          if (fd < best) { best = fd; best_c = col; }
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {               // minimum over the lanes, ties to the lower column
+          const float of = __shfl_xor_sync(0xffffffffu, best, o);
+          const int oc = __shfl_xor_sync(0xffffffffu, best_c, o);
+          if (oc >= 0 && (best_c < 0 || of < best || (of == best && oc < best_c))) { best = of; best_c = oc; }
+        }
+        if (lane == 0) {
+          int e = best_c >= 0 ? b0 + best_c : -1;
+          if (b0 > b_lo && best_e[r] >= 0 && !(best < best_f[r])) { best = best_f[r]; e = best_e[r]; }
+          best_f[r] = best;
+          best_e[r] = e;
+          if (b0 + R >= b_hi && e >= 0)
+            a.ws.a_key[size_t(b) * a.ws.cap_a + a0 + r] = ((unsigned long long)orderable(best) << 32) | (unsigned)e;
+        }
+      }
+      if (a0 + R < a_hi || b0 + R < b_hi) __syncthreads();   // the partial results are overwritten by the next block
+    }
+  }
+}
+
+template <int O, int S, int WARPS>
+static cudaError_t launch_fd_stream_o(const LayerLaunch& L, const FdStreamArgs& f) {
+  constexpr int smem = FdStreamSmem<O, S, WARPS>::BYTES;
+  const cudaError_t e = ensure_dynamic_smem(fd_stream_kernel<O, S, WARPS>, smem);
+  if (e != cudaSuccess) return e;
+  return launch_kernel(fd_stream_kernel<O, S, WARPS>, dim3(L.geo.n_windows, L.batch), 32 * WARPS, smem, L.stream, 1, f);
+}
+
+// Eight warps split the hidden dimension where each still gets a few chunks of it (hidden > 768); a narrow model gets
+// CTAs of two, so that the fixed cost of a window (its lists, the meeting of the warps) is paid by fewer threads.
+template <int O, int S>
+static cudaError_t launch_fd_stream_w(const LayerLaunch& L, const FdStreamArgs& f) {
+  return L.hidden > 768 ? launch_fd_stream_o<O, S, 8>(L, f) : launch_fd_stream_o<O, S, 2>(L, f);
+}
+
+// Largest window side (source or destination nodes) the plan may expect for this kernel: five groups of eight rows a
+// side is what the fragments of a thread hold at two CTAs per SM; beyond that the tcgen05 kernel shares the rows
+// between more pairs.
+bool fd_stream_supported(int fd_side) { return fd_side > 0 && fd_side <= 40; }
+
+cudaError_t launch_fd_stream(const LayerLaunch& L) {
+  const lightkv_layer_args_t* a = L.a;
+  FdStreamArgs f;
+  f.x = static_cast<const __nv_bfloat16*>(a->hidden) + size_t(a->vis_begin) * a->hidden_row_stride;
+  f.seq_start = a->seq_start;
+  f.batch_stride = a->hidden_batch_stride; f.row_stride = a->hidden_row_stride;
+  f.d = L.hidden; f.metric = L.divergence; f.ws = L.ws;
+  // chunks in flight per warp (S): as few as still leave enough CTAs on an SM; with more, fewer CTAs fit and the
+  // start and end of a window are less covered (S = 8, 6, 4 measured 39 / 33 / 25 us where 6, 4, 3 take 37 / 27 / 23)
+  switch ((L.fd_side + 7) / 8) {
+    case 1: return launch_fd_stream_w<1, 6>(L, f);
+    case 2: return launch_fd_stream_w<2, 4>(L, f);
+    case 3: return launch_fd_stream_w<3, 3>(L, f);
+    case 4: return launch_fd_stream_w<4, 2>(L, f);
+    default: return launch_fd_stream_w<5, 2>(L, f);
+  }
+}
+
+}  // namespace lkv

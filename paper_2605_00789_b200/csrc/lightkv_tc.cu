@@ -572,17 +572,6 @@ struct FdTcArgs {
   uint32_t* status;
 };
 
-// pair score from the inner product g and the norms of the two rows: the norms themselves for FD = 1 - cosine,
-// the squared norms for the Euclidean scores |a|^2 + |b|^2 - 2 g
-__device__ __forceinline__ float pair_score(int metric, float g, float na, float nb) {
-  if (metric == LIGHTKV_FD_COSINE) {
-    const float den = na * nb;
-    return 1.0f - (den > 0.f ? g / den : 0.f);
-  }
-  const float sq = fmaxf(fmaf(-2.0f, g, na + nb), 0.f);
-  return metric == LIGHTKV_FD_L2 ? sqrtf(sq) : sq;
-}
-
 constexpr int FT_LOADERS = 256;
 constexpr int FT_STAGES = 6;
 constexpr int FT_AHEAD = 4;                               // fills in flight

@@ -420,6 +420,30 @@ def test_fd_persistent_ctas_take_several_tiles(hidden, ragged):
     assert info.uses_tensor_cores == 1 and info.fd_tiles * wl.batch > 2 * _sm_count()
 
 
+@pytest.mark.parametrize("hidden", [72, 776])
+@pytest.mark.parametrize("grid", [(3, 3), (4, 4), (3, 6), (4, 8), (3, 11), (6, 8), (7, 7), (8, 8), (5, 13), (8, 10), (9, 9)])
+def test_fd_windows_around_groups_of_eight_nodes(grid, hidden):
+    # one window of rows x cols tokens: the larger side just below, at and above the 8, 16, 24, 32 and 40 nodes the
+    # streaming FD kernel's variants hold (41: the tcgen05 kernel); hidden sizes that end inside a chunk of columns
+    wl = S.Workload(name="fdside", config_id=132, batch=3, tiles=(grid,), n_text=4, hidden=hidden, n_q_heads=2,
+                    n_kv_heads=1, head_dim=64, n_layers=16, layers=(3,), windows=(1,), keep=(0.6,))
+    H.run_schedule(wl, xi_mode="uniform")
+    H.run_schedule(dataclasses.replace(wl, batch=1), xi_mode="uniform", direction="b2a", metric="l2")
+
+
+@pytest.mark.parametrize("grid,windows,seed", [((12, 20), (5, 3), 282), ((12, 32), (3, 2), 4)])
+def test_fd_window_larger_than_the_plan_expects(grid, windows, seed):
+    # a near-full subset of the grid moves tokens between windows: one window of the second stage has a node more a
+    # side than any window of the full grid (8, 24), so the streaming FD kernel walks it in blocks
+    wl = S.Workload(name="fdwalk", config_id=133, batch=2, tiles=(grid,), n_text=4, hidden=776, n_q_heads=2,
+                    n_kv_heads=1, head_dim=64, n_layers=16, layers=(3, 7), windows=windows, keep=(0.5, 0.5))
+    rng = np.random.default_rng(seed)
+    full = np.arange(grid[0] * grid[1], dtype=np.int32)
+    missing = int(rng.integers(4, 14))
+    subset = np.sort(rng.choice(full, full.size - missing, replace=False)).astype(np.int32)
+    H.run_schedule(wl, xi_mode="given", first_pos=[subset, full])
+
+
 # ---- subsets of the grid: capacities ---------------------------------------------------------------------------
 
 def _near_full_subset():
