@@ -251,8 +251,7 @@ typedef struct {
 
 /* Enqueue window build, xi, FD + best partner, selection + merge map and the weighted merge of the hidden states
  * (Steps 1-5 of Sec. "LightKV"; Eq. "attention-factor", "similarity", "message-passing").  Nothing is allocated or
- * synchronised; besides the kernels a 16-byte cudaMemsetAsync on `stream` clears the xi kernel's scheduler words
- * in the workspace.  Errors: INVALID_ARG (NULL or misaligned buffers, strides below the row width, a prompt set
+ * synchronised, and the workspace need not be cleared.  Errors: INVALID_ARG (NULL or misaligned buffers, strides below the row width, a prompt set
  * outside [0, vis_begin], aux_stream without its two events, lse_out outside ATTN_FULL, ...), WORKSPACE (too small
  * or not 256-byte aligned), CUDA (a launch failed).  Conditions only the device sees set bits of *status. */
 int lightkv_compress_layer(const lightkv_plan_t* plan, const lightkv_layer_args_t* args);
@@ -270,9 +269,8 @@ int lightkv_compress_layer(const lightkv_plan_t* plan, const lightkv_layer_args_
  *   - The first call on each device looks up the array's device address (cudaGetSymbolAddress, with
  *     that device current) and remembers it; make that first call outside any stream capture.
  *     LIGHTKV_ERR_CUDA if the lookup fails.
- *   - All calls on one device share the array, and it keeps what the previous call left.  The only
- *     words that have to start at zero (the ticket counters of the xi kernel) are cleared by a 16-byte
- *     cudaMemsetAsync on the stream inside every call; everything else is written before it is read.  But
+ *   - All calls on one device share the array, and it keeps what the previous call left (everything is
+ *     written before it is read).  But
  *     two calls whose kernels overlap on the GPU (different streams, no ordering between them)
  *     race on it: order such calls, or give all but one of them lightkv_compress_layer with their
  *     own workspace. */

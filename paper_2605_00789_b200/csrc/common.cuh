@@ -56,8 +56,8 @@ struct Workspace {
   int* partner;    // [B, cap_in]         token an A token is merged into, -1 = survives
   int* slot;       // [B, cap_in]         output slot of surviving tokens
   int* a_partner;  // [B, cap_a]          per A entry: token it is merged into, -1 = survives
-  unsigned int* xi_sched;   // [4]        ticket counters and list length of the tensor-core xi kernel
-  int* xi_redo;    // [ceil(cap_in / 128) * H * B]  its work items that need the second, safe launch
+  int* xi_redo;    // [ceil(cap_in / 128) * H * B]  links between the work items of the tensor-core xi kernel that a
+                   //                               CTA has to repeat with a running maximum
   int cap_in, cap_out, cap_a, cap_b, n_windows;
 };
 
@@ -71,6 +71,12 @@ struct TextSet {
     for (int i = 0; i < n; ++i)
       if (j >= lo[i] && j < hi[i]) return true;
     return false;
+  }
+  // bit c set <=> key j0 + c belongs to J (c < 32)
+  __device__ inline unsigned int mask32(int j0) const {
+    if (n != 1) return (unsigned int)mask64(j0);
+    const int a = begin > j0 ? begin - j0 : 0, b = end - j0 < 32 ? end - j0 : 32;
+    return a >= b ? 0u : (0xffffffffu >> (32 - b)) & (0xffffffffu << a);
   }
   // bit c set <=> key j0 + c belongs to J (c < 64)
   __host__ __device__ inline unsigned long long mask64(int j0) const {

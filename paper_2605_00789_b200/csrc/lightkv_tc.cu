@@ -48,61 +48,97 @@ static bool make_map_bhnd(CUtensorMap* map, const void* base, int width, int row
 // ======================================================================================================
 // xi per head on tensor cores (Eq. "attention-factor" over the softmax rows of Eq. "attention-matrix").
 //
-// A work item is (tile of 128 vision queries, head, sample).  Persistent CTAs, two per SM, draw items from a
-// ticket counter in global memory (the list interleaves groups of 64 (sample, head) pairs whose K stays in L2
-// together, longest rows first inside a group).  Warp 0 is the scheduler and the TMA producer: it
-// publishes the ticket to the other roles through a two-slot ring in shared memory, streams the item's Q tile
-// once and its K tiles (128 keys) through a 2-stage ring; the next item's Q and first K tiles are requested as
-// soon as the MMAs of the current item have drained, i.e. while its last tiles are still in the softmax warps.
-// Warp 1 issues S = Q K^T (128 x 128 x dh, bf16 -> fp32) into one of two TMEM accumulators.  Warps 2-9 are
-// the softmax warps, two threads per query row (= TMEM lane): a thread pulls 32 of the 64 logits of a half of the
-// accumulator into registers (the warp that takes the last piece releases the accumulator) and adds
-// exp(logit - reference) to two sums (all visible keys / prompt keys J); the two threads of a row combine their
-// references and sums once per item through shared memory.
-// Output per head: sum_J / sum_all.
+// A work item is (tile of 128 vision queries, head, sample).  The grid has one CTA per item, in an order that
+// interleaves groups of 64 (sample, head) pairs whose K stays in L2 together, longest rows first inside a group;
+// the CTAs that are resident (two per SM) take over the items of CTAs that have not started yet
+// (clusterlaunchcontrol.try_cancel), so a CTA is set up once, the next item's loads hide behind the current item's
+// last tiles, and no counter in global memory has to be cleared first.  Warp 0 is the scheduler and the TMA
+// producer: it decodes an item once, publishes it to the other roles through a two-slot ring in shared memory,
+// streams the item's Q tile once and its K tiles (128 keys) through a 2-stage ring; the next item's Q and first K
+// tiles are requested as soon as the MMAs of the current item have drained.  Warp 1 issues S = Q K^T
+// (128 x 128 x dh, bf16 -> fp32) into one of two TMEM accumulators.  Warps 2-9 are the softmax warps, two threads
+// per query row (= TMEM lane): a thread pulls 32 of the 64 logits of a half of the accumulator into registers (the
+// warp that takes the last piece releases the accumulator) and adds exp(logit - reference) to two sums (all
+// visible keys / prompt keys J); the two threads of a row combine their references and sums once per item through
+// shared memory.  Output per head: sum_J / sum_all.
 //
-// The kernel is bound by the exponentials (one per logit on the special-function unit, 16 per clock per SM,
-// against one MMA per tile), so the softmax arithmetic is kept to three instructions per logit:
+// One exponential per logit on the special-function unit (16 per clock per SM) against one MMA per tile; at full load
+// the SM clock drops to about 1.6 GHz (power), so what counts is instructions per logit (8 samples x 3008 keys x 32
+// heads: 11.0 clocks and 7.3 instructions per warp and logit before the points below, 8.5 and 5.9 with them, 422 -> 330 us):
 //   * the reference subtracted before the exponential is the thread's maximum over its FIRST 32 keys only
 //     (softmax is invariant to the reference; fp32 holds exp of any later logit up to 88 above it), so the
 //     other tiles need no maximum and no rescaling;
-//   * on halves that need neither the causal mask nor the prompt mask, every eighth exponential is evaluated
-//     on the FMA pipe instead (range reduction + cubic, relative error 7.5e-5).  With the softmax warps alone
-//     on an SM a quarter is the best share; in the whole kernel, which runs into the power limit (SM clock
-//     about 1.78 GHz instead of 1.965), the dozen instructions of the cubic cost more than the special-function
-//     slot they free, and an eighth measured fastest (none: +1 %, a quarter: +4 %, three eighths: +10 %).
+//   * runs of whole tiles that need no mask (all rows of the warp see every key; all or none are prompt keys) have a
+//     loop of their own: sharing one with the masked tiles cost a register move per logit and more;
+//   * scaling and summing take two logits per instruction (fma / add .f32x2: the same time on the FMA pipe, half the
+//     issue slots);
+//   * XT_POLY_PAIRS of every 16 pairs of exponentials are evaluated on the FMA pipe instead (range reduction + a
+//     polynomial of degree four, relative error 2.7e-6): 0 pairs 360 us, 2: 340, 3: 335, 4: 329, 5: 331;
+//   * an item is decoded once, by the scheduler, and masks are built only where the prompt set or the diagonal ends.
+// Tried and slower: the second half's TMEM load in flight behind the first half's arithmetic (350), the polynomial
+// on packed pairs (338).
 // A row whose sum left the fp32 range (a later logit more than 88 above the first keys' maximum) is found at
-// the end of its item, which is then appended to a list in global memory; a second launch of the kernel
-// (SAFE) walks that list with a running maximum and rescaling on every half, as an ordinary online softmax
-// does, and overwrites the item's results.  With an empty list that launch returns at once.
-// Halves that straddle the diagonal (or the end of the sample) are masked, and the columns no row of a warp
-// can see are skipped.  With the caller's row log-sum-exp (LSE) only the prompt key tiles are visited.
+// the end of its item; the CTA puts the item on its own list (links in global memory) and repeats it, once it has
+// run out of new ones, with a running maximum and rescaling on every half as an ordinary online softmax does.
+// With the caller's row log-sum-exp (LSE) only the prompt key tiles are visited.
 // ======================================================================================================
 __device__ __forceinline__ float ex2(float x) {          // one MUFU op, flush-to-zero
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-// 2^x on the FMA and integer pipes: x is clamped to [-126, 128], split into the nearest integer j (magic-number
-// add) and r in [-0.5, 0.5]; 2^r by a minimax cubic; j is added to the exponent field.  x = 128 gives the bit
-// pattern of a non-finite value, which the overflow check at the end of the item sees.
-__device__ __forceinline__ float ex2_fma(float x) {
-  x = fminf(fmaxf(x, -126.f), 128.f);
-  const float t = x + 12582912.f;                         // 1.5 * 2^23: the integer lands in the low mantissa bits
-  const float r = x - (t - 12582912.f);
-  float p = fmaf(r, 0.0551716685f, 0.2426111251f);
-  p = fmaf(p, r, 0.6932609677f);
-  p = fmaf(p, r, 0.9999280572f);
-  return __int_as_float(__float_as_int(p) + (__float_as_int(t) << 23));
+
+// two fp32 values in one 64-bit register, and arithmetic on both
+typedef unsigned long long f32x2;
+__device__ __forceinline__ f32x2 pack2(float lo, float hi) {
+  f32x2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void unpack2(f32x2 v, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(v));
+}
+__device__ __forceinline__ f32x2 fma2(f32x2 a, f32x2 b, f32x2 c) {
+  f32x2 r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+__device__ __forceinline__ f32x2 add2(f32x2 a, f32x2 b) {
+  f32x2 r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ float fma_sat(float a, float b, float c) {    // clamped to [0, 1] at no extra cost
+  float r;
+  asm("fma.rn.sat.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+  return r;
 }
 
-// Scheduler words in the workspace (zeroed on the stream before the first launch of a call).
-struct XiSched {
-  unsigned int ticket;               // next item of the first launch
-  unsigned int safe_ticket;          // next entry of the list, second launch
-  unsigned int n_redo;               // items appended to the list
-  unsigned int pad;
+// What the exponentials of a thread need: logits are scaled to log2 units, x = v * sc - ms.
+struct ExpRef {
+  f32x2 sc2, nms2;                   // {sc, sc}, {-ms, -ms}
+  float sc_y, c_y;                   // y = (x + 126) / 254 = v * sc_y + c_y, clamped to [0, 1] by the fma
+  __device__ __forceinline__ void set(float sc, float ms) {
+    sc2 = pack2(sc, sc);
+    nms2 = pack2(-ms, -ms);
+    sc_y = sc * (1.0f / 254.0f);
+    c_y = (126.0f - ms) * (1.0f / 254.0f);
+  }
 };
+// 2^x of two logits on the FMA pipe: x is clamped to [-126, 128] (as y in [0, 1]), split into the nearest integer j
+// (magic-number add) and r in [-0.5, 0.5]; 2^r by a minimax polynomial of degree four; j is added to the exponent
+// field.  x = 128 gives a value of 3.4e38 or more, which the overflow check at the end of the item sees.
+__device__ __forceinline__ float ex2_fma(float v, const ExpRef& e) {
+  constexpr float kMagic = 12582912.f - 126.f;            // 1.5 * 2^23: the integer lands in the low mantissa bits
+  const float y = fma_sat(v, e.sc_y, e.c_y);
+  const float t = fmaf(y, 254.f, kMagic);                 // bits: 0x4b400000 + j
+  const float r = fmaf(y, 254.f, kMagic - t);
+  float p = fmaf(r, 0.009570102207f, 0.05591785908f);
+  p = fmaf(p, r, 0.2402474433f);
+  p = fmaf(p, r, 0.6931217909f);
+  p = fmaf(p, r, 0.9999992847f);
+  return __int_as_float(__float_as_int(p) + (__float_as_int(t) << 23));
+}
 
 struct XiTcArgs {
   const int* n_vis;
@@ -118,8 +154,7 @@ struct XiTcArgs {
   int cap_in, vis_begin, n_q_heads, group;
   int batch, n_qt;                   // samples, query tiles of 128 rows per (sample, head)
   float scale2;                      // log2(e) / sqrt(dh)
-  XiSched* sched;
-  int* redo_list;                    // [n_qt * H * B] items whose sums left the fp32 range
+  int* redo_next;                    // [n_qt * H * B] links of the CTAs' lists of items whose sums left the fp32 range
 };
 
 constexpr int XT_STAGES = 2;         // K tiles in the shared-memory ring
@@ -128,17 +163,36 @@ constexpr int XT_CTAS = 2;           // CTAs per SM
 constexpr int XT_KEY_TILE = 128;     // keys per K tile and per MMA (the softmax warps read it as two halves of 64)
 constexpr int XT_SUB = 64;           // keys per half
 constexpr int XT_THREADS = 320;      // TMA / scheduler warp, MMA warp, eight softmax warps
-constexpr int XT_SAMPLE_CACHE = 256;  // samples whose token count and row offset are kept in shared memory
 constexpr int XT_HEAD_GROUP = 64;    // (sample, head) pairs whose work items are interleaved (their K: 64 x ~1 MB)
+constexpr int XT_POLY_PAIRS = 4;     // of 16 pairs of exponentials: on the FMA pipe
 
-// LSE: the caller supplied the row log-sum-exp (a.lse != nullptr).  SAFE: second launch, items from the list.
-template <int DH, bool LSE, bool SAFE>
+// adds exp over 32 logits of a thread to two pairs of sums (masked logits are -inf and add nothing that counts)
+__device__ __forceinline__ void exp_add32(const float (&v)[32], const ExpRef& e, f32x2 (&part)[2]) {
+#pragma unroll
+  for (int i = 0; i < 16; ++i) {
+    f32x2 p;
+    if ((i * XT_POLY_PAIRS) % 16 < XT_POLY_PAIRS) {
+      p = pack2(ex2_fma(v[2 * i], e), ex2_fma(v[2 * i + 1], e));
+    } else {
+      float x0, x1;
+      unpack2(fma2(pack2(v[2 * i], v[2 * i + 1]), e.sc2, e.nms2), x0, x1);
+      p = pack2(ex2(x0), ex2(x1));
+    }
+    part[i & 1] = add2(part[i & 1], p);
+  }
+}
+__device__ __forceinline__ float sum_pairs(const f32x2 (&part)[2]) {
+  float s0, s1;
+  unpack2(add2(part[0], part[1]), s0, s1);
+  return s0 + s1;
+}
+
+// LSE: the caller supplied the row log-sum-exp (a.lse != nullptr).
+template <int DH, bool LSE>
 __global__ void __launch_bounds__(XT_THREADS, XT_CTAS)
 xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ CUtensorMap k_map, XiTcArgs a) {
-  grid_dependency_sync();
   constexpr int BK = XT_KEY_TILE;
   static_assert(BK == 2 * XT_SUB && XT_SUB == 64, "a K tile is two halves of 64 keys; the prompt mask of a half is one 64-bit word");
-  static_assert(!(LSE && SAFE), "with the caller's normaliser no sum can leave the fp32 range");
   constexpr int HALVES = DH / 64;
   constexpr uint32_t TILE_BYTES = HALVES * 16384;          // Q tile: 128 rows x DH bf16
   constexpr uint32_t KHALF_BYTES = BK * 128;               // BK key rows x 64 columns
@@ -146,14 +200,15 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
   // With the caller's normaliser an item is one or two key tiles and the kernel is bound by reading Q from HBM:
   // then the Q tile is double buffered (two items' Q in flight per CTA) and one K stage is enough.
   constexpr int QBUF = LSE ? 2 : 1, KSTAGES = LSE ? 1 : XT_STAGES;
-  const unsigned int n_items = SAFE ? a.sched->n_redo : unsigned(a.n_qt) * a.n_q_heads * a.batch;
-  if (n_items == 0) return;                                // nothing on the list: the usual case of the second launch
 
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   unsigned char* q_s = base;                   // [QBUF] Q tiles
   unsigned char* k_s = base + QBUF * TILE_BYTES;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(base + QBUF * TILE_BYTES + KT_BYTES * KSTAGES);
+  unsigned char* ctl = base + QBUF * TILE_BYTES + KT_BYTES * KSTAGES;
+  int4* item_slot = reinterpret_cast<int4*>(ctl);          // [2][2] published items
+  uint4* clc_slot = reinterpret_cast<uint4*>(ctl + 64);    // answer to the request for another CTA's item
+  uint64_t* bars = reinterpret_cast<uint64_t*>(ctl + 80);
   uint64_t* q_full = bars;                     // [2]
   uint64_t* q_empty = bars + 2;                // [2] every MMA that reads the Q tile has completed
   uint64_t* k_full = bars + 4;                 // [XT_STAGES]
@@ -161,50 +216,23 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
   uint64_t* s_full = k_empty + XT_STAGES;      // [XT_SBUF]
   uint64_t* s_empty = s_full + XT_SBUF;        // [XT_SBUF]
   uint64_t* item_full = s_empty + XT_SBUF;     // [2] the scheduler published an item
-  uint64_t* item_empty = item_full + 2;        // [2] the MMA thread and the eight softmax warps have read it
+  uint64_t* item_empty = item_full + 2;        // [2] the MMA thread has read it, the eight softmax warps are done with it
   uint64_t* pair_full = item_empty + 2;        // the upper column group has stored its partial sums of an item
   uint64_t* pair_empty = pair_full + 1;        // the lower column group has read them
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(pair_empty + 1);
+  uint64_t* clc_full = pair_empty + 1;         // clc_slot has been written
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(clc_full + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  volatile int* item_slot = abort_flag + 1;    // [2]
-  int* redo_mark = const_cast<int*>(item_slot) + 2;      // last item this CTA put on the list
-  float* pair_m = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(bars) + 256);   // [128] each
+  int* redo_mark = const_cast<int*>(abort_flag) + 1;       // last item this CTA put on its list
+  int* redo_head = redo_mark + 1;                          // first item of the list, -1: empty
+  float* pair_m = reinterpret_cast<float*>(ctl + 384);     // [128] each
   float* pair_all = pair_m + 128;
   float* pair_txt = pair_all + 128;
-  // per-sample token counts and row offsets, read once (every role decodes every item; a trip to global memory
-  // per item would be a good part of a short item); samples beyond the cache are read from global memory
-  int* s_nvis = reinterpret_cast<int*>(pair_txt + 128);    // [XT_SAMPLE_CACHE]
-  int* s_row0 = s_nvis + XT_SAMPLE_CACHE;                   // [XT_SAMPLE_CACHE]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   // key tiles to visit: all tiles up to the last query's own key, or, when the caller supplies the row
   // log-sum-exp, only the tiles that hold prompt keys (J lies before the vision block, so it is visible)
   const int kt_lo = LSE ? a.text.begin / BK : 0;
   const int nkt_lse = a.text.end > a.text.begin ? (a.text.end - 1) / BK + 1 - kt_lo : 0;
-  struct Item { int h, b, t0, nq, s_first, nkt, n_seq, nsub, row0, bc; };   // nsub: halves of 64 keys the item visits;
-                                                                           // row0, bc: row offset and batch coordinate of the TMA loads
-  // item -> (query tile, head, sample).  The (sample, head) pairs are taken in groups of XT_HEAD_GROUP whose keys
-  // stay in L2 together; inside a group the list runs over the query tiles from the longest rows to the shortest,
-  // all pairs of the group for each, so that the work left for the last tickets is short.
-  auto decode = [&](int item, Item& it) -> bool {
-    const int n_hb = a.n_q_heads * a.batch, per_group = XT_HEAD_GROUP * a.n_qt;
-    const int grp = item / per_group, within = item - grp * per_group;
-    const int gsize = min(XT_HEAD_GROUP, n_hb - grp * XT_HEAD_GROUP);
-    const int hb = grp * XT_HEAD_GROUP + within % gsize, qt = a.n_qt - 1 - within / gsize;
-    it.h = hb % a.n_q_heads; it.b = hb / a.n_q_heads;
-    const int n = it.b < XT_SAMPLE_CACHE ? s_nvis[it.b] : (a.n_vis ? min(a.n_vis[it.b], a.cap_in) : a.cap_in);
-    it.t0 = qt * 128;
-    if (it.t0 >= n) return false;
-    it.nq = min(128, n - it.t0);
-    it.s_first = a.vis_begin + it.t0;
-    it.n_seq = a.vis_begin + n + a.n_text_after;
-    it.nsub = LSE ? 2 * nkt_lse : ((a.bidirectional ? it.n_seq : it.s_first + it.nq) - 1) / XT_SUB + 1;
-    it.nkt = (it.nsub + 1) / 2;
-    it.row0 = it.b < XT_SAMPLE_CACHE ? s_row0[it.b] : (a.seq_start ? a.seq_start[it.b] : 0);   // packed batch: one long
-                                                                                              // row axis, batch coordinate 0
-    it.bc = a.seq_start ? 0 : it.b;
-    return true;
-  };
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&q_full[i], 1); mbar_init(&q_empty[i], 1); }
@@ -213,60 +241,115 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
     for (int i = 0; i < 2; ++i) { mbar_init(&item_full[i], 1); mbar_init(&item_empty[i], 9); }
     mbar_init(pair_full, 4);
     mbar_init(pair_empty, 4);
+    mbar_init(clc_full, 1);
     *abort_flag = 0;
     *redo_mark = -1;
+    *redo_head = -1;
     fence_barrier_init();
+    prefetch_tensormap(&q_map);
+    prefetch_tensormap(&k_map);
   }
   if (warp == 1) { tmem_alloc(tmem_slot, XT_SBUF * BK); tmem_relinquish(); }
-  for (int i = threadIdx.x; i < min(a.batch, XT_SAMPLE_CACHE); i += blockDim.x) {
-    s_nvis[i] = a.n_vis ? min(a.n_vis[i], a.cap_in) : a.cap_in;
-    s_row0[i] = a.seq_start ? a.seq_start[i] : 0;
-  }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
+  grid_dependency_sync();                                  // from here on global memory is read and written
 
   if (warp == 0) {
     if (lane == 0) {
       // ---- scheduler + TMA producer
-      prefetch_tensormap(&q_map);
-      prefetch_tensormap(&k_map);
-      uint32_t kf = 0, n = 0, nq_loaded = 0;           // K tiles fetched / items published / Q tiles loaded
-      for (;;) {
+      struct Item { int h, b, t0, nq, n_seq, nsub, row0; };
+      // item -> (query tile, head, sample).  The (sample, head) pairs are taken in groups of XT_HEAD_GROUP whose
+      // keys stay in L2 together; inside a group the list runs over the query tiles from the longest rows to the
+      // shortest, all pairs of the group for each, so that the work left for the last items is short.
+      auto decode = [&](int item, Item& it) -> bool {
+        const int n_hb = a.n_q_heads * a.batch, per_group = XT_HEAD_GROUP * a.n_qt;
+        const int grp = item / per_group, within = item - grp * per_group;
+        const int gsize = min(XT_HEAD_GROUP, n_hb - grp * XT_HEAD_GROUP);
+        const int qi = within / gsize, hb = grp * XT_HEAD_GROUP + within - qi * gsize;
+        it.b = hb / a.n_q_heads; it.h = hb - it.b * a.n_q_heads;
+        const int n = a.n_vis ? min(a.n_vis[it.b], a.cap_in) : a.cap_in;
+        it.t0 = (a.n_qt - 1 - qi) * 128;
+        if (it.t0 >= n) return false;
+        it.nq = min(128, n - it.t0);
+        it.n_seq = a.vis_begin + n + a.n_text_after;
+        // halves of 64 keys the item visits
+        it.nsub = LSE ? 2 * nkt_lse : ((a.bidirectional ? it.n_seq : a.vis_begin + it.t0 + it.nq) - 1) / XT_SUB + 1;
+        it.row0 = a.seq_start ? a.seq_start[it.b] : 0;     // packed batch: one long row axis, batch coordinate 0
+        return true;
+      };
+      uint32_t kf = 0, n = 0, nq_loaded = 0, n_clc = 0;    // K tiles fetched / items published / Q tiles loaded / requests
+      auto publish = [&](int item, const Item& it, int safe) -> bool {
         const uint32_t slot = n & 1;
-        if (!mbar_wait(&item_empty[slot], ((n >> 1) & 1) ^ 1, abort_flag)) break;
-        // items of the LSE form are all alike: a fixed round-robin split balances them and saves the atomic's
-        // round trip, which would otherwise be a good part of such a short item
-        const unsigned int t = LSE ? blockIdx.x + n * gridDim.x
-                                   : atomicAdd(SAFE ? &a.sched->safe_ticket : &a.sched->ticket, 1u);
-        const int item = t < n_items ? (SAFE ? a.redo_list[t] : int(t)) : -1;
-        item_slot[slot] = item;
-        mbar_arrive(&item_full[slot]);                 // release: the slot is written before the arrival is seen
+        if (!mbar_wait(&item_empty[slot], ((n >> 1) & 1) ^ 1, abort_flag)) return false;
+        item_slot[2 * slot] = make_int4(item, it.h, it.b, it.t0 + safe);       // t0 is a multiple of 128
+        item_slot[2 * slot + 1] = make_int4(it.nq, it.n_seq, it.nsub, it.row0);
+        mbar_arrive(&item_full[slot]);                     // release: the slot is written before the arrival is seen
         ++n;
-        if (item < 0) break;
-        Item it;
-        if (!decode(item, it) || it.nkt == 0) continue;
+        return true;
+      };
+      bool asked = false;                                  // a request for another CTA's item is on its way
+      auto ask = [&]() {
+        if (LSE || asked) return;
+        mbar_expect_tx(clc_full, 16);
+        clc_try_cancel(clc_slot, clc_full);
+        asked = true;
+      };
+      auto feed = [&](const Item& it, bool last_asks) -> bool {    // the item's Q and K tiles
+        const int nkt = (it.nsub + 1) / 2;
+        if (nkt == 0) return true;
         // a Q buffer is free once every MMA of the item that used it last has completed
         const uint32_t qb = nq_loaded % QBUF, q_use = nq_loaded / QBUF;
-        if (q_use > 0 && !mbar_wait(&q_empty[qb], (q_use - 1) & 1, abort_flag)) break;
+        const int bc = a.seq_start ? 0 : it.b;
+        if (q_use > 0 && !mbar_wait(&q_empty[qb], (q_use - 1) & 1, abort_flag)) return false;
         mbar_expect_tx(&q_full[qb], TILE_BYTES);
 #pragma unroll
         for (int hf = 0; hf < HALVES; ++hf)
-          tma_load_4d(q_s + qb * TILE_BYTES + hf * 16384, &q_map, &q_full[qb], hf * 64, it.row0 + it.s_first, it.h, it.bc);
+          tma_load_4d(q_s + qb * TILE_BYTES + hf * 16384, &q_map, &q_full[qb], hf * 64, it.row0 + a.vis_begin + it.t0, it.h, bc);
         ++nq_loaded;
         const int hk = it.h / a.group;
-        bool ok = true;
-        for (int kt = 0; kt < it.nkt; ++kt, ++kf) {
+        for (int kt = 0; kt < nkt; ++kt, ++kf) {
           const uint32_t s = kf % KSTAGES;
-          if (!mbar_wait(&k_empty[s], ((kf / KSTAGES) & 1) ^ 1, abort_flag)) { ok = false; break; }
+          if (last_asks && kt == nkt - 1) ask();           // late, so that no CTA sits on an item others could start
+          if (!mbar_wait(&k_empty[s], ((kf / KSTAGES) & 1) ^ 1, abort_flag)) return false;
           mbar_expect_tx(&k_full[s], KT_BYTES);
 #pragma unroll
           for (int hf = 0; hf < HALVES; ++hf)
-            tma_load_4d(k_s + s * KT_BYTES + hf * KHALF_BYTES, &k_map, &k_full[s], hf * 64, it.row0 + (kt_lo + kt) * BK, hk, it.bc);
+            tma_load_4d(k_s + s * KT_BYTES + hf * KHALF_BYTES, &k_map, &k_full[s], hf * 64, it.row0 + (kt_lo + kt) * BK, hk, bc);
         }
-        if (!ok) break;
+        return true;
+      };
+      const int n_items = a.n_qt * a.n_q_heads * a.batch;
+      bool ok = true;
+      Item it;
+      for (int item = blockIdx.x; ok && item >= 0;) {
+        if (decode(item, it)) ok = publish(item, it, 0) && feed(it, true);
+        if (LSE) {
+          // items of the LSE form are all alike: a fixed round-robin split balances them
+          item = item + int(gridDim.x) < n_items ? item + int(gridDim.x) : -1;
+        } else {
+          ask();
+          ok = mbar_wait(clc_full, n_clc & 1, abort_flag) && ok;   // the answer is awaited even when the item failed
+          ++n_clc;
+          asked = false;
+          item = clc_canceled_cta(clc_slot);
+          fence_proxy_async();                             // the slot has been read before the next answer is written
+        }
       }
+      if (!LSE && ok) {
+        // all items handed out: once the softmax warps are done with the last two, the list of this CTA is complete
+        ok = mbar_wait(&item_empty[n & 1], ((n >> 1) & 1) ^ 1, abort_flag) &&
+             mbar_wait(&item_empty[(n + 1) & 1], (((n + 1) >> 1) & 1) ^ 1, abort_flag);
+        int item = ok ? *const_cast<volatile int*>(redo_head) : -1;
+        while (ok && item >= 0) {
+          const int next = __ldcg(a.redo_next + item);     // read before the item runs again
+          ok = decode(item, it) && publish(item, it, 1) && feed(it, false);
+          item = next;
+        }
+      }
+      it.h = it.b = it.t0 = it.nq = it.n_seq = it.nsub = it.row0 = 0;
+      if (ok) publish(-1, it, 0);
     }
   } else if (warp == 1) {
     if (lane == 0) {
@@ -284,17 +367,16 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
       for (;;) {
         const uint32_t slot = n & 1;
         if (!mbar_wait(&item_full[slot], (n >> 1) & 1, abort_flag)) break;
-        const int item = item_slot[slot];
+        const int item = item_slot[2 * slot].x, nsub = item_slot[2 * slot + 1].z, nkt = (nsub + 1) / 2;
         mbar_arrive(&item_empty[slot]);
         ++n;
         if (item < 0) break;
-        Item it;
-        if (!decode(item, it) || it.nkt == 0) continue;
+        if (nkt == 0) continue;
         const uint32_t qb = nq_used % QBUF;
         if (!mbar_wait(&q_full[qb], (nq_used / QBUF) & 1, abort_flag)) break;
         const uint64_t q_off = uint64_t(qb * (TILE_BYTES >> 4));
         bool ok = true;
-        for (int kt = 0; kt < it.nkt; ++kt, ++kc) {
+        for (int kt = 0; kt < nkt; ++kt, ++kc) {
           const uint32_t s = kc % KSTAGES, buf = kc % XT_SBUF;
           if (!mbar_wait(&s_empty[buf], ((kc / XT_SBUF) & 1) ^ 1, abort_flag) ||
               !mbar_wait(&k_full[s], (kc / KSTAGES) & 1, abort_flag)) { ok = false; break; }
@@ -302,7 +384,7 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
           const uint64_t stage_off = uint64_t(s * (KT_BYTES >> 4));     // the address field counts 16-byte units
           const uint32_t d_addr = tmem_base + buf * BK;
           // the last tile of an odd number of halves needs its first 64 keys only
-          const uint32_t idesc = (2 * kt + 2 > it.nsub) ? idesc_half : idesc_full;
+          const uint32_t idesc = (2 * kt + 2 > nsub) ? idesc_half : idesc_full;
 #pragma unroll
           for (int kk = 0; kk < DH / 16; ++kk) umma_bf16(d_addr, q_desc[kk] + q_off, k_desc[kk] + stage_off, idesc, kk > 0);
           umma_commit(&k_empty[s]);
@@ -327,125 +409,140 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
       const uint32_t slot = n & 1;
       const bool published = mbar_wait(&item_full[slot], (n >> 1) & 1, abort_flag);
       if (!__all_sync(0xffffffffu, published)) break;
-      const int item = item_slot[slot];
-      __syncwarp();                                     // every lane has read the slot
-      if (lane == 0) mbar_arrive(&item_empty[slot]);
+      const int4 i0 = item_slot[2 * slot], i1 = item_slot[2 * slot + 1];
       ++n;
+      const int item = i0.x, h = i0.y, b = i0.z, t0 = i0.w & ~1, nq = i1.x, nsub = i1.z, row0 = i1.w;
       if (item < 0) break;
-      Item it;
-      if (!decode(item, it)) continue;
-      const int h = it.h, b = it.b, nq = it.nq, s_first = it.s_first;
+      const bool safe = i0.w & 1;
+      const int s_first = a.vis_begin + t0;
+      // last key seen by the first row of this warp / by this thread's row
+      const int lim_lo = a.bidirectional ? i1.y - 1 : s_first + quad * 32;
+      const int lim_own = a.bidirectional ? i1.y - 1 : s_first + r;
       float m_run = -INFINITY, l_all = 0.f, l_txt = 0.f;
+      bool need_ref = !LSE;                             // some row of the warp has no reference yet
+      ExpRef er;
+      er.set(sc, 0.f);
       // the caller's normaliser of this row, in log2 units (fetched before the first wait: its latency hides there)
-      float l2 = 0.f;
-      if (LSE && r < nq) l2 = a.lse[size_t(b) * a.lse_bs + size_t(h) * a.lse_hs + it.row0 + s_first + r] * 1.4426950408889634f;
-      for (int kt = 0; kt < it.nkt; ++kt, ++kc) {
+      if (LSE) {
+        float l2 = 0.f;
+        if (r < nq) l2 = a.lse[size_t(b) * a.lse_bs + size_t(h) * a.lse_hs + row0 + s_first + r] * 1.4426950408889634f;
+        er.set(sc, l2);
+      }
+      const int nkt = (nsub + 1) / 2;
+      int kt = 0;
+      while (kt < nkt) {
+        if (!LSE && !need_ref) {
+          // The bulk: a run of whole tiles whose keys are visible to every row of the warp and all of which, or none of
+          // which, are prompt keys.  A loop of its own, without masks: two thirds and more of the logits pass here.
+          const int jt = kt * BK + cg * 32;             // first key of this thread's columns
+          const bool inside = a.text.n == 1 && jt >= a.text.begin;
+          const int end_key = min(inside && jt < a.text.end ? a.text.end : 0x7fffffff, lim_lo + 1);
+          const bool uniform = jt >= a.text.end || (inside && jt + XT_SUB + 32 <= a.text.end);
+          const int run_end = uniform ? min((end_key - cg * 32 - XT_SUB - 32 + BK) / BK, nsub / 2) : 0;
+          if (kt < run_end) {
+            const bool count = jt < a.text.end;
+            f32x2 part[2] = {0ull, 0ull};
+            do {
+              const uint32_t buf = kc % XT_SBUF;
+              const bool landed = mbar_wait(&s_full[buf], (kc / XT_SBUF) & 1, abort_flag);
+              if (!__all_sync(0xffffffffu, landed)) { alive = false; break; }   // the TMEM loads below are warp-wide
+              tc_fence_after();
+              float va[32], vb[32];
+              tmem_ld32(lane_addr + buf * BK, va);
+              tmem_ld_wait();
+              exp_add32(va, er, part);
+              tmem_ld32(lane_addr + buf * BK + XT_SUB, vb);
+              tmem_ld_wait();
+              tc_fence_before();
+              __syncwarp();
+              if (lane == 0) mbar_arrive(&s_empty[buf]);   // the accumulator is in registers: hand it back
+              exp_add32(vb, er, part);
+              ++kc;
+            } while (++kt < run_end);
+            if (!alive) break;
+            const float s = sum_pairs(part);
+            l_all += s;
+            if (count) l_txt += s;
+            continue;
+          }
+        }
         const uint32_t buf = kc % XT_SBUF;
         const bool landed = mbar_wait(&s_full[buf], (kc / XT_SBUF) & 1, abort_flag);
-        if (!__all_sync(0xffffffffu, landed)) { alive = false; break; }   // the TMEM loads below are warp-wide
+        if (!__all_sync(0xffffffffu, landed)) { alive = false; break; }
         tc_fence_after();
-        const int n_half = min(2, it.nsub - 2 * kt);     // halves of this tile the item needs
+        const int n_half = min(2, nsub - 2 * kt);       // halves of this tile the item needs
         for (int half = 0; half < n_half; ++half) {
           const int j0 = (kt_lo + kt) * BK + half * XT_SUB + cg * 32;      // first key of this thread's 32 columns
           float v[32];
           tmem_ld32(lane_addr + buf * BK + half * XT_SUB, v);
           tmem_ld_wait();
-          if (half == n_half - 1) {                       // the accumulator is in registers: hand it back
+          if (half == n_half - 1) {
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(&s_empty[buf]);
           }
-
-          if (LSE) {                                      // normaliser known: only the prompt columns count
-            const unsigned int tm = (unsigned int)a.text.mask64(j0);
-            l_all = 1.f;
-            if (tm == 0xffffffffu) {                      // all 32 keys are prompt keys: no tests, four chains
-              float part[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-              for (int i = 0; i < 32; ++i) part[i & 3] += ex2(fmaf(v[i], sc, -l2));
-              l_txt += (part[0] + part[1]) + (part[2] + part[3]);
-            } else if (tm != 0u) {
-              float st = 0.f;
+          // prompt keys among the 32 (warp-uniform)
+          const unsigned int tm = j0 < a.text.end && j0 + 32 > a.text.begin ? a.text.mask32(j0) : 0u;
+          if (LSE && tm == 0u) continue;
+          const int lim = lim_own - j0;                 // last visible column of this row
+          if (!LSE) {
+            if (j0 > lim_lo + (a.bidirectional ? 0 : 31)) continue;         // no row of this warp sees any of these keys
+            if (j0 + 31 > lim_lo) {                     // some row does not: the diagonal, or the end of the sample
 #pragma unroll
               for (int i = 0; i < 32; ++i)
-                if ((tm >> i) & 1u) st += ex2(fmaf(v[i], sc, -l2));
-              l_txt += st;
+                if (i > lim) v[i] = -INFINITY;
             }
-            continue;
-          }
-          const bool in_j = j0 < a.text.end && j0 + 32 > a.text.begin;     // the columns reach into the prompt set J
-          // some row does not see all of these keys: the diagonal, or the end of the sample
-          const bool edge = j0 + 31 > (a.bidirectional ? it.n_seq - 1 : s_first);
-          int lim_max = 32;                                // columns at least one row of this warp sees
-          if (edge) {
-            const int lim = (a.bidirectional ? it.n_seq - 1 : s_first + r) - j0;   // last visible column of this row
-            lim_max = __reduce_max_sync(0xffffffffu, lim);
-            if (lim_max < 0) continue;                     // no row of this warp sees any of these keys
+            if (need_ref) {
+              // reference of the thread: maximum of the first 32 columns of its own in which it sees a key (the
+              // first 64 keys of the row, unless the row is among the first 32 of a sequence), of every half when
+              // safe.  While some row of the warp has no reference yet the others update theirs, which is exact.
+              float mx[4] = {v[0], v[1], v[2], v[3]};
 #pragma unroll
-            for (int i = 0; i < 32; ++i)
-              if (i > lim) v[i] = -INFINITY;
-          }
-          if (SAFE || __any_sync(0xffffffffu, m_run == -INFINITY)) {
-            // reference of the thread: maximum of the first 32 columns of its own in which it sees a key (the
-            // first 64 keys of the row, unless the row is among the first 32 of a sequence), of every half when
-            // SAFE.  While some row of the warp has no reference yet the others update theirs, which is exact.
-            float mx[4];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-              mx[j] = v[j * 8];
-#pragma unroll
-              for (int i = 1; i < 8; ++i) mx[j] = fmaxf(mx[j], v[j * 8 + i]);
-            }
-            const float m_new = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), m_run);
-            if (m_new > -INFINITY) {                        // (a thread whose 32 columns are all masked keeps none)
-              const float resc = ex2((m_run - m_new) * sc); // 0 on the first half
-              l_all *= resc;
-              l_txt *= resc;
-              m_run = m_new;
+              for (int i = 4; i < 32; ++i) mx[i & 3] = fmaxf(mx[i & 3], v[i]);
+              const float m_new = fmaxf(fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])), m_run);
+              if (m_new > -INFINITY) {                  // (a thread whose 32 columns are all masked keeps none)
+                const float resc = ex2((m_run - m_new) * sc);   // 0 on the first half
+                l_all *= resc;
+                l_txt *= resc;
+                m_run = m_new;
+                er.set(sc, m_run * sc);
+              }
+              need_ref = safe || __any_sync(0xffffffffu, m_run == -INFINITY);
             }
           }
-          if (m_run == -INFINITY) continue;                // this thread has not seen a key yet
-          const float ms = m_run * sc;
-          if (!edge && !in_j) {
-            // the bulk: every eighth exponential on the FMA pipe
-            float part[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-            for (int i = 0; i < 32; ++i) {
-              const float x = fmaf(v[i], sc, -ms);
-              part[i & 3] += (i & 7) == 7 ? ex2_fma(x) : ex2(x);
-            }
-            l_all += (part[0] + part[1]) + (part[2] + part[3]);
-          } else {
-            const unsigned int tm = in_j ? (unsigned int)a.text.mask64(j0) : 0u;
+          if (tm == 0u || tm == 0xffffffffu) {
+            f32x2 part[2] = {0ull, 0ull};
+            exp_add32(v, er, part);
+            const float s = sum_pairs(part);
+            l_all += s;
+            if (tm) l_txt += s;
+          } else {                                      // the prompt set begins or ends among these keys
             float sa = 0.f, st = 0.f;
 #pragma unroll
-            for (int blk = 0; blk < 4; ++blk)
-              if (blk * 8 <= lim_max) {                     // warp-uniform: masked blocks cost no exponentials
-                float pa = 0.f, pt = 0.f;
-#pragma unroll
-                for (int i = 0; i < 8; ++i) {
-                  const float p = ex2(fmaf(v[blk * 8 + i], sc, -ms));   // exp2(-inf) = 0 on masked columns
-                  pa += p;
-                  if ((tm >> (blk * 8 + i)) & 1u) pt += p;
-                }
-                sa += pa;
-                st += pt;
-              }
+            for (int i = 0; i < 16; ++i) {
+              float x0, x1;
+              unpack2(fma2(pack2(v[2 * i], v[2 * i + 1]), er.sc2, er.nms2), x0, x1);
+              const float p0 = ex2(x0), p1 = ex2(x1);   // exp2(-inf) = 0 on masked columns
+              sa += p0 + p1;
+              if ((tm >> (2 * i)) & 1u) st += p0;
+              if ((tm >> (2 * i + 1)) & 1u) st += p1;
+            }
             l_all += sa;
             l_txt += st;
           }
         }  // halves
+        ++kt;
+        ++kc;
       }  // key tiles
       // ---- the two threads of a row meet: the upper column group hands its reference and sums over.  Every warp
       //      that entered the item takes part, also after a failed wait (the flag is raised, nothing is stored).
       if (cg == 1) {
         const bool free_again = np == 0 || mbar_wait(pair_empty, (np - 1) & 1, abort_flag);
         if (!__all_sync(0xffffffffu, free_again)) alive = false;
-        pair_m[r] = m_run; pair_all[r] = l_all; pair_txt[r] = l_txt;
+        if (alive) { pair_m[r] = m_run; pair_all[r] = l_all; pair_txt[r] = l_txt; }
         __syncwarp();
-        if (lane == 0) mbar_arrive(pair_full);
+        if (lane == 0) { mbar_arrive(pair_full); mbar_arrive(&item_empty[slot]); }
         ++np;
-        if (!alive) break;
         continue;
       }
       {
@@ -454,9 +551,14 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
         ++np;
         if (!alive) break;
         if (!LSE) {
-          const float m_o = pair_m[r], m_new = fmaxf(m_run, m_o);
+          const float m_o = pair_m[r], all_o = pair_all[r], m_new = fmaxf(m_run, m_o);
+          // a sum at the end of the fp32 range means some logit lay more than 88 above the reference: the item goes on
+          // the CTA's list, once (before the exchange buffers are handed back: no warp can be an item ahead here)
+          const bool bad = r < nq && !safe && !(l_all <= 3.0e38f && all_o <= 3.0e38f);
+          if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicExch(redo_mark, item) != item)
+            a.redo_next[item] = atomicExch(redo_head, item);
           const float f_own = ex2((m_run - m_new) * sc), f_o = m_o > -INFINITY ? ex2((m_o - m_new) * sc) : 0.f;
-          l_all = fmaf(l_all, f_own, pair_all[r] * f_o);
+          l_all = fmaf(l_all, f_own, all_o * f_o);
           l_txt = fmaf(l_txt, f_own, pair_txt[r] * f_o);
           m_run = m_new;
         } else {
@@ -465,19 +567,14 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
         __syncwarp();
         if (lane == 0) mbar_arrive(pair_empty);             // the exchange buffers are free for the next item
       }
-      if (!LSE && !SAFE) {
-        // a sum that is not a finite number means some logit lay more than 88 above the reference: the item
-        // goes on the list of the second launch (once per CTA)
-        const bool bad = r < nq && !(l_all <= 3.0e38f);
-        if (__any_sync(0xffffffffu, bad) && lane == 0 && atomicExch(redo_mark, item) != item)
-          a.redo_list[atomicAdd(&a.sched->n_redo, 1u)] = item;
-      }
       if (r < nq && !*abort_flag) {
-        a.xi_h[(size_t(b) * a.n_q_heads + h) * a.cap_in + it.t0 + r] = LSE ? l_txt : l_txt / l_all;
+        a.xi_h[(size_t(b) * a.n_q_heads + h) * a.cap_in + t0 + r] = LSE ? l_txt : l_txt / l_all;
         if (!LSE && a.lse_out)
-          a.lse_out[size_t(b) * a.lse_out_bs + size_t(h) * a.lse_out_hs + it.row0 + s_first + r] =
+          a.lse_out[size_t(b) * a.lse_out_bs + size_t(h) * a.lse_out_hs + row0 + s_first + r] =
               fmaf(m_run, sc, log2f(l_all)) * 0.6931471805599453f;
       }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&item_empty[slot]);
     }
   }
   tc_fence_before();
@@ -513,29 +610,22 @@ cudaError_t launch_xi_tc(const LayerLaunch& L) {
   x.n_q_heads = L.n_q_heads; x.group = L.n_q_heads / L.n_kv_heads;
   x.scale2 = 1.4426950408889634f / sqrtf((float)L.head_dim);
   x.batch = L.batch; x.n_qt = (L.ws.cap_in + 127) / 128;
-  x.sched = reinterpret_cast<XiSched*>(L.ws.xi_sched); x.redo_list = L.ws.xi_redo;
+  x.redo_next = L.ws.xi_redo;
   const long long n_items = (long long)x.n_qt * L.n_q_heads * L.batch;
   if (n_items > 0x7fffffffLL) return cudaErrorInvalidValue;
-  // As many CTAs as stay resident (two per SM) draw work items from a ticket counter; with the caller's
-  // log-sum-exp an item is one or two key tiles, otherwise up to the whole row.
-  const dim3 grid((unsigned)std::min<long long>(n_items, XT_CTAS * sm_count()));
-  // Q tiles + K ring (LSE: two Q tiles, one K stage; otherwise one Q tile, XT_STAGES K stages) + barriers + exchange
+  // One CTA per item, taken over by the resident ones; with the caller's log-sum-exp an item is one or two key tiles
+  // and as many CTAs as stay resident walk them round-robin.
+  const dim3 grid((unsigned)(x.lse ? std::min<long long>(n_items, XT_CTAS * sm_count()) : n_items));
+  // Q tiles + K ring (LSE: two Q tiles, one K stage; otherwise one Q tile, XT_STAGES K stages) + control block + exchange
   const size_t smem = size_t(L.head_dim / 64) * (x.lse ? 2 * 16384 + XT_KEY_TILE * 128
-                                                        : 16384 + size_t(XT_STAGES) * XT_KEY_TILE * 128) + 1024 + 256 + 1536 + 2 * XT_SAMPLE_CACHE * sizeof(int);
-  cudaError_t e = cudaMemsetAsync(x.sched, 0, sizeof(XiSched), L.stream);      // tickets and list length start at 0
-  if (e != cudaSuccess) return e;
-  auto launch = [&](auto kernel, dim3 g) -> cudaError_t {
+                                                        : 16384 + size_t(XT_STAGES) * XT_KEY_TILE * 128) + 1024 + 384 + 1536;
+  auto launch = [&](auto kernel) -> cudaError_t {
     const cudaError_t rc = ensure_dynamic_smem(kernel, (int)smem);
     if (rc != cudaSuccess) return rc;
-    return launch_kernel(kernel, g, XT_THREADS, smem, L.stream, 1, qm, km, x);
+    return launch_kernel(kernel, grid, XT_THREADS, smem, L.stream, 1, qm, km, x);
   };
-  if (x.lse) return L.head_dim == 128 ? launch(xi_tc_kernel<128, true, false>, grid) : launch(xi_tc_kernel<64, true, false>, grid);
-  e = L.head_dim == 128 ? launch(xi_tc_kernel<128, false, false>, grid) : launch(xi_tc_kernel<64, false, false>, grid);
-  if (e != cudaSuccess) return e;
-  // second launch: the items whose sums left the fp32 range, with a running maximum (returns at once when the
-  // list is empty; one CTA per SM is plenty for what is an exception)
-  const dim3 grid2((unsigned)std::min<long long>(n_items, sm_count()));
-  return L.head_dim == 128 ? launch(xi_tc_kernel<128, false, true>, grid2) : launch(xi_tc_kernel<64, false, true>, grid2);
+  if (x.lse) return L.head_dim == 128 ? launch(xi_tc_kernel<128, true>) : launch(xi_tc_kernel<64, true>);
+  return L.head_dim == 128 ? launch(xi_tc_kernel<128, false>) : launch(xi_tc_kernel<64, false>);
 }
 
 // ======================================================================================================

@@ -393,6 +393,26 @@ def test_lse_mode_persistent_ctas_walk_several_items(head_dim):
     H.run_schedule(wl, xi_mode="lse", text_ranges=[(2, 60), (70, 129)])
 
 
+@pytest.mark.parametrize("head_dim,text_ranges", [(64, None), (128, [(32, 96)]), (128, [(0, 64), (96, 129)])])
+def test_xi_items_taken_over_and_repeated(head_dim, text_ranges):
+    # 4 samples x 8 heads x 16 query tiles = 512 items for the 2 CTAs per SM that are resident: CTAs take over the
+    # items of others; one late key of a KV head is scaled so that a quarter of the items leave the fp32 range and are
+    # repeated from the CTAs' own lists; prompt sets that begin and end on and off the 32-key blocks of a thread
+    wl = S.Workload(name="xiwalk", config_id=134, batch=4, tiles=((64, 32),), n_text=130, hidden=64, n_q_heads=8,
+                    n_kv_heads=4, head_dim=head_dim, n_layers=16, layers=(3,), windows=(8,), keep=(0.5,))
+    assert 16 * wl.n_q_heads * wl.batch > 3 * _sm_count()
+    plan = H.make_plan(wl)
+    inp = H.prepare_stage(wl, 0)
+    late = wl.n_text + 700
+    inp["k"][:, 1, late] *= 256.0                              # a power of two: still bf16 values
+    gpu = H.gpu_stage(plan, wl, 0, inp, want_lse=True, text_ranges=text_ranges)
+    del gpu["k_out"], gpu["v_out"]      # the scaled key row is outside the value range the bf16 K/V tolerance is meant for
+    sub = {k: (v[[2]] if isinstance(v, np.ndarray) and v.shape[:1] == (4,) else v) for k, v in inp.items()}
+    H.compare_stage(wl, 0, inp, H.oracle_stage(wl, 0, sub, text_ranges=text_ranges), gpu, samples=[2])
+    H.check_lse_out(inp, gpu, wl.n_q_heads, wl.n_kv_heads, [2], atol=4e-2)
+    plan.close()
+
+
 def test_cfg2_lse_mode_full_size_sampled():
     # the benchmark shape in ATTN_LSE mode (5888 work items walked by 3 CTAs per SM), bench.py's streams; the
     # log-sum-exp input comes from plain torch ops, the oracle derives xi from Q and K alone
