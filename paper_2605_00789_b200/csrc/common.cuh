@@ -178,14 +178,19 @@ __device__ __forceinline__ float pair_score(int metric, float g, float na, float
   return metric == LIGHTKV_FD_L2 ? sqrtf(sq) : sq;
 }
 
-// Programmatic dependent launch.  Every kernel of the library is launched with programmatic stream
-// serialization and begins with this call: it lets the next kernel of the stream become resident, then
-// waits until the kernel before this one has completed and its writes are visible.  So a kernel's launch
-// latency hides behind its predecessor, and nothing is read or written before the predecessor is done.
-// Launched without the attribute, both instructions do nothing.
+// Programmatic dependent launch.  Every kernel of the library is launched with programmatic stream serialization:
+// it may start once every CTA of the kernel before it has called grid_launch_dependents() or exited, and
+// grid_dependency_wait() returns when that kernel has completed and its writes are visible.  Every kernel waits
+// before it exits, so a kernel's completion implies that of all before it.  Most wait before they touch global memory
+// (grid_dependency_sync: a launch's latency then hides behind its predecessor).  Two use the order further: the window
+// build lets the next kernel start only after its own wait, so everything before the call is complete when that
+// kernel starts; and the xi kernel, which reads nothing the window build or FD write, waits only at its end, i.e. runs
+// beside them.  Launched without the attribute, the instructions do nothing.
+__device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_sync() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  asm volatile("griddepcontrol.wait;" ::: "memory");
+  grid_launch_dependents();
+  grid_dependency_wait();
 }
 
 }  // namespace lkv

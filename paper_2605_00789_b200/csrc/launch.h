@@ -93,6 +93,7 @@ cudaError_t launch_kv_compact(const KvLaunch& K);
 bool tc_fd_supported(int hidden);
 bool tc_xi_supported(int head_dim);
 cudaError_t launch_fd_tc(const LayerLaunch& L);
-cudaError_t launch_xi_tc(const LayerLaunch& L);
+// wait_first: the stream's last kernel is not the window build or FD of the same call
+cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first);
 
 }  // namespace lkv

@@ -339,16 +339,18 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
     ok = ok && launch_window_build(La) == cudaSuccess;
     ok = ok && launch_fd(La) == cudaSuccess;
     const bool joined = cudaEventRecord(join, aux) == cudaSuccess;
-    ok = ok && (tc_xi ? launch_xi_tc(L) : launch_xi_simt(L)) == cudaSuccess;
+    ok = ok && (tc_xi ? launch_xi_tc(L, true) : launch_xi_simt(L)) == cudaSuccess;
     const bool waited = joined && cudaStreamWaitEvent(L.stream, join, 0) == cudaSuccess;
     if (!ok || !waited) return LIGHTKV_ERR_CUDA;
   } else {
+    // FD in front of xi, which runs beside it and the window build (programmatic launch order, see
+    // grid_dependency_sync); for per-kernel timing the two keep the order of the trace events
+    auto launch_xi = [&]() { return !attn ? cudaSuccess : tc_xi ? launch_xi_tc(L, false) : launch_xi_simt(L); };
     if (mark(0) != cudaSuccess) return LIGHTKV_ERR_CUDA;
     if (launch_window_build(L) != cudaSuccess || mark(1) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-    if (attn && (tc_xi ? launch_xi_tc(L) : launch_xi_simt(L)) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-    if (mark(2) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-    if (launch_fd(L) != cudaSuccess || mark(3) != cudaSuccess)
-      return LIGHTKV_ERR_CUDA;
+    if (!ev && launch_fd(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+    if (launch_xi() != cudaSuccess || mark(2) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+    if (ev && (launch_fd(L) != cudaSuccess || mark(3) != cudaSuccess)) return LIGHTKV_ERR_CUDA;
   }
   if (launch_select_map(L) != cudaSuccess || mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (a->map_event && cudaEventRecord(static_cast<cudaEvent_t>(a->map_event), L.stream) != cudaSuccess)

@@ -24,7 +24,8 @@ __device__ inline void set_status(uint32_t* status, uint32_t bit) {
 __global__ void __launch_bounds__(1024)
 window_build_kernel(Geometry g, const int* __restrict__ pos_all, const int* __restrict__ n_vis,
                     Workspace ws, uint32_t* status) {
-  grid_dependency_sync();
+  grid_dependency_wait();
+  grid_launch_dependents();                    // in this order: see grid_dependency_sync
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nW = g.n_windows;
   uint16_t* cnt = reinterpret_cast<uint16_t*>(smem_raw);                        // [32][nW]

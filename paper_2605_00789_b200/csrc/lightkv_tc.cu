@@ -154,6 +154,7 @@ struct XiTcArgs {
   int cap_in, vis_begin, n_q_heads, group;
   int batch, n_qt;                   // samples, query tiles of 128 rows per (sample, head)
   float scale2;                      // log2(e) / sqrt(dh)
+  int wait_first;                    // 1: the window build is not the kernel in front (see below)
   int* redo_next;                    // [n_qt * H * B] links of the CTAs' lists of items whose sums left the fp32 range
 };
 
@@ -254,7 +255,10 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem_base = *tmem_slot;
-  grid_dependency_sync();                                  // from here on global memory is read and written
+  // Behind the window build and FD of the same call everything this kernel reads is complete, and nothing reads what
+  // it writes before it has completed: it runs beside them and waits for them at its end (grid_dependency_sync).
+  grid_launch_dependents();
+  if (a.wait_first) grid_dependency_wait();
 
   if (warp == 0) {
     if (lane == 0) {
@@ -584,13 +588,14 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
     tmem_dealloc(tmem_base, XT_SBUF * BK);
   }
   if (threadIdx.x == 0 && *abort_flag && a.status) atomicOr(a.status, LIGHTKV_STATUS_TIMEOUT);
+  grid_dependency_wait();
 }
 
 bool tc_xi_supported(int head_dim) { return head_dim == 64 || head_dim == 128; }
 
 static int sm_count();
 
-cudaError_t launch_xi_tc(const LayerLaunch& L) {
+cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first) {
   const lightkv_layer_args_t* a = L.a;
   const int rows = a->seq_rows > 0 ? a->seq_rows : a->vis_begin + L.ws.cap_in + a->n_text_after;
   CUtensorMap qm, km;
@@ -610,7 +615,7 @@ cudaError_t launch_xi_tc(const LayerLaunch& L) {
   x.n_q_heads = L.n_q_heads; x.group = L.n_q_heads / L.n_kv_heads;
   x.scale2 = 1.4426950408889634f / sqrtf((float)L.head_dim);
   x.batch = L.batch; x.n_qt = (L.ws.cap_in + 127) / 128;
-  x.redo_next = L.ws.xi_redo;
+  x.redo_next = L.ws.xi_redo; x.wait_first = wait_first ? 1 : 0;
   const long long n_items = (long long)x.n_qt * L.n_q_heads * L.batch;
   if (n_items > 0x7fffffffLL) return cudaErrorInvalidValue;
   // One CTA per item, taken over by the resident ones; with the caller's log-sum-exp an item is one or two key tiles
