@@ -53,8 +53,10 @@ struct Workspace {
   FdTiling* fd_tiling;        // [B]         how the tensor-core FD kernel cuts this sample into tiles
   float* xi_h;     // [B, H, cap_in]      per-head attention mass on the prompt (ATTN modes)
   float* xi;       // [B, cap_in]
-  int* partner;    // [B, cap_in]         token an A token is merged into, -1 = survives
-  int* slot;       // [B, cap_in]         output slot of surviving tokens
+  int* partner;    // [B, cap_in]         token a source is merged into; negative: survives (-2: a source that was not
+                   //                     selected, where the streaming FD kernel wrote it)
+  int* slot;       // [B, cap_in]         output slot of surviving tokens; from the streaming FD kernel: a merged
+                   //                     token's rank among its partner's, or the number of tokens merged into this one
   int* a_partner;  // [B, cap_a]          per A entry: token it is merged into, -1 = survives
   int* xi_redo;    // [ceil(cap_in / 128) * H * B]  links between the work items of the tensor-core xi kernel that a
                    //                               CTA has to repeat with a running maximum

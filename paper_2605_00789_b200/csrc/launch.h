@@ -36,6 +36,8 @@ struct LayerLaunch {
   int dtype, xi_mode, divergence;
   double keep;
   int fd_side;                       // estimate of the larger side (A or B nodes) of a window: picks the FD kernel
+  int max_cell;                      // grid positions of the largest window
+  int n_grid;                        // ... of all tiles
   int fd_tiles;                      // estimate of FdTiling::n_tiles per sample (launch shape of the tensor-core FD kernel)
   Geometry geo;
   Workspace ws;
@@ -72,9 +74,13 @@ inline cudaError_t ensure_dynamic_smem(void (*kernel)(P...), int bytes) {
 cudaError_t launch_window_build(const LayerLaunch& L);
 // FD + best partner per A node (Step 2), fp32 FMA path
 cudaError_t launch_fd_simt(const LayerLaunch& L);
-// FD for bf16 windows of at most 40 nodes a side, rows straight from global memory into mma.sync fragments
-bool fd_stream_supported(int fd_side);
+// windows, FD and selection for bf16 windows of at most 40 nodes a side (Steps 1, 2 and 4): leaves every token's partner
+// and its place for launch_map
+bool fd_stream_supported(int fd_side, int max_cell, int cap_in);
 cudaError_t launch_fd_stream(const LayerLaunch& L);
+// head sum of xi, merge map, weights from the partners (Steps 4, 5); at most kMapMaxTokens per sample
+constexpr int kMapMaxTokens = 16384;
+cudaError_t launch_map(const LayerLaunch& L);
 // xi per head (Eq. "attention-factor"), fp32 FMA path; handles ATTN_FULL and ATTN_LSE
 cudaError_t launch_xi_simt(const LayerLaunch& L);
 // head sum of xi, ranking, merge map, weights (Steps 2-5)

@@ -17,6 +17,7 @@ struct StagePlan {
   bool exact;      // cap_in is the exact count (schedule so far is data independent)
   bool exact_out;  // cap_out too
   bool use_tc;
+  int max_cell;    // grid positions of the largest window
   int fd_side;     // larger side (A or B nodes) of a typical window: picks the FD kernel
   int fd_tiles;    // estimate of the tiles per sample of the tensor-core FD kernel (sizes its launch)
   Geometry geo;
@@ -168,6 +169,8 @@ int lightkv_plan(const lightkv_config_t* c, lightkv_plan_t** out) {
         delete p;
         return LIGHTKV_ERR_UNSUPPORTED;
       }
+    for (int t = 0; t < c->n_tiles; ++t)            // balanced cells: at most ceil(rows/w) x ceil(cols/w) positions
+      sp.max_cell = std::max(sp.max_cell, ((g.rows[t] + sp.w - 1) / sp.w) * ((g.cols[t] + sp.w - 1) / sp.w));
     sp.n_windows = g.n_windows;
     sp.cap_in = cap;
     sp.exact = exact;
@@ -202,13 +205,9 @@ int lightkv_plan(const lightkv_config_t* c, lightkv_plan_t** out) {
       sp.cap_b = g.src_par ? (sp.cap_in + sp.n_windows) / 2 : sp.cap_in / 2;
     }
     if (!sp.exact) {  // counts depend on the data: a window holds at most the tokens of its grid cell
-                      // (balanced cells: ceil(rows/w) x ceil(cols/w))
-      int cell = 0;
-      for (int t = 0; t < c->n_tiles; ++t)
-        cell = std::max(cell, ((g.rows[t] + sp.w - 1) / sp.w) * ((g.cols[t] + sp.w - 1) / sp.w));
-      sp.fd_tiles = fd_tile_count(g.n_windows, (std::min(cell, sp.cap_in) + 1) / 2, c->batch);
+      sp.fd_tiles = fd_tile_count(g.n_windows, (std::min(sp.max_cell, sp.cap_in) + 1) / 2, c->batch);
       // the tokens still alive are spread over the cells about evenly (the kernels walk larger windows in blocks)
-      sp.fd_side = (int)(((long long)cell * sp.cap_in / p->n_vis0 + 2) / 2);
+      sp.fd_side = (int)(((long long)sp.max_cell * sp.cap_in / p->n_vis0 + 2) / 2);
     }
     if (!exact) {   // data-dependent from here on: every window keeps at most ceil(keep n_w) tokens
       long long bound = (long long)ceil(sp.keep * sp.cap_in) + sp.n_windows;
@@ -314,18 +313,20 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
   L.batch = c.batch; L.hidden = c.hidden; L.n_q_heads = c.n_q_heads; L.n_kv_heads = c.n_kv_heads;
   L.head_dim = c.head_dim; L.dtype = c.dtype; L.xi_mode = c.xi_mode; L.divergence = c.divergence;
   L.keep = s.keep; L.geo = s.geo;
-  L.fd_tiles = s.fd_tiles; L.fd_side = s.fd_side;
+  L.fd_tiles = s.fd_tiles; L.fd_side = s.fd_side; L.max_cell = s.max_cell; L.n_grid = p->n_vis0;
   L.ws = bind_workspace(s, a->workspace); L.text = text; L.a = a; L.stream = static_cast<cudaStream_t>(a->stream);
 
   cudaEvent_t* ev = reinterpret_cast<cudaEvent_t*>(a->trace_events);
   auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], L.stream) : cudaSuccess; };
   const bool tc_xi = s.use_tc && attn && tc_xi_supported(c.head_dim);
   const bool tc_fd = s.use_tc && tc_fd_supported(c.hidden);
+  // Small windows: one kernel finds the windows, scores and selects, and the map kernel finishes (`streaming`; it
+  // addresses a sample's rows by 32-bit offsets of 16-byte units).  Otherwise window lists, a tiled FD kernel, selection.
+  const bool streaming = tc_fd && fd_stream_supported(s.fd_side, s.max_cell, s.cap_in) &&
+                         (long long)s.cap_in * a->hidden_row_stride / 8 < 0xffffffffll;
+  auto launch_windows = [&](const LayerLaunch& l) { return streaming ? cudaSuccess : launch_window_build(l); };
   auto launch_fd = [&](const LayerLaunch& l) {
-    if (!tc_fd) return launch_fd_simt(l);
-    // the streaming kernel addresses a sample's rows by 32-bit offsets of 16-byte units
-    const bool near = (long long)s.cap_in * a->hidden_row_stride / 8 < 0xffffffffll;
-    return near && fd_stream_supported(s.fd_side) ? launch_fd_stream(l) : launch_fd_tc(l);
+    return streaming ? launch_fd_stream(l) : tc_fd ? launch_fd_tc(l) : launch_fd_simt(l);
   };
   cudaStream_t aux = (a->aux_stream && attn && !ev) ? static_cast<cudaStream_t>(a->aux_stream) : nullptr;
   if (aux) {
@@ -336,7 +337,7 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
     La.stream = aux;
     if (cudaEventRecord(fork, L.stream) != cudaSuccess) return LIGHTKV_ERR_CUDA;
     bool ok = cudaStreamWaitEvent(aux, fork, 0) == cudaSuccess;
-    ok = ok && launch_window_build(La) == cudaSuccess;
+    ok = ok && launch_windows(La) == cudaSuccess;
     ok = ok && launch_fd(La) == cudaSuccess;
     const bool joined = cudaEventRecord(join, aux) == cudaSuccess;
     ok = ok && (tc_xi ? launch_xi_tc(L, true) : launch_xi_simt(L)) == cudaSuccess;
@@ -345,14 +346,14 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
   } else {
     // FD in front of xi, which runs beside it and the window build (programmatic launch order, see
     // grid_dependency_sync); for per-kernel timing the two keep the order of the trace events
-    auto launch_xi = [&]() { return !attn ? cudaSuccess : tc_xi ? launch_xi_tc(L, false) : launch_xi_simt(L); };
+    auto launch_xi = [&](bool first) { return !attn ? cudaSuccess : tc_xi ? launch_xi_tc(L, first) : launch_xi_simt(L); };
     if (mark(0) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-    if (launch_window_build(L) != cudaSuccess || mark(1) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+    if (launch_windows(L) != cudaSuccess || mark(1) != cudaSuccess) return LIGHTKV_ERR_CUDA;
     if (!ev && launch_fd(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-    if (launch_xi() != cudaSuccess || mark(2) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+    if (launch_xi(ev != nullptr) != cudaSuccess || mark(2) != cudaSuccess) return LIGHTKV_ERR_CUDA;
     if (ev && (launch_fd(L) != cudaSuccess || mark(3) != cudaSuccess)) return LIGHTKV_ERR_CUDA;
   }
-  if (launch_select_map(L) != cudaSuccess || mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+  if ((streaming ? launch_map(L) : launch_select_map(L)) != cudaSuccess || mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (a->map_event && cudaEventRecord(static_cast<cudaEvent_t>(a->map_event), L.stream) != cudaSuccess)
     return LIGHTKV_ERR_CUDA;
   if (launch_merge_rows(L) != cudaSuccess || mark(5) != cudaSuccess) return LIGHTKV_ERR_CUDA;

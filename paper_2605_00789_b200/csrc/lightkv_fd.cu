@@ -19,6 +19,8 @@ namespace lkv {
 // accumulate from the same registers (exact products, fp32 sums).  Partial inner products of the warps meet in
 // shared memory in warp order, then a warp per source row takes the minimum over the destinations (ties: lowest
 // index).  A window with more nodes than the template holds is walked in blocks of 8 * O by 8 * O.
+// Since the CTA has its whole window, it also finds the window's tokens (from the positions; no list has to be built
+// before) and makes the selection of Steps 2 and 4; what is left for the map kernel is one prefix sum per sample.
 // A lane's pieces wait in shared memory (cp.async, a ring of S chunks per warp that only this lane writes and reads,
 // so no barrier): loads in flight then cost no registers.  Against the tcgen05 kernel with its gathered 128-row tiles:
 // 8 samples x 2880 tokens x 4096 in windows of 16: 59 -> 37 us between events (189 MB: 5.1 TB/s), windows of 18:
@@ -29,7 +31,13 @@ struct FdStreamArgs {
   const int* seq_start;                // first row of each sample (packed batches) or nullptr
   int64_t batch_stride, row_stride;    // elements
   int d, metric;
-  Workspace ws;
+  double keep;
+  Geometry g;
+  const int* n_vis;                    // tokens of each sample, nullptr = cap_in
+  const int* pos;                      // grid positions, nullptr = identity
+  int cap_in, max_cell;                // max_cell: grid positions of the largest window
+  int* partner;                        // [B, cap_in] out, see Workspace
+  int* place;                          // [B, cap_in] out
 };
 
 __device__ __forceinline__ void mma_m16n8k16(float (&c)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
@@ -62,27 +70,107 @@ struct FdStreamSmem {
   static constexpr int R = 8 * O, PITCH = R + 2;
   static constexpr int RING = WARPS * S * 2 * O * 512;                              // bytes
   static constexpr int PART = (WARPS * R * PITCH + WARPS * 2 * R) * 4;              // over the drained ring
-  static constexpr int BYTES = (RING > PART ? RING : PART) + 2 * R * 4;
+  static constexpr int FIXED = RING > PART ? RING : PART;
+  // + per source of the window: key (8 bytes), best destination, per token of the window: its index; match masks
+  static size_t bytes(int max_cell, int cap_in) {
+    return FIXED + size_t((max_cell + 1) / 2) * 12 + size_t(max_cell) * 4 + size_t((cap_in + 31) / 32) * 4 + 16;
+  }
 };
 
 template <int O, int S, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(FdStreamArgs a) {
-  grid_dependency_sync();
+__global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_constant__ FdStreamArgs a) {
+  grid_dependency_wait();
+  grid_launch_dependents();                              // in this order: see grid_dependency_sync
   using M = FdStreamSmem<O, S, WARPS>;
-  constexpr int R = M::R, MT = (O + 1) / 2, PITCH = M::PITCH;
+  constexpr int R = M::R, MT = (O + 1) / 2, PITCH = M::PITCH, nwarps = WARPS, NT = 32 * WARPS;
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nwarps = WARPS;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* part = reinterpret_cast<float*>(smem_raw);      // [WARPS][R][PITCH] partial inner products
   float* nrm = part + WARPS * R * PITCH;                 // [WARPS][2 R] partial squared norms, row 0: the norms
-  float* best_f = reinterpret_cast<float*>(smem_raw + M::BYTES - 2 * R * 4);   // [R] running minimum over blocks of destinations
-  int* best_e = reinterpret_cast<int*>(best_f + R);      // [R]
-  const int w = blockIdx.x, b = blockIdx.y, nW = a.ws.n_windows;
-  const int* win_off = a.ws.win_off + size_t(b) * (nW + 1) + w;
-  const int* a_off = a.ws.a_off + size_t(b) * (nW + 1) + w;
-  const int a_lo = a_off[0], a_hi = a_off[1], b_lo = win_off[0] - a_lo, b_hi = win_off[1] - a_hi;
-  if (a_lo >= a_hi || b_lo >= b_hi) return;
-  const int* a_tok = a.ws.a_tok + size_t(b) * a.ws.cap_a;
-  const int* b_tok = a.ws.b_tok + size_t(b) * a.ws.cap_b;
+  const int max_src = (a.max_cell + 1) / 2;
+  unsigned int* key = reinterpret_cast<unsigned int*>(smem_raw + M::FIXED);   // [max_src] orderable lowest score of a source
+  int* best = reinterpret_cast<int*>(key + max_src);     // [max_src] destination (local index) that attains it
+  int* into = best + max_src;                            // [max_src] the same for selected sources, -1 for the others
+  int* tok = into + max_src;                             // [max_cell] token index of the window's tokens, in position order
+  unsigned int* match = reinterpret_cast<unsigned int*>(tok + a.max_cell);    // [ceil(cap_in / 32)] tokens of the window
+  __shared__ int warp_sum[WARPS + 1];
+  const int w = blockIdx.x, b = blockIdx.y;
+
+  // ---- the window's tokens in storage (= position) order
+  const int n = a.n_vis ? max(0, min(a.n_vis[b], a.cap_in)) : a.cap_in;
+  const int w2 = a.g.w * a.g.w, tile = w / w2, wr = (w - tile * w2) / a.g.w, wc = w - tile * w2 - wr * a.g.w;
+  const int rows = a.g.rows[tile], cols = a.g.cols[tile], first = a.g.tile_off[tile];
+  // rows r with r * w / rows == wr, columns c with c * w / cols == wc
+  const int r0 = (wr * rows + a.g.w - 1) / a.g.w, r1 = ((wr + 1) * rows + a.g.w - 1) / a.g.w;
+  const int c0 = (wc * cols + a.g.w - 1) / a.g.w, c1 = ((wc + 1) * cols + a.g.w - 1) / a.g.w;
+  int nw;
+  if (!a.pos && n == a.g.tile_off[a.g.n_tiles]) {        // the full grid: no list to search
+    nw = (r1 - r0) * (c1 - c0);
+    for (int l = tid; l < nw; l += NT) {
+      const int r = l / (c1 - c0);
+      tok[l] = first + (r0 + r) * cols + c0 + (l - r * (c1 - c0));
+    }
+    __syncthreads();
+  } else {
+    const int lo = first + r0 * cols, hi = first + r1 * cols, n_grid = a.g.tile_off[a.g.n_tiles];
+    const int* pos = a.pos ? a.pos + size_t(b) * a.cap_in : nullptr;
+    const int chunks = (n + 31) >> 5;
+#pragma unroll 4
+    for (int c = warp; c < chunks; c += WARPS) {
+      const int i = c * 32 + lane;
+      bool in = false;
+      if (i < n) {
+        const int p = pos ? pos[i] : i;
+        if (p >= lo && p < hi) {
+          const int col = (p - first) % cols;
+          in = col >= c0 && col < c1;
+        }
+        in = in || (w == 0 && (p < 0 || p >= n_grid));   // no such position: counted with window 0 (flagged elsewhere)
+      }
+      const unsigned int m = __ballot_sync(0xffffffffu, in);
+      if (lane == 0) match[c] = m;
+    }
+    __syncthreads();
+    nw = 0;
+    for (int base = 0; base < chunks; base += NT) {
+      const unsigned int m = base + tid < chunks ? match[base + tid] : 0u;
+      const int own = __popc(m);
+      int x = own;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int t = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += t;
+      }
+      if (lane == 31) warp_sum[warp] = x;
+      __syncthreads();
+      int before = nw, total = 0;
+#pragma unroll
+      for (int k = 0; k < WARPS; ++k) {
+        if (k < warp) before += warp_sum[k];
+        total += warp_sum[k];
+      }
+      int at = before + x - own;
+      for (unsigned int bits = m; bits; bits &= bits - 1) {
+        const int i = (base + tid) * 32 + __ffs(bits) - 1;
+        if (at < a.max_cell) {
+          tok[at] = i;
+        } else {                                         // only if positions repeat or lie outside the grid: survives
+          a.partner[size_t(b) * a.cap_in + i] = -1;
+          a.place[size_t(b) * a.cap_in + i] = 0;
+        }
+        ++at;
+      }
+      nw += total;
+      __syncthreads();
+    }
+    nw = min(nw, a.max_cell);
+  }
+  if (nw == 0) return;
+  const int par = a.g.src_par;
+  const int na_all = (nw + 1 - par) >> 1, nb_all = nw - na_all;   // sources: local ranks of parity `par`
+  const int removed = nb_all > 0 ? removal_count(nw, a.keep, par) : 0;
+  for (int e = tid; e < na_all; e += NT) { key[e] = 0xffffffffu; best[e] = -1; into[e] = -1; }
+
   const int g = lane >> 2, t = lane & 3;
   const int nc = (a.d + 31) >> 5, c_lo = warp * nc / WARPS, nk = (warp + 1) * nc / WARPS - c_lo;
   const __nv_bfloat16* base = a.x + size_t(b) * a.batch_stride + size_t(a.seq_start ? a.seq_start[b] : 0) * a.row_stride +
@@ -90,15 +178,15 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(FdStreamArgs a) {
   const uint32_t row16 = uint32_t(a.row_stride >> 3);    // row pitch in 16-byte units
   const uint32_t ring = tc::smem_u32(smem_raw) + (warp * S * 2 * O * 32 + lane) * 16;
 
-  for (int a0 = a_lo; a0 < a_hi; a0 += R) {
-    const int na = min(R, a_hi - a0);
-    for (int b0 = b_lo; b0 < b_hi; b0 += R) {
-      const int nb = min(R, b_hi - b0);
+  for (int a0 = 0; removed > 0 && a0 < na_all; a0 += R) {     // nothing to remove: no scores needed
+    const int na = min(R, na_all - a0);
+    for (int b0 = 0; b0 < nb_all; b0 += R) {
+      const int nb = min(R, nb_all - b0);
       uint32_t off[2 * O];                               // row offsets in 16-byte units, A rows first; all ones: no such row
 #pragma unroll
       for (int i = 0; i < O; ++i) {
-        off[i] = 8 * i + g < na ? uint32_t(a_tok[a0 + 8 * i + g]) * row16 : 0xffffffffu;
-        off[O + i] = 8 * i + g < nb ? uint32_t(b_tok[b0 + 8 * i + g]) * row16 : 0xffffffffu;
+        off[i] = 8 * i + g < na ? uint32_t(tok[2 * (a0 + 8 * i + g) + par]) * row16 : 0xffffffffu;
+        off[O + i] = 8 * i + g < nb ? uint32_t(tok[2 * (b0 + 8 * i + g) + 1 - par]) * row16 : 0xffffffffu;
       }
       // rows the block does not have stay zero in every stage
 #pragma unroll
@@ -176,38 +264,67 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(FdStreamArgs a) {
       __syncthreads();
       // ---- a warp per source row, lanes over the destinations
       for (int r = warp; r < na; r += nwarps) {
-        float best = 3.0e38f;
-        int best_c = -1;
+        float lowest = 3.0e38f;
+        int col_min = -1;
         for (int col = lane; col < nb; col += 32) {
           float s = part[r * PITCH + col];
           for (int k = 1; k < nwarps; ++k) s += part[(k * R + r) * PITCH + col];
           const float fd = pair_score(a.metric, s, nrm[r], nrm[R + col]);
-          if (fd < best) { best = fd; best_c = col; }
+          if (fd < lowest) { lowest = fd; col_min = col; }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) {               // minimum over the lanes, ties to the lower column
-          const float of = __shfl_xor_sync(0xffffffffu, best, o);
-          const int oc = __shfl_xor_sync(0xffffffffu, best_c, o);
-          if (oc >= 0 && (best_c < 0 || of < best || (of == best && oc < best_c))) { best = of; best_c = oc; }
+          const float of = __shfl_xor_sync(0xffffffffu, lowest, o);
+          const int oc = __shfl_xor_sync(0xffffffffu, col_min, o);
+          if (oc >= 0 && (col_min < 0 || of < lowest || (of == lowest && oc < col_min))) { lowest = of; col_min = oc; }
         }
-        if (lane == 0) {
-          int e = best_c >= 0 ? b0 + best_c : -1;
-          if (b0 > b_lo && best_e[r] >= 0 && !(best < best_f[r])) { best = best_f[r]; e = best_e[r]; }
-          best_f[r] = best;
-          best_e[r] = e;
-          if (b0 + R >= b_hi && e >= 0)
-            a.ws.a_key[size_t(b) * a.ws.cap_a + a0 + r] = ((unsigned long long)orderable(best) << 32) | (unsigned)e;
+        // later blocks of destinations hold higher indices: an equal score keeps the earlier one
+        if (lane == 0 && col_min >= 0 && orderable(lowest) < key[a0 + r]) {
+          key[a0 + r] = orderable(lowest);
+          best[a0 + r] = b0 + col_min;
         }
       }
-      if (a0 + R < a_hi || b0 + R < b_hi) __syncthreads();   // the partial results are overwritten by the next block
+      __syncthreads();                                   // the partial results are overwritten by the next block
     }
+  }
+
+  // ---- selection: the `removed` sources with the lowest (score, index) go into their best destination
+  if (removed == 0) __syncthreads();
+  for (int e = tid; e < na_all; e += NT) {
+    bool sel = removed >= na_all;
+    if (!sel && removed > 0) {
+      const unsigned int mine = key[e];
+      int rank = 0;
+      for (int k = 0; k < e; ++k) rank += key[k] <= mine;
+      for (int k = e + 1; k < na_all; ++k) rank += key[k] < mine;
+      sel = rank < removed;
+    }
+    if (sel) into[e] = best[e];
+  }
+  __syncthreads();
+  // ---- what the merge map needs of every token: its partner, and its place in the group or the group's size
+  int* partner = a.partner + size_t(b) * a.cap_in;
+  int* place = a.place + size_t(b) * a.cap_in;
+  for (int l = tid; l < nw; l += NT) {
+    const int e = l >> 1, i = tok[l];
+    int p = -1, q = 0;
+    if ((l & 1) == par) {
+      const int to = into[e];
+      p = to < 0 ? -2 : tok[2 * to + 1 - par];
+      if (to >= 0)
+        for (int k = 0; k < e; ++k) q += into[k] == to;
+    } else {
+      for (int k = 0; k < na_all; ++k) q += into[k] == e;
+    }
+    partner[i] = p;
+    place[i] = q;
   }
 }
 
 template <int O, int S, int WARPS>
 static cudaError_t launch_fd_stream_o(const LayerLaunch& L, const FdStreamArgs& f) {
-  constexpr int smem = FdStreamSmem<O, S, WARPS>::BYTES;
-  const cudaError_t e = ensure_dynamic_smem(fd_stream_kernel<O, S, WARPS>, smem);
+  const size_t smem = FdStreamSmem<O, S, WARPS>::bytes(f.max_cell, f.cap_in);
+  const cudaError_t e = ensure_dynamic_smem(fd_stream_kernel<O, S, WARPS>, (int)smem);
   if (e != cudaSuccess) return e;
   return launch_kernel(fd_stream_kernel<O, S, WARPS>, dim3(L.geo.n_windows, L.batch), 32 * WARPS, smem, L.stream, 1, f);
 }
@@ -219,10 +336,12 @@ static cudaError_t launch_fd_stream_w(const LayerLaunch& L, const FdStreamArgs& 
   return L.hidden > 768 ? launch_fd_stream_o<O, S, 8>(L, f) : launch_fd_stream_o<O, S, 2>(L, f);
 }
 
-// Largest window side (source or destination nodes) the plan may expect for this kernel: five groups of eight rows a
-// side is what the fragments of a thread hold at two CTAs per SM; beyond that the tcgen05 kernel shares the rows
-// between more pairs.
-bool fd_stream_supported(int fd_side) { return fd_side > 0 && fd_side <= 40; }
+// Five groups of eight rows a side is what the fragments of a thread hold at two CTAs per SM; beyond that the tcgen05
+// kernel shares the rows between more pairs.  The lists of a window and the search for its tokens have to fit in
+// shared memory beside the ring, and the map kernel behind takes two tokens per thread of eight CTAs.
+bool fd_stream_supported(int fd_side, int max_cell, int cap_in) {
+  return fd_side > 0 && fd_side <= 40 && max_cell <= 4096 && cap_in <= kMapMaxTokens;
+}
 
 cudaError_t launch_fd_stream(const LayerLaunch& L) {
   const lightkv_layer_args_t* a = L.a;
@@ -230,7 +349,8 @@ cudaError_t launch_fd_stream(const LayerLaunch& L) {
   f.x = static_cast<const __nv_bfloat16*>(a->hidden) + size_t(a->vis_begin) * a->hidden_row_stride;
   f.seq_start = a->seq_start;
   f.batch_stride = a->hidden_batch_stride; f.row_stride = a->hidden_row_stride;
-  f.d = L.hidden; f.metric = L.divergence; f.ws = L.ws;
+  f.d = L.hidden; f.metric = L.divergence; f.keep = L.keep; f.g = L.geo; f.n_vis = a->n_vis; f.pos = a->pos;
+  f.cap_in = L.ws.cap_in; f.max_cell = L.max_cell; f.partner = L.ws.partner; f.place = L.ws.slot;
   // chunks in flight per warp (S): as few as still leave enough CTAs on an SM; with more, fewer CTAs fit and the
   // start and end of a window are less covered (S = 8, 6, 4 measured 39 / 33 / 25 us where 6, 4, 3 take 37 / 27 / 23)
   switch ((L.fd_side + 7) / 8) {

@@ -746,6 +746,247 @@ cudaError_t launch_select_map(const LayerLaunch& L) {
 }
 
 // =====================================================================================================
+// Merge map behind the streaming FD kernel, which left every token's partner and its place (see Workspace).  One
+// cluster of 1-8 CTAs per sample, TPT consecutive tokens per thread, everything between the first loads and the last
+// stores in registers and (distributed) shared memory:
+//   1  xi = fixed-order sum over heads (or given / uniform); survivors and group sizes are counted in ONE pair of prefix
+//      sums: a survivor's slot, and the offset of its group (its members are 1 + place tokens)
+//   2  a merged token reads its partner's slot and offset from the CTA that owns it and stores its index and xi at its
+//      place in that CTA's member list (groups of one CTA's survivors are one contiguous range)
+//   3  weights xi_i / sum over the group, the sum taken in member order (survivor first)
+// Bound by latency: one round trip to L2 for the loads, three cluster barriers, one round of stores.  A merged token
+// that would need a kernel-wide search for its group costs one remote read here, because the streaming FD kernel holds
+// whole windows.  (select_map_kernel, which starts from keys, takes six dependent rounds through L2: 9 us at 576 and
+// 20 us at 2880 tokens per sample against 5 and 7.)
+// =====================================================================================================
+struct MapArgs {
+  int n_q_heads, xi_mode, cap_in, cap_out, cap_a, cap_b, n_grid;
+  const int* n_vis;
+  const int* pos;
+  const float* xi_in;
+  const float* xi_h;
+  const int* partner;
+  const int* place;
+  int* n_vis_out;
+  int* pos_out;
+  int* dst;
+  float* weight;
+  int* grp_off;
+  int* grp_src;
+  float* xi_out;
+  uint32_t* status;
+};
+
+template <bool CLUSTER, int TPT>
+__global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapArgs a) {
+  grid_dependency_sync();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  const int nthr = blockDim.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
+  const int span = nthr * TPT;                              // tokens a CTA can own
+  int* s_slot = reinterpret_cast<int*>(smem_raw);           // [span] slot of an owned survivor
+  int* s_at = s_slot + span;                                // [span] offset of its group inside this CTA's member list
+  int* m_tok = s_at + span;                                 // [cap_in] member list: token index
+  float* m_xi = reinterpret_cast<float*>(m_tok + a.cap_in); // [cap_in] ... and its xi
+  __shared__ int warp_sums[2][33];
+  __shared__ int cta_total[3];                              // survivors, members, sources of this CTA
+  __shared__ int base_off[8];                               // first member offset of every CTA
+  const int cs = CLUSTER ? (int)tc::cluster_nctarank() : 1, rank = CLUSTER ? (int)tc::cluster_ctarank() : 0;
+  auto sync_all = [&]() { if (CLUSTER) tc::cluster_sync(); else __syncthreads(); };
+  const int b = blockIdx.x / cs;
+  int n = a.n_vis ? a.n_vis[b] : a.cap_in;
+  if (n > a.cap_in) { n = a.cap_in; if (rank == 0 && tid == 0) set_status(a.status, LIGHTKV_STATUS_COUNT); }
+  if (n < 0) n = 0;
+  const size_t row = size_t(b) * a.cap_in;
+  const int chunk = ((n + cs - 1) / cs + TPT - 1) / TPT * TPT;   // tokens per CTA (whole threads)
+  const int lo = min(n, rank * chunk), hi = min(n, lo + chunk);
+  const int i0 = lo + tid * TPT;
+
+  // ---- loads
+  int prt[TPT], plc[TPT], ps[TPT];
+  float xi[TPT];
+  bool bad = false;
+#pragma unroll
+  for (int j = 0; j < TPT; ++j) {
+    const int i = i0 + j;
+    prt[j] = -1; plc[j] = 0; ps[j] = i; xi[j] = 0.f;
+    if (i < hi) {
+      prt[j] = a.partner[row + i];
+      plc[j] = a.place[row + i];
+      if (a.pos) {
+        ps[j] = a.pos[row + i];
+        bad = bad || ps[j] <= (i > 0 ? a.pos[row + i - 1] : -1) || ps[j] >= a.n_grid;
+      } else {
+        bad = bad || i >= a.n_grid;
+      }
+      if (a.xi_mode == LIGHTKV_XI_GIVEN) xi[j] = a.xi_in[row + i];
+      else if (a.xi_mode == LIGHTKV_XI_UNIFORM) xi[j] = 1.0f;
+      else {
+        const float* x = a.xi_h + size_t(b) * a.n_q_heads * a.cap_in + i;
+        for (int h0 = 0; h0 < a.n_q_heads; h0 += 16) {      // sixteen heads' loads in flight, added in head order
+          float v[16];
+#pragma unroll
+          for (int h = 0; h < 16; ++h) v[h] = h0 + h < a.n_q_heads ? x[size_t(h0 + h) * a.cap_in] : 0.f;
+#pragma unroll
+          for (int h = 0; h < 16; ++h) xi[j] += v[h];
+        }
+      }
+    }
+  }
+  if (__any_sync(0xffffffffu, bad) && lane == 0) set_status(a.status, LIGHTKV_STATUS_POS_ORDER);
+
+  // ---- survivors and group members in front of this thread
+  int ns = 0, nm = 0, nsrc = 0;
+#pragma unroll
+  for (int j = 0; j < TPT; ++j)
+    if (i0 + j < hi) {
+      if (prt[j] < 0) { ++ns; nm += 1 + plc[j]; }
+      if (prt[j] != -1) ++nsrc;
+    }
+  int xs = ns, xm = nm;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int ts = __shfl_up_sync(0xffffffffu, xs, o), tm = __shfl_up_sync(0xffffffffu, xm, o);
+    if (lane >= o) { xs += ts; xm += tm; }
+  }
+  nsrc = __reduce_add_sync(0xffffffffu, nsrc);
+  if (tid < 3) cta_total[tid] = 0;
+  if (lane == 31) { warp_sums[0][wp] = xs; warp_sums[1][wp] = xm; }
+  __syncthreads();
+  if (lane == 0 && nsrc) atomicAdd(&cta_total[2], nsrc);
+  if (wp == 0) {
+    const int nw = nthr >> 5;
+    int s = lane < nw ? warp_sums[0][lane] : 0, m = lane < nw ? warp_sums[1][lane] : 0;
+    const int own_s = s, own_m = m;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int ts = __shfl_up_sync(0xffffffffu, s, o), tm = __shfl_up_sync(0xffffffffu, m, o);
+      if (lane >= o) { s += ts; m += tm; }
+    }
+    warp_sums[0][lane] = s - own_s;
+    warp_sums[1][lane] = m - own_m;
+    if (lane == 31) { cta_total[0] = s; cta_total[1] = m; }
+  }
+  sync_all();
+  int before_s = 0, before_m = 0, survivors = 0, members = 0, sources = 0;
+  for (int j = 0; j < cs; ++j) {
+    auto total = [&](int k) {
+      return CLUSTER ? (int)tc::ld_cluster_u32(tc::map_to_cta(tc::smem_u32(&cta_total[k]), j)) : cta_total[k];
+    };
+    const int s = total(0), m = total(1);
+    if (tid == 0) base_off[j] = members;
+    if (j < rank) { before_s += s; before_m += m; }
+    survivors += s;
+    members += m;
+    sources += total(2);
+  }
+  // A sample whose A or B nodes do not fit the plan's capacities (a subset of the grid handed to a plan that was built
+  // for full grids) keeps all of its tokens, and the status word says so.
+  const bool over = sources > a.cap_a || n - sources > a.cap_b;
+  if (over) {
+    survivors = members = n;
+    before_s = before_m = lo;
+    xs = xm = ns = nm = 0;
+#pragma unroll
+    for (int j = 0; j < TPT; ++j) { prt[j] = -1; plc[j] = 0; }
+  }
+  const int n_out = min(survivors, a.cap_out);
+  if (rank == 0 && tid == 0) {
+    a.n_vis_out[b] = n_out;
+    if (n_out == survivors) a.grp_off[size_t(b) * (a.cap_out + 1) + n_out] = members;   // (cut at cap_out: set below)
+    if (over || survivors > a.cap_out) set_status(a.status, LIGHTKV_STATUS_COUNT);
+  }
+  int slot = over ? i0 : before_s + warp_sums[0][wp] + xs - ns, off = over ? i0 : before_m + warp_sums[1][wp] + xm - nm;
+#pragma unroll
+  for (int j = 0; j < TPT; ++j) {
+    const int i = i0 + j;
+    if (i < hi && prt[j] < 0) {
+      const int l = i - lo, at = off - before_m;
+      s_slot[l] = slot;
+      s_at[l] = at;
+      a.dst[row + i] = slot;
+      if (slot < a.cap_out) {
+        a.pos_out[size_t(b) * a.cap_out + slot] = ps[j];
+        a.grp_off[size_t(b) * (a.cap_out + 1) + slot] = off;
+        a.grp_src[row + off] = i;
+      } else if (slot == a.cap_out) {
+        a.grp_off[size_t(b) * (a.cap_out + 1) + slot] = off;   // the groups that are kept end here
+      }
+      m_tok[at] = i;
+      m_xi[at] = xi[j];
+      ++slot;
+      off += 1 + plc[j];
+    }
+  }
+  sync_all();
+  // ---- merged tokens join their partner's group
+#pragma unroll
+  for (int j = 0; j < TPT; ++j) {
+    const int i = i0 + j, p = prt[j];
+    if (i < hi && p >= 0) {
+      const int r = CLUSTER ? p / chunk : 0, l = p - r * chunk;
+      int o, at;
+      if (CLUSTER) {
+        o = (int)tc::ld_cluster_u32(tc::map_to_cta(tc::smem_u32(&s_slot[l]), r));
+        at = (int)tc::ld_cluster_u32(tc::map_to_cta(tc::smem_u32(&s_at[l]), r));
+      } else {
+        o = s_slot[l]; at = s_at[l];
+      }
+      at += 1 + plc[j];
+      a.dst[row + i] = o;
+      if (o < a.cap_out) a.grp_src[row + base_off[r] + at] = i;
+      if (CLUSTER) {
+        tc::st_cluster_u32(tc::map_to_cta(tc::smem_u32(&m_tok[at]), r), (uint32_t)i);
+        tc::st_cluster_u32(tc::map_to_cta(tc::smem_u32(&m_xi[at]), r), __float_as_uint(xi[j]));
+      } else {
+        m_tok[at] = i; m_xi[at] = xi[j];
+      }
+    }
+    if (i < hi && a.xi_out) a.xi_out[row + i] = xi[j];
+  }
+  sync_all();
+  // ---- weights
+#pragma unroll
+  for (int j = 0; j < TPT; ++j) {
+    const int i = i0 + j;
+    if (i < hi && prt[j] < 0 && s_slot[i - lo] < a.cap_out) {
+      const int at = s_at[i - lo], size = 1 + plc[j];
+      float den = 0.f;
+      for (int c = 0; c < size; ++c) den += m_xi[at + c];
+      if (den >= 1e-30f) {
+        for (int c = 0; c < size; ++c) a.weight[row + m_tok[at + c]] = m_xi[at + c] / den;
+      } else {
+        set_status(a.status, LIGHTKV_STATUS_ZERO_WEIGHT);
+        for (int c = 0; c < size; ++c) a.weight[row + m_tok[at + c]] = 1.0f / (float)size;
+      }
+    }
+  }
+}
+
+cudaError_t launch_map(const LayerLaunch& L) {
+  const lightkv_layer_args_t* a = L.a;
+  MapArgs m;
+  m.n_q_heads = L.n_q_heads; m.xi_mode = L.xi_mode; m.cap_in = L.ws.cap_in; m.cap_out = L.ws.cap_out;
+  m.cap_a = L.ws.cap_a; m.cap_b = L.ws.cap_b; m.n_grid = L.n_grid;
+  m.n_vis = a->n_vis; m.pos = a->pos; m.xi_in = a->xi; m.xi_h = L.ws.xi_h; m.partner = L.ws.partner; m.place = L.ws.slot;
+  m.n_vis_out = a->n_vis_out; m.pos_out = a->pos_out; m.dst = a->dst; m.weight = a->weight; m.grp_off = a->grp_off;
+  m.grp_src = a->grp_src; m.xi_out = a->xi_out; m.status = a->status;
+  // one cluster per sample: as many CTAs of up to 1024 threads as give every thread one token (two beyond 8192)
+  const int n = L.ws.cap_in;
+  int cs = 1;
+  while (cs < 8 && cs * 1024 < n) cs *= 2;
+  const int tpt = n > 8192 ? 2 : 1;
+  const int threads = std::min(1024, (((n + cs - 1) / cs + tpt - 1) / tpt + 31) / 32 * 32);
+  const size_t smem = (size_t(2) * threads * tpt + size_t(2) * n) * 4;
+  auto launch = [&](auto kernel) -> cudaError_t {
+    const cudaError_t e = ensure_dynamic_smem(kernel, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_kernel(kernel, L.batch * cs, threads, smem, L.stream, cs, m);
+  };
+  if (tpt == 2) return launch(map_kernel<true, 2>);
+  return cs > 1 ? launch(map_kernel<true, 1>) : launch(map_kernel<false, 1>);
+}
+
+// =====================================================================================================
 // Weighted merge of the hidden states (Eq. "message-passing", Steps 3-5): one CTA per output row.
 // Row o of the vision block is sum over its group of weight_i * x_i in fp32, rounded once to the
 // storage type; a group of one has weight exactly 1 and is therefore copied bit-exactly.  Text rows

@@ -464,6 +464,18 @@ def test_fd_window_larger_than_the_plan_expects(grid, windows, seed):
     H.run_schedule(wl, xi_mode="given", first_pos=[subset, full])
 
 
+@pytest.mark.parametrize("grid,w", [((32, 32), 5), ((25, 41), 4), ((32, 64), 8), ((45, 46), 7), ((64, 64), 11),
+                                    ((64, 65), 9), ((90, 91), 16), ((91, 91), 12), ((96, 100), 12)])
+def test_map_of_streaming_windows_over_cluster_sizes(grid, w):
+    # samples at the borders between one, two, four and eight CTAs and between one and two tokens per thread of the
+    # map kernel, one sample with the full grid and one with a subset of it (the cut between CTAs then falls elsewhere)
+    wl = S.Workload(name="mapcs", config_id=135, batch=2, tiles=(grid,), n_text=5, hidden=64, n_q_heads=2,
+                    n_kv_heads=1, head_dim=64, n_layers=16, layers=(3,), windows=(w,), keep=(0.57,))
+    full = np.arange(wl.n_vis, dtype=np.int32)
+    subset = np.sort(np.random.default_rng(w).choice(full, wl.n_vis * 5 // 7, replace=False)).astype(np.int32)
+    H.run_schedule(wl, xi_mode="given", ragged=True, first_pos=[full, subset])
+
+
 # ---- subsets of the grid: capacities ---------------------------------------------------------------------------
 
 def _near_full_subset():
