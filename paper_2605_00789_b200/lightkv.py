@@ -1,13 +1,14 @@
-"""ctypes binding of the liblightkv C ABI (include/lightkv.h): same names, argument marshalling only.
+"""Binding of the liblightkv C ABI (include/lightkv.h): same names, argument marshalling only.
 
 PyTorch is used for device memory and streams: tensors are handed over as data pointers plus element
-strides, the current CUDA stream as a raw handle.  No arithmetic of the method happens here.
+strides, the current CUDA stream as a raw handle.  No arithmetic of the method happens here.  Plans go
+through ctypes; the calls of every layer are marshalled natively (csrc/binding.c, module _binding).
 """
 from __future__ import annotations
 
 import ctypes as C
 import os
-from typing import Optional, Sequence, Tuple
+from typing import Sequence, Tuple
 
 BF16, FP32 = 0, 1
 XI_GIVEN, XI_ATTN_FULL, XI_ATTN_LSE, XI_UNIFORM = 0, 1, 2, 3
@@ -189,10 +190,6 @@ class Plan:
             pass
 
 
-def _ptr(t) -> Optional[int]:
-    return None if t is None else t.data_ptr()
-
-
 class StageBuffers:
     """Device outputs + workspace of one stage, allocated with torch (plumbing only)."""
 
@@ -219,68 +216,39 @@ class StageBuffers:
         return (p + 255) // 256 * 256
 
 
-def _stream_handle(stream) -> int:
+_BINDING = None
+
+
+def _fail(code: int, what: str) -> None:
+    _check(code, what)
+
+
+def _fork_join(out: StageBuffers):
+    """The fork / join events of a stage whose caller gave none (the library creates no events), kept with its buffers."""
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return s.cuda_stream
+    if not hasattr(out, "fork_join"):
+        out.fork_join = (torch.cuda.Event(), torch.cuda.Event())
+        for e in out.fork_join:
+            e.record()                # torch creates the CUDA event lazily; the C ABI needs a live handle
+    return out.fork_join
 
 
-def _layer_args(plan: Plan, stage: int, hidden, out: StageBuffers, *, vis_begin: int,
-                n_text_after: int = 0, text_begin: int = 0, text_end: Optional[int] = None,
-                q=None, k=None, lse=None, xi=None, n_vis=None, pos=None, stream=None,
-                trace_events=None, aux_stream=None, map_event=None, fork_event=None, join_event=None,
-                text_ranges=None, bidirectional: bool = False, lse_out=None, seq_start=None, seq_start_out=None,
-                hidden_out=None) -> _LayerArgs:
-    a = _LayerArgs()
-    a.struct_size = C.sizeof(_LayerArgs)
-    a.stage, a.vis_begin, a.n_text_after = stage, vis_begin, n_text_after
-    a.text_begin, a.text_end = text_begin, vis_begin if text_end is None else text_end
-    a.hidden, a.hidden_batch_stride, a.hidden_row_stride = hidden.data_ptr(), hidden.stride(0), hidden.stride(1)
-    ho = out.hidden_out if hidden_out is None else hidden_out
-    a.hidden_out, a.hidden_out_batch_stride, a.hidden_out_row_stride = ho.data_ptr(), ho.stride(0), ho.stride(1)
-    if q is not None:
-        a.seq_rows = q.shape[2]
-        a.q, a.q_batch_stride, a.q_head_stride, a.q_row_stride = q.data_ptr(), q.stride(0), q.stride(1), q.stride(2)
-    if k is not None:
-        a.k, a.k_batch_stride, a.k_head_stride, a.k_row_stride = k.data_ptr(), k.stride(0), k.stride(1), k.stride(2)
-    if lse is not None:
-        a.lse, a.lse_batch_stride, a.lse_head_stride = lse.data_ptr(), lse.stride(0), lse.stride(1)
-    a.xi, a.n_vis, a.pos = _ptr(xi), _ptr(n_vis), _ptr(pos)
-    a.n_vis_out, a.pos_out, a.dst, a.weight = _ptr(out.n_vis_out), _ptr(out.pos_out), _ptr(out.dst), _ptr(out.weight)
-    a.grp_off, a.grp_src, a.xi_out, a.status = _ptr(out.grp_off), _ptr(out.grp_src), _ptr(out.xi_out), _ptr(out.status)
-    a.workspace, a.workspace_bytes = out.workspace_ptr(), out.info.workspace_bytes
-    a.stream = _stream_handle(stream)
-    if aux_stream is not None:
-        # the library creates no events: the fork / join pair is the caller's (kept with the stage's buffers here)
+def _binding():
+    """The native marshalling module, bound to the loaded library.  There is no fallback: missing is an error."""
+    global _BINDING
+    if _BINDING is None:
         import torch
-        a.aux_stream = aux_stream.cuda_stream
-        if fork_event is None or join_event is None:
-            if not hasattr(out, "fork_join"):
-                out.fork_join = (torch.cuda.Event(), torch.cuda.Event())
-                for e in out.fork_join:
-                    e.record()            # torch creates the CUDA event lazily; the C ABI needs a live handle
-            fork_event, join_event = out.fork_join
-        a.fork_event, a.join_event = fork_event.cuda_event, join_event.cuda_event
-    if text_ranges is not None:       # [(begin, end), ...] instead of the single range text_begin / text_end
-        flat = [int(v) for r in text_ranges for v in r]
-        a._ranges = (C.c_int32 * len(flat))(*flat)          # kept alive by the struct object
-        a.text_ranges, a.n_text_ranges = a._ranges, len(flat) // 2
-    a.bidirectional = int(bool(bidirectional))
-    if lse_out is not None:
-        a.lse_out, a.lse_out_batch_stride, a.lse_out_head_stride = lse_out.data_ptr(), lse_out.stride(0), lse_out.stride(1)
-    if seq_start is not None:
-        # packed batch: tensors of shape [1, rows, ...] hold the samples back to back; sample b starts at row
-        # seq_start[b], so the batch strides are 0 and q / k span all rows
-        a.seq_start, a.seq_start_out = seq_start.data_ptr(), _ptr(seq_start_out)
-        a.hidden_batch_stride = a.q_batch_stride = a.k_batch_stride = a.lse_batch_stride = a.lse_out_batch_stride = 0
-        if seq_start_out is not None:
-            a.hidden_out_batch_stride = 0
-    if map_event is not None:         # a torch.cuda.Event that has been recorded once (torch creates it lazily)
-        a.map_event = map_event.cuda_event
-    if trace_events is not None:      # TRACE_EVENTS torch.cuda.Event objects (enable_timing=True), already created
-        assert len(trace_events) == TRACE_EVENTS
-        a.trace_events = (C.c_void_p * TRACE_EVENTS)(*[e.cuda_event for e in trace_events])
-    return a
+        lib = library()
+        try:
+            from . import _binding as native
+        except ImportError as exc:
+            raise LightKVError(f"_binding.so is missing: build it first (python -c 'import __graft_entry__ as g; g.build()'): {exc}")
+        address = lambda f: C.cast(f, C.c_void_p).value
+        native.bind(address(lib.lightkv_compress_layer), address(lib.lightkv_compress_layer_builtin_ws),
+                    address(lib.lightkv_compact_kv), _fail, _fork_join, torch._C._cuda_getCurrentRawStream,
+                    torch.cuda.current_device)
+        _BINDING = native
+    return _BINDING
 
 
 def compress_layer(plan: Plan, stage: int, hidden, out: StageBuffers, **kw) -> None:
@@ -288,19 +256,16 @@ def compress_layer(plan: Plan, stage: int, hidden, out: StageBuffers, **kw) -> N
     q [B,H,N,dh], k [B,H_kv,N,dh] (any strides with a contiguous last dimension), lse [B,H,N] fp32,
     xi [B,cap_in] fp32, n_vis [B] int32, pos [B,cap_in] int32, stream, trace_events, aux_stream, map_event,
     fork_event / join_event, text_ranges [(begin, end), ...], bidirectional, lse_out [B,H,N] fp32,
-    seq_start / seq_start_out [B] int32 (packed batches), hidden_out (instead of out.hidden_out)."""
-    a = _layer_args(plan, stage, hidden, out, **kw)
-    _check(library().lightkv_compress_layer(plan.handle, C.byref(a)), "lightkv_compress_layer")
+    seq_start / seq_start_out [B] int32 (packed batches), hidden_out (instead of out.hidden_out).
+    Events must have been recorded once (torch creates them lazily)."""
+    (_BINDING or _binding()).compress_layer(plan, stage, hidden, out, **kw)
 
 
 def compress_layer_builtin_ws(plan: Plan, stage: int, hidden, out: StageBuffers, **kw) -> None:
     """lightkv_compress_layer_builtin_ws: same call, but the stage's scratch is the fixed array inside
     the library (BUILTIN_WS_BYTES), so the workspace tensor of `out` is not used.  Meant for callers
     that may not allocate device memory; stages needing more scratch than that are refused."""
-    a = _layer_args(plan, stage, hidden, out, **kw)
-    a.workspace, a.workspace_bytes = None, 0
-    _check(library().lightkv_compress_layer_builtin_ws(plan.handle, C.byref(a)),
-           "lightkv_compress_layer_builtin_ws")
+    (_BINDING or _binding()).compress_layer_builtin_ws(plan, stage, hidden, out, **kw)
 
 
 def compact_kv(plan: Plan, stage: int, out: StageBuffers, k_src, v_src, k_dst, v_dst, *, vis_begin: int,
@@ -309,26 +274,5 @@ def compact_kv(plan: Plan, stage: int, out: StageBuffers, k_src, v_src, k_dst, v
                dst_seq_start=None) -> None:
     """lightkv_compact_kv.  Contiguous: k/v [B,H_kv,N,dh] views (any batch/head/row strides).
     Paged: k/v page pools [n_pages, H_kv, page_size, dh] views and int32 block tables [B, max_blocks]."""
-    a = _KvArgs()
-    a.struct_size = C.sizeof(_KvArgs)
-    a.stage, a.vis_begin, a.n_text_after, a.mode = stage, vis_begin, n_text_after, mode
-    a.n_vis, a.n_vis_out = _ptr(n_vis), _ptr(out.n_vis_out)
-    a.grp_off, a.grp_src, a.weight = _ptr(out.grp_off), _ptr(out.grp_src), _ptr(out.weight)
-    a.k_src, a.v_src, a.k_dst, a.v_dst = k_src.data_ptr(), v_src.data_ptr(), k_dst.data_ptr(), v_dst.data_ptr()
-    assert k_src.stride() == v_src.stride() and k_dst.stride() == v_dst.stride()
-    if page_size > 0:
-        a.src_page_stride, a.src_head_stride, a.src_row_stride = k_src.stride(0), k_src.stride(1), k_src.stride(2)
-        a.dst_page_stride, a.dst_head_stride, a.dst_row_stride = k_dst.stride(0), k_dst.stride(1), k_dst.stride(2)
-        a.page_size, a.max_blocks = page_size, src_block_table.shape[1]
-        assert dst_block_table.shape[1] == src_block_table.shape[1]
-        a.src_block_table, a.dst_block_table = src_block_table.data_ptr(), dst_block_table.data_ptr()
-    else:
-        a.src_batch_stride, a.src_head_stride, a.src_row_stride = k_src.stride(0), k_src.stride(1), k_src.stride(2)
-        a.dst_batch_stride, a.dst_head_stride, a.dst_row_stride = k_dst.stride(0), k_dst.stride(1), k_dst.stride(2)
-    a.status = _ptr(out.status)
-    a.stream = _stream_handle(stream)
-    if src_seq_start is not None:     # packed caches: sample b's first token; contiguous batch strides become 0
-        a.src_seq_start, a.src_batch_stride = src_seq_start.data_ptr(), 0
-    if dst_seq_start is not None:
-        a.dst_seq_start, a.dst_batch_stride = dst_seq_start.data_ptr(), 0
-    _check(library().lightkv_compact_kv(plan.handle, C.byref(a)), "lightkv_compact_kv")
+    (_BINDING or _binding()).compact_kv(plan, stage, out, k_src, v_src, k_dst, v_dst, vis_begin, n_text_after, mode, n_vis,
+                                        page_size, src_block_table, dst_block_table, stream, src_seq_start, dst_seq_start)
