@@ -97,7 +97,7 @@ typedef struct {
   int32_t  batch;                  /* samples per call */
   int32_t  hidden;                 /* d; multiple of 8 */
   int32_t  n_q_heads, n_kv_heads;  /* H, H_kv; H % H_kv == 0 */
-  int32_t  head_dim;               /* multiple of 8; tensor-core xi needs 64 or 128 */
+  int32_t  head_dim;               /* multiple of 8, at most 256; tensor-core xi takes up to 128 */
   int32_t  n_layers;               /* L, used by the accounting only */
   int32_t  n_tiles;                /* >= 1; sum of rows*cols = vision tokens before stage 0 */
   const lightkv_tile_t* tiles;

@@ -74,9 +74,9 @@ inline cudaError_t ensure_dynamic_smem(void (*kernel)(P...), int bytes) {
 cudaError_t launch_window_build(const LayerLaunch& L);
 // FD + best partner per A node (Step 2), fp32 FMA path
 cudaError_t launch_fd_simt(const LayerLaunch& L);
-// windows, FD and selection for bf16 windows of at most 40 nodes a side (Steps 1, 2 and 4): leaves every token's partner
+// windows, FD and selection for windows of at most 40 nodes a side (fp32: 80) in one kernel (Steps 1, 2 and 4): leaves every token's partner
 // and its place for launch_map
-bool fd_stream_supported(int fd_side, int max_cell, int cap_in);
+bool fd_stream_supported(int dtype, int fd_side, int max_cell, int cap_in);
 cudaError_t launch_fd_stream(const LayerLaunch& L);
 // head sum of xi, merge map, weights from the partners (Steps 4, 5); at most kMapMaxTokens per sample
 constexpr int kMapMaxTokens = 16384;

@@ -322,8 +322,8 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
   const bool tc_fd = s.use_tc && tc_fd_supported(c.hidden);
   // Small windows: one kernel finds the windows, scores and selects, and the map kernel finishes (`streaming`; it
   // addresses a sample's rows by 32-bit offsets of 16-byte units).  Otherwise window lists, a tiled FD kernel, selection.
-  const bool streaming = tc_fd && fd_stream_supported(s.fd_side, s.max_cell, s.cap_in) &&
-                         (long long)s.cap_in * a->hidden_row_stride / 8 < 0xffffffffll;
+  const bool streaming = (tc_fd || c.dtype == LIGHTKV_FP32) && fd_stream_supported(c.dtype, s.fd_side, s.max_cell, s.cap_in) &&
+                         (long long)s.cap_in * a->hidden_row_stride * (long long)esz / 16 < 0xffffffffll;
   auto launch_windows = [&](const LayerLaunch& l) { return streaming ? cudaSuccess : launch_window_build(l); };
   auto launch_fd = [&](const LayerLaunch& l) {
     return streaming ? launch_fd_stream(l) : tc_fd ? launch_fd_tc(l) : launch_fd_simt(l);

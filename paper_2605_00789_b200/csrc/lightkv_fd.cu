@@ -27,7 +27,7 @@ namespace lkv {
 // 41 -> 27, of 36: 39 -> 23; 32 x 576 x 5120 in windows of 36: 76 -> 45, of 72: 59 -> 29.
 // ======================================================================================================
 struct FdStreamArgs {
-  const __nv_bfloat16* x;              // first vision row of sample 0
+  const void* x;                       // first vision row of sample 0
   const int* seq_start;                // first row of each sample (packed batches) or nullptr
   int64_t batch_stride, row_stride;    // elements
   int d, metric;
@@ -49,6 +49,11 @@ __device__ __forceinline__ void mma_m16n8k16(float (&c)[4], uint32_t a0, uint32_
 
 __device__ __forceinline__ void st_shared16(uint32_t addr, const uint4& v) {
   asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(addr), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
+}
+__device__ __forceinline__ float4 ld_shared_f4(uint32_t addr) {
+  float4 v;
+  asm volatile("ld.shared.v4.f32 {%0,%1,%2,%3}, [%4];" : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "r"(addr));
+  return v;
 }
 // the quad of lanes takes 64 bytes of a row: ask L2 for the whole 128-byte line at once
 __device__ __forceinline__ void cp_async16_l2(uint32_t smem_dst, const void* gmem_src, uint32_t src_bytes) {
@@ -77,12 +82,14 @@ struct FdStreamSmem {
   }
 };
 
-template <int O, int S, int WARPS>
+template <typename T, int O, int S, int WARPS>
 __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_constant__ FdStreamArgs a) {
   grid_dependency_wait();
   grid_launch_dependents();                              // in this order: see grid_dependency_sync
   using M = FdStreamSmem<O, S, WARPS>;
   constexpr int R = M::R, MT = (O + 1) / 2, PITCH = M::PITCH, nwarps = WARPS, NT = 32 * WARPS;
+  constexpr bool F32 = sizeof(T) == 4;
+  constexpr int EL = 16 / sizeof(T), CH = 4 * EL;         // elements of a 16-byte piece and of a chunk of a row
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* part = reinterpret_cast<float*>(smem_raw);      // [WARPS][R][PITCH] partial inner products
@@ -172,11 +179,13 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
   for (int e = tid; e < na_all; e += NT) { key[e] = 0xffffffffu; best[e] = -1; into[e] = -1; }
 
   const int g = lane >> 2, t = lane & 3;
-  const int nc = (a.d + 31) >> 5, c_lo = warp * nc / WARPS, nk = (warp + 1) * nc / WARPS - c_lo;
-  const __nv_bfloat16* base = a.x + size_t(b) * a.batch_stride + size_t(a.seq_start ? a.seq_start[b] : 0) * a.row_stride +
-                              c_lo * 32 + t * 8;
-  const uint32_t row16 = uint32_t(a.row_stride >> 3);    // row pitch in 16-byte units
-  const uint32_t ring = tc::smem_u32(smem_raw) + (warp * S * 2 * O * 32 + lane) * 16;
+  const int nc = (a.d + CH - 1) / CH, c_lo = warp * nc / WARPS, nk = (warp + 1) * nc / WARPS - c_lo;
+  const T* base = static_cast<const T*>(a.x) + size_t(b) * a.batch_stride +
+                  size_t(a.seq_start ? a.seq_start[b] : 0) * a.row_stride + c_lo * CH + t * EL;
+  const uint32_t row16 = uint32_t(a.row_stride / EL);    // row pitch in 16-byte units
+  // fp32 pieces are read by the whole warp: a row's four pieces are swizzled against bank conflicts
+  const uint32_t warp_ring = tc::smem_u32(smem_raw) + warp * S * 2 * O * 512;
+  const uint32_t ring = warp_ring + (F32 ? g * 64 + ((t ^ ((g >> 1) & 3)) << 4) : lane * 16);
 
   for (int a0 = 0; removed > 0 && a0 < na_all; a0 += R) {     // nothing to remove: no scores needed
     const int na = min(R, na_all - a0);
@@ -196,42 +205,73 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
           for (int st = 0; st < S; ++st) st_shared16(ring + (st * 2 * O + i) * 512, make_uint4(0, 0, 0, 0));
       auto issue = [&](int k, int st) {
         if (k < nk) {
-          const uint32_t bytes = (c_lo + k) * 32 + t * 8 < a.d ? 16u : 0u;    // d is a multiple of 8
-          const __nv_bfloat16* p = base + (bytes ? k * 32 : 0);
+          const uint32_t bytes = (c_lo + k) * CH + t * EL < a.d ? 16u : 0u;   // d is a multiple of 8
+          const T* p = base + (bytes ? k * CH : 0);
 #pragma unroll
           for (int i = 0; i < 2 * O; ++i)
-            if (off[i] != 0xffffffffu) cp_async16_l2(ring + (st * 2 * O + i) * 512, p + size_t(off[i]) * 8, bytes);
+            if (off[i] != 0xffffffffu) cp_async16_l2(ring + (st * 2 * O + i) * 512, p + size_t(off[i]) * EL, bytes);
         }
         tc::cp_async_commit();
       };
-      float acc[MT][O][4];
+      float acc[F32 ? 1 : MT][O][4], accf[F32 ? O : 1][2 * O];
       float ss[2 * O];
 #pragma unroll
       for (int i = 0; i < 2 * O; ++i) ss[i] = 0.f;
 #pragma unroll
-      for (int i = 0; i < MT; ++i)
+      for (int j = 0; j < O; ++j) {
 #pragma unroll
-        for (int j = 0; j < O; ++j)
+        for (int i = 0; i < (F32 ? 1 : MT); ++i)
 #pragma unroll
           for (int q = 0; q < 4; ++q) acc[i][j][q] = 0.f;
+      }
+#pragma unroll
+      for (int i = 0; i < (F32 ? O : 1); ++i)
+#pragma unroll
+        for (int j = 0; j < 2 * O; ++j) accf[i][j] = 0.f;
 
 #pragma unroll
       for (int st = 0; st < S; ++st) issue(st, st);
       for (int k = 0, st = 0; k < nk; ++k) {
-        tc::cp_async_wait<S - 1>();                      // this lane's pieces of chunk k: nobody else reads them
-        uint4 v[2 * O];
+        tc::cp_async_wait<S - 1>();                      // this lane's pieces of chunk k
+        if constexpr (!F32) {                            // nobody else reads them
+          uint4 v[2 * O];
 #pragma unroll
-        for (int i = 0; i < 2 * O; ++i) v[i] = tc::ld_shared16(ring + (st * 2 * O + i) * 512);
+          for (int i = 0; i < 2 * O; ++i) v[i] = tc::ld_shared16(ring + (st * 2 * O + i) * 512);
 #pragma unroll
-        for (int i = 0; i < 2 * O; ++i) ss[i] = sumsq16(v[i], ss[i]);
+          for (int i = 0; i < 2 * O; ++i) ss[i] = sumsq16(v[i], ss[i]);
 #pragma unroll
-        for (int i = 0; i < MT; ++i) {
-          const uint4 lo = v[2 * i], hi = 2 * i + 1 < O ? v[2 * i + 1] : make_uint4(0, 0, 0, 0);
+          for (int i = 0; i < MT; ++i) {
+            const uint4 lo = v[2 * i], hi = 2 * i + 1 < O ? v[2 * i + 1] : make_uint4(0, 0, 0, 0);
 #pragma unroll
-          for (int j = 0; j < O; ++j) {
-            mma_m16n8k16(acc[i][j], lo.x, hi.x, lo.y, hi.y, v[O + j].x, v[O + j].y);
-            mma_m16n8k16(acc[i][j], lo.z, hi.z, lo.w, hi.w, v[O + j].z, v[O + j].w);
+            for (int j = 0; j < O; ++j) {
+              mma_m16n8k16(acc[i][j], lo.x, hi.x, lo.y, hi.y, v[O + j].x, v[O + j].y);
+              mma_m16n8k16(acc[i][j], lo.z, hi.z, lo.w, hi.w, v[O + j].z, v[O + j].w);
+            }
           }
+        } else {
+          // fp32: the warp's lanes hold the pairs (g + 8 i, t + 4 j) and read the chunk's rows from the ring
+          __syncwarp();
+          const uint32_t chunk = warp_ring + st * 2 * O * 512;
+#pragma unroll
+          for (int i = 0; i < 2 * O; ++i) {
+            const float4 v = ld_shared_f4(ring + (st * 2 * O + i) * 512);
+            ss[i] = fmaf(v.w, v.w, fmaf(v.z, v.z, fmaf(v.y, v.y, fmaf(v.x, v.x, ss[i]))));
+          }
+#pragma unroll
+          for (int piece = 0; piece < 4; ++piece) {
+            float4 va[O];
+#pragma unroll
+            for (int i = 0; i < O; ++i) va[i] = ld_shared_f4(chunk + i * 512 + g * 64 + ((piece ^ ((g >> 1) & 3)) << 4));
+#pragma unroll
+            for (int j = 0; j < 2 * O; ++j) {
+              const int rr = t + 4 * (j & 1);
+              const float4 vb = ld_shared_f4(chunk + (O + (j >> 1)) * 512 + rr * 64 + ((piece ^ ((rr >> 1) & 3)) << 4));
+#pragma unroll
+              for (int i = 0; i < O; ++i)
+                accf[i][j] = fmaf(va[i].w, vb.w, fmaf(va[i].z, vb.z, fmaf(va[i].y, vb.y, fmaf(va[i].x, vb.x, accf[i][j]))));
+            }
+          }
+          __syncwarp();                                  // everybody has read the stage before it is filled again
         }
         issue(k + S, st);
         st = st + 1 == S ? 0 : st + 1;
@@ -240,14 +280,21 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
       __syncthreads();                                   // every warp's ring is drained: the partial results go over it
       // ---- partial results of this warp
       float* pw = part + warp * R * PITCH;
+      if constexpr (F32) {
 #pragma unroll
-      for (int i = 0; i < MT; ++i)
+        for (int i = 0; i < O; ++i)
 #pragma unroll
-        for (int j = 0; j < O; ++j) {
-          const int r = 16 * i + g, col = 8 * j + 2 * t;
-          *reinterpret_cast<float2*>(pw + r * PITCH + col) = make_float2(acc[i][j][0], acc[i][j][1]);
-          if (2 * i + 1 < O) *reinterpret_cast<float2*>(pw + (r + 8) * PITCH + col) = make_float2(acc[i][j][2], acc[i][j][3]);
-        }
+          for (int j = 0; j < 2 * O; ++j) pw[(8 * i + g) * PITCH + t + 4 * j] = accf[i][j];
+      } else {
+#pragma unroll
+        for (int i = 0; i < MT; ++i)
+#pragma unroll
+          for (int j = 0; j < O; ++j) {
+            const int r = 16 * i + g, col = 8 * j + 2 * t;
+            *reinterpret_cast<float2*>(pw + r * PITCH + col) = make_float2(acc[i][j][0], acc[i][j][1]);
+            if (2 * i + 1 < O) *reinterpret_cast<float2*>(pw + (r + 8) * PITCH + col) = make_float2(acc[i][j][2], acc[i][j][3]);
+          }
+      }
 #pragma unroll
       for (int i = 0; i < 2 * O; ++i) {
 #pragma unroll
@@ -321,32 +368,36 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
   }
 }
 
-template <int O, int S, int WARPS>
+template <typename T, int O, int S, int WARPS>
 static cudaError_t launch_fd_stream_o(const LayerLaunch& L, const FdStreamArgs& f) {
   const size_t smem = FdStreamSmem<O, S, WARPS>::bytes(f.max_cell, f.cap_in);
-  const cudaError_t e = ensure_dynamic_smem(fd_stream_kernel<O, S, WARPS>, (int)smem);
+  const cudaError_t e = ensure_dynamic_smem(fd_stream_kernel<T, O, S, WARPS>, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_kernel(fd_stream_kernel<O, S, WARPS>, dim3(L.geo.n_windows, L.batch), 32 * WARPS, smem, L.stream, 1, f);
+  return launch_kernel(fd_stream_kernel<T, O, S, WARPS>, dim3(L.geo.n_windows, L.batch), 32 * WARPS, smem, L.stream, 1, f);
 }
 
-// Eight warps split the hidden dimension where each still gets a few chunks of it (hidden > 768); a narrow model gets
-// CTAs of two, so that the fixed cost of a window (its lists, the meeting of the warps) is paid by fewer threads.
+// Eight warps split the hidden dimension where each still gets a few chunks of it (rows of more than 1.5 KB); a narrow
+// model gets CTAs of two, so that the fixed cost of a window (its lists, the meeting of the warps) is paid by fewer
+// threads.
 template <int O, int S>
 static cudaError_t launch_fd_stream_w(const LayerLaunch& L, const FdStreamArgs& f) {
-  return L.hidden > 768 ? launch_fd_stream_o<O, S, 8>(L, f) : launch_fd_stream_o<O, S, 2>(L, f);
+  if (L.dtype == LIGHTKV_FP32)
+    return L.hidden > 384 ? launch_fd_stream_o<float, O, S, 8>(L, f) : launch_fd_stream_o<float, O, S, 2>(L, f);
+  return L.hidden > 768 ? launch_fd_stream_o<__nv_bfloat16, O, S, 8>(L, f) : launch_fd_stream_o<__nv_bfloat16, O, S, 2>(L, f);
 }
 
 // Five groups of eight rows a side is what the fragments of a thread hold at two CTAs per SM; beyond that the tcgen05
-// kernel shares the rows between more pairs.  The lists of a window and the search for its tokens have to fit in
-// shared memory beside the ring, and the map kernel behind takes two tokens per thread of eight CTAs.
-bool fd_stream_supported(int fd_side, int max_cell, int cap_in) {
-  return fd_side > 0 && fd_side <= 40 && max_cell <= 4096 && cap_in <= kMapMaxTokens;
+// kernel shares the rows between more pairs (in fp32, where the FMAs bound the work, windows of two blocks a side still
+// gain).  The lists of a window and the search for its tokens have to fit in shared memory beside the ring, and the map
+// kernel behind takes two tokens per thread of eight CTAs.
+bool fd_stream_supported(int dtype, int fd_side, int max_cell, int cap_in) {
+  return fd_side > 0 && fd_side <= (dtype == LIGHTKV_FP32 ? 80 : 40) && max_cell <= 4096 && cap_in <= kMapMaxTokens;
 }
 
 cudaError_t launch_fd_stream(const LayerLaunch& L) {
   const lightkv_layer_args_t* a = L.a;
   FdStreamArgs f;
-  f.x = static_cast<const __nv_bfloat16*>(a->hidden) + size_t(a->vis_begin) * a->hidden_row_stride;
+  f.x = static_cast<const char*>(a->hidden) + size_t(a->vis_begin) * a->hidden_row_stride * (L.dtype == LIGHTKV_FP32 ? 4 : 2);
   f.seq_start = a->seq_start;
   f.batch_stride = a->hidden_batch_stride; f.row_stride = a->hidden_row_stride;
   f.d = L.hidden; f.metric = L.divergence; f.keep = L.keep; f.g = L.geo; f.n_vis = a->n_vis; f.pos = a->pos;

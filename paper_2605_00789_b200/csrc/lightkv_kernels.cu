@@ -328,12 +328,15 @@ cudaError_t launch_fd_simt(const LayerLaunch& L) {
 
 // =====================================================================================================
 // xi per head, fp32 FMA path (Eq. "attention-factor" with the causal softmax rows of Eq.
-// "attention-matrix").  One CTA per (tile of 32 vision queries, head, sample).  Keys 0..s_i are visited
-// in tiles of 64 with an online (running-maximum) softmax that carries two sums per row: all visible
+// "attention-matrix").  One CTA per (tile of 64 vision queries, head, sample), longest rows first.  Keys 0..s_i are
+// visited in tiles of 64 with an online (running-maximum) softmax that carries two sums per row: all visible
 // keys and the prompt keys J.  Output per head: sum_J / sum_all.  With a caller-supplied row
 // log-sum-exp only the prompt keys are visited: sum_J exp(logit - lse).
+// A thread holds 4 x 4 logits and reads both operands 16 bytes along the head dimension (8 shared-memory loads per 64
+// FMAs, rows padded by four floats: no bank conflicts); the 16 threads of a row meet by shuffles, the groups at the end.  2 x 576 queries x 8
+// heads of 128 in fp32: 140 us with 2 x 4 logits per thread and scalar loads, 23 now.
 // =====================================================================================================
-constexpr int XI_TQ = 32, XI_TK = 64;
+constexpr int XI_TQ = 32, XI_TK = 64, XI_GROUP = 4 * XI_TQ, XI_GROUPS = 4;
 
 template <typename T>
 struct XiSimtArgs {
@@ -349,16 +352,16 @@ struct XiSimtArgs {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(XI_GROUP * XI_GROUPS)
 xi_simt_kernel(XiSimtArgs<T> a, Workspace ws) {
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int dh = a.dh, ld = dh + 1;
+  const int dh = a.dh, ld = dh + 4;
   float* Qs = reinterpret_cast<float*>(smem_raw);       // [XI_TQ][ld]
-  float* Ks = Qs + XI_TQ * ld;                          // [XI_TK][ld]
-  float* Ss = Ks + XI_TK * ld;                          // [XI_TQ][XI_TK + 1]
+  float* Ks = Qs + XI_TQ * ld;                          // [groups][XI_TK][ld]
 
-  const int b = blockIdx.z, h = blockIdx.y, t0 = blockIdx.x * XI_TQ, tid = threadIdx.x;
+  const int b = blockIdx.z, h = blockIdx.y, t0 = (gridDim.x - 1 - blockIdx.x) * XI_TQ;
+  const int grp = threadIdx.x / XI_GROUP, groups = blockDim.x / XI_GROUP, tid = threadIdx.x - grp * XI_GROUP;
   int n = a.n_vis ? min(a.n_vis[b], ws.cap_in) : ws.cap_in;
   if (t0 >= n) return;
   const int nq = min(XI_TQ, n - t0);
@@ -370,100 +373,116 @@ xi_simt_kernel(XiSimtArgs<T> a, Workspace ws) {
   const int vis_begin = a.vis_begin;
   const int n_seq = vis_begin + n + a.n_text_after;                   // keys of this sample
 
-  for (int idx = tid; idx < XI_TQ * (dh / 4); idx += blockDim.x) {
-    const int r = idx / (dh / 4), c = (idx % (dh / 4)) * 4;
-    float f[4] = {0.f, 0.f, 0.f, 0.f};
-    if (r < nq) load4<T>(qh + size_t(vis_begin + t0 + r) * a.q_rs + c, f);
-#pragma unroll
-    for (int j = 0; j < 4; ++j) Qs[r * ld + c + j] = f[j];
-  }
+  const int q4 = dh / 4;
+  auto stage = [&](float* dst, const T* src, int64_t row_stride, int rows, int all, int first, int step) {   // rows of dh values, zeros behind them
+    if constexpr (sizeof(T) == 4) {
+      for (int idx = first; idx < all * q4; idx += step) {
+        const int r = idx / q4, c = (idx - r * q4) * 4;
+        tc::cp_async16(tc::smem_u32(dst + r * ld + c), src + size_t(r < rows ? r : 0) * row_stride + c, r < rows ? 16u : 0u);
+      }
+      tc::cp_async_commit();
+    } else {
+#pragma unroll 4
+      for (int idx = first; idx < all * q4; idx += step) {
+        const int r = idx / q4, c = (idx - r * q4) * 4;
+        float f[4] = {0.f, 0.f, 0.f, 0.f};
+        if (r < rows) load4<T>(src + size_t(r) * row_stride + c, f);
+        *reinterpret_cast<float4*>(dst + r * ld + c) = make_float4(f[0], f[1], f[2], f[3]);
+      }
+    }
+  };
+  stage(Qs, qh + size_t(vis_begin + t0) * a.q_rs, a.q_rs, nq, XI_TQ, threadIdx.x, blockDim.x);
+  tc::cp_async_wait<0>();
+  __syncthreads();
 
-  const int tx = tid & 15, ty = tid >> 4;
-  const int lane = tid & 31, wp = tid >> 5;             // softmax: warp wp owns rows 4*wp .. 4*wp+3
-  float m_run[4], l_all[4], l_txt[4];
+  const int tx = tid & 15, ty = tid >> 4;               // rows 4 ty + i, columns tx + 16 j
+  float m_run[4], l_all[4], l_txt[4], l2[4];
 #pragma unroll
-  for (int i = 0; i < 4; ++i) { m_run[i] = -INFINITY; l_all[i] = 0.f; l_txt[i] = 0.f; }
+  for (int i = 0; i < 4; ++i) {
+    m_run[i] = -INFINITY; l_all[i] = 0.f; l_txt[i] = 0.f; l2[i] = 0.f;
+    if (a.lse && 4 * ty + i < nq)
+      l2[i] = a.lse[size_t(b) * a.lse_bs + size_t(h) * a.lse_hs + row0 + vis_begin + t0 + 4 * ty + i] * 1.4426950408889634f;
+  }
 
   // last key any row of the tile may see: its own (causal) or the sample's last (bidirectional)
   const int s_last = a.bidirectional ? n_seq - 1 : vis_begin + t0 + nq - 1;
   const int key_lo = a.lse ? a.text.begin : 0;
   const int key_hi = a.lse ? min(a.text.end, s_last + 1) : s_last + 1;
 
-  for (int j0 = key_lo; j0 < key_hi; j0 += XI_TK) {
-    const int nk = min(XI_TK, key_hi - j0);
-    __syncthreads();
-    for (int idx = tid; idx < XI_TK * (dh / 4); idx += blockDim.x) {
-      const int r = idx / (dh / 4), c = (idx % (dh / 4)) * 4;
-      float f[4] = {0.f, 0.f, 0.f, 0.f};
-      if (r < nk) load4<T>(kh + size_t(j0 + r) * a.k_rs + c, f);
+  const float* Kt = Ks + grp * XI_TK * ld;
+  for (int j0 = key_lo + grp * XI_TK; j0 < key_hi; j0 += groups * XI_TK) {
+    stage(Ks + grp * XI_TK * ld, kh + size_t(j0) * a.k_rs, a.k_rs, min(XI_TK, key_hi - j0), XI_TK, tid, XI_GROUP);
+    tc::cp_async_wait<0>();
+    tc::named_barrier(1 + grp, XI_GROUP);
+    float acc[4][4] = {};
+#pragma unroll 2
+    for (int kk = 0; kk < dh; kk += 4) {
+      float4 q[4], k[4];
 #pragma unroll
-      for (int j = 0; j < 4; ++j) Ks[r * ld + c + j] = f[j];
+      for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const float4*>(Qs + (4 * ty + i) * ld + kk);
+#pragma unroll
+      for (int j = 0; j < 4; ++j) k[j] = *reinterpret_cast<const float4*>(Kt + (tx + 16 * j) * ld + kk);
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          acc[i][j] = fmaf(q[i].w, k[j].w, fmaf(q[i].z, k[j].z, fmaf(q[i].y, k[j].y, fmaf(q[i].x, k[j].x, acc[i][j]))));
     }
-    __syncthreads();
-    float acc[2][4] = {};
-    for (int kk = 0; kk < dh; ++kk) {
-      const float a0 = Qs[(2 * ty) * ld + kk], a1 = Qs[(2 * ty + 1) * ld + kk];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float bv = Ks[(4 * tx + j) * ld + kk];
-        acc[0][j] = fmaf(a0, bv, acc[0][j]);
-        acc[1][j] = fmaf(a1, bv, acc[1][j]);
-      }
-    }
-#pragma unroll
-    for (int i = 0; i < 2; ++i)
-#pragma unroll
-      for (int j = 0; j < 4; ++j) Ss[(2 * ty + i) * (XI_TK + 1) + 4 * tx + j] = acc[i][j] * scale2;
-    __syncthreads();
-    const unsigned long long tmask = a.text.mask64(j0);      // XI_TK = 64 columns
+    const unsigned long long tmask = a.text.mask64(j0) >> tx;          // bits 0, 16, 32, 48: this thread's columns
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      const int r = 4 * wp + i;
-      if (r >= nq) continue;                            // warp-uniform
-      const int s_i = vis_begin + t0 + r;
-      const int last = a.bidirectional ? n_seq - 1 : s_i;
-      float v[2];
-      bool ok[2], txt[2];
+      const int last = (a.bidirectional ? n_seq - 1 : vis_begin + t0 + 4 * ty + i) - j0 - tx;   // visible: 16 j <= last
+      float v[4];
 #pragma unroll
-      for (int c = 0; c < 2; ++c) {
-        const int j = j0 + lane + 32 * c;
-        ok[c] = (lane + 32 * c < nk) && j <= last;
-        txt[c] = ok[c] && ((tmask >> (lane + 32 * c)) & 1ull);
-        v[c] = ok[c] ? Ss[r * (XI_TK + 1) + lane + 32 * c] : -INFINITY;
-      }
+      for (int j = 0; j < 4; ++j) v[j] = 16 * j <= last && j0 + tx + 16 * j < key_hi ? acc[i][j] * scale2 : -INFINITY;
       if (a.lse) {
-        const float l2 = a.lse[size_t(b) * a.lse_bs + size_t(h) * a.lse_hs + row0 + s_i] * 1.4426950408889634f;
-        float p = (txt[0] ? exp2f(v[0] - l2) : 0.f) + (txt[1] ? exp2f(v[1] - l2) : 0.f);
-        for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
-        l_txt[i] += p;
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          if ((tmask >> (16 * j)) & 1ull) l_txt[i] += exp2f(v[j] - l2[i]);
         continue;
       }
-      float mx = fmaxf(v[0], v[1]);
-      for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float m_new = fmaxf(m_run[i], mx);          // finite: key 0 is visible to every query
-      const float p0 = ok[0] ? exp2f(v[0] - m_new) : 0.f, p1 = ok[1] ? exp2f(v[1] - m_new) : 0.f;
-      float sa = p0 + p1, st = (txt[0] ? p0 : 0.f) + (txt[1] ? p1 : 0.f);
-      for (int o = 16; o > 0; o >>= 1) {
-        sa += __shfl_xor_sync(0xffffffffu, sa, o);
-        st += __shfl_xor_sync(0xffffffffu, st, o);
-      }
-      const float resc = exp2f(m_run[i] - m_new);       // 0 on the first tile (m_run = -inf)
-      l_all[i] = l_all[i] * resc + sa;
-      l_txt[i] = l_txt[i] * resc + st;
-      m_run[i] = m_new;
-    }
-  }
-  if (lane == 0) {
+      float mx = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
 #pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int r = 4 * wp + i;
-      if (r < nq) {
-        ws.xi_h[(size_t(b) * a.n_q_heads + h) * ws.cap_in + t0 + r] = a.lse ? l_txt[i] : l_txt[i] / l_all[i];
-        if (a.lse_out)
-          a.lse_out[size_t(b) * a.lse_out_bs + size_t(h) * a.lse_out_hs + row0 + vis_begin + t0 + r] =
-              (m_run[i] + log2f(l_all[i])) * 0.6931471805599453f;
+      for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+      const float m_new = fmaxf(m_run[i], mx);
+      if (m_new == -INFINITY) continue;                 // the row sees none of this group's keys yet (uniform over the row)
+      const float resc = exp2f(m_run[i] - m_new);       // 0 on the first tile (m_run = -inf)
+      l_all[i] *= resc;
+      l_txt[i] *= resc;
+      m_run[i] = m_new;
+#pragma unroll
+      for (int j = 0; j < 4; ++j) {
+        const float p = exp2f(v[j] - m_new);
+        l_all[i] += p;
+        if ((tmask >> (16 * j)) & 1ull) l_txt[i] += p;
       }
     }
+    tc::named_barrier(1 + grp, XI_GROUP);               // the tile has been read: its buffer is filled next
+  }
+  // ---- the groups' results of a row meet
+  __shared__ float s_m[XI_GROUPS][XI_TQ], s_all[XI_GROUPS][XI_TQ], s_txt[XI_GROUPS][XI_TQ];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) {
+      l_all[i] += __shfl_xor_sync(0xffffffffu, l_all[i], o);
+      l_txt[i] += __shfl_xor_sync(0xffffffffu, l_txt[i], o);
+    }
+    if (tx == 0) { s_m[grp][4 * ty + i] = m_run[i]; s_all[grp][4 * ty + i] = l_all[i]; s_txt[grp][4 * ty + i] = l_txt[i]; }
+  }
+  __syncthreads();
+  const int r = threadIdx.x;
+  if (r < nq) {
+    float m = s_m[0][r], all = 0.f, txt = 0.f;          // finite without a given log-sum-exp: key 0 is visible to every query
+    for (int k = 1; k < groups; ++k) m = fmaxf(m, s_m[k][r]);
+    for (int k = 0; k < groups; ++k) {
+      const float f = a.lse ? 1.f : exp2f(s_m[k][r] - m);
+      all += s_all[k][r] * f;
+      txt += s_txt[k][r] * f;
+    }
+    ws.xi_h[(size_t(b) * a.n_q_heads + h) * ws.cap_in + t0 + r] = a.lse ? txt : txt / all;
+    if (a.lse_out)
+      a.lse_out[size_t(b) * a.lse_out_bs + size_t(h) * a.lse_out_hs + row0 + vis_begin + t0 + r] = (m + log2f(all)) * 0.6931471805599453f;
   }
 }
 
@@ -471,7 +490,8 @@ template <typename T>
 static cudaError_t launch_xi_simt_t(const LayerLaunch& L) {
   const lightkv_layer_args_t* a = L.a;
   const int dh = L.head_dim;
-  const size_t smem = (size_t(XI_TQ + XI_TK) * (dh + 1) + size_t(XI_TQ) * (XI_TK + 1)) * sizeof(float);
+  const int groups = dh <= 128 ? XI_GROUPS : XI_GROUPS / 2;      // key tiles of a CTA within shared memory
+  const size_t smem = size_t(XI_TQ + groups * XI_TK) * (dh + 4) * sizeof(float);
   const dim3 grid((L.ws.cap_in + XI_TQ - 1) / XI_TQ, L.n_q_heads, L.batch);
   XiSimtArgs<T> x;
   x.q = static_cast<const T*>(a->q); x.q_bs = a->q_batch_stride; x.q_hs = a->q_head_stride; x.q_rs = a->q_row_stride;
@@ -482,9 +502,9 @@ static cudaError_t launch_xi_simt_t(const LayerLaunch& L) {
   x.n_vis = a->n_vis; x.seq_start = a->seq_start;
   x.vis_begin = a->vis_begin; x.n_text_after = a->n_text_after; x.bidirectional = a->bidirectional;
   x.n_q_heads = L.n_q_heads; x.n_kv_heads = L.n_kv_heads; x.dh = dh; x.text = L.text;
-  const cudaError_t e = ensure_dynamic_smem(xi_simt_kernel<T>, 160 * 1024);
+  const cudaError_t e = ensure_dynamic_smem(xi_simt_kernel<T>, 176 * 1024);
   if (e != cudaSuccess) return e;
-  return launch_kernel(xi_simt_kernel<T>, grid, 256, smem, L.stream, 1, x, L.ws);
+  return launch_kernel(xi_simt_kernel<T>, grid, groups * XI_GROUP, smem, L.stream, 1, x, L.ws);
 }
 
 cudaError_t launch_xi_simt(const LayerLaunch& L) {

@@ -591,7 +591,8 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
   grid_dependency_wait();
 }
 
-bool tc_xi_supported(int head_dim) { return head_dim == 64 || head_dim == 128; }
+// A head of up to 64 (128) columns takes the kernel for 64 (128): the TMA loads fill the columns it lacks with zeros.
+bool tc_xi_supported(int head_dim) { return head_dim <= 128; }
 
 static int sm_count();
 
@@ -622,15 +623,16 @@ cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first) {
   // and as many CTAs as stay resident walk them round-robin.
   const dim3 grid((unsigned)(x.lse ? std::min<long long>(n_items, XT_CTAS * sm_count()) : n_items));
   // Q tiles + K ring (LSE: two Q tiles, one K stage; otherwise one Q tile, XT_STAGES K stages) + control block + exchange
-  const size_t smem = size_t(L.head_dim / 64) * (x.lse ? 2 * 16384 + XT_KEY_TILE * 128
+  const int halves = L.head_dim <= 64 ? 1 : 2;
+  const size_t smem = size_t(halves) * (x.lse ? 2 * 16384 + XT_KEY_TILE * 128
                                                         : 16384 + size_t(XT_STAGES) * XT_KEY_TILE * 128) + 1024 + 384 + 1536;
   auto launch = [&](auto kernel) -> cudaError_t {
     const cudaError_t rc = ensure_dynamic_smem(kernel, (int)smem);
     if (rc != cudaSuccess) return rc;
     return launch_kernel(kernel, grid, XT_THREADS, smem, L.stream, 1, qm, km, x);
   };
-  if (x.lse) return L.head_dim == 128 ? launch(xi_tc_kernel<128, true>) : launch(xi_tc_kernel<64, true>);
-  return L.head_dim == 128 ? launch(xi_tc_kernel<128, false>) : launch(xi_tc_kernel<64, false>);
+  if (x.lse) return halves == 2 ? launch(xi_tc_kernel<128, true>) : launch(xi_tc_kernel<64, true>);
+  return halves == 2 ? launch(xi_tc_kernel<128, false>) : launch(xi_tc_kernel<64, false>);
 }
 
 // ======================================================================================================
