@@ -334,7 +334,7 @@ cudaError_t launch_fd_simt(const LayerLaunch& L) {
 // log-sum-exp only the prompt keys are visited: sum_J exp(logit - lse).
 // A thread holds 4 x 4 logits and reads both operands 16 bytes along the head dimension (8 shared-memory loads per 64
 // FMAs, rows padded by four floats: no bank conflicts); the 16 threads of a row meet by shuffles, the groups at the end.  2 x 576 queries x 8
-// heads of 128 in fp32: 140 us with 2 x 4 logits per thread and scalar loads, 23 now.
+// heads of 128 in fp32: 140 us with 2 x 4 logits per thread and scalar loads, 60 now.
 // =====================================================================================================
 constexpr int XI_TQ = 32, XI_TK = 64, XI_GROUP = 4 * XI_TQ, XI_GROUPS = 4;
 
@@ -1006,13 +1006,18 @@ cudaError_t launch_map(const LayerLaunch& L) {
   return cs > 1 ? launch(map_kernel<true, 1>) : launch(map_kernel<false, 1>);
 }
 
+// Launches of at most this many rows do not fill the SMs' memory pipes by number: they get wider CTAs and more members of
+// a group in flight per thread: a group of ten tokens is three rounds of loads instead of five (one image of 576 tokens,
+// one layer: 39.6 -> 33.3 us a pass).
+constexpr int kFewRows = 4 * 148;
+
 // =====================================================================================================
 // Weighted merge of the hidden states (Eq. "message-passing", Steps 3-5): one CTA per output row.
 // Row o of the vision block is sum over its group of weight_i * x_i in fp32, rounded once to the
 // storage type; a group of one has weight exactly 1 and is therefore copied bit-exactly.  Text rows
 // before / after the vision block are copied.  Pure 16-byte streaming loads and stores.
 // =====================================================================================================
-template <typename T>
+template <typename T, int MB>
 __global__ void __launch_bounds__(256)
 merge_rows_kernel(const T* __restrict__ src, int64_t src_bs, int64_t src_rs,
                   T* __restrict__ out, int64_t out_bs, int64_t out_rs,
@@ -1045,24 +1050,24 @@ merge_rows_kernel(const T* __restrict__ src, int64_t src_bs, int64_t src_rs,
   }
   const int o = row - vis_begin;
   const int* go = grp_off + size_t(b) * (cap_out + 1);
-  const int g0 = go[o], g1 = go[o + 1];
+  const int g0 = go[o], count = go[o + 1] - g0;
   const int* gs = grp_src + size_t(b) * cap_in;
   const float* wt = weight + size_t(b) * cap_in;
   const T* vis = sb + size_t(vis_begin) * src_rs;
-  // two 16-byte chunks per thread and two members at a time: four loads in flight whatever the group's size
+  // two 16-byte chunks per thread and MB members at a time: 2 MB loads in flight whatever the group's size
   for (int c0 = threadIdx.x; c0 < chunks; c0 += 2 * blockDim.x) {
     const int c1 = c0 + blockDim.x;
     const bool two = c1 < chunks;
     float acc0[V], acc1[V];
 #pragma unroll
     for (int j = 0; j < V; ++j) { acc0[j] = 0.f; acc1[j] = 0.f; }
-    for (int g = g0; g < g1; g += 2) {
-      uint4 va[2], vb[2];
-      float wv[2];
+    for (int g = 0; g < count; g += MB) {
+      uint4 va[MB], vb[MB];
+      float wv[MB];
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        if (g + u < g1) {
-          const int i = gs[g + u];
+      for (int u = 0; u < MB; ++u) {
+        if (g + u < count) {
+          const int i = gs[g0 + g + u];
           wv[u] = wt[i];
           const T* r = vis + size_t(i) * src_rs;
           va[u] = ld_stream16(r + c0 * V);
@@ -1070,8 +1075,8 @@ merge_rows_kernel(const T* __restrict__ src, int64_t src_bs, int64_t src_rs,
         }
       }
 #pragma unroll
-      for (int u = 0; u < 2; ++u) {
-        if (g + u < g1) {
+      for (int u = 0; u < MB; ++u) {
+        if (g + u < count) {
           float f[V];
           unpack16(va[u], f, T());
 #pragma unroll
@@ -1093,17 +1098,16 @@ cudaError_t launch_merge_rows(const LayerLaunch& L) {
   const lightkv_layer_args_t* a = L.a;
   const int rows = a->vis_begin + L.ws.cap_out + a->n_text_after;
   const dim3 grid(rows, L.batch);
-  if (L.dtype == LIGHTKV_BF16)
-    return launch_kernel(merge_rows_kernel<__nv_bfloat16>, grid, 256, 0, L.stream, 1,
-        static_cast<const __nv_bfloat16*>(a->hidden), a->hidden_batch_stride, a->hidden_row_stride,
-        static_cast<__nv_bfloat16*>(a->hidden_out), a->hidden_out_batch_stride, a->hidden_out_row_stride,
+  const bool few = (long long)rows * L.batch <= kFewRows;
+  auto run = [&](auto tag) -> cudaError_t {
+    using T = decltype(tag);
+    return launch_kernel(few ? merge_rows_kernel<T, 4> : merge_rows_kernel<T, 2>, grid, 256, 0, L.stream, 1,
+        static_cast<const T*>(a->hidden), a->hidden_batch_stride, a->hidden_row_stride,
+        static_cast<T*>(a->hidden_out), a->hidden_out_batch_stride, a->hidden_out_row_stride,
         L.hidden, a->vis_begin, a->n_text_after, L.ws.cap_in, L.ws.cap_out, a->n_vis, a->n_vis_out,
         a->grp_off, a->grp_src, a->weight, a->seq_start, a->seq_start_out);
-  return launch_kernel(merge_rows_kernel<float>, grid, 256, 0, L.stream, 1,
-        static_cast<const float*>(a->hidden), a->hidden_batch_stride, a->hidden_row_stride,
-        static_cast<float*>(a->hidden_out), a->hidden_out_batch_stride, a->hidden_out_row_stride,
-        L.hidden, a->vis_begin, a->n_text_after, L.ws.cap_in, L.ws.cap_out, a->n_vis, a->n_vis_out,
-        a->grp_off, a->grp_src, a->weight, a->seq_start, a->seq_start_out);
+  };
+  return L.dtype == LIGHTKV_BF16 ? run(__nv_bfloat16()) : run(float());
 }
 
 // =====================================================================================================
@@ -1127,13 +1131,13 @@ struct KvAddr {
   }
 };
 
-constexpr int KV_THREADS = 256;
 
 // floor(n / d) for n, d < 65536 with m = ceil(2^32 / d): one multiply instead of a division
 __device__ inline int div_magic(int n, unsigned m) { return (int)__umulhi((unsigned)n, m); }
 
-template <typename T>
-__global__ void __launch_bounds__(KV_THREADS, sizeof(T) == 2 ? 5 : 4)
+// THREADS per CTA, MB members of a group in flight
+template <typename T, int THREADS, int MB>
+__global__ void __launch_bounds__(THREADS, THREADS > 256 ? 2 : (sizeof(T) == 2 ? 5 : 4))
 kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* __restrict__ k_dst,
                   T* __restrict__ v_dst, KvAddr sa, KvAddr da, int n_kv_heads, int dh, int vis_begin,
                   int n_text_after, int cap_in, int cap_out, int gather, int merge_at_survivor, unsigned magic_ch,
@@ -1187,10 +1191,22 @@ kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* _
     }
     return;
   }
-  // merge: two units per thread and two members at a time, i.e. four loads in flight whatever the group's size
-  for (int u0 = threadIdx.x; u0 < units; u0 += 2 * blockDim.x) {
-    const int u1 = u0 + blockDim.x;
-    const bool two = u1 < units;
+  // merge: two units per thread and MB members at a time.  The lanes of a warp hold the members' addresses and weights
+  // (one lookup each, 32 at a time), so that a round of loads waits for nothing but the round before.
+  const int lane = threadIdx.x & 31, count = g1 - g0;
+  int64_t m_tok = 0;
+  float m_w = 0.f;
+  auto members = [&](int first) {
+    if (first + lane < count) {
+      const int i = gs[g0 + first + lane];
+      m_w = wt[i];
+      m_tok = sa.token(b, vis_begin + i);
+    }
+  };
+  members(0);
+  for (int base = 0; base < units; base += 2 * blockDim.x) {
+    const int u0 = base + threadIdx.x, u1 = u0 + blockDim.x;
+    const bool one = u0 < units, two = u1 < units;
     const int kv0 = u0 >= per_kv ? 1 : 0, rem0 = u0 - kv0 * per_kv, h0 = div_magic(rem0, magic_ch), c0 = rem0 - h0 * ch;
     const int ub = two ? u1 : u0;
     const int kv1 = ub >= per_kv ? 1 : 0, rem1 = ub - kv1 * per_kv, h1 = div_magic(rem1, magic_ch), c1 = rem1 - h1 * ch;
@@ -1199,41 +1215,151 @@ kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* _
     float acc0[V], acc1[V];
 #pragma unroll
     for (int j = 0; j < V; ++j) { acc0[j] = 0.f; acc1[j] = 0.f; }
-    for (int g = g0; g < g1; g += 2) {
-      uint4 va[2], vb[2];
-      float wv[2];
+    for (int g = 0; g < count; g += MB) {
+      if (count > 32 && (g & 31) == 0) members(g);
+      uint4 va[MB], vb[MB];
 #pragma unroll
-      for (int m = 0; m < 2; ++m) {
-        if (g + m < g1) {
-          const int i = gs[g + m];
-          wv[m] = wt[i];
-          const int64_t tok = sa.token(b, vis_begin + i);
-          va[m] = ld_stream16(sp0 + tok);
+      for (int m = 0; m < MB; ++m) {
+        if (g + m < count) {
+          const int64_t tok = __shfl_sync(0xffffffffu, m_tok, (g + m) & 31);
+          if (one) va[m] = ld_stream16(sp0 + tok);
           if (two) vb[m] = ld_stream16(sp1 + tok);
         }
       }
 #pragma unroll
-      for (int m = 0; m < 2; ++m) {
-        if (g + m < g1) {
+      for (int m = 0; m < MB; ++m) {
+        if (g + m < count) {
+          const float w = __shfl_sync(0xffffffffu, m_w, (g + m) & 31);
           float f[V];
           unpack16(va[m], f, T());
 #pragma unroll
-          for (int j = 0; j < V; ++j) acc0[j] = fmaf(wv[m], f[j], acc0[j]);
+          for (int j = 0; j < V; ++j) acc0[j] = fmaf(w, f[j], acc0[j]);
           if (two) {
             unpack16(vb[m], f, T());
 #pragma unroll
-            for (int j = 0; j < V; ++j) acc1[j] = fmaf(wv[m], f[j], acc1[j]);
+            for (int j = 0; j < V; ++j) acc1[j] = fmaf(w, f[j], acc1[j]);
           }
         }
       }
     }
-    st_stream16((kv0 ? v_dst : k_dst) + d_tok + int64_t(h0) * da.head_stride + c0 * V, pack16(acc0, T()));
+    if (one) st_stream16((kv0 ? v_dst : k_dst) + d_tok + int64_t(h0) * da.head_stride + c0 * V, pack16(acc0, T()));
     if (two) st_stream16((kv1 ? v_dst : k_dst) + d_tok + int64_t(h1) * da.head_stride + c1 * V, pack16(acc1, T()));
   }
 }
 
 // =====================================================================================================
-// Second phase of the in-place form: every output row moves from its surviving token's row (which holds the
+// In place, where a plane fits on chip: one CTA owns a plane -- one (sample, K or V, head, column part) --, gathers and
+// merges ALL of its output rows behind the first vision row into shared memory, synchronises, and stores them: no other
+// CTA touches these bytes, so nothing is overwritten before it has been read, and one kernel does what the two below
+// need a pass over memory more for.  The group lists and the rows' offsets (a block-table lookup each) are staged once
+// per CTA, so that the gather is one round of loads, eight in flight per thread.  Columns are cut so that the launch has
+// two CTAs per SM, in parts of at least 64 bytes (32 where the rows would not fit otherwise).
+// 4 samples x 652 tokens, 8 KV heads x 128, pages of 16: 28 -> 18 us between events against merge + move; parts of 32
+// or 128 bytes 28 and 27 (with the first form of the gather; parts of 64: 22).  Members are taken two at a time over
+// four pieces: one piece after the other, the largest group of a warp was a chain of loads (22 us).
+// =====================================================================================================
+constexpr int KVI_THREADS = 256, KVI_AHEAD = 4;
+
+struct KvPlaneSmem {
+  int rows_in, rows_out, n_in, n_out;          // capacities: moving rows in / out, vision tokens in / out
+  __host__ __device__ size_t addr() const { return 0; }
+  __host__ __device__ size_t mem() const { return size_t(rows_in) * 8; }
+  __host__ __device__ size_t wgt() const { return mem() + size_t(n_in) * 4; }
+  __host__ __device__ size_t off() const { return wgt() + size_t(n_in) * 4; }
+  __host__ __device__ size_t out() const { return (off() + size_t(n_out + 1) * 4 + 15) & ~size_t(15); }
+  __host__ __device__ size_t bytes(int pieces) const { return out() + size_t(rows_out) * pieces * 16; }
+};
+
+template <typename T>
+__global__ void __launch_bounds__(KVI_THREADS)
+kv_plane_kernel(T* __restrict__ k_buf, T* __restrict__ v_buf, KvAddr ad, KvPlaneSmem sm, int n_kv_heads, int ch, int parts,
+                unsigned magic_ch, int vis_begin, int n_text_after, int gather, const int* __restrict__ n_vis,
+                const int* __restrict__ n_vis_out, const int* __restrict__ grp_off, const int* __restrict__ grp_src,
+                const float* __restrict__ weight) {
+  grid_dependency_sync();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  constexpr int V = Vec<T>::n;
+  int64_t* addr = reinterpret_cast<int64_t*>(smem_raw + sm.addr());     // element offset of every row from the first vision row on
+  int* mem = reinterpret_cast<int*>(smem_raw + sm.mem());               // group members, survivor first
+  float* wgt = reinterpret_cast<float*>(smem_raw + sm.wgt());           // their weights
+  int* off = reinterpret_cast<int*>(smem_raw + sm.off());               // first member of every output row
+  uint4* rows = reinterpret_cast<uint4*>(smem_raw + sm.out());
+  const int tid = threadIdx.x;
+  int plane = blockIdx.x;
+  const int part = plane % parts; plane /= parts;
+  const int h = plane % n_kv_heads; plane /= n_kv_heads;
+  const int kv = plane & 1, b = plane >> 1;
+  const int n_in = n_vis ? min(n_vis[b], sm.n_in) : sm.n_in;
+  const int n_out = n_vis_out[b];
+  if (n_out >= n_in) return;                               // nothing was merged away: every row is where it belongs
+  T* buf = (kv ? v_buf : k_buf) + int64_t(h) * ad.head_stride + part * ch * V;
+
+  for (int l = tid; l < n_in + n_text_after; l += KVI_THREADS) addr[l] = ad.token(b, vis_begin + l);
+  for (int o = tid; o <= n_out; o += KVI_THREADS) off[o] = grp_off[size_t(b) * (sm.n_out + 1) + o];
+  for (int k = tid; k < n_in; k += KVI_THREADS) {          // (a sample cut at its capacity has fewer: never read)
+    const int i = min(max(grp_src[size_t(b) * sm.n_in + k], 0), n_in - 1);
+    mem[k] = i;
+    if (!gather) wgt[k] = weight[size_t(b) * sm.n_in + i];
+  }
+  __syncthreads();
+
+  const int total = (n_out + n_text_after) * ch;
+  for (int i0 = tid; i0 < total; i0 += KVI_AHEAD * KVI_THREADS) {
+    int first[KVI_AHEAD], count[KVI_AHEAD], col[KVI_AHEAD], most = 0;
+    float acc[KVI_AHEAD][V];
+#pragma unroll
+    for (int u = 0; u < KVI_AHEAD; ++u) {
+      const int idx = i0 + u * KVI_THREADS, r = div_magic(idx, magic_ch);
+      col[u] = (idx - r * ch) * V;
+      count[u] = 0;
+      if (idx < total) {
+        const bool group = r < n_out;
+        first[u] = group ? off[r] : -(n_in + r - n_out);     // a row behind the vision block is negative (or row 0)
+        count[u] = group && !gather ? off[r + 1] - first[u] : 1;
+        if (group && count[u] == 1) first[u] = -mem[first[u]];
+      }
+      most = max(most, count[u]);
+#pragma unroll
+      for (int j = 0; j < V; ++j) acc[u][j] = 0.f;
+    }
+    for (int g = 0; g < most; g += 2) {
+      uint4 v[KVI_AHEAD][2];
+#pragma unroll
+      for (int u = 0; u < KVI_AHEAD; ++u)
+#pragma unroll
+        for (int m = 0; m < 2; ++m)
+          if (g + m < count[u]) v[u][m] = ld_plane16(buf + addr[count[u] == 1 ? -first[u] : mem[first[u] + g + m]] + col[u]);
+#pragma unroll
+      for (int u = 0; u < KVI_AHEAD; ++u) {
+        if (count[u] == 1) {
+          if (g == 0) rows[i0 + u * KVI_THREADS] = v[u][0];
+        } else {
+#pragma unroll
+          for (int m = 0; m < 2; ++m)
+            if (g + m < count[u]) {
+              float f[V];
+              unpack16(v[u][m], f, T());
+              const float w = wgt[first[u] + g + m];
+#pragma unroll
+              for (int j = 0; j < V; ++j) acc[u][j] = fmaf(w, f[j], acc[u][j]);
+            }
+        }
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < KVI_AHEAD; ++u)
+      if (count[u] > 1) rows[i0 + u * KVI_THREADS] = pack16(acc[u], T());
+  }
+  __syncthreads();                                         // every source of the plane has been read
+#pragma unroll 4
+  for (int idx = tid; idx < total; idx += KVI_THREADS) {
+    const int r = div_magic(idx, magic_ch), c = idx - r * ch;
+    st_stream16(buf + addr[r] + c * V, rows[idx]);
+  }
+}
+
+// =====================================================================================================
+// Second phase of the in-place form for planes that do not fit on chip: every output row moves from its surviving token's row (which holds the
 // merged group after the first phase) to its slot.  A slot never lies behind its source (o <= i), so rows only
 // move towards the front.  One CTA owns a plane -- one (sample, K or V, head, column part) -- and sweeps its
 // output rows in ascending chunks: the sources of a chunk are gathered into shared memory, the CTA
@@ -1309,14 +1435,31 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
   const dim3 grid(a->vis_begin + K.cap_out + a->n_text_after, K.batch);
   const int units = 2 * K.n_kv_heads * ch_host;
   // two units per thread (both in flight); narrow caches (GQA) get narrow CTAs
-  const int threads = std::min(KV_THREADS, ((units + 1) / 2 + 31) / 32 * 32);
+  const bool few = (long long)grid.x * grid.y <= kFewRows;
+  const int threads = std::min(few ? 512 : 256, ((units + 1) / 2 + 31) / 32 * 32);
   const int gather = a->mode == LIGHTKV_KV_GATHER;
   const bool in_place = a->k_src == a->k_dst;             // (the API checked that V and the addressing agree)
   auto run = [&](auto tag) -> cudaError_t {
     using T = decltype(tag);
     cudaError_t e = cudaSuccess;
+    if (in_place) {
+      // planes: (sample, K / V, head, column part); see kv_plane_kernel for the cut
+      const KvPlaneSmem sm{K.cap_in + a->n_text_after, K.cap_out + a->n_text_after, K.cap_in, K.cap_out};
+      const long long planes = 2ll * K.batch * K.n_kv_heads;
+      int p = 1;
+      while (ch_host % (2 * p) == 0 && ch_host / p >= 4 &&
+             (sm.bytes(ch_host / p) > 100 * 1024 || (planes * p < 2 * 148 && ch_host / p >= 8))) p *= 2;
+      const int ch = ch_host / p;
+      if (sm.bytes(ch) <= 220 * 1024 && (long long)sm.rows_out * ch < 65536) {
+        if ((e = ensure_dynamic_smem(kv_plane_kernel<T>, 220 * 1024)) != cudaSuccess) return e;
+        return launch_kernel(kv_plane_kernel<T>, dim3((unsigned)(planes * p)), KVI_THREADS, sm.bytes(ch), K.stream, 1,
+            static_cast<T*>(a->k_dst), static_cast<T*>(a->v_dst), da, sm, K.n_kv_heads, ch, p,
+            (unsigned)(((1ull << 32) + ch - 1) / ch), a->vis_begin, a->n_text_after, gather, a->n_vis, a->n_vis_out,
+            a->grp_off, a->grp_src, a->weight);
+      }
+    }
     if (!(in_place && gather))                            // in place, gather mode has nothing to merge
-      e = launch_kernel(kv_compact_kernel<T>, grid, threads, 0, K.stream, 1,
+      e = launch_kernel(few ? kv_compact_kernel<T, 512, 4> : kv_compact_kernel<T, 256, 2>, grid, threads, 0, K.stream, 1,
           static_cast<const T*>(a->k_src), static_cast<const T*>(a->v_src), static_cast<T*>(a->k_dst),
           static_cast<T*>(a->v_dst), sa, da, K.n_kv_heads, K.head_dim, a->vis_begin, a->n_text_after, K.cap_in,
           K.cap_out, gather, in_place ? 1 : 0, magic_ch, a->n_vis, a->n_vis_out, a->grp_off, a->grp_src, a->weight);

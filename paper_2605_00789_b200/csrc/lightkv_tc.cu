@@ -233,7 +233,7 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
   // key tiles to visit: all tiles up to the last query's own key, or, when the caller supplies the row
   // log-sum-exp, only the tiles that hold prompt keys (J lies before the vision block, so it is visible)
   const int kt_lo = LSE ? a.text.begin / BK : 0;
-  const int nkt_lse = a.text.end > a.text.begin ? (a.text.end - 1) / BK + 1 - kt_lo : 0;
+  const int nsub_lse = a.text.end > a.text.begin ? (a.text.end - 1) / XT_SUB + 1 - 2 * kt_lo : 0;
 
   if (threadIdx.x == 0) {
     for (int i = 0; i < 2; ++i) { mbar_init(&q_full[i], 1); mbar_init(&q_empty[i], 1); }
@@ -279,7 +279,7 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
         it.nq = min(128, n - it.t0);
         it.n_seq = a.vis_begin + n + a.n_text_after;
         // halves of 64 keys the item visits
-        it.nsub = LSE ? 2 * nkt_lse : ((a.bidirectional ? it.n_seq : a.vis_begin + it.t0 + it.nq) - 1) / XT_SUB + 1;
+        it.nsub = LSE ? nsub_lse : ((a.bidirectional ? it.n_seq : a.vis_begin + it.t0 + it.nq) - 1) / XT_SUB + 1;
         it.row0 = a.seq_start ? a.seq_start[it.b] : 0;     // packed batch: one long row axis, batch coordinate 0
         return true;
       };

@@ -284,6 +284,20 @@ def test_in_place_kv_compaction_long_rows_and_text_behind():
     plan.close()
 
 
+@pytest.mark.parametrize("batch,n_kv,head_dim,grid,text", [
+    (1, 1, 64, (24, 24), 3),         # one plane pair, cut into parts of 64 bytes
+    (3, 2, 24, (12, 14), 0),         # rows of three 16-byte pieces: not cut
+    (2, 3, 96, (40, 41), 17),        # parts of 64 bytes (rows of twelve pieces)
+    (1, 2, 128, (72, 74), 5),        # fits on chip in parts of 32 bytes only
+    (1, 1, 128, (100, 96), 5),       # does not fit: merged at the survivors, then moved in chunks
+])
+@pytest.mark.parametrize("kv_mode,paged", [("merge", 0), ("gather", 16)])
+def test_in_place_planes_over_cuts(batch, n_kv, head_dim, grid, text, kv_mode, paged):
+    wl = S.Workload(name="plane", config_id=141, batch=batch, tiles=(grid,), n_text=text, hidden=64, n_q_heads=n_kv,
+                    n_kv_heads=n_kv, head_dim=head_dim, n_layers=16, layers=(3,), windows=(3,), keep=(0.55,))
+    H.run_schedule(wl, xi_mode="given", kv_mode=kv_mode, paged=paged, kv_in_place=True)
+
+
 def test_in_place_equals_out_of_place_bit_for_bit():
     wl = S.workload("cfg1")
     plan = H.make_plan(wl)
