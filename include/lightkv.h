@@ -134,9 +134,8 @@ typedef struct {
   int32_t uses_tensor_cores;       /* 1: the FD and xi contractions of this stage run on tcgen05  */
   size_t  workspace_bytes;         /* DEVICE scratch lightkv_compress_layer needs                 */
   int32_t cap_a, cap_b;            /* upper bounds on the A / B nodes of one sample               */
-  int32_t fd_tiles;                /* tiles per sample the plan expects the tensor-core FD kernel
-                                      to cut (sizes its launch; the kernel walks whatever tiling
-                                      the device derives from the actual windows)                 */
+  int32_t fd_tiles;                /* tiles (of nodes of one window) per sample the plan expects the FD
+                                      kernel to score                                              */
   int32_t reserved;
 } lightkv_stage_info_t;
 

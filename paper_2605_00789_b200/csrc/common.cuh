@@ -9,7 +9,6 @@
 namespace lkv {
 
 constexpr int kMaxTiles = 32;          // image tiles / frames per sample
-constexpr int kFdTile = 128;           // A (and B) entries per tile of the tensor-core FD kernel
 constexpr int kMaxWindows = 2048;      // windows per sample (window-build kernel keeps 32 x n_windows u16 counters in smem)
 constexpr int kMaxWindowTokens = 65535;  // tokens of one window (range of those counters)
 
@@ -24,21 +23,6 @@ struct Geometry {
   int cols[kMaxTiles];
 };
 
-// Tiling of one sample's A x B pairs for the tensor-core FD kernel.  Consecutive groups of `wpt`
-// windows share one tile while every window has at most 128 A entries; larger windows are cut into
-// blocks_a x blocks_b blocks of 128 x 128 entries (wpt = 1).  `passes` * 32 bounds the A (and B)
-// entries of any tile; the kernel sizes its shared-memory stages from it.
-struct FdTiling {
-  int n_tiles;                         // groups * blocks_a * blocks_b
-  int wpt;                             // windows per group
-  int blocks_a, blocks_b;
-  int passes;                          // 1, 2 or 4
-  int pad[3];
-};
-
-// Groups are kept small enough that the whole batch yields about this many tiles (two per SM).
-constexpr int kFdTargetTiles = 296;
-
 // Per-stage views into the caller's workspace (all DEVICE pointers, per-sample row strides in elements).
 struct Workspace {
   int* win_off;    // [B, n_windows + 1]  first window-sorted slot of each window
@@ -49,8 +33,10 @@ struct Workspace {
   int* a_win;      // [B, cap_a]          window of each A entry
   int* b_tok;      // [B, cap_b]          token index of each B entry
   unsigned long long* a_key;  // [B, cap_a]  (orderable(lowest FD) << 32) | B entry index of the best partner;
-                              //             all ones while no partner is known (set by the window build)
-  FdTiling* fd_tiling;        // [B]         how the tensor-core FD kernel cuts this sample into tiles
+                              //             all ones while no partner is known (set by the window build).  Without window
+                              //             lists: [B, fd blocks, cap_in], by token and block of destinations, see
+                              //             fd_tc_kernel
+  int* win_tok;    // [B, n_windows, max_cell + 1]  tiled FD kernel: the number of tokens of a window, then the tokens
   float* xi_h;     // [B, H, cap_in]      per-head attention mass on the prompt (ATTN modes)
   float* xi;       // [B, cap_in]
   int* partner;    // [B, cap_in]         token a source is merged into; negative: survives (-2: a source that was not
@@ -150,6 +136,16 @@ __device__ inline uint4 pack16(const float (&f)[4], float) {
 }
 __device__ inline float to_float(__nv_bfloat16 v) { return __bfloat162float(v); }
 __device__ inline float to_float(float v) { return v; }
+
+// acc += lo^2 + hi^2 over the four bf16 pairs of v; every product is exact in fp32
+__device__ __forceinline__ float sumsq16(const uint4& v, float acc) {
+  const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int j = 0; j < 4; ++j)
+    asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %1;\n\t"
+        "fma.rn.f32.bf16 %0, lo, lo, %0;\n\tfma.rn.f32.bf16 %0, hi, hi, %0;\n\t}" : "+f"(acc) : "r"(u[j]));
+  return acc;
+}
 
 // streaming 16-byte load / store (read-once data: do not keep in L1)
 __device__ inline uint4 ld_stream16(const void* p) {

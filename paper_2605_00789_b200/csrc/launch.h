@@ -36,9 +36,9 @@ struct LayerLaunch {
   int dtype, xi_mode, divergence;
   double keep;
   int fd_side;                       // estimate of the larger side (A or B nodes) of a window: picks the FD kernel
-  int max_cell;                      // grid positions of the largest window
-  int n_grid;                        // ... of all tiles
-  int fd_tiles;                      // estimate of FdTiling::n_tiles per sample (launch shape of the tensor-core FD kernel)
+  int fd_blocks;                     // tiles of fd_tile_side(fd_side) nodes a side the largest window may have
+  int max_cell;                      // most tokens a window can hold
+  int n_grid;                        // grid positions of all tiles
   Geometry geo;
   Workspace ws;
   TextSet text;                      // prompt-token set J of this call
@@ -76,11 +76,12 @@ cudaError_t launch_window_build(const LayerLaunch& L);
 cudaError_t launch_fd_simt(const LayerLaunch& L);
 // windows, FD and selection for windows of at most 40 nodes a side (fp32: 80) in one kernel (Steps 1, 2 and 4): leaves every token's partner
 // and its place for launch_map
-bool fd_stream_supported(int dtype, int fd_side, int max_cell, int cap_in);
+bool fd_stream_supported(int dtype, int fd_side);
 cudaError_t launch_fd_stream(const LayerLaunch& L);
-// head sum of xi, merge map, weights from the partners (Steps 4, 5); at most kMapMaxTokens per sample
+// head sum of xi, merge map, weights from the partners (Steps 4, 5), with `select` from the keys of launch_fd_tc; at most
+// kMapMaxTokens per sample
 constexpr int kMapMaxTokens = 16384;
-cudaError_t launch_map(const LayerLaunch& L);
+cudaError_t launch_map(const LayerLaunch& L, bool select);
 // xi per head (Eq. "attention-factor"), fp32 FMA path; handles ATTN_FULL and ATTN_LSE
 cudaError_t launch_xi_simt(const LayerLaunch& L);
 // head sum of xi, ranking, merge map, weights (Steps 2-5)
@@ -98,7 +99,9 @@ cudaError_t launch_kv_compact(const KvLaunch& K);
 // tcgen05 paths (lightkv_tc.cu).  `supported` queries are host-only.
 bool tc_fd_supported(int hidden);
 bool tc_xi_supported(int head_dim);
-cudaError_t launch_fd_tc(const LayerLaunch& L);
+// lists: windows from launch_window_build, keys by source entry for launch_select_map; else by token for launch_map
+cudaError_t launch_fd_tc(const LayerLaunch& L, bool lists);
+int fd_tile_side(int fd_side);
 // wait_first: the stream's last kernel is not the window build or FD of the same call
 cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first);
 

@@ -17,9 +17,10 @@ struct StagePlan {
   bool exact;      // cap_in is the exact count (schedule so far is data independent)
   bool exact_out;  // cap_out too
   bool use_tc;
-  int max_cell;    // grid positions of the largest window
+  int max_cell;    // most tokens a window can hold (grid positions of the largest cell, or the whole sample)
   int fd_side;     // larger side (A or B nodes) of a typical window: picks the FD kernel
-  int fd_tiles;    // estimate of the tiles per sample of the tensor-core FD kernel (sizes its launch)
+  int fd_blocks;   // tiles a side the largest window may have, tensor-core FD kernel
+  int fd_tiles;    // tiles of the FD kernel per sample, at windows of fd_side nodes
   Geometry geo;
   size_t ws_bytes;
   size_t off[15];     // byte offsets of the Workspace arrays
@@ -38,27 +39,20 @@ namespace lkv {
 
 static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Tiles per sample the window-build kernel reports when the largest window has max_a A entries (same
-// rule as the kernel).  Only the launch shape of the persistent FD kernel depends on it, so an estimate
-// is enough: the kernel itself walks whatever tiles the device-side tiling holds.
-static int fd_tile_count(int n_windows, int max_a, int batch) {
-  if (max_a <= 0) return 0;
-  if (max_a <= kFdTile) {
-    const int want = (n_windows * batch + kFdTargetTiles - 1) / kFdTargetTiles;
-    const int wpt = std::max(1, std::min(std::min(kFdTile / max_a, n_windows), want));
-    return (n_windows + wpt - 1) / wpt;
-  }
-  const int blocks = (max_a + kFdTile - 1) / kFdTile;
-  return n_windows * blocks * blocks;
-}
+// Whether one CTA can hold a window's lists and one cluster a sample: the FD kernels then work without window lists.
+static bool windows_in_ctas(const StagePlan& s) { return s.max_cell <= 4096 && s.cap_in <= kMapMaxTokens; }
 
 static void layout_workspace(const lightkv_plan_t& p, StagePlan& s) {
   const size_t B = p.cfg.batch, nW1 = s.n_windows + 1;
   const bool attn = p.cfg.xi_mode == LIGHTKV_XI_ATTN_FULL || p.cfg.xi_mode == LIGHTKV_XI_ATTN_LSE;
   const size_t xi_items = attn ? size_t((s.cap_in + 127) / 128) * p.cfg.n_q_heads * B : 0;
+  // keys: one per source, or, for the tiled FD kernel without lists, one per token and block of destinations
+  const bool by_token = s.use_tc && windows_in_ctas(s) && !fd_stream_supported(p.cfg.dtype, s.fd_side);
+  const size_t keys = std::max(B * s.cap_a, by_token ? B * s.fd_blocks * s.cap_in : size_t(0));
+  const size_t win_tok = by_token ? B * s.n_windows * (size_t(s.max_cell) + 1) : 0;
   const size_t sizes[15] = {
       B * nW1 * 4, B * nW1 * 4, B * s.cap_in * 4, B * s.cap_in * 4, B * s.cap_a * 4, B * s.cap_a * 4,
-      B * s.cap_b * 4, B * s.cap_a * 8, B * sizeof(FdTiling),
+      B * s.cap_b * 4, keys * 8, win_tok * 4,
       attn ? B * p.cfg.n_q_heads * s.cap_in * 4 : 0, B * s.cap_in * 4, B * s.cap_in * 4, B * s.cap_in * 4,
       B * s.cap_a * 4, xi_items * 4};
   size_t off = 0;
@@ -77,7 +71,7 @@ static Workspace bind_workspace(const StagePlan& s, void* base) {
   w.a_win = reinterpret_cast<int*>(p + s.off[5]);
   w.b_tok = reinterpret_cast<int*>(p + s.off[6]);
   w.a_key = reinterpret_cast<unsigned long long*>(p + s.off[7]);
-  w.fd_tiling = reinterpret_cast<FdTiling*>(p + s.off[8]);
+  w.win_tok = reinterpret_cast<int*>(p + s.off[8]);
   w.xi_h = reinterpret_cast<float*>(p + s.off[9]);
   w.xi = reinterpret_cast<float*>(p + s.off[10]);
   w.partner = reinterpret_cast<int*>(p + s.off[11]);
@@ -169,8 +163,10 @@ int lightkv_plan(const lightkv_config_t* c, lightkv_plan_t** out) {
         delete p;
         return LIGHTKV_ERR_UNSUPPORTED;
       }
-    for (int t = 0; t < c->n_tiles; ++t)            // balanced cells: at most ceil(rows/w) x ceil(cols/w) positions
-      sp.max_cell = std::max(sp.max_cell, ((g.rows[t] + sp.w - 1) / sp.w) * ((g.cols[t] + sp.w - 1) / sp.w));
+    int cell = 0;                                   // balanced cells: at most ceil(rows/w) x ceil(cols/w) positions
+    for (int t = 0; t < c->n_tiles; ++t)
+      cell = std::max(cell, ((g.rows[t] + sp.w - 1) / sp.w) * ((g.cols[t] + sp.w - 1) / sp.w));
+    sp.max_cell = std::min(cell, cap);
     sp.n_windows = g.n_windows;
     sp.cap_in = cap;
     sp.exact = exact;
@@ -190,7 +186,6 @@ int lightkv_plan(const lightkv_config_t* c, lightkv_plan_t** out) {
         else still = false;
       }
       sp.cap_a = cap_a; sp.cap_b = cap_b;
-      sp.fd_tiles = fd_tile_count(g.n_windows, max_a, c->batch);
       sp.fd_side = max_a;
       if (still) {
         std::sort(next.begin(), next.end());
@@ -204,11 +199,12 @@ int lightkv_plan(const lightkv_config_t* c, lightkv_plan_t** out) {
       sp.cap_a = g.src_par ? sp.cap_in / 2 : (sp.cap_in + sp.n_windows) / 2;
       sp.cap_b = g.src_par ? (sp.cap_in + sp.n_windows) / 2 : sp.cap_in / 2;
     }
-    if (!sp.exact) {  // counts depend on the data: a window holds at most the tokens of its grid cell
-      sp.fd_tiles = fd_tile_count(g.n_windows, (std::min(sp.max_cell, sp.cap_in) + 1) / 2, c->batch);
-      // the tokens still alive are spread over the cells about evenly (the kernels walk larger windows in blocks)
-      sp.fd_side = (int)(((long long)sp.max_cell * sp.cap_in / p->n_vis0 + 2) / 2);
-    }
+    // where counts depend on the data: the tokens still alive are spread over the cells about evenly (the kernels walk
+    // larger windows, up to a whole cell, in blocks)
+    if (!sp.exact) sp.fd_side = (int)(((long long)cell * sp.cap_in / p->n_vis0 + 2) / 2);
+    const int side = fd_tile_side(sp.fd_side), typical = (std::max(sp.fd_side, 1) + side - 1) / side;
+    sp.fd_blocks = ((sp.max_cell + 1) / 2 + side - 1) / side;
+    sp.fd_tiles = (int)std::min<long long>((long long)g.n_windows * typical * typical, 0x7fffffff);
     if (!exact) {   // data-dependent from here on: every window keeps at most ceil(keep n_w) tokens
       long long bound = (long long)ceil(sp.keep * sp.cap_in) + sp.n_windows;
       sp.cap_out = (int)std::min<long long>(bound, sp.cap_in);
@@ -313,20 +309,25 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
   L.batch = c.batch; L.hidden = c.hidden; L.n_q_heads = c.n_q_heads; L.n_kv_heads = c.n_kv_heads;
   L.head_dim = c.head_dim; L.dtype = c.dtype; L.xi_mode = c.xi_mode; L.divergence = c.divergence;
   L.keep = s.keep; L.geo = s.geo;
-  L.fd_tiles = s.fd_tiles; L.fd_side = s.fd_side; L.max_cell = s.max_cell; L.n_grid = p->n_vis0;
+  L.fd_side = s.fd_side; L.fd_blocks = s.fd_blocks; L.max_cell = s.max_cell; L.n_grid = p->n_vis0;
   L.ws = bind_workspace(s, a->workspace); L.text = text; L.a = a; L.stream = static_cast<cudaStream_t>(a->stream);
 
   cudaEvent_t* ev = reinterpret_cast<cudaEvent_t*>(a->trace_events);
   auto mark = [&](int i) { return ev ? cudaEventRecord(ev[i], L.stream) : cudaSuccess; };
   const bool tc_xi = s.use_tc && attn && tc_xi_supported(c.head_dim);
   const bool tc_fd = s.use_tc && tc_fd_supported(c.hidden);
-  // Small windows: one kernel finds the windows, scores and selects, and the map kernel finishes (`streaming`; it
-  // addresses a sample's rows by 32-bit offsets of 16-byte units).  Otherwise window lists, a tiled FD kernel, selection.
-  const bool streaming = (tc_fd || c.dtype == LIGHTKV_FP32) && fd_stream_supported(c.dtype, s.fd_side, s.max_cell, s.cap_in) &&
-                         (long long)s.cap_in * a->hidden_row_stride * (long long)esz / 16 < 0xffffffffll;
-  auto launch_windows = [&](const LayerLaunch& l) { return streaming ? cudaSuccess : launch_window_build(l); };
+  // How windows, FD and selection are split over kernels (rows of a sample are addressed by 32-bit offsets of 16-byte
+  // units where CTAs gather them):
+  //   streaming  small windows: one kernel finds the windows, scores and selects; the map kernel finishes
+  //   tiled      larger windows on tensor cores: tiles of windows are scored, the map kernel selects and finishes
+  //   otherwise  samples or windows too large for the lists of a CTA, and the fp32-FMA engine: window lists, FD, selection
+  const bool near = (long long)s.cap_in * a->hidden_row_stride * (long long)esz / 16 < 0xffffffffll;
+  const bool in_ctas = near && windows_in_ctas(s);
+  const bool streaming = in_ctas && (tc_fd || c.dtype == LIGHTKV_FP32) && fd_stream_supported(c.dtype, s.fd_side);
+  const bool tiled = in_ctas && tc_fd && !streaming;
+  auto launch_windows = [&](const LayerLaunch& l) { return streaming || tiled ? cudaSuccess : launch_window_build(l); };
   auto launch_fd = [&](const LayerLaunch& l) {
-    return streaming ? launch_fd_stream(l) : tc_fd ? launch_fd_tc(l) : launch_fd_simt(l);
+    return streaming ? launch_fd_stream(l) : tc_fd && near ? launch_fd_tc(l, !tiled) : launch_fd_simt(l);
   };
   cudaStream_t aux = (a->aux_stream && attn && !ev) ? static_cast<cudaStream_t>(a->aux_stream) : nullptr;
   if (aux) {
@@ -353,7 +354,8 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
     if (launch_xi(ev != nullptr) != cudaSuccess || mark(2) != cudaSuccess) return LIGHTKV_ERR_CUDA;
     if (ev && (launch_fd(L) != cudaSuccess || mark(3) != cudaSuccess)) return LIGHTKV_ERR_CUDA;
   }
-  if ((streaming ? launch_map(L) : launch_select_map(L)) != cudaSuccess || mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+  const cudaError_t mapped = streaming || tiled ? launch_map(L, tiled) : launch_select_map(L);
+  if (mapped != cudaSuccess || mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (a->map_event && cudaEventRecord(static_cast<cudaEvent_t>(a->map_event), L.stream) != cudaSuccess)
     return LIGHTKV_ERR_CUDA;
   if (launch_merge_rows(L) != cudaSuccess || mark(5) != cudaSuccess) return LIGHTKV_ERR_CUDA;

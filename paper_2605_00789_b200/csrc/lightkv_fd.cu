@@ -3,6 +3,7 @@
 
 #include "launch.h"
 #include "tc_common.cuh"
+#include "windows.cuh"
 
 namespace lkv {
 
@@ -35,7 +36,7 @@ struct FdStreamArgs {
   Geometry g;
   const int* n_vis;                    // tokens of each sample, nullptr = cap_in
   const int* pos;                      // grid positions, nullptr = identity
-  int cap_in, max_cell;                // max_cell: grid positions of the largest window
+  int cap_in, max_cell;                // max_cell: most tokens a window can hold
   int* partner;                        // [B, cap_in] out, see Workspace
   int* place;                          // [B, cap_in] out
 };
@@ -59,16 +60,6 @@ __device__ __forceinline__ float4 ld_shared_f4(uint32_t addr) {
 __device__ __forceinline__ void cp_async16_l2(uint32_t smem_dst, const void* gmem_src, uint32_t src_bytes) {
   asm volatile("cp.async.cg.shared.global.L2::128B [%0], [%1], 16, %2;" ::"r"(smem_dst), "l"(gmem_src), "r"(src_bytes) : "memory");
 }
-// acc += lo^2 + hi^2 over the four bf16 pairs of v; every product is exact in fp32
-__device__ __forceinline__ float sumsq16(const uint4& v, float acc) {
-  const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int j = 0; j < 4; ++j)
-    asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %1;\n\t"
-        "fma.rn.f32.bf16 %0, lo, lo, %0;\n\tfma.rn.f32.bf16 %0, hi, hi, %0;\n\t}" : "+f"(acc) : "r"(u[j]));
-  return acc;
-}
-
 // O: groups of eight rows a side; S: 32-column chunks in flight per warp; WARPS: warps of a CTA
 template <int O, int S, int WARPS>
 struct FdStreamSmem {
@@ -76,9 +67,9 @@ struct FdStreamSmem {
   static constexpr int RING = WARPS * S * 2 * O * 512;                              // bytes
   static constexpr int PART = (WARPS * R * PITCH + WARPS * 2 * R) * 4;              // over the drained ring
   static constexpr int FIXED = RING > PART ? RING : PART;
-  // + per source of the window: key (8 bytes), best destination, per token of the window: its index; match masks
+  // + the window's lists and the match masks of the search
   static size_t bytes(int max_cell, int cap_in) {
-    return FIXED + size_t((max_cell + 1) / 2) * 12 + size_t(max_cell) * 4 + size_t((cap_in + 31) / 32) * 4 + 16;
+    return FIXED + WindowLists::bytes(max_cell) + size_t((cap_in + 31) / 32) * 4;
   }
 };
 
@@ -94,92 +85,34 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   float* part = reinterpret_cast<float*>(smem_raw);      // [WARPS][R][PITCH] partial inner products
   float* nrm = part + WARPS * R * PITCH;                 // [WARPS][2 R] partial squared norms, row 0: the norms
-  const int max_src = (a.max_cell + 1) / 2;
-  unsigned int* key = reinterpret_cast<unsigned int*>(smem_raw + M::FIXED);   // [max_src] orderable lowest score of a source
-  int* best = reinterpret_cast<int*>(key + max_src);     // [max_src] destination (local index) that attains it
-  int* into = best + max_src;                            // [max_src] the same for selected sources, -1 for the others
-  int* tok = into + max_src;                             // [max_cell] token index of the window's tokens, in position order
-  unsigned int* match = reinterpret_cast<unsigned int*>(tok + a.max_cell);    // [ceil(cap_in / 32)] tokens of the window
-  __shared__ int warp_sum[WARPS + 1];
-  const int w = blockIdx.x, b = blockIdx.y;
+  const WindowLists lists = WindowLists::at(smem_raw + M::FIXED, a.max_cell);
+  unsigned int* match = reinterpret_cast<unsigned int*>(smem_raw + M::FIXED + WindowLists::bytes(a.max_cell));
+  __shared__ int warp_sum[WARPS];
+  // a cluster of ks CTAs shares a window: CTA `rank` contracts its part of the hidden dimension and finishes every ks-th row
+  const int ks = (int)tc::cluster_nctarank(), rank = (int)tc::cluster_ctarank();
+  const int w = blockIdx.x / ks, b = blockIdx.y;
+  int* partner = a.partner + size_t(b) * a.cap_in;
+  int* place = a.place + size_t(b) * a.cap_in;
 
-  // ---- the window's tokens in storage (= position) order
   const int n = a.n_vis ? max(0, min(a.n_vis[b], a.cap_in)) : a.cap_in;
-  const int w2 = a.g.w * a.g.w, tile = w / w2, wr = (w - tile * w2) / a.g.w, wc = w - tile * w2 - wr * a.g.w;
-  const int rows = a.g.rows[tile], cols = a.g.cols[tile], first = a.g.tile_off[tile];
-  // rows r with r * w / rows == wr, columns c with c * w / cols == wc
-  const int r0 = (wr * rows + a.g.w - 1) / a.g.w, r1 = ((wr + 1) * rows + a.g.w - 1) / a.g.w;
-  const int c0 = (wc * cols + a.g.w - 1) / a.g.w, c1 = ((wc + 1) * cols + a.g.w - 1) / a.g.w;
-  int nw;
-  if (!a.pos && n == a.g.tile_off[a.g.n_tiles]) {        // the full grid: no list to search
-    nw = (r1 - r0) * (c1 - c0);
-    for (int l = tid; l < nw; l += NT) {
-      const int r = l / (c1 - c0);
-      tok[l] = first + (r0 + r) * cols + c0 + (l - r * (c1 - c0));
+  const int nw = min(a.max_cell, window_tokens<WARPS>(a.g, a.pos ? a.pos + size_t(b) * a.cap_in : nullptr, n, w, match, warp_sum, [&](int l, int i) {
+    if (l < a.max_cell) {
+      lists.tok[l] = i;
+    } else {                                             // only if positions repeat or lie outside the grid: survives
+      partner[i] = -1;
+      place[i] = 0;
     }
-    __syncthreads();
-  } else {
-    const int lo = first + r0 * cols, hi = first + r1 * cols, n_grid = a.g.tile_off[a.g.n_tiles];
-    const int* pos = a.pos ? a.pos + size_t(b) * a.cap_in : nullptr;
-    const int chunks = (n + 31) >> 5;
-#pragma unroll 4
-    for (int c = warp; c < chunks; c += WARPS) {
-      const int i = c * 32 + lane;
-      bool in = false;
-      if (i < n) {
-        const int p = pos ? pos[i] : i;
-        if (p >= lo && p < hi) {
-          const int col = (p - first) % cols;
-          in = col >= c0 && col < c1;
-        }
-        in = in || (w == 0 && (p < 0 || p >= n_grid));   // no such position: counted with window 0 (flagged elsewhere)
-      }
-      const unsigned int m = __ballot_sync(0xffffffffu, in);
-      if (lane == 0) match[c] = m;
-    }
-    __syncthreads();
-    nw = 0;
-    for (int base = 0; base < chunks; base += NT) {
-      const unsigned int m = base + tid < chunks ? match[base + tid] : 0u;
-      const int own = __popc(m);
-      int x = own;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int t = __shfl_up_sync(0xffffffffu, x, o);
-        if (lane >= o) x += t;
-      }
-      if (lane == 31) warp_sum[warp] = x;
-      __syncthreads();
-      int before = nw, total = 0;
-#pragma unroll
-      for (int k = 0; k < WARPS; ++k) {
-        if (k < warp) before += warp_sum[k];
-        total += warp_sum[k];
-      }
-      int at = before + x - own;
-      for (unsigned int bits = m; bits; bits &= bits - 1) {
-        const int i = (base + tid) * 32 + __ffs(bits) - 1;
-        if (at < a.max_cell) {
-          tok[at] = i;
-        } else {                                         // only if positions repeat or lie outside the grid: survives
-          a.partner[size_t(b) * a.cap_in + i] = -1;
-          a.place[size_t(b) * a.cap_in + i] = 0;
-        }
-        ++at;
-      }
-      nw += total;
-      __syncthreads();
-    }
-    nw = min(nw, a.max_cell);
-  }
+  }));
   if (nw == 0) return;
   const int par = a.g.src_par;
   const int na_all = (nw + 1 - par) >> 1, nb_all = nw - na_all;   // sources: local ranks of parity `par`
   const int removed = nb_all > 0 ? removal_count(nw, a.keep, par) : 0;
-  for (int e = tid; e < na_all; e += NT) { key[e] = 0xffffffffu; best[e] = -1; into[e] = -1; }
+  for (int e = tid; e < na_all; e += NT) { lists.key[e] = 0xffffffffu; lists.best[e] = -1; }
+  __syncthreads();
 
   const int g = lane >> 2, t = lane & 3;
-  const int nc = (a.d + CH - 1) / CH, c_lo = warp * nc / WARPS, nk = (warp + 1) * nc / WARPS - c_lo;
+  const int nc = (a.d + CH - 1) / CH, part_id = rank * WARPS + warp, parts = ks * WARPS;
+  const int c_lo = part_id * nc / parts, nk = (part_id + 1) * nc / parts - c_lo;
   const T* base = static_cast<const T*>(a.x) + size_t(b) * a.batch_stride +
                   size_t(a.seq_start ? a.seq_start[b] : 0) * a.row_stride + c_lo * CH + t * EL;
   const uint32_t row16 = uint32_t(a.row_stride / EL);    // row pitch in 16-byte units
@@ -194,8 +127,8 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
       uint32_t off[2 * O];                               // row offsets in 16-byte units, A rows first; all ones: no such row
 #pragma unroll
       for (int i = 0; i < O; ++i) {
-        off[i] = 8 * i + g < na ? uint32_t(tok[2 * (a0 + 8 * i + g) + par]) * row16 : 0xffffffffu;
-        off[O + i] = 8 * i + g < nb ? uint32_t(tok[2 * (b0 + 8 * i + g) + 1 - par]) * row16 : 0xffffffffu;
+        off[i] = 8 * i + g < na ? uint32_t(lists.tok[2 * (a0 + 8 * i + g) + par]) * row16 : 0xffffffffu;
+        off[O + i] = 8 * i + g < nb ? uint32_t(lists.tok[2 * (b0 + 8 * i + g) + 1 - par]) * row16 : 0xffffffffu;
       }
       // rows the block does not have stay zero in every stage
 #pragma unroll
@@ -302,20 +235,51 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
         if (t == 0) nrm[warp * 2 * R + 8 * i + g] = ss[i];
       }
       __syncthreads();
-      // ---- norms and inner products over the warps, in warp order
-      for (int i = tid; i < 2 * R; i += blockDim.x) {
-        float s = nrm[i];
-        for (int k = 1; k < nwarps; ++k) s += nrm[k * 2 * R + i];
-        nrm[i] = a.metric == LIGHTKV_FD_COSINE ? sqrtf(s) : s;
+      // ---- norms and inner products over the warps (and the CTAs of the cluster), in that order
+      if (ks == 1) {
+        for (int i = tid; i < 2 * R; i += NT) {
+          float s = nrm[i];
+          for (int k = 1; k < nwarps; ++k) s += nrm[k * 2 * R + i];
+          nrm[i] = a.metric == LIGHTKV_FD_COSINE ? sqrtf(s) : s;
+        }
+        __syncthreads();
+      } else {
+        for (int i = tid; i < 2 * R; i += NT) {
+          float s = nrm[i];
+          for (int k = 1; k < nwarps; ++k) s += nrm[k * 2 * R + i];
+          nrm[2 * R + i] = s;                            // (row 0 takes the sum over the cluster)
+        }
+        for (int i = tid; i < na * R; i += NT) {
+          const int r = i / R, col = i - r * R;
+          if (col >= nb) continue;
+          float s = part[r * PITCH + col];
+          for (int k = 1; k < nwarps; ++k) s += part[(k * R + r) * PITCH + col];
+          part[r * PITCH + col] = s;
+        }
+        tc::cluster_sync();
+        for (int i = tid; i < 2 * R; i += NT) {
+          float s = 0.f;
+          for (int j = 0; j < ks; ++j) s += tc::ld_cluster_f32(tc::map_to_cta(tc::smem_u32(nrm + 2 * R + i), j));
+          nrm[i] = a.metric == LIGHTKV_FD_COSINE ? sqrtf(s) : s;
+        }
+        __syncthreads();
       }
-      __syncthreads();
       // ---- a warp per source row, lanes over the destinations
-      for (int r = warp; r < na; r += nwarps) {
+      for (int r = rank + warp * ks; r < na; r += nwarps * ks) {
         float lowest = 3.0e38f;
         int col_min = -1;
         for (int col = lane; col < nb; col += 32) {
-          float s = part[r * PITCH + col];
-          for (int k = 1; k < nwarps; ++k) s += part[(k * R + r) * PITCH + col];
+          float s = 0.f;
+          if (ks == 1) {
+            s = part[r * PITCH + col];
+            for (int k = 1; k < nwarps; ++k) s += part[(k * R + r) * PITCH + col];
+          } else {
+            float v[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = j < ks ? tc::ld_cluster_f32(tc::map_to_cta(tc::smem_u32(part + r * PITCH + col), j)) : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s += v[j];
+          }
           const float fd = pair_score(a.metric, s, nrm[r], nrm[R + col]);
           if (fd < lowest) { lowest = fd; col_min = col; }
         }
@@ -326,46 +290,19 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
           if (oc >= 0 && (col_min < 0 || of < lowest || (of == lowest && oc < col_min))) { lowest = of; col_min = oc; }
         }
         // later blocks of destinations hold higher indices: an equal score keeps the earlier one
-        if (lane == 0 && col_min >= 0 && orderable(lowest) < key[a0 + r]) {
-          key[a0 + r] = orderable(lowest);
-          best[a0 + r] = b0 + col_min;
+        if (lane == 0 && col_min >= 0 && orderable(lowest) < lists.key[a0 + r]) {
+          lists.key[a0 + r] = orderable(lowest);
+          lists.best[a0 + r] = b0 + col_min;
+          if (rank > 0) {                                // CTA 0 selects
+            tc::st_cluster_u32(tc::map_to_cta(tc::smem_u32(lists.key + a0 + r), 0), orderable(lowest));
+            tc::st_cluster_u32(tc::map_to_cta(tc::smem_u32(lists.best + a0 + r), 0), uint32_t(b0 + col_min));
+          }
         }
       }
-      __syncthreads();                                   // the partial results are overwritten by the next block
+      if (ks == 1) __syncthreads(); else tc::cluster_sync();   // the partial results are overwritten by the next block
     }
   }
-
-  // ---- selection: the `removed` sources with the lowest (score, index) go into their best destination
-  if (removed == 0) __syncthreads();
-  for (int e = tid; e < na_all; e += NT) {
-    bool sel = removed >= na_all;
-    if (!sel && removed > 0) {
-      const unsigned int mine = key[e];
-      int rank = 0;
-      for (int k = 0; k < e; ++k) rank += key[k] <= mine;
-      for (int k = e + 1; k < na_all; ++k) rank += key[k] < mine;
-      sel = rank < removed;
-    }
-    if (sel) into[e] = best[e];
-  }
-  __syncthreads();
-  // ---- what the merge map needs of every token: its partner, and its place in the group or the group's size
-  int* partner = a.partner + size_t(b) * a.cap_in;
-  int* place = a.place + size_t(b) * a.cap_in;
-  for (int l = tid; l < nw; l += NT) {
-    const int e = l >> 1, i = tok[l];
-    int p = -1, q = 0;
-    if ((l & 1) == par) {
-      const int to = into[e];
-      p = to < 0 ? -2 : tok[2 * to + 1 - par];
-      if (to >= 0)
-        for (int k = 0; k < e; ++k) q += into[k] == to;
-    } else {
-      for (int k = 0; k < na_all; ++k) q += into[k] == e;
-    }
-    partner[i] = p;
-    place[i] = q;
-  }
+  if (rank == 0) select_window(lists, nw, a.keep, par, partner, place);
 }
 
 template <typename T, int O, int S, int WARPS>
@@ -373,26 +310,28 @@ static cudaError_t launch_fd_stream_o(const LayerLaunch& L, const FdStreamArgs& 
   const size_t smem = FdStreamSmem<O, S, WARPS>::bytes(f.max_cell, f.cap_in);
   const cudaError_t e = ensure_dynamic_smem(fd_stream_kernel<T, O, S, WARPS>, (int)smem);
   if (e != cudaSuccess) return e;
-  return launch_kernel(fd_stream_kernel<T, O, S, WARPS>, dim3(L.geo.n_windows, L.batch), 32 * WARPS, smem, L.stream, 1, f);
+  // few windows: clusters of 2, 4 or 8 CTAs split the hidden dimension further, while that fills no SM twice and leaves a
+  // CTA 32 KB to read (fp32, bound by its FMAs: 8 KB) beside the two cluster barriers it costs
+  const long long window_bytes = 2ll * L.fd_side * L.hidden * (long long)sizeof(T) * (sizeof(T) == 4 ? 4 : 1);
+  int ks = 1;
+  while (ks < 8 && (long long)L.geo.n_windows * L.batch * 2 * ks <= 148 && window_bytes >= 2 * ks * (32ll << 10)) ks *= 2;
+  return launch_kernel(fd_stream_kernel<T, O, S, WARPS>, dim3(L.geo.n_windows * ks, L.batch), 32 * WARPS, smem, L.stream, ks, f);
 }
 
-// Eight warps split the hidden dimension where each still gets a few chunks of it (rows of more than 1.5 KB); a narrow
-// model gets CTAs of two, so that the fixed cost of a window (its lists, the meeting of the warps) is paid by fewer
-// threads.
+// Eight warps split the hidden dimension where each still gets a few chunks of it (rows of more than 1.5 KB) or the
+// windows are too few to fill the SMs; a large batch of a narrow model gets CTAs of two, so that the fixed cost of a
+// window (its lists, the meeting of the warps) is paid by fewer threads.
 template <int O, int S>
 static cudaError_t launch_fd_stream_w(const LayerLaunch& L, const FdStreamArgs& f) {
-  if (L.dtype == LIGHTKV_FP32)
-    return L.hidden > 384 ? launch_fd_stream_o<float, O, S, 8>(L, f) : launch_fd_stream_o<float, O, S, 2>(L, f);
-  return L.hidden > 768 ? launch_fd_stream_o<__nv_bfloat16, O, S, 8>(L, f) : launch_fd_stream_o<__nv_bfloat16, O, S, 2>(L, f);
+  const bool wide = L.hidden * (L.dtype == LIGHTKV_FP32 ? 4 : 2) > 1536 || (long long)L.geo.n_windows * L.batch <= 148;
+  if (L.dtype == LIGHTKV_FP32) return wide ? launch_fd_stream_o<float, O, S, 8>(L, f) : launch_fd_stream_o<float, O, S, 2>(L, f);
+  return wide ? launch_fd_stream_o<__nv_bfloat16, O, S, 8>(L, f) : launch_fd_stream_o<__nv_bfloat16, O, S, 2>(L, f);
 }
 
 // Five groups of eight rows a side is what the fragments of a thread hold at two CTAs per SM; beyond that the tcgen05
 // kernel shares the rows between more pairs (in fp32, where the FMAs bound the work, windows of two blocks a side still
-// gain).  The lists of a window and the search for its tokens have to fit in shared memory beside the ring, and the map
-// kernel behind takes two tokens per thread of eight CTAs.
-bool fd_stream_supported(int dtype, int fd_side, int max_cell, int cap_in) {
-  return fd_side > 0 && fd_side <= (dtype == LIGHTKV_FP32 ? 80 : 40) && max_cell <= 4096 && cap_in <= kMapMaxTokens;
-}
+// gain).
+bool fd_stream_supported(int dtype, int fd_side) { return fd_side > 0 && fd_side <= (dtype == LIGHTKV_FP32 ? 80 : 40); }
 
 cudaError_t launch_fd_stream(const LayerLaunch& L) {
   const lightkv_layer_args_t* a = L.a;

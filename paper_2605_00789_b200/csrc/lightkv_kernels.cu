@@ -4,6 +4,7 @@
 
 #include "launch.h"
 #include "tc_common.cuh"
+#include "windows.cuh"
 
 namespace lkv {
 
@@ -43,7 +44,6 @@ window_build_kernel(Geometry g, const int* __restrict__ pos_all, const int* __re
   int* a_win = ws.a_win + size_t(b) * ws.cap_a;
   int* b_tok = ws.b_tok + size_t(b) * ws.cap_b;
   unsigned long long* a_key = ws.a_key + size_t(b) * ws.cap_a;
-  __shared__ int max_ab[2][32];
 
   for (int i = tid; i < 32 * nW; i += blockDim.x) cnt[i] = 0;
   __syncthreads();
@@ -110,43 +110,6 @@ window_build_kernel(Geometry g, const int* __restrict__ pos_all, const int* __re
     ws.win_off[size_t(b) * (nW + 1) + w] = over ? 0 : wsum[w];
     ws.a_off[size_t(b) * (nW + 1) + w] = over ? 0 : asum[w];
   }
-  {  // largest A and B side of any window -> tiling of the tensor-core FD kernel
-    int ma = 0, mb = 0;
-    for (int w = tid; w < nW; w += blockDim.x) {
-      const int na = asum[w + 1] - asum[w];
-      ma = max(ma, na);
-      mb = max(mb, wsum[w + 1] - wsum[w] - na);
-    }
-    ma = __reduce_max_sync(0xffffffffu, ma);
-    mb = __reduce_max_sync(0xffffffffu, mb);
-    if (lane == 0) { max_ab[0][wp] = ma; max_ab[1][wp] = mb; }
-    __syncthreads();
-    if (wp == 0) {
-      ma = __reduce_max_sync(0xffffffffu, max_ab[0][lane]);
-      mb = __reduce_max_sync(0xffffffffu, max_ab[1][lane]);
-      if (lane == 0) {
-        FdTiling t;
-        const int mm = max(ma, mb);                      // either side of a window (the destinations outnumber the
-                                                         // sources by one per odd window in the reverse direction)
-        if (mm <= kFdTile) {
-          // as few windows per tile as still gives the batch about kFdTargetTiles tiles, at most 128 entries a side
-          const int want = (nW * (int)gridDim.x + kFdTargetTiles - 1) / kFdTargetTiles;
-          t.wpt = mm > 0 ? max(1, min(min(kFdTile / mm, nW), want)) : nW;
-          t.blocks_a = 1; t.blocks_b = 1;
-          const int rows = t.wpt * mm;
-          t.passes = rows <= 32 ? 1 : (rows <= 64 ? 2 : 4);
-        } else {
-          t.wpt = 1;
-          t.blocks_a = (ma + kFdTile - 1) / kFdTile; t.blocks_b = (mb + kFdTile - 1) / kFdTile;
-          t.passes = 4;
-        }
-        t.n_tiles = (ma > 0 && mb > 0 && !over) ? ((nW + t.wpt - 1) / t.wpt) * t.blocks_a * t.blocks_b : 0;
-        t.pad[0] = t.pad[1] = t.pad[2] = 0;
-        ws.fd_tiling[b] = t;
-      }
-    }
-  }
-
   // pass B: local rank, A / B entry lists
   for (int base = s0; base < s1; base += 32) {
     const int i = base + lane;
@@ -766,7 +729,9 @@ cudaError_t launch_select_map(const LayerLaunch& L) {
 }
 
 // =====================================================================================================
-// Merge map behind the streaming FD kernel, which left every token's partner and its place (see Workspace).  One
+// Merge map behind the streaming FD kernel, which left every token's partner and its place (see Workspace), or, with
+// SELECT, behind the tiled one, which left the windows' tokens and keys: the CTAs of a sample then first take its windows
+// in turn and select.  One
 // cluster of 1-8 CTAs per sample, TPT consecutive tokens per thread, everything between the first loads and the last
 // stores in registers and (distributed) shared memory:
 //   1  xi = fixed-order sum over heads (or given / uniform); survivors and group sizes are counted in ONE pair of prefix
@@ -785,8 +750,12 @@ struct MapArgs {
   const int* pos;
   const float* xi_in;
   const float* xi_h;
-  const int* partner;
-  const int* place;
+  int* partner;
+  int* place;
+  const unsigned long long* key;       // SELECT: [B, blocks, cap_in]
+  const int* win_tok;                  // SELECT: [B, n_windows, max_cell + 1]
+  int blocks, max_cell, n_windows, src_par, tile_side;
+  double keep;
   int* n_vis_out;
   int* pos_out;
   int* dst;
@@ -797,7 +766,7 @@ struct MapArgs {
   uint32_t* status;
 };
 
-template <bool CLUSTER, int TPT>
+template <bool CLUSTER, int TPT, bool SELECT>
 __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapArgs a) {
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -821,6 +790,28 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
   const int lo = min(n, rank * chunk), hi = min(n, lo + chunk);
   const int i0 = lo + tid * TPT;
 
+  if (SELECT) {
+    const WindowLists lists = WindowLists::at(smem_raw, a.max_cell);          // (before the arrays above are in use)
+    for (int w = rank; w < a.n_windows; w += cs) {
+      const int* win_tok = a.win_tok + (size_t(b) * a.n_windows + w) * (a.max_cell + 1);
+      const int nw = win_tok[0], par = a.src_par, na = (nw + 1 - par) >> 1, nb = nw - na;
+      for (int l = tid; l < nw; l += nthr) lists.tok[l] = win_tok[1 + l];
+      const bool scored = nb > 0 && removal_count(nw, a.keep, par) > 0;
+      for (int e = tid; e < na; e += nthr) {
+        const int i = win_tok[1 + 2 * e + par];
+        unsigned long long key = ~0ull;
+        for (int ib = 0; scored && ib * a.tile_side < nb; ++ib)
+          key = min(key, a.key[(size_t(b) * a.blocks + ib) * a.cap_in + i]);
+        lists.key[e] = (unsigned int)(key >> 32);
+        lists.best[e] = (unsigned int)key == 0xffffffffu ? -1 : (int)(unsigned int)key;
+      }
+      __syncthreads();
+      select_window(lists, nw, a.keep, par, a.partner + row, a.place + row);
+      __syncthreads();
+    }
+    sync_all();
+  }
+
   // ---- loads
   int prt[TPT], plc[TPT], ps[TPT];
   float xi[TPT];
@@ -830,8 +821,8 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
     const int i = i0 + j;
     prt[j] = -1; plc[j] = 0; ps[j] = i; xi[j] = 0.f;
     if (i < hi) {
-      prt[j] = a.partner[row + i];
-      plc[j] = a.place[row + i];
+      prt[j] = __ldcg(a.partner + row + i);
+      plc[j] = __ldcg(a.place + row + i);
       if (a.pos) {
         ps[j] = a.pos[row + i];
         bad = bad || ps[j] <= (i > 0 ? a.pos[row + i - 1] : -1) || ps[j] >= a.n_grid;
@@ -982,28 +973,33 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
   }
 }
 
-cudaError_t launch_map(const LayerLaunch& L) {
+cudaError_t launch_map(const LayerLaunch& L, bool select) {
   const lightkv_layer_args_t* a = L.a;
   MapArgs m;
   m.n_q_heads = L.n_q_heads; m.xi_mode = L.xi_mode; m.cap_in = L.ws.cap_in; m.cap_out = L.ws.cap_out;
   m.cap_a = L.ws.cap_a; m.cap_b = L.ws.cap_b; m.n_grid = L.n_grid;
   m.n_vis = a->n_vis; m.pos = a->pos; m.xi_in = a->xi; m.xi_h = L.ws.xi_h; m.partner = L.ws.partner; m.place = L.ws.slot;
+  m.key = L.ws.a_key; m.win_tok = L.ws.win_tok; m.blocks = L.fd_blocks; m.max_cell = L.max_cell; m.n_windows = L.geo.n_windows;
+  m.src_par = L.geo.src_par; m.tile_side = fd_tile_side(L.fd_side); m.keep = L.keep;
   m.n_vis_out = a->n_vis_out; m.pos_out = a->pos_out; m.dst = a->dst; m.weight = a->weight; m.grp_off = a->grp_off;
   m.grp_src = a->grp_src; m.xi_out = a->xi_out; m.status = a->status;
-  // one cluster per sample: as many CTAs of up to 1024 threads as give every thread one token (two beyond 8192)
+  // one cluster per sample: as many CTAs of up to 1024 threads as give every thread one token (two beyond 8192), and
+  // with windows to select in, as many as there are windows (up to eight) of at least 256 threads
   const int n = L.ws.cap_in;
   int cs = 1;
-  while (cs < 8 && cs * 1024 < n) cs *= 2;
+  while (cs < 8 && (cs * 1024 < n || (select && cs < L.geo.n_windows))) cs *= 2;
   const int tpt = n > 8192 ? 2 : 1;
-  const int threads = std::min(1024, (((n + cs - 1) / cs + tpt - 1) / tpt + 31) / 32 * 32);
-  const size_t smem = (size_t(2) * threads * tpt + size_t(2) * n) * 4;
+  const int threads = std::max(select ? 256 : 32, std::min(1024, (((n + cs - 1) / cs + tpt - 1) / tpt + 31) / 32 * 32));
+  size_t smem = (size_t(2) * threads * tpt + size_t(2) * n) * 4;
+  if (select) smem = std::max(smem, WindowLists::bytes(L.max_cell));
   auto launch = [&](auto kernel) -> cudaError_t {
     const cudaError_t e = ensure_dynamic_smem(kernel, (int)smem);
     if (e != cudaSuccess) return e;
     return launch_kernel(kernel, L.batch * cs, threads, smem, L.stream, cs, m);
   };
-  if (tpt == 2) return launch(map_kernel<true, 2>);
-  return cs > 1 ? launch(map_kernel<true, 1>) : launch(map_kernel<false, 1>);
+  if (tpt == 2) return select ? launch(map_kernel<true, 2, true>) : launch(map_kernel<true, 2, false>);
+  if (cs > 1) return select ? launch(map_kernel<true, 1, true>) : launch(map_kernel<true, 1, false>);
+  return select ? launch(map_kernel<false, 1, true>) : launch(map_kernel<false, 1, false>);
 }
 
 // Launches of at most this many rows do not fill the SMs' memory pipes by number: they get wider CTAs and more members of

@@ -3,6 +3,7 @@
 
 #include "launch.h"
 #include "tc_common.cuh"
+#include "windows.cuh"
 
 namespace lkv {
 
@@ -636,112 +637,91 @@ cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first) {
 }
 
 // ======================================================================================================
-// FD + best partner on tensor cores (Eq. "similarity", Step 2).
+// FD + best partner for larger windows on tensor cores (Eq. "similarity", Step 2).
 //
-// Persistent CTAs, two per SM; a work item is a tile of up to 128 A entries x 128 B entries (see
-// FdTiling): a group of whole windows, or one 128 x 128 block of a large window.  The rows of a tile are
-// scattered over the sequence (they are listed by a_tok / b_tok), so eight warps gather them with 16-byte
-// cp.async copies, eight threads per 128-byte row segment, straight into the 128-byte-swizzled K-major
-// layout tcgen05 reads.  The copies go through a ring of six 16 KB stages; a stage is 128 row slots of
-// 128 bytes (64 columns) and every loader thread fills four slots of it.  What the slots hold depends
-// on the tile's size (passes = 1, 2, 4 <=> at most 32, 64, 128 entries per operand):
-//   passes 4: even fills = the 128 A rows of a chunk, odd fills = its 128 B rows   (2 fills per chunk)
-//   passes 2: [64 A rows | 64 B rows] of one chunk                                  (1 fill per chunk)
-//   passes 1: [32 A rows, chunk c | 32 A rows, chunk c+1 | 32 B rows, c | 32 B rows, c+1]   (2 chunks per fill)
-// Four fills are in flight while a fifth is being consumed and a sixth may still be held by the tensor
-// core, so the loaders never wait for an MMA on their critical path.  Each thread re-reads the pieces
-// it fetched to accumulate the rows' squared norms: X is read from HBM exactly once.  A ninth warp
-// issues G += X_A X_B^T (128 x N x 64 per chunk, N = B entries rounded up to 16, bf16 -> fp32 in TMEM).
-// The MMA always reads 128 A rows (16 KB) from the start of a chunk's A block: rows the tile does not
-// have are never written, may overlap other blocks or the 4 KB pad behind the ring, and only feed
-// accumulator rows nobody reads.  After the last chunk the loader warps turn into the epilogue: one
-// thread per A row scans the FD of the columns that belong to the row's own window and keeps the
-// minimum (ties: lowest B index).  Blocks of a large window combine through a 64-bit atomicMin on
-// (orderable FD, B index), which is order independent.
+// A CTA (or a cluster of ks CTAs that split the hidden dimension, where there are few tiles) takes one tile of up to
+// BLK sources x BLK destinations of one window, BLK = 128 or, for larger windows, 256.  The rows of a tile are scattered
+// over the sequence; the CTA finds them from the positions (window_tokens) or, for samples too long for that, in the
+// lists the window build left.  Eight warps gather them with 16-byte cp.async copies, eight threads per 128-byte row
+// segment, straight into the 128-byte-swizzled K-major layout tcgen05 reads, through a ring of three stages (64 columns
+// of both operands), and re-read their pieces to accumulate the squared norms.  A ninth warp issues
+// G += X_A X_B^T (128 x N x 64 per half of 128 sources and chunk, bf16 -> fp32 in TMEM).  The MMA always reads 128 A
+// rows: rows the tile does not have are never written and only feed accumulator rows nobody reads.  After the last chunk
+// the loader warps turn into the epilogue: minimum over the destinations (ties: lowest index) of every source, one key
+// per (source, block of destinations), of which the map kernel takes the lowest.
+//
+// Every tile reads its rows again, so the kernel is bound by the way from L2 through shared memory (a 64-column chunk of
+// a 128 x 128 tile: 32 KB written, read by the norms and read by the MMA), not by HBM or the tensor pipe; a tile of 256
+// halves that.  The launch has as many tiles as windows of the expected size need; a CTA goes on with the blocks of a
+// window that has grown beyond that.
+// FD_TC_FIGURES
 // ======================================================================================================
 struct FdTcArgs {
   const __nv_bfloat16* x;              // first vision row of sample 0
   const int* seq_start;                // first row of each sample (packed batches) or nullptr
   int64_t batch_stride, row_stride;    // elements
-  int d, batch;
+  int d;
   int metric;                          // LIGHTKV_FD_*
+  double keep;
+  Geometry g;
+  const int* n_vis;
+  const int* pos;
+  int cap_in, max_cell;
+  int blocks;                          // blocks a side the largest window may have (row pitch of key)
+  int grid_blocks;                     // ... a window of the expected size has (the launch)
+  int lists;                           // 1: windows from ws (window build), keys by source entry through atomics
   Workspace ws;
   uint32_t* status;
 };
 
-constexpr int FT_LOADERS = 256;
-constexpr int FT_STAGES = 6;
-constexpr int FT_AHEAD = 4;                               // fills in flight
-constexpr int kFdPitch = kFdTile + 1;                     // row pitch (floats) of a partial G in shared memory
-constexpr uint32_t FT_STAGE_BYTES = 16 * 1024;
-constexpr uint32_t FT_RING_BYTES = FT_STAGES * FT_STAGE_BYTES + 4096;   // + pad for the 16 KB A read
-constexpr size_t FT_SMEM = size_t(FT_RING_BYTES) + 1024 /* alignment */ + 128 /* barriers */ +
-                           4 * kFdTile * sizeof(float);
+constexpr int FT_LOADERS = 256, FT_WARPS = 9;
+constexpr int FT_STAGES = 3;
+constexpr int FT_AHEAD = FT_STAGES - 1;                   // fills in flight beside the one being consumed
 
-// Second half of the cluster epilogue (kept out of line so that it does not weigh on the registers of the
-// streaming loop): full norms = partial squared sums added in rank order; then CTA `rank` finishes rows
-// [rank * 128 / ks, (rank + 1) * 128 / ks), a warp per row, lanes over the columns of the row's window.
-__device__ __noinline__ void fd_cluster_finish(int metric, const int* a_win, unsigned long long* a_key, int ks, int rank, int a0, int a1,
-                                               int b0, int b1,
-                                               bool combine, const int* win_off, const int* a_off, uint32_t p0,
-                                               const float* a_nrm, const float* b_nrm, float* nrm_a, float* nrm_b,
-                                               volatile int* abort_flag) {
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  {
-    const int i = tid & (kFdTile - 1);
-    const uint32_t src = smem_u32(tid < kFdTile ? a_nrm + i : b_nrm + i);
-    float ss = 0.f;
-    for (int j = 0; j < ks; ++j) ss += ld_cluster_f32(map_to_cta(src, j));
-    (tid < kFdTile ? nrm_a : nrm_b)[i] = metric == LIGHTKV_FD_COSINE ? sqrtf(ss) : ss;
+template <int BLK>
+struct FdTcSmem {
+  static constexpr int PITCH = BLK + 1;                   // row pitch (floats) of a partial G
+  static constexpr uint32_t STAGE = BLK * 256;            // BLK A rows | BLK B rows of 64 columns
+  static constexpr uint32_t CTL = 128 + 4 * BLK * 4 + 2 * 128 * 4 + 2 * BLK * 4 + 16 * 4;
+  static_assert(128 * PITCH * 4 <= FT_STAGES * STAGE, "a partial G of 128 rows fits over the drained ring");
+  static size_t bytes(int cap_in, bool lists) {
+    return 1024 /* alignment */ + FT_STAGES * STAGE + CTL + (lists ? 0 : size_t((cap_in + 31) / 32) * 4);
   }
-  named_barrier(1, FT_LOADERS);
-  // CTA `rank` finishes rows [rank * 128 / ks, (rank + 1) * 128 / ks): a warp per row, lanes over the
-  // columns of the row's window, partial sums added in rank order
-  const int rows_mine = kFdTile / ks, r0 = rank * rows_mine;
-  for (int rr = warp; rr < rows_mine; rr += 8) {
-    const int row = r0 + rr, e = a0 + row;
-    if (e >= a1) break;                               // warp-uniform; later rows are further out
-    const int w = a_win[e];
-    const int lo = max(win_off[w] - a_off[w], b0) - b0, hi = min(win_off[w + 1] - a_off[w + 1], b1) - b0;
-    const float na = nrm_a[row];
-    float best = 3.0e38f;
-    int best_c = -1;
-    for (int col = lo + lane; col < hi; col += 32) {
-      const uint32_t src = p0 + uint32_t(row * kFdPitch + col) * 4;
-      float gsum = 0.f;
-      for (int j = 0; j < ks; ++j) gsum += ld_cluster_f32(map_to_cta(src, j));
-      const float fd = pair_score(metric, gsum, na, nrm_b[col]);
-      if (fd < best) { best = fd; best_c = col; }
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {                // minimum over the lanes, ties to the lower column
-      const float of = __shfl_xor_sync(0xffffffffu, best, o);
-      const int oc = __shfl_xor_sync(0xffffffffu, best_c, o);
-      if (oc >= 0 && (best_c < 0 || of < best || (of == best && oc < best_c))) { best = of; best_c = oc; }
-    }
-    if (lane == 0 && best_c >= 0 && !*abort_flag) {
-      const unsigned long long key = ((unsigned long long)orderable(best) << 32) | (unsigned)(b0 + best_c);
-      unsigned long long* dst = a_key + e;
-      if (combine) atomicMin(dst, key); else *dst = key;
-    }
-  }
+};
+
+// the best destination of source `row` of tile (ia, ib) of sample b
+template <int BLK>
+__device__ __forceinline__ void store_key(const FdTcArgs& a, int b, int ia, int ib, int row, const int* row_a, int a_first,
+                                          int b_first, float best, int best_c) {
+  unsigned long long key = ~0ull;
+  if (best_c >= 0)
+    key = ((unsigned long long)orderable(best) << 32) | (unsigned)((a.lists ? b_first : 0) + ib * BLK + best_c);
+  if (a.lists) atomicMin(a.ws.a_key + size_t(b) * a.ws.cap_a + a_first + ia * BLK + row, key);
+  else a.ws.a_key[(size_t(b) * a.blocks + ib) * a.cap_in + row_a[row]] = key;
 }
 
 // CLUSTER = false is the plain launch (ks = 1) with the cluster code compiled out.
-template <bool CLUSTER>
-__global__ void __launch_bounds__(FT_LOADERS + 32, 2) fd_tc_kernel(FdTcArgs a) {
+template <int BLK, bool CLUSTER>
+__global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kernel(const __grid_constant__ FdTcArgs a) {
+  using M = FdTcSmem<BLK>;
+  constexpr int NR = BLK / 32;                  // rows of an operand per loader thread
+  constexpr int PITCH = M::PITCH;
   extern __shared__ unsigned char smem_raw[];
   unsigned char* base = reinterpret_cast<unsigned char*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* bars = reinterpret_cast<uint64_t*>(base + FT_RING_BYTES);
-  uint64_t* full = bars;                        // [FT_STAGES] fill landed (one arrival per loader warp)
+  unsigned char* ctl = base + FT_STAGES * M::STAGE;
+  uint64_t* full = reinterpret_cast<uint64_t*>(ctl);   // [FT_STAGES] fill landed (one arrival per loader warp)
   uint64_t* empty = full + FT_STAGES;           // [FT_STAGES] fill consumed (MMA commit)
   uint64_t* acc_full = empty + FT_STAGES;       // accumulator complete
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_full + 1);
   volatile int* abort_flag = reinterpret_cast<volatile int*>(tmem_slot + 1);
-  float* a_nrm = reinterpret_cast<float*>(reinterpret_cast<unsigned char*>(bars) + 128);   // [128]
-  float* b_nrm = a_nrm + kFdTile;                                                          // [128]
-  float* red_f = b_nrm + kFdTile;                                                          // [128]
-  int* red_c = reinterpret_cast<int*>(red_f + kFdTile);                                    // [128]
+  float* sq = reinterpret_cast<float*>(ctl + 128);     // [2 BLK] squared norms of A, B rows over this CTA's columns
+  float* nrm = sq + 2 * BLK;                           // [2 BLK] whole norms
+  float* red_f = nrm + 2 * BLK;                        // [128]
+  int* red_c = reinterpret_cast<int*>(red_f + 128);    // [128]
+  int* row_a = red_c + 128;                            // [BLK] token index of the tile's rows
+  int* row_b = row_a + BLK;                            // [BLK]
+  int* warp_sum = row_b + BLK;                         // [FT_WARPS]
+  unsigned int* match = reinterpret_cast<unsigned int*>(warp_sum + 16);
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   if (tid == 0) {
@@ -750,296 +730,279 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, 2) fd_tc_kernel(FdTcArgs a) {
     *abort_flag = 0;
     fence_barrier_init();
   }
-  if (warp == 8) { tmem_alloc(tmem_slot, kFdTile); tmem_relinquish(); }
+  if (warp == 8) { tmem_alloc(tmem_slot, BLK == 128 ? 128 : 512); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   // barriers and tensor memory are set up while the kernel before this one may still be running; from here on
   // global memory is read (and written), so that kernel must have completed
-  grid_dependency_sync();
+  grid_dependency_wait();
+  grid_launch_dependents();                     // in this order: see grid_dependency_sync
   const uint32_t tmem_base = *tmem_slot;
   const uint32_t ring = smem_u32(base);
-  const int nW = a.ws.n_windows;
-  // A cluster of ks CTAs shares every tile: CTA `rank` contracts chunks [c_lo, c_lo + nk) of the hidden
-  // dimension and the partial results are combined through distributed shared memory (ks = 1: no cluster).
   const int ks = CLUSTER ? (int)cluster_nctarank() : 1, rank = CLUSTER ? (int)cluster_ctarank() : 0;
+  const int b = blockIdx.y, tile = blockIdx.x / ks, per_window = a.grid_blocks * a.grid_blocks;
+  const int w = tile / per_window, rem = tile - w * per_window, ia0 = rem / a.grid_blocks, ib0 = rem - ia0 * a.grid_blocks;
+  const int par = a.g.src_par;
+  const int n = a.n_vis ? max(0, min(a.n_vis[b], a.cap_in)) : a.cap_in;
   const int nk_all = (a.d + 63) >> 6;           // 64-column chunks of the whole hidden dimension
   const int c_lo = rank * nk_all / ks, nk = (rank + 1) * nk_all / ks - c_lo;
+  int* win_tok = a.lists ? nullptr : a.ws.win_tok + (size_t(b) * a.g.n_windows + w) * (a.max_cell + 1);
 
-  // Work items are the (sample, tile) pairs of the whole batch in sample order; this CTA takes items
-  // cluster id, cluster id + number of clusters, ...  Barrier phases run on across items: `done` counts the
-  // fills this CTA has completed, `n_items` its finished tiles.
-  uint32_t done = 0, n_items = 0;
-  for (int item = blockIdx.x / ks;; item += gridDim.x / ks) {
-  int b = 0, tile = item;
-  while (b < a.batch) {
-    const int nt = a.ws.fd_tiling[b].n_tiles;
-    if (tile < nt) break;
-    tile -= nt;
-    ++b;
-  }
-  if (b >= a.batch) break;                      // same for every thread of the CTA
-  const FdTiling tl = a.ws.fd_tiling[b];
-  const int* win_off = a.ws.win_off + size_t(b) * (nW + 1);
-  const int* a_off = a.ws.a_off + size_t(b) * (nW + 1);
-  const int per_group = tl.blocks_a * tl.blocks_b;
-  const int grp = tile / per_group, rem = tile - grp * per_group;
-  const int ia = rem / tl.blocks_b, ib = rem - ia * tl.blocks_b;
-  const int w0 = min(grp * tl.wpt, nW), w1 = min(nW, w0 + tl.wpt);
-  const int passes = tl.passes;                                      // 1, 2 or 4
-  const int cap_rows = 32 * passes;
-  const int a0 = a_off[w0] + ia * kFdTile, a1 = min(a_off[w1], a0 + cap_rows);
-  const int b0 = win_off[w0] - a_off[w0] + ib * kFdTile, b1 = min(win_off[w1] - a_off[w1], b0 + cap_rows);
-  if (a0 >= a1 || b0 >= b1) continue;           // same for every thread of the CTA
-  const int n_cols = (b1 - b0 + 15) & ~15;      // MMA N
-  const int nf = passes == 4 ? 2 * nk : (passes == 2 ? nk : (nk + 1) >> 1);   // fills of this tile
-
-  if (warp < 8) {
-    // ---- gather: thread = 16-byte piece c of row slots g, g + 32, g + 64, g + 96 of every fill
-    const int c = tid & 7, g = tid >> 3;
-    const unsigned char* xb = reinterpret_cast<const unsigned char*>(
-        a.x + size_t(b) * a.batch_stride + size_t(a.seq_start ? a.seq_start[b] : 0) * a.row_stride) + size_t(c_lo) * 128;
-    const int* a_tok = a.ws.a_tok + size_t(b) * a.ws.cap_a;
-    const int* b_tok = a.ws.b_tok + size_t(b) * a.ws.cap_b;
-    // source row of slot t on even / odd fills (they differ only when passes = 4), validity bits, and the
-    // chunk of slot t relative to the fill's first chunk (passes = 1 packs two chunks into a fill)
-    const unsigned char* src_e[4];
-    const unsigned char* src_o[4];
-    uint32_t ok_e = 0, ok_o = 0;
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-      const int i = passes == 4 ? t : (passes == 2 ? (t & 1) : 0);          // row g + 32 i of the operand
-      const bool slot_b = passes == 4 ? false : (t >> 1) != 0;              // operand of slot t on even fills
-      const int ea = a0 + g + 32 * i, eb = b0 + g + 32 * i;
-      const int ta = ea < a1 ? a_tok[ea] : -1, tb = eb < b1 ? b_tok[eb] : -1;
-      const unsigned char* pa = xb + (size_t(max(ta, 0)) * a.row_stride + c * 8) * 2;
-      const unsigned char* pb = xb + (size_t(max(tb, 0)) * a.row_stride + c * 8) * 2;
-      const size_t sub = passes == 1 ? size_t(t & 1) * 128 : 0;             // second chunk of the fill
-      src_e[t] = (slot_b ? pb : pa) + sub;
-      src_o[t] = (passes == 4 ? pb : (slot_b ? pb : pa)) + sub;
-      ok_e |= ((slot_b ? tb : ta) >= 0 ? 1u : 0u) << t;
-      ok_o |= ((passes == 4 ? tb : (slot_b ? tb : ta)) >= 0 ? 1u : 0u) << t;
-    }
-    const uint32_t slot0 = uint32_t(g) * 128 + (uint32_t(c ^ (g & 7)) << 4);   // swizzled offset of slot g; slot g+32t is 4096 t further
-    const int chunk_shift = passes == 4 ? 1 : 0, chunk_mul = passes == 1 ? 2 : 1;
-    float acc_e[4] = {0.f, 0.f, 0.f, 0.f}, acc_o[4] = {0.f, 0.f, 0.f, 0.f};
-    // columns of this thread's A row in the epilogue (row = TMEM lane): the B entries of the row's own window.
-    // Fetched here, two dependent loads deep, so that their latency hides behind the rows that stream below.
-    const int q = warp & 3, half = warp >> 2, row = q * 32 + lane, e = a0 + row;
-    int lo = 0x7fffffff, hi = 0;
-    if (e < a1) {
-      const int w = a.ws.a_win[size_t(b) * a.ws.cap_a + e];
-      lo = max(win_off[w] - a_off[w], b0) - b0;
-      hi = min(win_off[w + 1] - a_off[w + 1], b1) - b0;
-    }
-
-    // rows the tile does not have and chunks past the hidden size are not fetched at all; the pieces of
-    // the last chunk that lie past the hidden size are zero-filled
-    auto issue = [&](int f, uint32_t stage) {
-      const uint32_t sb = ring + stage * FT_STAGE_BYTES + slot0;
-      const bool odd = passes == 4 && (f & 1);
-      const int kc0 = (f >> chunk_shift) * chunk_mul;
-      const uint32_t okm = odd ? ok_o : ok_e;
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int kc = kc0 + (passes == 1 ? (t & 1) : 0);
-        if (kc >= nk || !((okm >> t) & 1)) continue;
-        const uint32_t bytes = ((c_lo + kc) * 64 + c * 8 < a.d) ? 16u : 0u;   // d is a multiple of 8
-        const unsigned char* p = odd ? src_o[t] : src_e[t];
-        cp_async16(sb + t * 4096, p + (bytes ? size_t(kc0) * 128 : 0), bytes);
-      }
-    };
-    // acc += lo^2 + hi^2 for the four bf16 pairs of v, each product exact in fp32 and added with one rounding
-    // (the mixed-precision fma reads the bf16 halves directly: no unpacking instructions)
-    auto sumsq = [](const uint4& v, float acc) {
-      const uint32_t u[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-      for (int j = 0; j < 4; ++j)
-        asm("{\n\t.reg .b16 lo, hi;\n\tmov.b32 {lo, hi}, %1;\n\t"
-            "fma.rn.f32.bf16 %0, lo, lo, %0;\n\tfma.rn.f32.bf16 %0, hi, hi, %0;\n\t}" : "+f"(acc) : "r"(u[j]));
-      return acc;
-    };
-
-    // fill F of this CTA (counted across tiles) uses stage F % 6; it may be written once the MMAs that read
-    // fill F - 6 have completed, and is complete for the MMA warp on phase (F / 6) & 1 of full[]
-    bool ok = true;
-    for (int f = 0; f < FT_AHEAD; ++f) {
-      if (f < nf && ok) {
-        const uint32_t F = done + f;
-        ok = mbar_wait(&empty[F % FT_STAGES], ((F / FT_STAGES) & 1) ^ 1, abort_flag);
-        if (ok) issue(f, F % FT_STAGES);
-      }
-      cp_async_commit();
-    }
-    for (int f = 0; ok && f < nf; ++f) {
-      const int fn = f + FT_AHEAD;
-      if (fn < nf) {
-        const uint32_t F = done + fn;
-        if (!mbar_wait(&empty[F % FT_STAGES], ((F / FT_STAGES) & 1) ^ 1, abort_flag)) { ok = false; break; }
-        issue(fn, F % FT_STAGES);
-      }
-      cp_async_commit();
-      cp_async_wait<FT_AHEAD>();                          // this thread's pieces of fill f have landed
-      const uint32_t s_cur = (done + f) % FT_STAGES;
-      const uint32_t sb = ring + s_cur * FT_STAGE_BYTES + slot0;
-      const bool odd = passes == 4 && (f & 1);
-      const int kc0 = (f >> chunk_shift) * chunk_mul;
-      const uint32_t okm = odd ? ok_o : ok_e;
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        if (kc0 + (passes == 1 ? (t & 1) : 0) >= nk || !((okm >> t) & 1)) continue;
-        const uint4 v = ld_shared16(sb + t * 4096);
-        if (odd) acc_o[t] = sumsq(v, acc_o[t]); else acc_e[t] = sumsq(v, acc_e[t]);
-      }
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&full[s_cur]);           // the MMA warp fences the proxies after its wait
-    }
-    cp_async_wait<0>();
-
-    // ---- norms: squared sums of A row g + 32 i and B row g + 32 i, then across the eight threads of a row
-    float ssa[4], ssb[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) { ssa[i] = acc_e[i]; ssb[i] = acc_o[i]; }                 // passes 4
-    if (passes == 2) { ssb[0] = acc_e[2]; ssb[1] = acc_e[3]; }
-    if (passes == 1) { ssa[0] = acc_e[0] + acc_e[1]; ssb[0] = acc_e[2] + acc_e[3]; }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-#pragma unroll
-      for (int o = 1; o < 8; o <<= 1) {
-        ssa[i] += __shfl_xor_sync(0xffffffffu, ssa[i], o);
-        ssb[i] += __shfl_xor_sync(0xffffffffu, ssb[i], o);
-      }
-      if (c == 0 && i < passes) {                         // a cluster exchanges the squared partial sums
-        const bool root = ks == 1 && a.metric == LIGHTKV_FD_COSINE;
-        a_nrm[g + 32 * i] = root ? sqrtf(ssa[i]) : ssa[i];
-        b_nrm[g + 32 * i] = root ? sqrtf(ssb[i]) : ssb[i];
-      }
-    }
-    named_barrier(1, FT_LOADERS);
-
-    // ---- epilogue: thread = A row (TMEM lane); warps 0-3 scan columns 0-63, warps 4-7 columns 64-127
-    ok = ok && mbar_wait(acc_full, n_items & 1, abort_flag);
-    ok = __all_sync(0xffffffffu, ok);                     // the TMEM loads below are warp-wide
-    tc_fence_after();
-    // columns some row of this warp needs: blocks of eight outside that range are skipped as a whole
-    const int lo_w = __reduce_min_sync(0xffffffffu, lo), hi_w = __reduce_max_sync(0xffffffffu, hi);
-    const float na = row < cap_rows ? a_nrm[row] : 0.f;
-    float best = 3.0e38f;
-    int best_c = -1;
-    if (CLUSTER && ok && ks > 1) {
-      // cluster: this CTA's partial G goes to shared memory as float [128][kFdPitch] over the drained ring
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int c0 = half * 64 + j * 32;
-        if (c0 >= n_cols) break;                          // warp-uniform
-        float v[32];
-        tmem_ld32(tmem_base + (uint32_t(q * 32) << 16) + c0, v);
-        tmem_ld_wait();
-        float* prow = reinterpret_cast<float*>(base) + row * kFdPitch + c0;
-#pragma unroll
-        for (int i = 0; i < 32; ++i) prow[i] = v[i];
-      }
-    }
-    if (ok && ks == 1) {
-#pragma unroll
-      for (int j = 0; j < 2; ++j) {
-        const int c0 = half * 64 + j * 32;
-        if (c0 >= n_cols) break;                          // warp-uniform
-        if (c0 + 32 <= lo_w || c0 >= hi_w) continue;      // warp-uniform
-        float v[32];
-        tmem_ld32(tmem_base + (uint32_t(q * 32) << 16) + c0, v);
-        tmem_ld_wait();
-#pragma unroll
-        for (int blk = 0; blk < 4; ++blk) {
-          if (c0 + blk * 8 + 8 <= lo_w || c0 + blk * 8 >= hi_w) continue;   // warp-uniform
-#pragma unroll
-          for (int i = blk * 8; i < blk * 8 + 8; ++i) {
-            const int col = c0 + i;
-            if (col >= lo && col < hi) {
-              const float fd = pair_score(a.metric, v[i], na, b_nrm[col]);
-              if (fd < best) { best = fd; best_c = col; }
-            }
-          }
-        }
-      }
-    }
-    if (ks == 1) {
-    if (half == 1) { red_f[row] = best; red_c[row] = best_c; }
-    named_barrier(1, FT_LOADERS);
-    if (half == 0 && ok && e < a1) {
-      if (red_f[row] < best) { best = red_f[row]; best_c = red_c[row]; }   // ties stay with the lower column
-      if (best_c >= 0) {
-        const unsigned long long key = ((unsigned long long)orderable(best) << 32) | (unsigned)(b0 + best_c);
-        unsigned long long* dst = a.ws.a_key + size_t(b) * a.ws.cap_a + e;
-        if (tl.blocks_b > 1) atomicMin(dst, key); else *dst = key;
-      }
-    }
-    }
-    tc_fence_before();                                    // TMEM reads done before the next tile's MMAs
-  } else if (lane == 0) {
-    // ---- MMA issue: one chunk = four K = 16 steps inside the 128-byte rows
-    const uint32_t idesc = idesc_bf16(kFdTile, n_cols);
-    auto chunk_mma = [&](uint32_t a_addr, uint32_t b_addr, bool first) {
-#pragma unroll
-      for (int kk = 0; kk < 4; ++kk)
-        umma_bf16(tmem_base, smem_desc_sw128(a_addr + kk * 32), smem_desc_sw128(b_addr + kk * 32), idesc,
-                  !(first && kk == 0));
-    };
-    if (passes == 4) {
-      for (int k = 0; k < nk; ++k) {
-        const uint32_t FA = done + 2 * k, FB = FA + 1, sA = FA % FT_STAGES, sB = FB % FT_STAGES;
-        if (!mbar_wait(&full[sA], (FA / FT_STAGES) & 1, abort_flag)) break;
-        if (!mbar_wait(&full[sB], (FB / FT_STAGES) & 1, abort_flag)) break;
-        fence_proxy_async();                              // the loaders' cp.async writes -> visible to the tensor core
-        tc_fence_after();
-        chunk_mma(ring + sA * FT_STAGE_BYTES, ring + sB * FT_STAGE_BYTES, k == 0);
-        umma_commit(&empty[sA]);
-        umma_commit(&empty[sB]);
+  uint32_t done = 0, tiles = 0;                 // fills and tiles completed (phases of the barriers)
+  for (int ia = ia0;; ia += a.grid_blocks) {
+  bool more_a = false;
+  for (int ib = ib0;; ib += a.grid_blocks) {
+    // ---- the tile's rows
+    int na, nb, a_first = 0, b_first = 0;       // sources and destinations of the whole window; list mode: first entries
+    bool wanted = true;                         // the window loses tokens at all
+    if (a.lists) {
+      const int nW = a.ws.n_windows;
+      const int* win_off = a.ws.win_off + size_t(b) * (nW + 1) + w;
+      const int* a_off = a.ws.a_off + size_t(b) * (nW + 1) + w;
+      a_first = a_off[0];
+      b_first = win_off[0] - a_first;
+      na = a_off[1] - a_first;
+      nb = win_off[1] - win_off[0] - na;
+      for (int r = tid; r < 2 * BLK; r += FT_LOADERS + 32) {
+        const int e = r < BLK ? ia * BLK + r : ib * BLK + r - BLK;
+        if (r < BLK) { if (e < na) row_a[r] = a.ws.a_tok[size_t(b) * a.ws.cap_a + a_first + e]; }
+        else if (e < nb) row_b[r - BLK] = a.ws.b_tok[size_t(b) * a.ws.cap_b + b_first + e];
       }
     } else {
-      for (int f = 0; f < nf; ++f) {
-        const uint32_t F = done + f, s = F % FT_STAGES;
-        if (!mbar_wait(&full[s], (F / FT_STAGES) & 1, abort_flag)) break;
-        fence_proxy_async();
-        tc_fence_after();
-        const uint32_t sa = ring + s * FT_STAGE_BYTES;
-        if (passes == 2) {
-          chunk_mma(sa, sa + 8192, f == 0);
-        } else {
-          chunk_mma(sa, sa + 8192, f == 0);
-          if (2 * f + 1 < nk) chunk_mma(sa + 4096, sa + 12288, false);
+      const bool publish = rank == 0 && ia == 0 && ib == 0;   // the map kernel reads the window's tokens
+      const int nw = min(a.max_cell, window_tokens<FT_WARPS>(a.g, a.pos ? a.pos + size_t(b) * a.cap_in : nullptr, n, w, match, warp_sum, [&](int l, int i) {
+        if (l < a.max_cell) {
+          const bool src = (l & 1) == par;
+          const int r = (l >> 1) - (src ? ia : ib) * BLK;
+          if (r >= 0 && r < BLK) (src ? row_a : row_b)[r] = i;
+          if (publish) win_tok[1 + l] = i;
+        } else if (publish) {                   // only if positions repeat or lie outside the grid: survives
+          a.ws.partner[size_t(b) * a.cap_in + i] = -1;
+          a.ws.slot[size_t(b) * a.cap_in + i] = 0;
         }
-        umma_commit(&empty[s]);
-      }
+      }));
+      if (publish && tid == 0) win_tok[0] = nw;
+      na = (nw + 1 - par) >> 1;
+      nb = nw - na;
+      wanted = nb > 0 && removal_count(nw, a.keep, par) > 0;
     }
-    umma_commit(acc_full);
+    const bool more_b = wanted && nb > (ib + a.grid_blocks) * BLK;
+    more_a = wanted && na > (ia + a.grid_blocks) * BLK;
+    wanted = wanted && na > ia * BLK && nb > ib * BLK;
+    __syncthreads();
+    if (wanted) {                               // the same for every thread of the CTA and of its cluster
+      na = min(na - ia * BLK, BLK);
+      nb = min(nb - ib * BLK, BLK);
+      if (warp < 8) {
+        // ---- gather: thread = 16-byte piece c of rows g + 32 i of both operands
+        const int c = tid & 7, g = tid >> 3;
+        const __nv_bfloat16* xb = a.x + size_t(b) * a.batch_stride + size_t(a.seq_start ? a.seq_start[b] : 0) * a.row_stride +
+                                  c_lo * 64 + c * 8;
+        const uint32_t row16 = uint32_t(a.row_stride >> 3);                   // row pitch in 16-byte units
+        uint32_t off[2 * NR];                                                 // A rows, B rows; all ones: no such row
+#pragma unroll
+        for (int i = 0; i < NR; ++i) {
+          off[i] = g + 32 * i < na ? uint32_t(row_a[g + 32 * i]) * row16 : 0xffffffffu;
+          off[NR + i] = g + 32 * i < nb ? uint32_t(row_b[g + 32 * i]) * row16 : 0xffffffffu;
+        }
+        const uint32_t slot0 = uint32_t(g) * 128 + (uint32_t(c ^ (g & 7)) << 4);   // swizzled offset of row g; row g + 32 i is 4096 i further
+        float ss[2 * NR];
+#pragma unroll
+        for (int i = 0; i < 2 * NR; ++i) ss[i] = 0.f;
+        auto issue = [&](int k) {
+          const uint32_t F = done + k, sb = ring + (F % FT_STAGES) * M::STAGE + slot0;
+          const uint32_t bytes = (c_lo + k) * 64 + c * 8 < a.d ? 16u : 0u;    // d is a multiple of 8
+          const __nv_bfloat16* p = xb + (bytes ? k * 64 : 0);
+#pragma unroll
+          for (int i = 0; i < 2 * NR; ++i)
+            if (off[i] != 0xffffffffu) cp_async16(sb + i * 4096, p + size_t(off[i]) * 8, bytes);
+        };
+        bool ok = true;
+        auto fill = [&](int k) {                            // once the MMAs that read the stage before have completed
+          if (ok && k < nk) {
+            const uint32_t F = done + k;
+            ok = F < FT_STAGES || mbar_wait(&empty[F % FT_STAGES], ((F / FT_STAGES) & 1) ^ 1, abort_flag);
+            if (ok) issue(k);
+          }
+          cp_async_commit();
+        };
+#pragma unroll
+        for (int k = 0; k < FT_AHEAD; ++k) fill(k);
+        for (int k = 0; ok && k < nk; ++k) {
+          cp_async_wait<FT_AHEAD - 1>();                    // this thread's pieces of chunk k have landed
+          const uint32_t s = (done + k) % FT_STAGES, sb = ring + s * M::STAGE + slot0;
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&full[s]);             // the MMA warp fences the proxies after its wait
+#pragma unroll
+          for (int i = 0; i < 2 * NR; ++i)
+            if (off[i] != 0xffffffffu) ss[i] = sumsq16(ld_shared16(sb + i * 4096), ss[i]);
+          fill(k + FT_AHEAD);                               // the stage of chunk k - 1, whose MMAs ran beside the norms
+        }
+        cp_async_wait<0>();
+
+        // ---- squared norms of the rows (this CTA's columns)
+#pragma unroll
+        for (int i = 0; i < 2 * NR; ++i) {
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) ss[i] += __shfl_xor_sync(0xffffffffu, ss[i], o);
+          if (c == 0) sq[(i < NR ? 0 : BLK) + g + 32 * (i % NR)] = ss[i];
+        }
+        named_barrier(1, FT_LOADERS);
+        ok = ok && mbar_wait(acc_full, tiles & 1, abort_flag);
+        ok = __all_sync(0xffffffffu, ok);                   // the TMEM loads below are warp-wide
+        tc_fence_after();
+        const int q = warp & 3, half = warp >> 2;
+        if (!CLUSTER) {
+          for (int i = tid; i < 2 * BLK; i += FT_LOADERS) nrm[i] = a.metric == LIGHTKV_FD_COSINE ? sqrtf(sq[i]) : sq[i];
+          named_barrier(1, FT_LOADERS);
+          // ---- thread = A row (TMEM lane).  BLK 128: warps 0-3 scan columns 0-63, warps 4-7 columns 64-127 of the row; BLK 256:
+          //      warps 0-3 take the first 128 rows, warps 4-7 the others
+          const int row = (BLK > 128 ? half * 128 : 0) + q * 32 + lane, col0 = BLK > 128 ? 0 : half * 64;
+          float best = 3.0e38f;
+          int best_c = -1;
+          if (ok && row - lane < na) {
+            const float na_row = nrm[row];
+            for (int c0 = col0; c0 < min(nb, col0 + (BLK > 128 ? 256 : 64)); c0 += 32) {   // warp-uniform
+              float v[32];
+              tmem_ld32(tmem_base + (uint32_t(q * 32) << 16) + (BLK > 128 ? half * 256 : 0) + c0, v);
+              tmem_ld_wait();
+#pragma unroll
+              for (int i = 0; i < 32; ++i) {
+                if (c0 + i < nb) {                          // warp-uniform
+                  const float fd = pair_score(a.metric, v[i], na_row, nrm[BLK + c0 + i]);
+                  if (fd < best) { best = fd; best_c = c0 + i; }
+                }
+              }
+            }
+          }
+          if (BLK > 128) {
+            if (row < na && ok) store_key<BLK>(a, b, ia, ib, row, row_a, a_first, b_first, best, best_c);
+          } else {
+            if (half == 1) { red_f[row] = best; red_c[row] = best_c; }
+            named_barrier(1, FT_LOADERS);
+            if (half == 0 && row < na && ok) {
+              if (red_f[row] < best) { best = red_f[row]; best_c = red_c[row]; }   // ties stay with the lower column
+              store_key<BLK>(a, b, ia, ib, row, row_a, a_first, b_first, best, best_c);
+            }
+          }
+        } else {
+          // ---- cluster: for 128 rows at a time every CTA puts its partial G into shared memory (float [128][PITCH], over
+          //      the drained ring), then CTA `rank` finishes every ks-th row.  All loader threads of every CTA pass all
+          //      barriers, whatever happened before (an aborted CTA contributes garbage and the status bit, never a hang).
+          //      The MMA warp joins them below.
+          for (int m0 = 0; m0 < na; m0 += 128) {
+            if (ok && q * 32 + m0 < na) {
+              for (int c0 = half * 32; c0 < nb; c0 += 64) {
+                float v[32];
+                tmem_ld32(tmem_base + (uint32_t(q * 32) << 16) + (m0 ? 256 : 0) + c0, v);
+                tmem_ld_wait();
+                float* prow = reinterpret_cast<float*>(base) + (q * 32 + lane) * PITCH + c0;
+#pragma unroll
+                for (int i = 0; i < 32; ++i) prow[i] = v[i];
+              }
+            }
+            __syncwarp();
+            cluster_sync();                                 // all partial G and squared norms are in shared memory
+            if (m0 == 0) {
+              for (int i = tid; i < 2 * BLK; i += FT_LOADERS) {
+                const uint32_t src = smem_u32(sq + i);
+                float part[8], sum = 0.f;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) part[j] = j < ks ? ld_cluster_f32(map_to_cta(src, j)) : 0.f;
+#pragma unroll
+                for (int j = 0; j < 8; ++j) sum += part[j];
+                nrm[i] = a.metric == LIGHTKV_FD_COSINE ? sqrtf(sum) : sum;
+              }
+              named_barrier(1, FT_LOADERS);
+            }
+            // a warp per row, four columns per lane at a time, their remote reads all in flight
+            for (int r = rank + warp * ks; r < min(128, na - m0); r += 8 * ks) {
+              float best = 3.0e38f;
+              int best_c = -1;
+              for (int cc = 0; cc < nb; cc += 128) {
+                float v[8][4];
+#pragma unroll
+                for (int j = 0; j < 8; ++j)
+#pragma unroll
+                  for (int t = 0; t < 4; ++t)
+                    v[j][t] = j < ks && cc + lane + 32 * t < nb
+                                  ? ld_cluster_f32(map_to_cta(ring + uint32_t(r * PITCH + cc + lane + 32 * t) * 4, j)) : 0.f;
+#pragma unroll
+                for (int t = 0; t < 4; ++t) {
+                  const int col = cc + lane + 32 * t;
+                  float gsum = 0.f;
+#pragma unroll
+                  for (int j = 0; j < 8; ++j) gsum += v[j][t];   // in rank order
+                  if (col < nb) {
+                    const float fd = pair_score(a.metric, gsum, nrm[m0 + r], nrm[BLK + col]);
+                    if (fd < best) { best = fd; best_c = col; }
+                  }
+                }
+              }
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) {            // minimum over the lanes, ties to the lower column
+                const float of = __shfl_xor_sync(0xffffffffu, best, o);
+                const int oc = __shfl_xor_sync(0xffffffffu, best_c, o);
+                if (oc >= 0 && (best_c < 0 || of < best || (of == best && oc < best_c))) { best = of; best_c = oc; }
+              }
+              if (lane == 0 && !*abort_flag) store_key<BLK>(a, b, ia, ib, m0 + r, row_a, a_first, b_first, best, best_c);
+            }
+            __syncwarp();
+            cluster_sync();                                 // nobody reads this CTA's shared memory any more
+          }
+        }
+        tc_fence_before();                                  // TMEM reads done before the next tile's MMAs
+      } else {
+        if (lane == 0) {
+          // ---- MMA issue: one chunk = four K = 16 steps inside the 128-byte rows
+          const uint32_t idesc = idesc_bf16(128, (nb + 15) & ~15);
+          for (int k = 0; k < nk; ++k) {
+            const uint32_t F = done + k, s = F % FT_STAGES, sa = ring + s * M::STAGE;
+            if (!mbar_wait(&full[s], (F / FT_STAGES) & 1, abort_flag)) break;
+            fence_proxy_async();                            // the loaders' cp.async writes -> visible to the tensor core
+            tc_fence_after();
+#pragma unroll
+            for (int m = 0; m < BLK / 128; ++m) {
+              if (m * 128 >= na) break;
+#pragma unroll
+              for (int kk = 0; kk < 4; ++kk)
+                umma_bf16(tmem_base + m * 256, smem_desc_sw128(sa + m * 16384 + kk * 32),
+                          smem_desc_sw128(sa + BLK * 128 + kk * 32), idesc, k > 0 || kk > 0);
+            }
+            umma_commit(&empty[s]);
+          }
+          umma_commit(acc_full);
+        }
+        if (CLUSTER)
+          for (int m0 = 0; m0 < na; m0 += 128) {
+            __syncwarp();
+            cluster_sync();
+            cluster_sync();
+          }
+      }
+      done += nk;
+      ++tiles;
+      __syncthreads();                                      // the tile's lists and accumulators are free
+    }
+    if (!more_b || (!CLUSTER && *abort_flag)) break;     // (the CTAs of a cluster stay together)
   }
-  if (CLUSTER && ks > 1) {
-    // ---- cluster epilogue.  Every thread of every CTA of the cluster passes both barriers for every tile,
-    //      whatever happened before (an aborted CTA contributes garbage and the status bit, never a hang).
-    __syncwarp();
-    cluster_sync();                                       // all partial G and squared norms are in shared memory
-    if (warp < 8)
-      fd_cluster_finish(a.metric, a.ws.a_win + size_t(b) * a.ws.cap_a, a.ws.a_key + size_t(b) * a.ws.cap_a, ks, rank, a0, a1, b0, b1,
-                        tl.blocks_b > 1, win_off, a_off, smem_u32(base), a_nrm, b_nrm, red_f,
-                        reinterpret_cast<float*>(red_c), abort_flag);
-    __syncwarp();
-    cluster_sync();                                       // nobody reads this CTA's shared memory any more
+  if (!more_a || (!CLUSTER && *abort_flag)) break;
   }
-  done += nf;
-  ++n_items;
-  if (*abort_flag && ks == 1) break;
-  }  // work items
   tc_fence_before();
   __syncthreads();
   if (warp == 8) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, kFdTile);
+    tmem_dealloc(tmem_base, BLK == 128 ? 128 : 512);
   }
   if (tid == 0 && *abort_flag && a.status) atomicOr(a.status, LIGHTKV_STATUS_TIMEOUT);
 }
 
 bool tc_fd_supported(int hidden) { return hidden % 8 == 0; }
+
+// Nodes a side of a tile: 256 where windows are expected to have more than 128 (at most half as many rows are read), else
+// 128, of which two fit on an SM.
+int fd_tile_side(int fd_side) { return fd_side > 128 ? 256 : 128; }
 
 // SMs of the current device (cached per device ordinal).
 static int sm_count() {
@@ -1054,27 +1017,33 @@ static int sm_count() {
   return cached[dev];
 }
 
-cudaError_t launch_fd_tc(const LayerLaunch& L) {
+cudaError_t launch_fd_tc(const LayerLaunch& L, bool lists) {
   const lightkv_layer_args_t* a = L.a;
   FdTcArgs f;
   f.x = static_cast<const __nv_bfloat16*>(a->hidden) + size_t(a->vis_begin) * a->hidden_row_stride;
   f.seq_start = a->seq_start;
-  f.batch_stride = a->hidden_batch_stride; f.row_stride = a->hidden_row_stride; f.d = L.hidden; f.batch = L.batch;
-  f.metric = L.divergence; f.ws = L.ws; f.status = a->status;
-  // Persistent CTAs, two per SM, no more than the plan expects tiles.  When that estimate leaves SMs idle,
-  // clusters of 2, 4 or 8 CTAs split the hidden dimension of every tile.
-  const long long bound = std::max<long long>(1, (long long)L.fd_tiles * L.batch);   // an estimate, see the plan
-  const int slots = 2 * sm_count(), nk_all = (L.hidden + 63) / 64;
+  f.batch_stride = a->hidden_batch_stride; f.row_stride = a->hidden_row_stride; f.d = L.hidden;
+  f.metric = L.divergence; f.keep = L.keep; f.g = L.geo; f.n_vis = a->n_vis; f.pos = a->pos; f.cap_in = L.ws.cap_in;
+  f.max_cell = L.max_cell; f.blocks = L.fd_blocks; f.lists = lists ? 1 : 0; f.ws = L.ws; f.status = a->status;
+  const int side = fd_tile_side(L.fd_side);
+  f.grid_blocks = std::max(1, (L.fd_side + side - 1) / side);
+  // While there are fewer tiles than CTAs that fit, clusters of 2, 4 or 8 CTAs split the hidden dimension of every tile.
+  const long long tiles = (long long)L.geo.n_windows * f.grid_blocks * f.grid_blocks;
+  const int slots = (side > 128 ? 1 : 2) * sm_count(), nk_all = (L.hidden + 63) / 64;
   int ks = 1;
-  while (ks < 8 && bound * (2 * ks) <= slots && 2 * ks <= nk_all) ks *= 2;
-  const int clusters = (int)std::min<long long>(bound, slots / ks);
-  cudaError_t e;
-  if (ks == 1) {
-    if ((e = ensure_dynamic_smem(fd_tc_kernel<false>, (int)FT_SMEM)) != cudaSuccess) return e;
-    return launch_kernel(fd_tc_kernel<false>, clusters, FT_LOADERS + 32, FT_SMEM, L.stream, 1, f);
+  while (ks < 8 && tiles * L.batch * (2 * ks) <= slots && 4 * ks <= nk_all) ks *= 2;
+  if (tiles * ks > 0x7fffffffLL) return cudaErrorInvalidValue;
+  auto launch = [&](auto kernel, size_t smem) -> cudaError_t {
+    const cudaError_t e = ensure_dynamic_smem(kernel, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_kernel(kernel, dim3((unsigned)(tiles * ks), L.batch), FT_LOADERS + 32, smem, L.stream, ks, f);
+  };
+  if (side > 128) {
+    const size_t smem = FdTcSmem<256>::bytes(f.cap_in, lists);
+    return ks == 1 ? launch(fd_tc_kernel<256, false>, smem) : launch(fd_tc_kernel<256, true>, smem);
   }
-  if ((e = ensure_dynamic_smem(fd_tc_kernel<true>, (int)FT_SMEM)) != cudaSuccess) return e;
-  return launch_kernel(fd_tc_kernel<true>, clusters * ks, FT_LOADERS + 32, FT_SMEM, L.stream, ks, f);
+  const size_t smem = FdTcSmem<128>::bytes(f.cap_in, lists);
+  return ks == 1 ? launch(fd_tc_kernel<128, false>, smem) : launch(fd_tc_kernel<128, true>, smem);
 }
 
 }  // namespace lkv

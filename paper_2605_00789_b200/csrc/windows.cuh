@@ -1,0 +1,164 @@
+// Windows inside a CTA: the tokens of one window from the positions, and the selection of its merged sources (Steps 1, 2
+// and 4).  Used by the FD kernels, which take one window (or a tile of one) per CTA, and by the map kernel.
+#pragma once
+#include "common.cuh"
+
+namespace lkv {
+
+// Calls emit(l, i) for every token i of window w, l its rank inside the window in storage (= position) order, from
+// whatever thread holds it, and returns the number of tokens.  All threads of the CTA (WARPS warps) take part; the caller
+// synchronises before it uses what emit wrote.  A full grid is counted out; otherwise every position is looked at (the
+// position arrays are small, and an unsorted one is still taken apart without a gap: it only raises a status bit).
+// match: [ceil(n / 32)], warp_sum: [WARPS], both in shared memory.
+template <int WARPS, typename Emit>
+__device__ __forceinline__ int window_tokens(const Geometry& g, const int* __restrict__ pos, int n, int w,
+                                             unsigned int* match, int* warp_sum, Emit emit) {
+  constexpr int NT = 32 * WARPS;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int w2 = g.w * g.w, tile = w / w2, wr = (w - tile * w2) / g.w, wc = w - tile * w2 - wr * g.w;
+  const int rows = g.rows[tile], cols = g.cols[tile], first = g.tile_off[tile], n_grid = g.tile_off[g.n_tiles];
+  // rows r with r * w / rows == wr, columns c with c * w / cols == wc
+  const int r0 = (wr * rows + g.w - 1) / g.w, r1 = ((wr + 1) * rows + g.w - 1) / g.w;
+  const int c0 = (wc * cols + g.w - 1) / g.w, c1 = ((wc + 1) * cols + g.w - 1) / g.w;
+  if (!pos && n == n_grid) {
+    const int nw = (r1 - r0) * (c1 - c0);
+    for (int l = tid; l < nw; l += NT) {
+      const int r = l / (c1 - c0);
+      emit(l, first + (r0 + r) * cols + c0 + (l - r * (c1 - c0)));
+    }
+    return nw;
+  }
+  const int lo = first + r0 * cols, hi = first + r1 * cols;
+  const int chunks = (n + 31) >> 5;
+#pragma unroll 4
+  for (int c = warp; c < chunks; c += WARPS) {
+    const int i = c * 32 + lane;
+    bool in = false;
+    if (i < n) {
+      const int p = pos ? pos[i] : i;
+      if (p >= lo && p < hi) {
+        const int col = (p - first) % cols;
+        in = col >= c0 && col < c1;
+      }
+      in = in || (w == 0 && (p < 0 || p >= n_grid));     // no such position: counted with window 0
+    }
+    const unsigned int m = __ballot_sync(0xffffffffu, in);
+    if (lane == 0) match[c] = m;
+  }
+  __syncthreads();
+  int nw = 0;
+  for (int base = 0; base < chunks; base += NT) {
+    const unsigned int m = base + tid < chunks ? match[base + tid] : 0u;
+    const int own = __popc(m);
+    int x = own;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += t;
+    }
+    if (lane == 31) warp_sum[warp] = x;
+    __syncthreads();
+    int before = nw, total = 0;
+#pragma unroll
+    for (int k = 0; k < WARPS; ++k) {
+      const int s = warp_sum[k];
+      if (k < warp) before += s;
+      total += s;
+    }
+    int l = before + x - own;
+    for (unsigned int bits = m; bits; bits &= bits - 1) emit(l++, (base + tid) * 32 + __ffs(bits) - 1);
+    nw += total;
+    __syncthreads();
+  }
+  return nw;
+}
+
+// The lists of one window in shared memory.
+struct WindowLists {
+  unsigned int* key;     // [max_src + 4] orderable lowest score of every source
+  int* best;             // [max_src] destination (rank among the destinations) that attains it, -1: none
+  int* into;             // [max_src] the same for selected sources, -1 for the others
+  int* count;            // [max_dst] sources merged into a destination
+  int* tok;              // [max_cell] token index by local rank
+  static __host__ __device__ size_t bytes(int max_cell) {
+    const size_t src = (max_cell + 1) / 2;
+    return (((src + 7) & ~size_t(3)) + 3 * src + max_cell) * 4;
+  }
+  __device__ static WindowLists at(void* p, int max_cell) {     // p: 16-byte aligned
+    const int src = (max_cell + 1) / 2;
+    WindowLists w;
+    w.key = static_cast<unsigned int*>(p);
+    w.best = reinterpret_cast<int*>(w.key + ((src + 7) & ~3));
+    w.into = w.best + src;
+    w.count = w.into + src;
+    w.tok = w.count + src;
+    return w;
+  }
+};
+
+// Selection: the removal_count(nw) sources with the lowest (score, index) are merged into their best destination.  Writes
+// every token's partner and place (see Workspace).  key / best / tok are complete in shared memory (synchronised) on
+// entry; all threads take part.  A source's rank among the sources of its destination is counted by its own thread in
+// windows of up to 128 sources; in larger ones a warp walks the sources in order, 32 at a time (match_any gives the rank
+// within the 32, a counter per destination the ones before).
+__device__ __forceinline__ void select_window(const WindowLists& s, int nw, double keep, int par, int* __restrict__ partner,
+                                              int* __restrict__ place) {
+  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int na = (nw + 1 - par) >> 1, nb = nw - na;      // sources: local ranks of parity `par`
+  const int removed = nb > 0 ? removal_count(nw, keep, par) : 0;
+  const bool ranked = removed > 0 && removed < na;
+  if (ranked) {
+    if (tid < 4) s.key[na + tid] = 0xffffffffu;          // the last group of four keys
+    __syncthreads();
+  }
+  for (int e = tid; e < na; e += nthr) {
+    bool sel = removed >= na;
+    if (ranked) {
+      const unsigned int mine = s.key[e];
+      int rank = 0;
+      for (int k = 0; k < na; k += 4) {
+        const uint4 v = *reinterpret_cast<const uint4*>(s.key + k);
+        rank += (v.x < mine) + (v.y < mine) + (v.z < mine) + (v.w < mine);
+        if (k < e) rank += (v.x == mine) + (k + 1 < e && v.y == mine) + (k + 2 < e && v.z == mine) + (k + 3 < e && v.w == mine);
+      }
+      sel = rank < removed;
+    }
+    s.into[e] = sel ? s.best[e] : -1;
+  }
+  for (int e = tid; e < nb; e += nthr) s.count[e] = 0;
+  __syncthreads();
+  if (na <= 128) {
+    for (int e = tid; e < na; e += nthr) {
+      const int to = s.into[e], i = s.tok[2 * e + par];
+      int q = 0;
+      if (to >= 0) {
+        for (int k = 0; k < e; ++k) q += s.into[k] == to;
+        atomicAdd(&s.count[to], 1);
+      }
+      partner[i] = to < 0 ? -2 : s.tok[2 * to + 1 - par];
+      place[i] = q;
+    }
+  } else if (tid < 32) {
+    for (int base = 0; base < na; base += 32) {
+      const int e = base + tid, to = e < na ? s.into[e] : -1;
+      const unsigned int peers = __match_any_sync(0xffffffffu, to);
+      const int before = to >= 0 ? s.count[to] : 0;
+      __syncwarp();
+      if (to >= 0 && tid == __ffs(peers) - 1) s.count[to] = before + __popc(peers);
+      __syncwarp();
+      if (e < na) {
+        const int i = s.tok[2 * e + par];
+        partner[i] = to < 0 ? -2 : s.tok[2 * to + 1 - par];
+        place[i] = to < 0 ? 0 : before + __popc(peers & ((1u << tid) - 1u));
+      }
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < nb; e += nthr) {
+    const int i = s.tok[2 * e + 1 - par];
+    partner[i] = -1;
+    place[i] = s.count[e];
+  }
+}
+
+}  // namespace lkv
