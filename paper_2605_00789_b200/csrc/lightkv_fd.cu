@@ -69,7 +69,7 @@ struct FdStreamSmem {
   static constexpr int FIXED = RING > PART ? RING : PART;
   // + the window's lists and the match masks of the search
   static size_t bytes(int max_cell, int cap_in) {
-    return FIXED + WindowLists::bytes(max_cell) + size_t((cap_in + 31) / 32) * 4;
+    return FIXED + WindowLists::bytes(max_cell) + window_search_bytes(cap_in);
   }
 };
 

@@ -680,12 +680,13 @@ constexpr int FT_AHEAD = FT_STAGES - 1;                   // fills in flight bes
 
 template <int BLK>
 struct FdTcSmem {
-  static constexpr int PITCH = BLK + 1;                   // row pitch (floats) of a partial G
+  static constexpr int PITCH = BLK + 4;                   // row pitch (floats) of a partial G: 16-byte pieces of eight rows
+                                                          // in a row of lanes meet no bank conflict
   static constexpr uint32_t STAGE = BLK * 256;            // BLK A rows | BLK B rows of 64 columns
   static constexpr uint32_t CTL = 128 + 4 * BLK * 4 + 2 * 128 * 4 + 2 * BLK * 4 + 16 * 4;
   static_assert(128 * PITCH * 4 <= FT_STAGES * STAGE, "a partial G of 128 rows fits over the drained ring");
   static size_t bytes(int cap_in, bool lists) {
-    return 1024 /* alignment */ + FT_STAGES * STAGE + CTL + (lists ? 0 : size_t((cap_in + 31) / 32) * 4);
+    return 1024 /* alignment */ + FT_STAGES * STAGE + CTL + (lists ? 0 : window_search_bytes(cap_in));
   }
 };
 
@@ -834,9 +835,16 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kern
           const uint32_t s = (done + k) % FT_STAGES, sb = ring + s * M::STAGE + slot0;
           __syncwarp();
           if (lane == 0) mbar_arrive(&full[s]);             // the MMA warp fences the proxies after its wait
+          // (rows the tile does not have hold whatever is there: their norms are not used.  Eight loads in flight and no test:
+          // row after row the norms took 1.4 us a chunk, twice the MMAs)
 #pragma unroll
-          for (int i = 0; i < 2 * NR; ++i)
-            if (off[i] != 0xffffffffu) ss[i] = sumsq16(ld_shared16(sb + i * 4096), ss[i]);
+          for (int i0 = 0; i0 < 2 * NR; i0 += 8) {
+            uint4 v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) v[i] = ld_shared16(sb + (i0 + i) * 4096);
+#pragma unroll
+            for (int i = 0; i < 8; ++i) ss[i0 + i] = sumsq16(v[i], ss[i0 + i]);
+          }
           fill(k + FT_AHEAD);                               // the stage of chunk k - 1, whose MMAs ran beside the norms
         }
         cp_async_wait<0>();
@@ -897,9 +905,9 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kern
                 float v[32];
                 tmem_ld32(tmem_base + (uint32_t(q * 32) << 16) + (m0 ? 256 : 0) + c0, v);
                 tmem_ld_wait();
-                float* prow = reinterpret_cast<float*>(base) + (q * 32 + lane) * PITCH + c0;
+                float4* prow = reinterpret_cast<float4*>(reinterpret_cast<float*>(base) + (q * 32 + lane) * PITCH + c0);
 #pragma unroll
-                for (int i = 0; i < 32; ++i) prow[i] = v[i];
+                for (int i = 0; i < 8; ++i) prow[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
               }
             }
             __syncwarp();
@@ -916,37 +924,52 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kern
               }
               named_barrier(1, FT_LOADERS);
             }
-            // a warp per row, four columns per lane at a time, their remote reads all in flight
-            for (int r = rank + warp * ks; r < min(128, na - m0); r += 8 * ks) {
-              float best = 3.0e38f;
-              int best_c = -1;
-              for (int cc = 0; cc < nb; cc += 128) {
-                float v[8][4];
+            // a warp per row, two rows at a time, four columns per lane and piece, all of their remote reads in flight; the
+            // CTAs start with different peers
+            const int r_end = min(128, na - m0);
+            for (int r = rank + warp * ks; r < r_end; r += 16 * ks) {
+              float4 v[2][8][BLK / 128];
+#pragma unroll
+              for (int t = 0; t < 2; ++t)
 #pragma unroll
                 for (int j = 0; j < 8; ++j)
 #pragma unroll
-                  for (int t = 0; t < 4; ++t)
-                    v[j][t] = j < ks && cc + lane + 32 * t < nb
-                                  ? ld_cluster_f32(map_to_cta(ring + uint32_t(r * PITCH + cc + lane + 32 * t) * 4, j)) : 0.f;
+                  for (int cc = 0; cc < BLK / 128; ++cc) {
+                    const int rr = r + t * 8 * ks;
+                    v[t][j][cc] = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (j < ks && rr < r_end && cc * 128 + 4 * lane < nb)
+                      v[t][j][cc] = ld_cluster_f32x4(map_to_cta(ring + uint32_t(rr * PITCH + cc * 128 + 4 * lane) * 4, (rank + j) & (ks - 1)));
+                  }
 #pragma unroll
-                for (int t = 0; t < 4; ++t) {
-                  const int col = cc + lane + 32 * t;
-                  float gsum = 0.f;
+              for (int t = 0; t < 2; ++t) {
+                const int rr = r + t * 8 * ks;
+                if (rr >= r_end) break;                     // warp-uniform
+                float best = 3.0e38f;
+                int best_c = -1;
 #pragma unroll
-                  for (int j = 0; j < 8; ++j) gsum += v[j][t];   // in rank order
-                  if (col < nb) {
-                    const float fd = pair_score(a.metric, gsum, nrm[m0 + r], nrm[BLK + col]);
-                    if (fd < best) { best = fd; best_c = col; }
+                for (int cc = 0; cc < BLK / 128; ++cc) {
+                  float g4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+                  for (int j = 0; j < 8; ++j) {             // in a fixed order: from this CTA's own part on
+                    g4[0] += v[t][j][cc].x; g4[1] += v[t][j][cc].y; g4[2] += v[t][j][cc].z; g4[3] += v[t][j][cc].w;
+                  }
+#pragma unroll
+                  for (int k = 0; k < 4; ++k) {
+                    const int col = cc * 128 + 4 * lane + k;
+                    if (col < nb) {
+                      const float fd = pair_score(a.metric, g4[k], nrm[m0 + rr], nrm[BLK + col]);
+                      if (fd < best) { best = fd; best_c = col; }
+                    }
                   }
                 }
-              }
 #pragma unroll
-              for (int o = 16; o > 0; o >>= 1) {            // minimum over the lanes, ties to the lower column
-                const float of = __shfl_xor_sync(0xffffffffu, best, o);
-                const int oc = __shfl_xor_sync(0xffffffffu, best_c, o);
-                if (oc >= 0 && (best_c < 0 || of < best || (of == best && oc < best_c))) { best = of; best_c = oc; }
+                for (int o = 16; o > 0; o >>= 1) {          // minimum over the lanes, ties to the lower column
+                  const float of = __shfl_xor_sync(0xffffffffu, best, o);
+                  const int oc = __shfl_xor_sync(0xffffffffu, best_c, o);
+                  if (oc >= 0 && (best_c < 0 || of < best || (of == best && oc < best_c))) { best = of; best_c = oc; }
+                }
+                if (lane == 0 && !*abort_flag) store_key<BLK>(a, b, ia, ib, m0 + rr, row_a, a_first, b_first, best, best_c);
               }
-              if (lane == 0 && !*abort_flag) store_key<BLK>(a, b, ia, ib, m0 + r, row_a, a_first, b_first, best, best_c);
             }
             __syncwarp();
             cluster_sync();                                 // nobody reads this CTA's shared memory any more

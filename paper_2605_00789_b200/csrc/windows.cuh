@@ -9,7 +9,9 @@ namespace lkv {
 // whatever thread holds it, and returns the number of tokens.  All threads of the CTA (WARPS warps) take part; the caller
 // synchronises before it uses what emit wrote.  A full grid is counted out; otherwise every position is looked at (the
 // position arrays are small, and an unsorted one is still taken apart without a gap: it only raises a status bit).
-// match: [ceil(n / 32)], warp_sum: [WARPS], both in shared memory.
+// match: window_search_bytes(cap_in), warp_sum: [WARPS], both in shared memory.
+__host__ __device__ inline size_t window_search_bytes(int cap_in) { return size_t((cap_in + 31) / 32) * 8; }
+
 template <int WARPS, typename Emit>
 __device__ __forceinline__ int window_tokens(const Geometry& g, const int* __restrict__ pos, int n, int w,
                                              unsigned int* match, int* warp_sum, Emit emit) {
@@ -30,20 +32,29 @@ __device__ __forceinline__ int window_tokens(const Geometry& g, const int* __res
   }
   const int lo = first + r0 * cols, hi = first + r1 * cols;
   const int chunks = (n + 31) >> 5;
+  // four consecutive tokens per lane, 128 per warp and step: enough loads in flight that a sample of a few thousand tokens
+  // is one or two round trips
 #pragma unroll 4
-  for (int c = warp; c < chunks; c += WARPS) {
-    const int i = c * 32 + lane;
-    bool in = false;
-    if (i < n) {
-      const int p = pos ? pos[i] : i;
-      if (p >= lo && p < hi) {
-        const int col = (p - first) % cols;
+  for (int c = warp * 4; c < chunks; c += WARPS * 4) {
+    const int i = c * 32 + lane * 4;
+    int p[4];
+#pragma unroll
+    for (int k = 0; k < 4; ++k) p[k] = i + k < n ? (pos ? pos[i + k] : i + k) : 0;
+    unsigned int m = 0;
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+      bool in = false;
+      if (p[k] >= lo && p[k] < hi) {
+        const int col = (p[k] - first) % cols;
         in = col >= c0 && col < c1;
       }
-      in = in || (w == 0 && (p < 0 || p >= n_grid));     // no such position: counted with window 0
+      in = in || (w == 0 && (p[k] < 0 || p[k] >= n_grid));   // no such position: counted with window 0
+      if (in && i + k < n) m |= 1u << ((lane & 7) * 4 + k);
     }
-    const unsigned int m = __ballot_sync(0xffffffffu, in);
-    if (lane == 0) match[c] = m;
+    m |= __shfl_xor_sync(0xffffffffu, m, 1);
+    m |= __shfl_xor_sync(0xffffffffu, m, 2);
+    m |= __shfl_xor_sync(0xffffffffu, m, 4);
+    if ((lane & 7) == 0 && c + (lane >> 3) < chunks) match[c + (lane >> 3)] = m;
   }
   __syncthreads();
   int nw = 0;
@@ -65,10 +76,13 @@ __device__ __forceinline__ int window_tokens(const Geometry& g, const int* __res
       if (k < warp) before += s;
       total += s;
     }
-    int l = before + x - own;
-    for (unsigned int bits = m; bits; bits &= bits - 1) emit(l++, (base + tid) * 32 + __ffs(bits) - 1);
+    if (base + tid < chunks) match[chunks + base + tid] = before + x - own;   // tokens of the window in front of the word
     nw += total;
     __syncthreads();
+  }
+  for (int c = warp; c < chunks; c += WARPS) {           // a lane per token: a window may be as dense as the sample
+    const unsigned int m = match[c];
+    if ((m >> lane) & 1u) emit((int)match[chunks + c] + __popc(m & ((1u << lane) - 1u)), c * 32 + lane);
   }
   return nw;
 }
