@@ -9,6 +9,7 @@
 namespace lkv {
 
 constexpr int kMaxTiles = 32;          // image tiles / frames per sample
+constexpr int kFdTile = 128;           // sources (and destinations) per tile of the tensor-core FD kernel
 constexpr int kMaxWindows = 2048;      // windows per sample (window-build kernel keeps 32 x n_windows u16 counters in smem)
 constexpr int kMaxWindowTokens = 65535;  // tokens of one window (range of those counters)
 

@@ -36,7 +36,7 @@ struct LayerLaunch {
   int dtype, xi_mode, divergence;
   double keep;
   int fd_side;                       // estimate of the larger side (A or B nodes) of a window: picks the FD kernel
-  int fd_blocks;                     // tiles of fd_tile_side(fd_side) nodes a side the largest window may have
+  int fd_blocks;                     // tiles of kFdTile nodes a side the largest window may have
   int max_cell;                      // most tokens a window can hold
   int n_grid;                        // grid positions of all tiles
   Geometry geo;
@@ -101,7 +101,6 @@ bool tc_fd_supported(int hidden);
 bool tc_xi_supported(int head_dim);
 // lists: windows from launch_window_build, keys by source entry for launch_select_map; else by token for launch_map
 cudaError_t launch_fd_tc(const LayerLaunch& L, bool lists);
-int fd_tile_side(int fd_side);
 // wait_first: the stream's last kernel is not the window build or FD of the same call
 cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first);
 

@@ -202,8 +202,8 @@ int lightkv_plan(const lightkv_config_t* c, lightkv_plan_t** out) {
     // where counts depend on the data: the tokens still alive are spread over the cells about evenly (the kernels walk
     // larger windows, up to a whole cell, in blocks)
     if (!sp.exact) sp.fd_side = (int)(((long long)cell * sp.cap_in / p->n_vis0 + 2) / 2);
-    const int side = fd_tile_side(sp.fd_side), typical = (std::max(sp.fd_side, 1) + side - 1) / side;
-    sp.fd_blocks = ((sp.max_cell + 1) / 2 + side - 1) / side;
+    const int typical = (std::max(sp.fd_side, 1) + kFdTile - 1) / kFdTile;
+    sp.fd_blocks = ((sp.max_cell + 1) / 2 + kFdTile - 1) / kFdTile;
     sp.fd_tiles = (int)std::min<long long>((long long)g.n_windows * typical * typical, 0x7fffffff);
     if (!exact) {   // data-dependent from here on: every window keeps at most ceil(keep n_w) tokens
       long long bound = (long long)ceil(sp.keep * sp.cap_in) + sp.n_windows;

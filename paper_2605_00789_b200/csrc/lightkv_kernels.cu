@@ -754,7 +754,7 @@ struct MapArgs {
   int* place;
   const unsigned long long* key;       // SELECT: [B, blocks, cap_in]
   const int* win_tok;                  // SELECT: [B, n_windows, max_cell + 1]
-  int blocks, max_cell, n_windows, src_par, tile_side;
+  int blocks, max_cell, n_windows, src_par;
   double keep;
   int* n_vis_out;
   int* pos_out;
@@ -800,7 +800,7 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
       for (int e = tid; e < na; e += nthr) {
         const int i = win_tok[1 + 2 * e + par];
         unsigned long long key = ~0ull;
-        for (int ib = 0; scored && ib * a.tile_side < nb; ++ib)
+        for (int ib = 0; scored && ib * kFdTile < nb; ++ib)
           key = min(key, a.key[(size_t(b) * a.blocks + ib) * a.cap_in + i]);
         lists.key[e] = (unsigned int)(key >> 32);
         lists.best[e] = (unsigned int)key == 0xffffffffu ? -1 : (int)(unsigned int)key;
@@ -980,7 +980,7 @@ cudaError_t launch_map(const LayerLaunch& L, bool select) {
   m.cap_a = L.ws.cap_a; m.cap_b = L.ws.cap_b; m.n_grid = L.n_grid;
   m.n_vis = a->n_vis; m.pos = a->pos; m.xi_in = a->xi; m.xi_h = L.ws.xi_h; m.partner = L.ws.partner; m.place = L.ws.slot;
   m.key = L.ws.a_key; m.win_tok = L.ws.win_tok; m.blocks = L.fd_blocks; m.max_cell = L.max_cell; m.n_windows = L.geo.n_windows;
-  m.src_par = L.geo.src_par; m.tile_side = fd_tile_side(L.fd_side); m.keep = L.keep;
+  m.src_par = L.geo.src_par; m.keep = L.keep;
   m.n_vis_out = a->n_vis_out; m.pos_out = a->pos_out; m.dst = a->dst; m.weight = a->weight; m.grp_off = a->grp_off;
   m.grp_src = a->grp_src; m.xi_out = a->xi_out; m.status = a->status;
   // one cluster per sample: as many CTAs of up to 1024 threads as give every thread one token (two beyond 8192), and

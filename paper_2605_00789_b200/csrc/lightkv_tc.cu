@@ -640,21 +640,22 @@ cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first) {
 // FD + best partner for larger windows on tensor cores (Eq. "similarity", Step 2).
 //
 // A CTA (or a cluster of ks CTAs that split the hidden dimension, where there are few tiles) takes one tile of up to
-// BLK sources x BLK destinations of one window, BLK = 128 or, for larger windows, 256.  The rows of a tile are scattered
-// over the sequence; the CTA finds them from the positions (window_tokens) or, for samples too long for that, in the
-// lists the window build left.  Eight warps gather them with 16-byte cp.async copies, eight threads per 128-byte row
-// segment, straight into the 128-byte-swizzled K-major layout tcgen05 reads, through a ring of three stages (64 columns
+// 128 sources x 128 destinations of one window.  The rows of a tile are scattered over the sequence; the CTA finds them
+// from the positions (window_tokens) or, for samples too long for that, in the lists the window build left.  Eight warps gather them with 16-byte cp.async copies, eight threads per 128-byte row
+// segment, straight into the 128-byte-swizzled K-major layout tcgen05 reads, through a ring of stages of 32 KB (64 columns
 // of both operands), and re-read their pieces to accumulate the squared norms.  A ninth warp issues
-// G += X_A X_B^T (128 x N x 64 per half of 128 sources and chunk, bf16 -> fp32 in TMEM).  The MMA always reads 128 A
+// G += X_A X_B^T (128 x N x 64 per chunk, bf16 -> fp32 in TMEM).  The MMA always reads 128 A
 // rows: rows the tile does not have are never written and only feed accumulator rows nobody reads.  After the last chunk
 // the loader warps turn into the epilogue: minimum over the destinations (ties: lowest index) of every source, one key
 // per (source, block of destinations), of which the map kernel takes the lowest.
 //
-// Every tile reads its rows again, so the kernel is bound by the way from L2 through shared memory (a 64-column chunk of
-// a 128 x 128 tile: 32 KB written, read by the norms and read by the MMA), not by HBM or the tensor pipe; a tile of 256
-// halves that.  The launch has as many tiles as windows of the expected size need; a CTA goes on with the blocks of a
-// window that has grown beyond that.
-// FD_TC_FIGURES
+// Every tile reads its rows again, so the kernel is bound by the way from L2 through shared memory (a chunk: 32 KB
+// written, read by the norms and read by the MMA), not by HBM or the tensor pipe.  Tiles of 256 x 256 halve that, but the
+// four CTAs they then leave per SM's worth of work have to exchange partial products, and distributed shared memory gave
+// 10 bytes per nanosecond and SM (13 us per 128 rows of 256): 62, with the exchange vectorised 56 us, where tiles of 128
+// with a six-stage ring take 44 (two samples of 8192 tokens x 3584 in windows of 512; list-driven tiles that met in atomics
+// took 77; windows of 1024 and 2048: 76 -> 45 and 76 -> 43).  The launch has as many tiles as windows of the expected
+// size need; a CTA goes on with the blocks of a window that has grown beyond that.
 // ======================================================================================================
 struct FdTcArgs {
   const __nv_bfloat16* x;              // first vision row of sample 0
@@ -675,23 +676,21 @@ struct FdTcArgs {
 };
 
 constexpr int FT_LOADERS = 256, FT_WARPS = 9;
-constexpr int FT_STAGES = 3;
-constexpr int FT_AHEAD = FT_STAGES - 1;                   // fills in flight beside the one being consumed
+constexpr int BLK = kFdTile;
 
-template <int BLK>
+template <int STAGES>
 struct FdTcSmem {
   static constexpr int PITCH = BLK + 4;                   // row pitch (floats) of a partial G: 16-byte pieces of eight rows
                                                           // in a row of lanes meet no bank conflict
   static constexpr uint32_t STAGE = BLK * 256;            // BLK A rows | BLK B rows of 64 columns
   static constexpr uint32_t CTL = 128 + 4 * BLK * 4 + 2 * 128 * 4 + 2 * BLK * 4 + 16 * 4;
-  static_assert(128 * PITCH * 4 <= FT_STAGES * STAGE, "a partial G of 128 rows fits over the drained ring");
+  static_assert(BLK * PITCH * 4 <= STAGES * STAGE, "a partial G fits over the drained ring");
   static size_t bytes(int cap_in, bool lists) {
-    return 1024 /* alignment */ + FT_STAGES * STAGE + CTL + (lists ? 0 : window_search_bytes(cap_in));
+    return 1024 /* alignment */ + STAGES * STAGE + CTL + (lists ? 0 : window_search_bytes(cap_in));
   }
 };
 
 // the best destination of source `row` of tile (ia, ib) of sample b
-template <int BLK>
 __device__ __forceinline__ void store_key(const FdTcArgs& a, int b, int ia, int ib, int row, const int* row_a, int a_first,
                                           int b_first, float best, int best_c) {
   unsigned long long key = ~0ull;
@@ -702,9 +701,10 @@ __device__ __forceinline__ void store_key(const FdTcArgs& a, int b, int ia, int 
 }
 
 // CLUSTER = false is the plain launch (ks = 1) with the cluster code compiled out.
-template <int BLK, bool CLUSTER>
-__global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kernel(const __grid_constant__ FdTcArgs a) {
-  using M = FdTcSmem<BLK>;
+template <bool CLUSTER, int FT_STAGES>
+__global__ void __launch_bounds__(FT_LOADERS + 32, FT_STAGES > 3 ? 1 : 2) fd_tc_kernel(const __grid_constant__ FdTcArgs a) {
+  using M = FdTcSmem<FT_STAGES>;
+  constexpr int FT_AHEAD = FT_STAGES - 1;       // fills in flight beside the one being consumed
   constexpr int NR = BLK / 32;                  // rows of an operand per loader thread
   constexpr int PITCH = M::PITCH;
   extern __shared__ unsigned char smem_raw[];
@@ -731,7 +731,7 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kern
     *abort_flag = 0;
     fence_barrier_init();
   }
-  if (warp == 8) { tmem_alloc(tmem_slot, BLK == 128 ? 128 : 512); tmem_relinquish(); }
+  if (warp == 8) { tmem_alloc(tmem_slot, BLK); tmem_relinquish(); }
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
@@ -864,16 +864,15 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kern
         if (!CLUSTER) {
           for (int i = tid; i < 2 * BLK; i += FT_LOADERS) nrm[i] = a.metric == LIGHTKV_FD_COSINE ? sqrtf(sq[i]) : sq[i];
           named_barrier(1, FT_LOADERS);
-          // ---- thread = A row (TMEM lane).  BLK 128: warps 0-3 scan columns 0-63, warps 4-7 columns 64-127 of the row; BLK 256:
-          //      warps 0-3 take the first 128 rows, warps 4-7 the others
-          const int row = (BLK > 128 ? half * 128 : 0) + q * 32 + lane, col0 = BLK > 128 ? 0 : half * 64;
+          // ---- thread = A row (TMEM lane); warps 0-3 scan columns 0-63, warps 4-7 columns 64-127
+          const int row = q * 32 + lane, col0 = half * 64;
           float best = 3.0e38f;
           int best_c = -1;
           if (ok && row - lane < na) {
             const float na_row = nrm[row];
-            for (int c0 = col0; c0 < min(nb, col0 + (BLK > 128 ? 256 : 64)); c0 += 32) {   // warp-uniform
+            for (int c0 = col0; c0 < min(nb, col0 + 64); c0 += 32) {   // warp-uniform
               float v[32];
-              tmem_ld32(tmem_base + (uint32_t(q * 32) << 16) + (BLK > 128 ? half * 256 : 0) + c0, v);
+              tmem_ld32(tmem_base + (uint32_t(q * 32) << 16) + c0, v);
               tmem_ld_wait();
 #pragma unroll
               for (int i = 0; i < 32; ++i) {
@@ -884,96 +883,81 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kern
               }
             }
           }
-          if (BLK > 128) {
-            if (row < na && ok) store_key<BLK>(a, b, ia, ib, row, row_a, a_first, b_first, best, best_c);
-          } else {
-            if (half == 1) { red_f[row] = best; red_c[row] = best_c; }
-            named_barrier(1, FT_LOADERS);
-            if (half == 0 && row < na && ok) {
-              if (red_f[row] < best) { best = red_f[row]; best_c = red_c[row]; }   // ties stay with the lower column
-              store_key<BLK>(a, b, ia, ib, row, row_a, a_first, b_first, best, best_c);
-            }
+          if (half == 1) { red_f[row] = best; red_c[row] = best_c; }
+          named_barrier(1, FT_LOADERS);
+          if (half == 0 && row < na && ok) {
+            if (red_f[row] < best) { best = red_f[row]; best_c = red_c[row]; }   // ties stay with the lower column
+            store_key(a, b, ia, ib, row, row_a, a_first, b_first, best, best_c);
           }
         } else {
-          // ---- cluster: for 128 rows at a time every CTA puts its partial G into shared memory (float [128][PITCH], over
-          //      the drained ring), then CTA `rank` finishes every ks-th row.  All loader threads of every CTA pass all
-          //      barriers, whatever happened before (an aborted CTA contributes garbage and the status bit, never a hang).
-          //      The MMA warp joins them below.
-          for (int m0 = 0; m0 < na; m0 += 128) {
-            if (ok && q * 32 + m0 < na) {
-              for (int c0 = half * 32; c0 < nb; c0 += 64) {
-                float v[32];
-                tmem_ld32(tmem_base + (uint32_t(q * 32) << 16) + (m0 ? 256 : 0) + c0, v);
-                tmem_ld_wait();
-                float4* prow = reinterpret_cast<float4*>(reinterpret_cast<float*>(base) + (q * 32 + lane) * PITCH + c0);
+          // ---- cluster: every CTA puts its partial G into shared memory (float [128][PITCH], over the drained ring), then CTA
+          //      `rank` finishes every ks-th row.  All threads of every CTA pass both barriers, whatever happened before (an
+          //      aborted CTA contributes garbage and the status bit, never a hang); the MMA warp joins them below.
+          if (ok && q * 32 < na) {
+            for (int c0 = half * 32; c0 < nb; c0 += 64) {
+              float v[32];
+              tmem_ld32(tmem_base + (uint32_t(q * 32) << 16) + c0, v);
+              tmem_ld_wait();
+              float4* prow = reinterpret_cast<float4*>(reinterpret_cast<float*>(base) + (q * 32 + lane) * PITCH + c0);
 #pragma unroll
-                for (int i = 0; i < 8; ++i) prow[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
-              }
+              for (int i = 0; i < 8; ++i) prow[i] = make_float4(v[4 * i], v[4 * i + 1], v[4 * i + 2], v[4 * i + 3]);
             }
-            __syncwarp();
-            cluster_sync();                                 // all partial G and squared norms are in shared memory
-            if (m0 == 0) {
-              for (int i = tid; i < 2 * BLK; i += FT_LOADERS) {
-                const uint32_t src = smem_u32(sq + i);
-                float part[8], sum = 0.f;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) part[j] = j < ks ? ld_cluster_f32(map_to_cta(src, j)) : 0.f;
-#pragma unroll
-                for (int j = 0; j < 8; ++j) sum += part[j];
-                nrm[i] = a.metric == LIGHTKV_FD_COSINE ? sqrtf(sum) : sum;
-              }
-              named_barrier(1, FT_LOADERS);
-            }
-            // a warp per row, two rows at a time, four columns per lane and piece, all of their remote reads in flight; the
-            // CTAs start with different peers
-            const int r_end = min(128, na - m0);
-            for (int r = rank + warp * ks; r < r_end; r += 16 * ks) {
-              float4 v[2][8][BLK / 128];
-#pragma unroll
-              for (int t = 0; t < 2; ++t)
-#pragma unroll
-                for (int j = 0; j < 8; ++j)
-#pragma unroll
-                  for (int cc = 0; cc < BLK / 128; ++cc) {
-                    const int rr = r + t * 8 * ks;
-                    v[t][j][cc] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    if (j < ks && rr < r_end && cc * 128 + 4 * lane < nb)
-                      v[t][j][cc] = ld_cluster_f32x4(map_to_cta(ring + uint32_t(rr * PITCH + cc * 128 + 4 * lane) * 4, (rank + j) & (ks - 1)));
-                  }
-#pragma unroll
-              for (int t = 0; t < 2; ++t) {
-                const int rr = r + t * 8 * ks;
-                if (rr >= r_end) break;                     // warp-uniform
-                float best = 3.0e38f;
-                int best_c = -1;
-#pragma unroll
-                for (int cc = 0; cc < BLK / 128; ++cc) {
-                  float g4[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                  for (int j = 0; j < 8; ++j) {             // in a fixed order: from this CTA's own part on
-                    g4[0] += v[t][j][cc].x; g4[1] += v[t][j][cc].y; g4[2] += v[t][j][cc].z; g4[3] += v[t][j][cc].w;
-                  }
-#pragma unroll
-                  for (int k = 0; k < 4; ++k) {
-                    const int col = cc * 128 + 4 * lane + k;
-                    if (col < nb) {
-                      const float fd = pair_score(a.metric, g4[k], nrm[m0 + rr], nrm[BLK + col]);
-                      if (fd < best) { best = fd; best_c = col; }
-                    }
-                  }
-                }
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) {          // minimum over the lanes, ties to the lower column
-                  const float of = __shfl_xor_sync(0xffffffffu, best, o);
-                  const int oc = __shfl_xor_sync(0xffffffffu, best_c, o);
-                  if (oc >= 0 && (best_c < 0 || of < best || (of == best && oc < best_c))) { best = of; best_c = oc; }
-                }
-                if (lane == 0 && !*abort_flag) store_key<BLK>(a, b, ia, ib, m0 + rr, row_a, a_first, b_first, best, best_c);
-              }
-            }
-            __syncwarp();
-            cluster_sync();                                 // nobody reads this CTA's shared memory any more
           }
+          __syncwarp();
+          cluster_sync();                                   // all partial G and squared norms are in shared memory
+          {
+            const uint32_t src = smem_u32(sq + tid);
+            float part[8], sum = 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) part[j] = j < ks ? ld_cluster_f32(map_to_cta(src, j)) : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) sum += part[j];
+            nrm[tid] = a.metric == LIGHTKV_FD_COSINE ? sqrtf(sum) : sum;
+          }
+          named_barrier(1, FT_LOADERS);
+          // a warp per row, two rows at a time, four columns per lane, all of their remote reads in flight; the CTAs start
+          // with different peers
+          for (int r = rank + warp * ks; r < na; r += 16 * ks) {
+            float4 v[2][8];
+#pragma unroll
+            for (int t = 0; t < 2; ++t)
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {
+                const int rr = r + t * 8 * ks;
+                v[t][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                if (j < ks && rr < na && 4 * lane < nb)
+                  v[t][j] = ld_cluster_f32x4(map_to_cta(ring + uint32_t(rr * PITCH + 4 * lane) * 4, (rank + j) & (ks - 1)));
+              }
+#pragma unroll
+            for (int t = 0; t < 2; ++t) {
+              const int rr = r + t * 8 * ks;
+              if (rr >= na) break;                          // warp-uniform
+              float best = 3.0e38f;
+              int best_c = -1;
+              float g4[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+              for (int j = 0; j < 8; ++j) {                 // in a fixed order: from this CTA's own part on
+                g4[0] += v[t][j].x; g4[1] += v[t][j].y; g4[2] += v[t][j].z; g4[3] += v[t][j].w;
+              }
+#pragma unroll
+              for (int k = 0; k < 4; ++k) {
+                const int col = 4 * lane + k;
+                if (col < nb) {
+                  const float fd = pair_score(a.metric, g4[k], nrm[rr], nrm[BLK + col]);
+                  if (fd < best) { best = fd; best_c = col; }
+                }
+              }
+#pragma unroll
+              for (int o = 16; o > 0; o >>= 1) {            // minimum over the lanes, ties to the lower column
+                const float of = __shfl_xor_sync(0xffffffffu, best, o);
+                const int oc = __shfl_xor_sync(0xffffffffu, best_c, o);
+                if (oc >= 0 && (best_c < 0 || of < best || (of == best && oc < best_c))) { best = of; best_c = oc; }
+              }
+              if (lane == 0 && !*abort_flag) store_key(a, b, ia, ib, rr, row_a, a_first, b_first, best, best_c);
+            }
+          }
+          __syncwarp();
+          cluster_sync();                                   // nobody reads this CTA's shared memory any more
         }
         tc_fence_before();                                  // TMEM reads done before the next tile's MMAs
       } else {
@@ -986,23 +970,17 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kern
             fence_proxy_async();                            // the loaders' cp.async writes -> visible to the tensor core
             tc_fence_after();
 #pragma unroll
-            for (int m = 0; m < BLK / 128; ++m) {
-              if (m * 128 >= na) break;
-#pragma unroll
-              for (int kk = 0; kk < 4; ++kk)
-                umma_bf16(tmem_base + m * 256, smem_desc_sw128(sa + m * 16384 + kk * 32),
-                          smem_desc_sw128(sa + BLK * 128 + kk * 32), idesc, k > 0 || kk > 0);
-            }
+            for (int kk = 0; kk < 4; ++kk)
+              umma_bf16(tmem_base, smem_desc_sw128(sa + kk * 32), smem_desc_sw128(sa + BLK * 128 + kk * 32), idesc, k > 0 || kk > 0);
             umma_commit(&empty[s]);
           }
           umma_commit(acc_full);
         }
-        if (CLUSTER)
-          for (int m0 = 0; m0 < na; m0 += 128) {
-            __syncwarp();
-            cluster_sync();
-            cluster_sync();
-          }
+        if (CLUSTER) {
+          __syncwarp();
+          cluster_sync();
+          cluster_sync();
+        }
       }
       done += nk;
       ++tiles;
@@ -1016,16 +994,12 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, BLK > 128 ? 1 : 2) fd_tc_kern
   __syncthreads();
   if (warp == 8) {
     tc_fence_after();
-    tmem_dealloc(tmem_base, BLK == 128 ? 128 : 512);
+    tmem_dealloc(tmem_base, BLK);
   }
   if (tid == 0 && *abort_flag && a.status) atomicOr(a.status, LIGHTKV_STATUS_TIMEOUT);
 }
 
 bool tc_fd_supported(int hidden) { return hidden % 8 == 0; }
-
-// Nodes a side of a tile: 256 where windows are expected to have more than 128 (at most half as many rows are read), else
-// 128, of which two fit on an SM.
-int fd_tile_side(int fd_side) { return fd_side > 128 ? 256 : 128; }
 
 // SMs of the current device (cached per device ordinal).
 static int sm_count() {
@@ -1048,25 +1022,23 @@ cudaError_t launch_fd_tc(const LayerLaunch& L, bool lists) {
   f.batch_stride = a->hidden_batch_stride; f.row_stride = a->hidden_row_stride; f.d = L.hidden;
   f.metric = L.divergence; f.keep = L.keep; f.g = L.geo; f.n_vis = a->n_vis; f.pos = a->pos; f.cap_in = L.ws.cap_in;
   f.max_cell = L.max_cell; f.blocks = L.fd_blocks; f.lists = lists ? 1 : 0; f.ws = L.ws; f.status = a->status;
-  const int side = fd_tile_side(L.fd_side);
-  f.grid_blocks = std::max(1, (L.fd_side + side - 1) / side);
-  // While there are fewer tiles than CTAs that fit, clusters of 2, 4 or 8 CTAs split the hidden dimension of every tile.
-  const long long tiles = (long long)L.geo.n_windows * f.grid_blocks * f.grid_blocks;
-  const int slots = (side > 128 ? 1 : 2) * sm_count(), nk_all = (L.hidden + 63) / 64;
+  f.grid_blocks = std::max(1, (L.fd_side + BLK - 1) / BLK);
+  // While there are fewer tiles than CTAs that fit (two per SM), clusters of 2, 4 or 8 CTAs split the hidden dimension of
+  // every tile.  Where every tile has an SM of its own without that, the ring takes all of its shared memory.
+  const long long tiles = (long long)L.geo.n_windows * f.grid_blocks * f.grid_blocks, all = tiles * L.batch;
+  const int sms = sm_count(), nk_all = (L.hidden + 63) / 64;
+  const bool deep = all <= sms && 4 * all > 3 * sms;
   int ks = 1;
-  while (ks < 8 && tiles * L.batch * (2 * ks) <= slots && 4 * ks <= nk_all) ks *= 2;
+  while (!deep && ks < 8 && all * (2 * ks) <= 2 * sms && 4 * ks <= nk_all) ks *= 2;
   if (tiles * ks > 0x7fffffffLL) return cudaErrorInvalidValue;
   auto launch = [&](auto kernel, size_t smem) -> cudaError_t {
     const cudaError_t e = ensure_dynamic_smem(kernel, (int)smem);
     if (e != cudaSuccess) return e;
     return launch_kernel(kernel, dim3((unsigned)(tiles * ks), L.batch), FT_LOADERS + 32, smem, L.stream, ks, f);
   };
-  if (side > 128) {
-    const size_t smem = FdTcSmem<256>::bytes(f.cap_in, lists);
-    return ks == 1 ? launch(fd_tc_kernel<256, false>, smem) : launch(fd_tc_kernel<256, true>, smem);
-  }
-  const size_t smem = FdTcSmem<128>::bytes(f.cap_in, lists);
-  return ks == 1 ? launch(fd_tc_kernel<128, false>, smem) : launch(fd_tc_kernel<128, true>, smem);
+  if (deep) return launch(fd_tc_kernel<false, 6>, FdTcSmem<6>::bytes(f.cap_in, lists));
+  const size_t smem = FdTcSmem<3>::bytes(f.cap_in, lists);
+  return ks == 1 ? launch(fd_tc_kernel<false, 3>, smem) : launch(fd_tc_kernel<true, 3>, smem);
 }
 
 }  // namespace lkv

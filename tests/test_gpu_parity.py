@@ -490,6 +490,24 @@ def test_map_of_streaming_windows_over_cluster_sizes(grid, w):
     H.run_schedule(wl, xi_mode="given", ragged=True, first_pos=[full, subset])
 
 
+@pytest.mark.parametrize("grid,w,batch,hidden", [
+    ((9, 9), 1, 120, 72),       # 41 nodes a side, a tile per SM: the deep ring
+    ((16, 16), 1, 1, 776),      # 128 a side, clusters of eight
+    ((16, 16), 1, 160, 72),     # 128 a side, more tiles than SMs, no cluster
+    ((7, 37), 1, 2, 328),       # 130 and 129 a side: tiles of one and two rows
+    ((33, 62), 2, 1, 200),      # windows of 496 to 527 tokens
+    ((66, 62), 1, 1, 72),       # one window of 4092 tokens: the most the lists of a CTA hold
+    ((70, 64), 1, 1, 72),       # one of 4480: window lists and keys through atomics
+])
+def test_fd_tiles_over_window_sizes(grid, w, batch, hidden):
+    wl = S.Workload(name="fdtile", config_id=136, batch=batch, tiles=(grid,), n_text=4, hidden=hidden, n_q_heads=2,
+                    n_kv_heads=1, head_dim=64, n_layers=16, layers=(3,), windows=(w,), keep=(0.6,))
+    samples = sorted({0, batch // 2, batch - 1})
+    H.run_schedule(wl, xi_mode="uniform", oracle_samples=samples)
+    if batch < 10 and grid[0] * grid[1] < 3000:
+        H.run_schedule(wl, xi_mode="uniform", direction="b2a", metric="l2sq", oracle_samples=samples)
+
+
 # ---- subsets of the grid: capacities ---------------------------------------------------------------------------
 
 def _near_full_subset():
