@@ -1350,7 +1350,13 @@ kv_plane_kernel(T* __restrict__ k_buf, T* __restrict__ v_buf, KvAddr ad, KvPlane
 #pragma unroll 4
   for (int idx = tid; idx < total; idx += KVI_THREADS) {
     const int r = div_magic(idx, magic_ch), c = idx - r * ch;
-    st_stream16(buf + addr[r] + c * V, rows[idx]);
+    const uint4 v = rows[idx];
+    st_stream16(buf + addr[r] + c * V, v);
+    // a merged group also replaces its survivor's row where that lies behind the new end, as the two-phase form leaves it
+    if (r < n_out && !gather && off[r + 1] - off[r] > 1) {
+      const int s = mem[off[r]];
+      if (s >= n_out + n_text_after) st_stream16(buf + addr[s] + c * V, v);
+    }
   }
 }
 

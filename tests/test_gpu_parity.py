@@ -298,6 +298,28 @@ def test_in_place_planes_over_cuts(batch, n_kv, head_dim, grid, text, kv_mode, p
     H.run_schedule(wl, xi_mode="given", kv_mode=kv_mode, paged=paged, kv_in_place=True)
 
 
+def test_in_place_rows_behind_the_new_end():
+    # a merged group replaces its survivor's row also where that row lies behind the new end of the sample; all other
+    # rows there keep what they held (the one-kernel form leaves the cache as the merge-then-move form does)
+    import torch
+    import paper_2605_00789_b200 as L
+    wl = dataclasses.replace(S.workload("cfg1"), hidden=64, n_q_heads=2, n_kv_heads=2)
+    plan = H.make_plan(wl, xi_mode="uniform")
+    inp = H.prepare_stage(wl, 0)
+    gpu = H.gpu_stage(plan, wl, 0, inp, xi_mode="uniform")
+    k = H.to_device(inp["k"], "bf16")
+    v = H.to_device(inp["v"], "bf16")
+    L.compact_kv(plan, 0, gpu["out"], k, v, k, v, vis_begin=wl.n_text)
+    got = k.float().cpu().numpy()[0]
+    n_out, off, src = int(gpu["n_vis_out"][0]), gpu["grp_off"][0], gpu["grp_src"][0]
+    want = inp["k"][0].copy()
+    for o in range(n_out):
+        if off[o + 1] - off[o] > 1:
+            want[:, wl.n_text + src[off[o]]] = gpu["k_out"][0][:, wl.n_text + o]
+    np.testing.assert_array_equal(got[:, wl.n_text + n_out:], want[:, wl.n_text + n_out:])
+    plan.close()
+
+
 def test_in_place_equals_out_of_place_bit_for_bit():
     wl = S.workload("cfg1")
     plan = H.make_plan(wl)
