@@ -18,7 +18,7 @@ namespace lkv {
 // an MMA is free as long as both operands agree, so the eight bf16 of a 16-byte piece serve as the lane's k
 // elements of two MMA steps, for the row's role as an A operand and as a B operand alike.  The squared norms
 // accumulate from the same registers (exact products, fp32 sums).  Partial inner products of the warps meet in
-// shared memory in warp order, then a warp per source row takes the minimum over the destinations (ties: lowest
+// shared memory in warp order, then eight lanes per source row take the minimum over the destinations (ties: lowest
 // index).  A window with more nodes than the template holds is walked in blocks of 8 * O by 8 * O.
 // Since the CTA has its whole window, it also finds the window's tokens (from the positions; no list has to be built
 // before) and makes the selection of Steps 2 and 4; what is left for the map kernel is one prefix sum per sample.
@@ -264,33 +264,43 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
         }
         __syncthreads();
       }
-      // ---- a warp per source row, lanes over the destinations
-      for (int r = rank + warp * ks; r < na; r += nwarps * ks) {
+      // ---- scores of the rows this CTA finishes (every ks-th), a thread per pair, over the pair's first partial product
+      const int nr = rank < na ? (na - rank + ks - 1) / ks : 0;
+      for (int idx = tid; idx < nr * nb; idx += NT) {
+        const int i = idx / nb, col = idx - i * nb, r = rank + i * ks;
+        float v[8], s = 0.f;
+        if (ks == 1) {
+#pragma unroll
+          for (int k = 0; k < nwarps; ++k) v[k] = part[(k * R + r) * PITCH + col];
+#pragma unroll
+          for (int k = 0; k < nwarps; ++k) s += v[k];
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) v[j] = j < ks ? tc::ld_cluster_f32(tc::map_to_cta(tc::smem_u32(part + r * PITCH + col), j)) : 0.f;
+#pragma unroll
+          for (int j = 0; j < 8; ++j) s += v[j];
+        }
+        part[r * PITCH + col] = pair_score(a.metric, s, nrm[r], nrm[R + col]);
+      }
+      __syncthreads();
+      // ---- eight lanes per row
+      for (int i0 = 0; i0 < nr; i0 += NT / 8) {
+        const int i = i0 + (tid >> 3), r = rank + i * ks;
         float lowest = 3.0e38f;
         int col_min = -1;
-        for (int col = lane; col < nb; col += 32) {
-          float s = 0.f;
-          if (ks == 1) {
-            s = part[r * PITCH + col];
-            for (int k = 1; k < nwarps; ++k) s += part[(k * R + r) * PITCH + col];
-          } else {
-            float v[8];
-#pragma unroll
-            for (int j = 0; j < 8; ++j) v[j] = j < ks ? tc::ld_cluster_f32(tc::map_to_cta(tc::smem_u32(part + r * PITCH + col), j)) : 0.f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) s += v[j];
+        if (i < nr)
+          for (int col = tid & 7; col < nb; col += 8) {
+            const float fd = part[r * PITCH + col];
+            if (fd < lowest) { lowest = fd; col_min = col; }
           }
-          const float fd = pair_score(a.metric, s, nrm[r], nrm[R + col]);
-          if (fd < lowest) { lowest = fd; col_min = col; }
-        }
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {               // minimum over the lanes, ties to the lower column
+        for (int o = 4; o > 0; o >>= 1) {                // minimum over the lanes, ties to the lower column
           const float of = __shfl_xor_sync(0xffffffffu, lowest, o);
           const int oc = __shfl_xor_sync(0xffffffffu, col_min, o);
           if (oc >= 0 && (col_min < 0 || of < lowest || (of == lowest && oc < col_min))) { lowest = of; col_min = oc; }
         }
         // later blocks of destinations hold higher indices: an equal score keeps the earlier one
-        if (lane == 0 && col_min >= 0 && orderable(lowest) < lists.key[a0 + r]) {
+        if (i < nr && (tid & 7) == 0 && col_min >= 0 && orderable(lowest) < lists.key[a0 + r]) {
           lists.key[a0 + r] = orderable(lowest);
           lists.best[a0 + r] = b0 + col_min;
           if (rank > 0) {                                // CTA 0 selects
@@ -302,7 +312,7 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
       if (ks == 1) __syncthreads(); else tc::cluster_sync();   // the partial results are overwritten by the next block
     }
   }
-  if (rank == 0) select_window(lists, nw, a.keep, par, partner, place);
+  if (rank == 0) select_window(lists, nw, removed, par, partner, place);
 }
 
 template <typename T, int O, int S, int WARPS>

@@ -796,17 +796,17 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
       const int* win_tok = a.win_tok + (size_t(b) * a.n_windows + w) * (a.max_cell + 1);
       const int nw = win_tok[0], par = a.src_par, na = (nw + 1 - par) >> 1, nb = nw - na;
       for (int l = tid; l < nw; l += nthr) lists.tok[l] = win_tok[1 + l];
-      const bool scored = nb > 0 && removal_count(nw, a.keep, par) > 0;
+      const int removed = nb > 0 ? removal_count(nw, a.keep, par) : 0;
       for (int e = tid; e < na; e += nthr) {
         const int i = win_tok[1 + 2 * e + par];
         unsigned long long key = ~0ull;
-        for (int ib = 0; scored && ib * kFdTile < nb; ++ib)
+        for (int ib = 0; removed > 0 && ib * kFdTile < nb; ++ib)
           key = min(key, a.key[(size_t(b) * a.blocks + ib) * a.cap_in + i]);
         lists.key[e] = (unsigned int)(key >> 32);
         lists.best[e] = (unsigned int)key == 0xffffffffu ? -1 : (int)(unsigned int)key;
       }
       __syncthreads();
-      select_window(lists, nw, a.keep, par, a.partner + row, a.place + row);
+      select_window(lists, nw, removed, par, a.partner + row, a.place + row);
       __syncthreads();
     }
     sync_all();

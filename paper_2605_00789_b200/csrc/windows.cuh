@@ -90,36 +90,35 @@ __device__ __forceinline__ int window_tokens(const Geometry& g, const int* __res
 // The lists of one window in shared memory.
 struct WindowLists {
   unsigned int* key;     // [max_src + 4] orderable lowest score of every source
-  int* best;             // [max_src] destination (rank among the destinations) that attains it, -1: none
-  int* into;             // [max_src] the same for selected sources, -1 for the others
+  int* into;             // [max_src + 4] destination (rank among the destinations) of selected sources, -1 for the others
+  int* best;             // [max_src] destination that attains the lowest score, -1: none
   int* count;            // [max_dst] sources merged into a destination
   int* tok;              // [max_cell] token index by local rank
   static __host__ __device__ size_t bytes(int max_cell) {
     const size_t src = (max_cell + 1) / 2;
-    return (((src + 7) & ~size_t(3)) + 3 * src + max_cell) * 4;
+    return (2 * ((src + 7) & ~size_t(3)) + 2 * src + max_cell) * 4;
   }
   __device__ static WindowLists at(void* p, int max_cell) {     // p: 16-byte aligned
     const int src = (max_cell + 1) / 2;
     WindowLists w;
     w.key = static_cast<unsigned int*>(p);
-    w.best = reinterpret_cast<int*>(w.key + ((src + 7) & ~3));
-    w.into = w.best + src;
-    w.count = w.into + src;
+    w.into = reinterpret_cast<int*>(w.key + ((src + 7) & ~3));
+    w.best = w.into + ((src + 7) & ~3);
+    w.count = w.best + src;
     w.tok = w.count + src;
     return w;
   }
 };
 
-// Selection: the removal_count(nw) sources with the lowest (score, index) are merged into their best destination.  Writes
-// every token's partner and place (see Workspace).  key / best / tok are complete in shared memory (synchronised) on
-// entry; all threads take part.  A source's rank among the sources of its destination is counted by its own thread in
-// windows of up to 128 sources; in larger ones a warp walks the sources in order, 32 at a time (match_any gives the rank
-// within the 32, a counter per destination the ones before).
-__device__ __forceinline__ void select_window(const WindowLists& s, int nw, double keep, int par, int* __restrict__ partner,
+// Selection: the `removed` sources with the lowest (score, index) are merged into their best destination.  Writes every
+// token's partner and place (see Workspace).  key / best / tok are complete in shared memory (synchronised) on entry; all
+// threads take part.  A source's rank among the sources of its destination is counted by its own thread in windows of up
+// to 128 sources; in larger ones a warp walks the sources in order, 32 at a time (match_any gives the rank within the 32, a
+// counter per destination the ones before).
+__device__ __forceinline__ void select_window(const WindowLists& s, int nw, int removed, int par, int* __restrict__ partner,
                                               int* __restrict__ place) {
   const int tid = threadIdx.x, nthr = blockDim.x;
   const int na = (nw + 1 - par) >> 1, nb = nw - na;      // sources: local ranks of parity `par`
-  const int removed = nb > 0 ? removal_count(nw, keep, par) : 0;
   const bool ranked = removed > 0 && removed < na;
   if (ranked) {
     if (tid < 4) s.key[na + tid] = 0xffffffffu;          // the last group of four keys
@@ -146,7 +145,10 @@ __device__ __forceinline__ void select_window(const WindowLists& s, int nw, doub
       const int to = s.into[e], i = s.tok[2 * e + par];
       int q = 0;
       if (to >= 0) {
-        for (int k = 0; k < e; ++k) q += s.into[k] == to;
+        for (int k = 0; k < e; k += 4) {
+          const int4 v = *reinterpret_cast<const int4*>(s.into + k);
+          q += (v.x == to) + (k + 1 < e && v.y == to) + (k + 2 < e && v.z == to) + (k + 3 < e && v.w == to);
+        }
         atomicAdd(&s.count[to], 1);
       }
       partner[i] = to < 0 ? -2 : s.tok[2 * to + 1 - par];
