@@ -18,7 +18,7 @@ namespace lkv {
 // an MMA is free as long as both operands agree, so the eight bf16 of a 16-byte piece serve as the lane's k
 // elements of two MMA steps, for the row's role as an A operand and as a B operand alike.  The squared norms
 // accumulate from the same registers (exact products, fp32 sums).  Partial inner products of the warps meet in
-// shared memory in warp order, then eight lanes per source row take the minimum over the destinations (ties: lowest
+// shared memory in warp order, then 8 to 32 lanes per source row take the minimum over the destinations (ties: lowest
 // index).  A window with more nodes than the template holds is walked in blocks of 8 * O by 8 * O.
 // Since the CTA has its whole window, it also finds the window's tokens (from the positions; no list has to be built
 // before) and makes the selection of Steps 2 and 4; what is left for the map kernel is one prefix sum per sample.
@@ -264,43 +264,37 @@ __global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_cons
         }
         __syncthreads();
       }
-      // ---- scores of the rows this CTA finishes (every ks-th), a thread per pair, over the pair's first partial product
+      // ---- the rows this CTA finishes (every ks-th), each by as many lanes as leave a lane for every row, at least eight
       const int nr = rank < na ? (na - rank + ks - 1) / ks : 0;
-      for (int idx = tid; idx < nr * nb; idx += NT) {
-        const int i = idx / nb, col = idx - i * nb, r = rank + i * ks;
-        float v[8], s = 0.f;
-        if (ks == 1) {
-#pragma unroll
-          for (int k = 0; k < nwarps; ++k) v[k] = part[(k * R + r) * PITCH + col];
-#pragma unroll
-          for (int k = 0; k < nwarps; ++k) s += v[k];
-        } else {
-#pragma unroll
-          for (int j = 0; j < 8; ++j) v[j] = j < ks ? tc::ld_cluster_f32(tc::map_to_cta(tc::smem_u32(part + r * PITCH + col), j)) : 0.f;
-#pragma unroll
-          for (int j = 0; j < 8; ++j) s += v[j];
-        }
-        part[r * PITCH + col] = pair_score(a.metric, s, nrm[r], nrm[R + col]);
-      }
-      __syncthreads();
-      // ---- eight lanes per row
-      for (int i0 = 0; i0 < nr; i0 += NT / 8) {
-        const int i = i0 + (tid >> 3), r = rank + i * ks;
+      int width = 8;
+      while (width < 32 && width < nb && 2 * width * nr <= NT) width *= 2;
+      for (int i0 = 0; i0 < nr; i0 += NT / width) {
+        const int i = i0 + tid / width, r = rank + i * ks;
         float lowest = 3.0e38f;
         int col_min = -1;
-        if (i < nr)
-          for (int col = tid & 7; col < nb; col += 8) {
-            const float fd = part[r * PITCH + col];
-            if (fd < lowest) { lowest = fd; col_min = col; }
-          }
+        for (int col = tid & (width - 1); i < nr && col < nb; col += width) {
+          float v[8], s = 0.f;
+          if (ks == 1) {
 #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) {                // minimum over the lanes, ties to the lower column
+            for (int k = 0; k < nwarps; ++k) v[k] = part[(k * R + r) * PITCH + col];
+#pragma unroll
+            for (int k = 0; k < nwarps; ++k) s += v[k];
+          } else {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) v[j] = j < ks ? tc::ld_cluster_f32(tc::map_to_cta(tc::smem_u32(part + r * PITCH + col), j)) : 0.f;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) s += v[j];
+          }
+          const float fd = pair_score(a.metric, s, nrm[r], nrm[R + col]);
+          if (fd < lowest) { lowest = fd; col_min = col; }
+        }
+        for (int o = width >> 1; o > 0; o >>= 1) {       // minimum over the lanes, ties to the lower column
           const float of = __shfl_xor_sync(0xffffffffu, lowest, o);
           const int oc = __shfl_xor_sync(0xffffffffu, col_min, o);
           if (oc >= 0 && (col_min < 0 || of < lowest || (of == lowest && oc < col_min))) { lowest = of; col_min = oc; }
         }
         // later blocks of destinations hold higher indices: an equal score keeps the earlier one
-        if (i < nr && (tid & 7) == 0 && col_min >= 0 && orderable(lowest) < lists.key[a0 + r]) {
+        if (i < nr && (tid & (width - 1)) == 0 && col_min >= 0 && orderable(lowest) < lists.key[a0 + r]) {
           lists.key[a0 + r] = orderable(lowest);
           lists.best[a0 + r] = b0 + col_min;
           if (rank > 0) {                                // CTA 0 selects
