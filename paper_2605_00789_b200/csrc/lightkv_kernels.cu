@@ -291,15 +291,22 @@ cudaError_t launch_fd_simt(const LayerLaunch& L) {
 
 // =====================================================================================================
 // xi per head, fp32 FMA path (Eq. "attention-factor" with the causal softmax rows of Eq.
-// "attention-matrix").  One CTA per (tile of 64 vision queries, head, sample), longest rows first.  Keys 0..s_i are
-// visited in tiles of 64 with an online (running-maximum) softmax that carries two sums per row: all visible
+// "attention-matrix").  One CTA per (tile of 32 vision queries, head, sample), longest rows first.  Keys 0..s_i are
+// visited in tiles of 32 with an online (running-maximum) softmax that carries two sums per row: all visible
 // keys and the prompt keys J.  Output per head: sum_J / sum_all.  With a caller-supplied row
 // log-sum-exp only the prompt keys are visited: sum_J exp(logit - lse).
-// A thread holds 4 x 4 logits and reads both operands 16 bytes along the head dimension (8 shared-memory loads per 64
-// FMAs, rows padded by four floats: no bank conflicts); the 16 threads of a row meet by shuffles, the groups at the end.  2 x 576 queries x 8
-// heads of 128 in fp32: 140 us with 2 x 4 logits per thread and scalar loads, 60 now.
+// The eight warps of a CTA take every eighth tile of keys, on their own: a warp loads its keys 32 dimensions at a time
+// (cp.async, the next chunk during this one), a lane holds 4 x 8 logits (12 shared-memory loads of 16 bytes per 128 FMAs)
+// and keeps its own maximum and sums of its four queries; lanes and warps meet once, at the end.  Two CTAs per SM, for
+// any head size.  Bound by latency: four warps per scheduler issue 0.6 instructions a clock (packed FMAs, half as many,
+// take the same time).
+// 2 x 576 queries x 8 heads of 128 in fp32: 38 us, the next stage with 317 queries 27; with four groups of 128 threads at
+// a barrier per key tile of 64 (4 x 4 logits a lane) 60 and 33 (bf16, heads of 256: 152 -> 65); 8 x 8 logits a lane, two warps per scheduler: 43 and 33;
+// the head dimension cut over the warps: 46 and 31; two CTAs of a cluster per query tile: 50 and 30.
 // =====================================================================================================
-constexpr int XI_TQ = 32, XI_TK = 64, XI_GROUP = 4 * XI_TQ, XI_GROUPS = 4;
+constexpr int XI_TQ = 32, XI_TK = 32, XI_WARPS = 8, XI_DIMS = 32;
+constexpr int XI_LD = XI_DIMS + 4;                       // pitch of a chunk's rows: eight of them in different banks
+__host__ __device__ inline int xi_q_pitch(int dh) { return (dh + 7) / 8 * 8 + 4; }
 
 template <typename T>
 struct XiSimtArgs {
@@ -315,17 +322,23 @@ struct XiSimtArgs {
 };
 
 template <typename T>
-__global__ void __launch_bounds__(XI_GROUP * XI_GROUPS)
+__global__ void __launch_bounds__(32 * XI_WARPS, 2)
 xi_simt_kernel(XiSimtArgs<T> a, Workspace ws) {
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int dh = a.dh, ld = dh + 4;
-  float* Qs = reinterpret_cast<float*>(smem_raw);       // [XI_TQ][ld]
-  float* Ks = Qs + XI_TQ * ld;                          // [groups][XI_TK][ld]
+  const int dh = a.dh, ldq = xi_q_pitch(dh);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float* ring = reinterpret_cast<float*>(smem_raw) + warp * 2 * XI_TK * XI_LD;            // [warps][2][XI_TK][XI_LD]
+  float* Qs = reinterpret_cast<float*>(smem_raw) + XI_WARPS * 2 * XI_TK * XI_LD;          // [XI_TQ][ldq]
 
-  const int b = blockIdx.z, h = blockIdx.y, t0 = (gridDim.x - 1 - blockIdx.x) * XI_TQ;
-  const int grp = threadIdx.x / XI_GROUP, groups = blockDim.x / XI_GROUP, tid = threadIdx.x - grp * XI_GROUP;
-  int n = a.n_vis ? min(a.n_vis[b], ws.cap_in) : ws.cap_in;
+  // The queries with the most keys first.  Where every CTA is resident at once, two to an SM, the second half starts with
+  // the fewest and hands its tiles to the warps in the other direction: the SMs, and the schedulers of an SM, have about
+  // the same to do.
+  const bool second = gridDim.x <= 2 * 148 && blockIdx.x >= 148;
+  const int item = second ? gridDim.x - 1 - (blockIdx.x - 148) : blockIdx.x;
+  const int tiles = (ws.cap_in + XI_TQ - 1) / XI_TQ, heads = gridDim.x / tiles;           // (heads of all samples)
+  const int b = item % heads / a.n_q_heads, h = item % heads % a.n_q_heads, t0 = (tiles - 1 - item / heads) * XI_TQ;
+  const int n = a.n_vis ? min(a.n_vis[b], ws.cap_in) : ws.cap_in;
   if (t0 >= n) return;
   const int nq = min(XI_TQ, n - t0);
   const int hk = h / (a.n_q_heads / a.n_kv_heads);
@@ -333,119 +346,149 @@ xi_simt_kernel(XiSimtArgs<T> a, Workspace ws) {
   const T* qh = a.q + size_t(b) * a.q_bs + size_t(h) * a.q_hs + size_t(row0) * a.q_rs;
   const T* kh = a.k + size_t(b) * a.k_bs + size_t(hk) * a.k_hs + size_t(row0) * a.k_rs;
   const float scale2 = 1.4426950408889634f / sqrtf((float)dh);      // logits in log2 units
-  const int vis_begin = a.vis_begin;
-  const int n_seq = vis_begin + n + a.n_text_after;                   // keys of this sample
+  const int q_pos = a.vis_begin + t0;                                 // of the first query
+  const int n_seq = a.vis_begin + n + a.n_text_after;                 // keys of this sample
 
-  const int q4 = dh / 4;
-  auto stage = [&](float* dst, const T* src, int64_t row_stride, int rows, int all, int first, int step) {   // rows of dh values, zeros behind them
+  auto put = [](float* dst, const T* p, bool in) {      // four values, zeros if not `in`
     if constexpr (sizeof(T) == 4) {
-      for (int idx = first; idx < all * q4; idx += step) {
-        const int r = idx / q4, c = (idx - r * q4) * 4;
-        tc::cp_async16(tc::smem_u32(dst + r * ld + c), src + size_t(r < rows ? r : 0) * row_stride + c, r < rows ? 16u : 0u);
-      }
-      tc::cp_async_commit();
+      tc::cp_async16(tc::smem_u32(dst), p, in ? 16u : 0u);
     } else {
-#pragma unroll 4
-      for (int idx = first; idx < all * q4; idx += step) {
-        const int r = idx / q4, c = (idx - r * q4) * 4;
-        float f[4] = {0.f, 0.f, 0.f, 0.f};
-        if (r < rows) load4<T>(src + size_t(r) * row_stride + c, f);
-        *reinterpret_cast<float4*>(dst + r * ld + c) = make_float4(f[0], f[1], f[2], f[3]);
-      }
+      float f[4] = {0.f, 0.f, 0.f, 0.f};
+      if (in) load4<T>(p, f);
+      *reinterpret_cast<float4*>(dst) = make_float4(f[0], f[1], f[2], f[3]);
     }
   };
-  stage(Qs, qh + size_t(vis_begin + t0) * a.q_rs, a.q_rs, nq, XI_TQ, threadIdx.x, blockDim.x);
-  tc::cp_async_wait<0>();
-  __syncthreads();
-
-  const int tx = tid & 15, ty = tid >> 4;               // rows 4 ty + i, columns tx + 16 j
-  float m_run[4], l_all[4], l_txt[4], l2[4];
-#pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    m_run[i] = -INFINITY; l_all[i] = 0.f; l_txt[i] = 0.f; l2[i] = 0.f;
-    if (a.lse && 4 * ty + i < nq)
-      l2[i] = a.lse[size_t(b) * a.lse_bs + size_t(h) * a.lse_hs + row0 + vis_begin + t0 + 4 * ty + i] * 1.4426950408889634f;
+  for (int idx = threadIdx.x; idx < XI_TQ * (dh / 4); idx += blockDim.x) {
+    const int r = idx / (dh / 4), d = (idx - r * (dh / 4)) * 4;
+    put(Qs + r * ldq + d, qh + size_t(q_pos + (r < nq ? r : 0)) * a.q_rs + d, r < nq);
   }
-
   // last key any row of the tile may see: its own (causal) or the sample's last (bidirectional)
-  const int s_last = a.bidirectional ? n_seq - 1 : vis_begin + t0 + nq - 1;
+  const int s_last = a.bidirectional ? n_seq - 1 : q_pos + nq - 1;
   const int key_lo = a.lse ? a.text.begin : 0;
   const int key_hi = a.lse ? min(a.text.end, s_last + 1) : s_last + 1;
+  const int j_first = key_lo + (second ? XI_WARPS - 1 - warp : warp) * XI_TK;
+  // the warp's next chunk: lane (lr, ld4) loads 16 bytes of the rows lr + 4 k
+  const int lr = lane >> 3, ld4 = (lane & 7) * 4;
+  int load_j = j_first, load_d = 0;
+  auto load = [&](int st) {
+    if (load_j < key_hi) {
+      const int rows = load_d + ld4 < dh ? min(XI_TK, key_hi - load_j) : 0;
+      const T* p = kh + size_t(load_j) * a.k_rs + load_d;
+      const T* pr = p + size_t(lr) * a.k_rs + ld4;
+      float* dst = ring + st * XI_TK * XI_LD + lr * XI_LD + ld4;
+#pragma unroll
+      for (int k = 0; k < XI_TK / 4; ++k) {
+        const bool in = lr + 4 * k < rows;
+        put(dst + 4 * k * XI_LD, in ? pr : p, in);
+        pr += 4 * a.k_rs;
+      }
+      load_d += XI_DIMS;
+      if (load_d >= dh) { load_d = 0; load_j += XI_WARPS * XI_TK; }
+    }
+    tc::cp_async_commit();
+  };
+  tc::cp_async_commit();
+  load(0);
+  tc::cp_async_wait<1>();
+  __syncthreads();                                      // the queries are there
 
-  const float* Kt = Ks + grp * XI_TK * ld;
-  for (int j0 = key_lo + grp * XI_TK; j0 < key_hi; j0 += groups * XI_TK) {
-    stage(Ks + grp * XI_TK * ld, kh + size_t(j0) * a.k_rs, a.k_rs, min(XI_TK, key_hi - j0), XI_TK, tid, XI_GROUP);
-    tc::cp_async_wait<0>();
-    tc::named_barrier(1 + grp, XI_GROUP);
-    float acc[4][4] = {};
-#pragma unroll 2
-    for (int kk = 0; kk < dh; kk += 4) {
-      float4 q[4], k[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const float4*>(Qs + (4 * ty + i) * ld + kk);
-#pragma unroll
-      for (int j = 0; j < 4; ++j) k[j] = *reinterpret_cast<const float4*>(Kt + (tx + 16 * j) * ld + kk);
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          acc[i][j] = fmaf(q[i].w, k[j].w, fmaf(q[i].z, k[j].z, fmaf(q[i].y, k[j].y, fmaf(q[i].x, k[j].x, acc[i][j]))));
-    }
-    const unsigned long long tmask = a.text.mask64(j0) >> tx;          // bits 0, 16, 32, 48: this thread's columns
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const int last = (a.bidirectional ? n_seq - 1 : vis_begin + t0 + 4 * ty + i) - j0 - tx;   // visible: 16 j <= last
-      float v[4];
-#pragma unroll
-      for (int j = 0; j < 4; ++j) v[j] = 16 * j <= last && j0 + tx + 16 * j < key_hi ? acc[i][j] * scale2 : -INFINITY;
-      if (a.lse) {
-#pragma unroll
-        for (int j = 0; j < 4; ++j)
-          if ((tmask >> (16 * j)) & 1ull) l_txt[i] += exp2f(v[j] - l2[i]);
-        continue;
-      }
-      float mx = fmaxf(fmaxf(v[0], v[1]), fmaxf(v[2], v[3]));
-#pragma unroll
-      for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-      const float m_new = fmaxf(m_run[i], mx);
-      if (m_new == -INFINITY) continue;                 // the row sees none of this group's keys yet (uniform over the row)
-      const float resc = exp2f(m_run[i] - m_new);       // 0 on the first tile (m_run = -inf)
-      l_all[i] *= resc;
-      l_txt[i] *= resc;
-      m_run[i] = m_new;
-#pragma unroll
-      for (int j = 0; j < 4; ++j) {
-        const float p = exp2f(v[j] - m_new);
-        l_all[i] += p;
-        if ((tmask >> (16 * j)) & 1ull) l_txt[i] += p;
-      }
-    }
-    tc::named_barrier(1 + grp, XI_GROUP);               // the tile has been read: its buffer is filled next
-  }
-  // ---- the groups' results of a row meet
-  __shared__ float s_m[XI_GROUPS][XI_TQ], s_all[XI_GROUPS][XI_TQ], s_txt[XI_GROUPS][XI_TQ];
+  const int tx = lane & 3, ty = lane >> 2;              // queries ty + 8 i, keys tx + 4 j
+  float m_run[4], l_all[4], l_txt[4];                   // maximum in log2 units (given log-sum-exp: that); sums
 #pragma unroll
   for (int i = 0; i < 4; ++i) {
+    m_run[i] = -INFINITY; l_all[i] = 0.f; l_txt[i] = 0.f;
+    if (a.lse) {
+      const int r = ty + 8 * i;
+      m_run[i] = r < nq ? a.lse[size_t(b) * a.lse_bs + size_t(h) * a.lse_hs + row0 + q_pos + r] * 1.4426950408889634f : 0.f;
+    }
+  }
+  for (int j0 = j_first, st = 0; j0 < key_hi; j0 += XI_WARPS * XI_TK) {
+    float acc[4][8] = {};
+    for (int d0 = 0; d0 < dh; d0 += XI_DIMS, st ^= 1) {
+      load(st ^ 1);
+      tc::cp_async_wait<1>();
+      __syncwarp();                                     // the chunk is there for all lanes
+      const float* Kt = ring + st * XI_TK * XI_LD + tx * XI_LD;
+      const float* Qt = Qs + ty * ldq + d0;
+      const int dims = min(XI_DIMS, dh - d0);
+#pragma unroll 1
+      for (int kk = 0; kk < dims; kk += 4) {
+        float4 q[4];
 #pragma unroll
-    for (int o = 8; o > 0; o >>= 1) {
+        for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const float4*>(Qt + 8 * i * ldq + kk);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float4 k = *reinterpret_cast<const float4*>(Kt + 4 * j * XI_LD + kk);
+#pragma unroll
+          for (int i = 0; i < 4; ++i)
+            acc[i][j] = fmaf(q[i].w, k.w, fmaf(q[i].z, k.z, fmaf(q[i].y, k.y, fmaf(q[i].x, k.x, acc[i][j]))));
+        }
+      }
+      __syncwarp();                                     // every lane has read it: it is filled next
+    }
+    const unsigned tile_text = a.text.mask32(j0), text = tile_text >> tx;                  // bits 4 j: this lane's keys
+    const bool whole = j0 + XI_TK <= key_hi && (a.bidirectional || j0 + XI_TK - 1 <= q_pos);   // every query sees every key
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int last = min(a.bidirectional ? n_seq - 1 : q_pos + ty + 8 * i, key_hi - 1) - j0 - tx;   // visible: 4 j <= last
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[i][j] = whole || 4 * j <= last ? acc[i][j] * scale2 : -INFINITY;
+      float ref = m_run[i];
+      if (!a.lse) {
+#pragma unroll
+        for (int j = 0; j < 8; ++j) ref = fmaxf(ref, acc[i][j]);
+        const float old = m_run[i];
+        m_run[i] = ref;
+        if (ref == -INFINITY) ref = 0.f;                // none of the lane's keys is visible so far: all terms are 0
+        const float resc = exp2f(old - ref);
+        l_all[i] *= resc;
+        l_txt[i] *= resc;
+      }
+#pragma unroll
+      for (int j = 0; j < 8; ++j) acc[i][j] = exp2f(acc[i][j] - ref);
+#pragma unroll
+      for (int j = 0; j < 8; ++j) l_all[i] += acc[i][j];
+      if (tile_text)
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          if ((text >> (4 * j)) & 1u) l_txt[i] += acc[i][j];
+    }
+  }
+  // ---- the lanes' and the warps' results of a query meet
+  __shared__ float s_m[XI_WARPS][XI_TQ], s_all[XI_WARPS][XI_TQ], s_txt[XI_WARPS][XI_TQ];
+#pragma unroll
+  for (int i = 0; i < 4; ++i) {
+    float m = m_run[i];
+    if (!a.lse) {
+#pragma unroll
+      for (int o = 2; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+      const float f = m == -INFINITY ? 0.f : exp2f(m_run[i] - m);
+      l_all[i] *= f;
+      l_txt[i] *= f;
+    }
+#pragma unroll
+    for (int o = 2; o > 0; o >>= 1) {
       l_all[i] += __shfl_xor_sync(0xffffffffu, l_all[i], o);
       l_txt[i] += __shfl_xor_sync(0xffffffffu, l_txt[i], o);
     }
-    if (tx == 0) { s_m[grp][4 * ty + i] = m_run[i]; s_all[grp][4 * ty + i] = l_all[i]; s_txt[grp][4 * ty + i] = l_txt[i]; }
+    if (tx == 0) { s_m[warp][ty + 8 * i] = m; s_all[warp][ty + 8 * i] = l_all[i]; s_txt[warp][ty + 8 * i] = l_txt[i]; }
   }
+  tc::cp_async_wait<0>();
   __syncthreads();
   const int r = threadIdx.x;
   if (r < nq) {
     float m = s_m[0][r], all = 0.f, txt = 0.f;          // finite without a given log-sum-exp: key 0 is visible to every query
-    for (int k = 1; k < groups; ++k) m = fmaxf(m, s_m[k][r]);
-    for (int k = 0; k < groups; ++k) {
+#pragma unroll
+    for (int k = 1; k < XI_WARPS; ++k) m = fmaxf(m, s_m[k][r]);
+#pragma unroll
+    for (int k = 0; k < XI_WARPS; ++k) {
       const float f = a.lse ? 1.f : exp2f(s_m[k][r] - m);
       all += s_all[k][r] * f;
       txt += s_txt[k][r] * f;
     }
     ws.xi_h[(size_t(b) * a.n_q_heads + h) * ws.cap_in + t0 + r] = a.lse ? txt : txt / all;
     if (a.lse_out)
-      a.lse_out[size_t(b) * a.lse_out_bs + size_t(h) * a.lse_out_hs + row0 + vis_begin + t0 + r] = (m + log2f(all)) * 0.6931471805599453f;
+      a.lse_out[size_t(b) * a.lse_out_bs + size_t(h) * a.lse_out_hs + row0 + q_pos + r] = (m + log2f(all)) * 0.6931471805599453f;
   }
 }
 
@@ -453,9 +496,8 @@ template <typename T>
 static cudaError_t launch_xi_simt_t(const LayerLaunch& L) {
   const lightkv_layer_args_t* a = L.a;
   const int dh = L.head_dim;
-  const int groups = dh <= 128 ? XI_GROUPS : XI_GROUPS / 2;      // key tiles of a CTA within shared memory
-  const size_t smem = size_t(XI_TQ + groups * XI_TK) * (dh + 4) * sizeof(float);
-  const dim3 grid((L.ws.cap_in + XI_TQ - 1) / XI_TQ, L.n_q_heads, L.batch);
+  const size_t smem = size_t(XI_WARPS * 2 * XI_TK * XI_LD + XI_TQ * xi_q_pitch(dh)) * sizeof(float);   // at most 105 KB: two CTAs per SM
+  const unsigned ctas = unsigned((L.ws.cap_in + XI_TQ - 1) / XI_TQ) * unsigned(L.n_q_heads) * unsigned(L.batch);
   XiSimtArgs<T> x;
   x.q = static_cast<const T*>(a->q); x.q_bs = a->q_batch_stride; x.q_hs = a->q_head_stride; x.q_rs = a->q_row_stride;
   x.k = static_cast<const T*>(a->k); x.k_bs = a->k_batch_stride; x.k_hs = a->k_head_stride; x.k_rs = a->k_row_stride;
@@ -465,9 +507,9 @@ static cudaError_t launch_xi_simt_t(const LayerLaunch& L) {
   x.n_vis = a->n_vis; x.seq_start = a->seq_start;
   x.vis_begin = a->vis_begin; x.n_text_after = a->n_text_after; x.bidirectional = a->bidirectional;
   x.n_q_heads = L.n_q_heads; x.n_kv_heads = L.n_kv_heads; x.dh = dh; x.text = L.text;
-  const cudaError_t e = ensure_dynamic_smem(xi_simt_kernel<T>, 176 * 1024);
+  const cudaError_t e = ensure_dynamic_smem(xi_simt_kernel<T>, 108 * 1024);
   if (e != cudaSuccess) return e;
-  return launch_kernel(xi_simt_kernel<T>, grid, groups * XI_GROUP, smem, L.stream, 1, x, L.ws);
+  return launch_kernel(xi_simt_kernel<T>, dim3(ctas), 32 * XI_WARPS, smem, L.stream, 1, x, L.ws);
 }
 
 cudaError_t launch_xi_simt(const LayerLaunch& L) {

@@ -429,6 +429,23 @@ def test_lse_mode_persistent_ctas_walk_several_items(head_dim):
     H.run_schedule(wl, xi_mode="lse", text_ranges=[(2, 60), (70, 129)])
 
 
+@pytest.mark.parametrize("head_dim,grid,text,batch,heads", [
+    (8, (1, 2), 1, 1, 1),           # less than a query tile; two of four warps have no dimension of the head
+    (72, (4, 8), 32, 2, 2),         # one full query tile; keys end on a tile; slices end within the head's last piece
+    (80, (3, 11), 63, 2, 4),        # a query more than a tile
+    (256, (8, 9), 57, 3, 2),        # largest head: one CTA per SM
+    (64, (24, 24), 35, 4, 4),       # 288 CTAs: two per SM, paired from both ends
+    (128, (24, 25), 5, 4, 4),       # 304 CTAs: more than are resident
+])
+@pytest.mark.parametrize("xi_mode", ["attn", "lse"])
+def test_xi_fma_tiles(head_dim, grid, text, batch, heads, xi_mode):
+    wl = S.Workload(name="xifma", config_id=142, batch=batch, tiles=(grid,), n_text=text, hidden=64, n_q_heads=heads,
+                    n_kv_heads=heads if heads < 4 else 2, head_dim=head_dim, n_layers=16, layers=(3,), windows=(1,),
+                    keep=(0.55,))
+    H.run_schedule(wl, xi_mode=xi_mode, dtype="fp32", engine="simt")
+    H.run_schedule(wl, xi_mode=xi_mode, dtype="bf16", engine="simt")
+
+
 @pytest.mark.parametrize("head_dim,text_ranges", [(64, None), (128, [(32, 96)]), (128, [(0, 64), (96, 129)])])
 def test_xi_items_taken_over_and_repeated(head_dim, text_ranges):
     # 4 samples x 8 heads x 16 query tiles = 512 items for the 2 CTAs per SM that are resident: CTAs take over the
