@@ -916,7 +916,9 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, FT_STAGES > 3 ? 1 : 2) fd_tc_
           }
           named_barrier(1, FT_LOADERS);
           // a warp per row, two rows at a time, four columns per lane, all of their remote reads in flight; the CTAs start
-          // with different peers
+          // with different peers (rank ^ j).  The parts are added as a balanced tree: its pairs are the same peers in every
+          // CTA, whatever the rank, so equal rows get equal scores bit for bit wherever they are finished (the tie rule
+          // needs that; added from the CTA's own part on they differed in the last digit).
           for (int r = rank + warp * ks; r < na; r += 16 * ks) {
             float4 v[2][8];
 #pragma unroll
@@ -926,7 +928,7 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, FT_STAGES > 3 ? 1 : 2) fd_tc_
                 const int rr = r + t * 8 * ks;
                 v[t][j] = make_float4(0.f, 0.f, 0.f, 0.f);
                 if (j < ks && rr < na && 4 * lane < nb)
-                  v[t][j] = ld_cluster_f32x4(map_to_cta(ring + uint32_t(rr * PITCH + 4 * lane) * 4, (rank + j) & (ks - 1)));
+                  v[t][j] = ld_cluster_f32x4(map_to_cta(ring + uint32_t(rr * PITCH + 4 * lane) * 4, rank ^ j));
               }
 #pragma unroll
             for (int t = 0; t < 2; ++t) {
@@ -934,11 +936,14 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, FT_STAGES > 3 ? 1 : 2) fd_tc_
               if (rr >= na) break;                          // warp-uniform
               float best = 3.0e38f;
               int best_c = -1;
-              float g4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-              for (int j = 0; j < 8; ++j) {                 // in a fixed order: from this CTA's own part on
-                g4[0] += v[t][j].x; g4[1] += v[t][j].y; g4[2] += v[t][j].z; g4[3] += v[t][j].w;
-              }
+              for (int step = 1; step < 8; step *= 2)
+#pragma unroll
+                for (int j = 0; j < 8; j += 2 * step) {
+                  v[t][j].x += v[t][j + step].x; v[t][j].y += v[t][j + step].y;
+                  v[t][j].z += v[t][j + step].z; v[t][j].w += v[t][j + step].w;
+                }
+              const float g4[4] = {v[t][0].x, v[t][0].y, v[t][0].z, v[t][0].w};
 #pragma unroll
               for (int k = 0; k < 4; ++k) {
                 const int col = 4 * lane + k;

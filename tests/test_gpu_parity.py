@@ -549,6 +549,38 @@ def test_fd_tiles_over_window_sizes(grid, w, batch, hidden):
 
 # ---- subsets of the grid: capacities ---------------------------------------------------------------------------
 
+@pytest.mark.parametrize("grid,hidden", [((8, 8), 1024), ((12, 16), 256), ((12, 16), 768), ((12, 16), 1024),
+                                         ((13, 17), 2056), ((16, 32), 4096)])
+def test_repeated_source_rows_merge_by_index(grid, hidden):
+    """Every source row of the one window is the same, so all of them have the same lowest score bit for bit and only the
+    tie rule decides: the lowest source indices go, into one destination.  Few windows: the FD kernel splits the hidden
+    dimension over clusters of 2, 4 or 8 CTAs (256 / 768 / 1024 channels and more) that each finish some of the rows."""
+    import torch
+    import paper_2605_00789_b200 as L
+    wl = S.Workload(name="ties", config_id=131, batch=1, tiles=(grid,), n_text=5, hidden=hidden, n_q_heads=2,
+                    n_kv_heads=2, head_dim=64, n_layers=4, layers=(2,), windows=(1,), keep=(0.75,))
+    n = grid[0] * grid[1]
+    plan = H.make_plan(wl, xi_mode="uniform")
+    gen = torch.Generator(device="cuda")
+    for seed in range(3):
+        gen.manual_seed(seed)
+        src = torch.randn((hidden,), generator=gen, device="cuda")
+        hidden_in = torch.randn((1, wl.n_text + n, hidden), generator=gen, device="cuda")
+        vis = hidden_in[:, wl.n_text:]
+        vis.mul_(0.3).add_(src)                      # destinations near the source: scores far from 1, with all their digits
+        vis[:, 0::2] = src
+        out = L.StageBuffers(plan, 0, wl.n_text + plan.stage_info(0).cap_out, "cuda")
+        L.compress_layer(plan, 0, hidden_in.bfloat16(), out, vis_begin=wl.n_text)
+        removed = n - int(np.ceil(0.75 * n))
+        assert int(out.status) == 0 and int(out.n_vis_out) == n - removed
+        dst = out.dst[0].cpu().numpy()
+        left = np.ones(n, dtype=bool)
+        left[0:2 * removed:2] = False                # the first `removed` sources
+        np.testing.assert_array_equal(out.pos_out[0, :n - removed].cpu().numpy(), np.nonzero(left)[0])
+        assert len(set(dst[0:2 * removed:2])) == 1
+    plan.close()
+
+
 def _near_full_subset():
     """576-token grid, windows 6 / 4 / 2 (not nested): a sample that misses 8 positions reaches the second stage
     with 146 A nodes, two more than the full grid's 144 (found with the oracle, seed fixed)."""
