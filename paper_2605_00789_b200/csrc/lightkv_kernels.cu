@@ -845,7 +845,7 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
         for (int ib = 0; removed > 0 && ib * kFdTile < nb; ++ib)
           key = min(key, a.key[(size_t(b) * a.blocks + ib) * a.cap_in + i]);
         lists.key[e] = (unsigned int)(key >> 32);
-        lists.best[e] = (unsigned int)key == 0xffffffffu ? -1 : (int)(unsigned int)key;
+        lists.best[e] = key_partner(key, nb);
       }
       __syncthreads();
       select_window(lists, nw, removed, par, a.partner + row, a.place + row);

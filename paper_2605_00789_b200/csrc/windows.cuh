@@ -110,6 +110,13 @@ struct WindowLists {
   }
 };
 
+// The destination (rank among the window's nb) a key of the tiled FD kernel names, -1: none.  A tile whose waits expired
+// stores no key, so what stands in its place is whatever the workspace held: it must not become an index.
+__host__ __device__ inline int key_partner(unsigned long long key, int nb) {
+  const unsigned int to = (unsigned int)key;
+  return to < (unsigned int)nb ? (int)to : -1;
+}
+
 // Selection: the `removed` sources with the lowest (score, index) are merged into their best destination.  Writes every
 // token's partner and place (see Workspace).  key / best / tok are complete in shared memory (synchronised) on entry; all
 // threads take part.  A source's rank among the sources of its destination is counted by its own thread in windows of up
