@@ -263,8 +263,10 @@ int lightkv_compress_layer(const lightkv_plan_t* plan, const lightkv_layer_args_
  * is a fixed device array of LIGHTKV_BUILTIN_WS_BYTES that is part of the library image (each GPU
  * that loads the library keeps that much memory until the process exits).  This function and
  * everything below it call no cudaMalloc / cudaFree and no allocating library routine.
- *   - A stage whose lightkv_plan_stage_info().workspace_bytes exceeds LIGHTKV_BUILTIN_WS_BYTES is
- *     rejected with LIGHTKV_ERR_WORKSPACE before anything is launched.
+ *   - Stages with large windows whose lightkv_plan_stage_info().workspace_bytes exceeds
+ *     LIGHTKV_BUILTIN_WS_BYTES run in the list form (window lists, FD, selection as separate kernels: the
+ *     same results, slower) when that fits; what does not fit in any form is rejected with
+ *     LIGHTKV_ERR_WORKSPACE before anything is launched.
  *   - The first call on each device looks up the array's device address (cudaGetSymbolAddress, with
  *     that device current) and remembers it; make that first call outside any stream capture.
  *     LIGHTKV_ERR_CUDA if the lookup fails.

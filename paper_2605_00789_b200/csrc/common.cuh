@@ -34,9 +34,9 @@ struct Workspace {
   int* a_win;      // [B, cap_a]          window of each A entry
   int* b_tok;      // [B, cap_b]          token index of each B entry
   unsigned long long* a_key;  // [B, cap_a]  (orderable(lowest FD) << 32) | B entry index of the best partner;
-                              //             all ones while no partner is known (set by the window build).  Without window
-                              //             lists: [B, fd blocks, cap_in], by token and block of destinations, see
-                              //             fd_tc_kernel
+                              //             all ones while no partner is known (set by the window build)
+  // tiled FD kernel without window lists (these two lie over the arrays of the list form)
+  unsigned long long* tile_key;  // [B, fd blocks, cap_in]  such keys by token and block of destinations, see fd_tc_kernel
   int* win_tok;    // [B, n_windows, max_cell + 1]  tiled FD kernel: the number of tokens of a window, then the tokens
   float* xi_h;     // [B, H, cap_in]      per-head attention mass on the prompt (ATTN modes)
   float* xi;       // [B, cap_in]

@@ -104,4 +104,9 @@ cudaError_t launch_fd_tc(const LayerLaunch& L, bool lists);
 // wait_first: the stream's last kernel is not the window build or FD of the same call
 cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first);
 
+// lightkv_compress_layer.  `least`: a workspace of least_workspace() bytes will do; where the tiled FD kernel's keys do not
+// fit it, the call takes the list form.
+size_t least_workspace(const lightkv_plan_t* p, int stage);
+int compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* a, bool least);
+
 }  // namespace lkv

@@ -10,6 +10,13 @@
 
 namespace lkv {
 
+// byte offsets of the Workspace arrays
+struct WorkspaceOffsets {
+  size_t xi_h, partner, slot, xi_redo;                                                      // every form
+  size_t win_off, a_off, tok_win, tok_l, a_tok, a_win, b_tok, a_key, xi, a_partner;         // list form
+  size_t tile_key, win_tok;                                                                 // tiled form
+};
+
 struct StagePlan {
   int layer, w;
   double keep;
@@ -22,8 +29,10 @@ struct StagePlan {
   int fd_blocks;   // tiles a side the largest window may have, tensor-core FD kernel
   int fd_tiles;    // tiles of the FD kernel per sample, at windows of fd_side nodes
   Geometry geo;
-  size_t ws_bytes;
-  size_t off[15];     // byte offsets of the Workspace arrays
+  size_t ws_list;     // workspace of the list form (the streaming form needs less)
+  size_t ws_tiled;    // ... of the tiled form
+  size_t ws_bytes;    // the larger of the two
+  WorkspaceOffsets off;
 };
 
 }  // namespace lkv
@@ -42,42 +51,59 @@ static size_t align_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // Whether one CTA can hold a window's lists and one cluster a sample: the FD kernels then work without window lists.
 static bool windows_in_ctas(const StagePlan& s) { return s.max_cell <= 4096 && s.cap_in <= kMapMaxTokens; }
 
+// The scratch of a stage: what every form needs, then the arrays of the list form and, over them, those of the tiled form
+// (a call takes one or the other).
 static void layout_workspace(const lightkv_plan_t& p, StagePlan& s) {
   const size_t B = p.cfg.batch, nW1 = s.n_windows + 1;
   const bool attn = p.cfg.xi_mode == LIGHTKV_XI_ATTN_FULL || p.cfg.xi_mode == LIGHTKV_XI_ATTN_LSE;
   const size_t xi_items = attn ? size_t((s.cap_in + 127) / 128) * p.cfg.n_q_heads * B : 0;
-  // keys: one per source, or, for the tiled FD kernel without lists, one per token and block of destinations
   const bool by_token = s.use_tc && windows_in_ctas(s) && !fd_stream_supported(p.cfg.dtype, s.fd_side);
-  const size_t keys = std::max(B * s.cap_a, by_token ? B * s.fd_blocks * s.cap_in : size_t(0));
-  const size_t win_tok = by_token ? B * s.n_windows * (size_t(s.max_cell) + 1) : 0;
-  const size_t sizes[15] = {
-      B * nW1 * 4, B * nW1 * 4, B * s.cap_in * 4, B * s.cap_in * 4, B * s.cap_a * 4, B * s.cap_a * 4,
-      B * s.cap_b * 4, keys * 8, win_tok * 4,
-      attn ? B * p.cfg.n_q_heads * s.cap_in * 4 : 0, B * s.cap_in * 4, B * s.cap_in * 4, B * s.cap_in * 4,
-      B * s.cap_a * 4, xi_items * 4};
-  size_t off = 0;
-  for (int i = 0; i < 15; ++i) { s.off[i] = off; off += align_up(sizes[i], 256); }
-  s.ws_bytes = std::max<size_t>(off, 256);
+  WorkspaceOffsets& o = s.off;
+  size_t end = 0;
+  auto place = [&](size_t bytes) { const size_t at = end; end += align_up(bytes, 256); return at; };
+  o.xi_h = place(attn ? B * p.cfg.n_q_heads * s.cap_in * 4 : 0);
+  o.partner = place(B * s.cap_in * 4);
+  o.slot = place(B * s.cap_in * 4);
+  o.xi_redo = place(xi_items * 4);
+  const size_t forms = end;
+  o.win_off = place(B * nW1 * 4);
+  o.a_off = place(B * nW1 * 4);
+  o.tok_win = place(B * s.cap_in * 4);
+  o.tok_l = place(B * s.cap_in * 4);
+  o.a_tok = place(B * s.cap_a * 4);
+  o.a_win = place(B * s.cap_a * 4);
+  o.b_tok = place(B * s.cap_b * 4);
+  o.a_key = place(B * s.cap_a * 8);
+  o.xi = place(B * s.cap_in * 4);
+  o.a_partner = place(B * s.cap_a * 4);
+  s.ws_list = end;
+  end = forms;
+  o.tile_key = place(by_token ? B * s.fd_blocks * s.cap_in * 8 : 0);
+  o.win_tok = place(by_token ? B * s.n_windows * (size_t(s.max_cell) + 1) * 4 : 0);
+  s.ws_tiled = end;
+  s.ws_bytes = std::max(s.ws_list, s.ws_tiled);
 }
 
 static Workspace bind_workspace(const StagePlan& s, void* base) {
   char* p = static_cast<char*>(base);
+  const WorkspaceOffsets& o = s.off;
   Workspace w;
-  w.win_off = reinterpret_cast<int*>(p + s.off[0]);
-  w.a_off = reinterpret_cast<int*>(p + s.off[1]);
-  w.tok_win = reinterpret_cast<int*>(p + s.off[2]);
-  w.tok_l = reinterpret_cast<int*>(p + s.off[3]);
-  w.a_tok = reinterpret_cast<int*>(p + s.off[4]);
-  w.a_win = reinterpret_cast<int*>(p + s.off[5]);
-  w.b_tok = reinterpret_cast<int*>(p + s.off[6]);
-  w.a_key = reinterpret_cast<unsigned long long*>(p + s.off[7]);
-  w.win_tok = reinterpret_cast<int*>(p + s.off[8]);
-  w.xi_h = reinterpret_cast<float*>(p + s.off[9]);
-  w.xi = reinterpret_cast<float*>(p + s.off[10]);
-  w.partner = reinterpret_cast<int*>(p + s.off[11]);
-  w.slot = reinterpret_cast<int*>(p + s.off[12]);
-  w.a_partner = reinterpret_cast<int*>(p + s.off[13]);
-  w.xi_redo = reinterpret_cast<int*>(p + s.off[14]);
+  w.win_off = reinterpret_cast<int*>(p + o.win_off);
+  w.a_off = reinterpret_cast<int*>(p + o.a_off);
+  w.tok_win = reinterpret_cast<int*>(p + o.tok_win);
+  w.tok_l = reinterpret_cast<int*>(p + o.tok_l);
+  w.a_tok = reinterpret_cast<int*>(p + o.a_tok);
+  w.a_win = reinterpret_cast<int*>(p + o.a_win);
+  w.b_tok = reinterpret_cast<int*>(p + o.b_tok);
+  w.a_key = reinterpret_cast<unsigned long long*>(p + o.a_key);
+  w.tile_key = reinterpret_cast<unsigned long long*>(p + o.tile_key);
+  w.win_tok = reinterpret_cast<int*>(p + o.win_tok);
+  w.xi_h = reinterpret_cast<float*>(p + o.xi_h);
+  w.xi = reinterpret_cast<float*>(p + o.xi);
+  w.partner = reinterpret_cast<int*>(p + o.partner);
+  w.slot = reinterpret_cast<int*>(p + o.slot);
+  w.a_partner = reinterpret_cast<int*>(p + o.a_partner);
+  w.xi_redo = reinterpret_cast<int*>(p + o.xi_redo);
   w.cap_in = s.cap_in; w.cap_out = s.cap_out; w.cap_a = s.cap_a; w.cap_b = s.cap_b;
   w.n_windows = s.n_windows;
   return w;
@@ -253,7 +279,13 @@ double lightkv_plan_retention(const lightkv_plan_t* p) {
 
 static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15) == 0; }
 
-int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* a) {
+}  // extern "C"
+
+namespace lkv {
+
+size_t least_workspace(const lightkv_plan_t* p, int stage) { return p->stages[stage].ws_list; }
+
+int compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* a, bool least) {
   if (!p || !a || a->struct_size != sizeof(lightkv_layer_args_t)) return LIGHTKV_ERR_INVALID_ARG;
   if (a->stage < 0 || a->stage >= (int)p->stages.size()) return LIGHTKV_ERR_INVALID_ARG;
   const StagePlan& s = p->stages[a->stage];
@@ -290,7 +322,7 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
       (a->hidden_out_batch_stride * esz) % 16 || a->hidden_row_stride < c.hidden ||
       a->hidden_out_row_stride < c.hidden)
     return LIGHTKV_ERR_INVALID_ARG;
-  if ((reinterpret_cast<uintptr_t>(a->workspace) & 255) != 0 || a->workspace_bytes < s.ws_bytes)
+  if ((reinterpret_cast<uintptr_t>(a->workspace) & 255) != 0 || a->workspace_bytes < (least ? s.ws_list : s.ws_bytes))
     return LIGHTKV_ERR_WORKSPACE;
   const bool attn = c.xi_mode == LIGHTKV_XI_ATTN_FULL || c.xi_mode == LIGHTKV_XI_ATTN_LSE;
   if (attn) {
@@ -320,11 +352,12 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
   // units where CTAs gather them):
   //   streaming  small windows: one kernel finds the windows, scores and selects; the map kernel finishes
   //   tiled      larger windows on tensor cores: tiles of windows are scored, the map kernel selects and finishes
-  //   otherwise  samples or windows too large for the lists of a CTA, and the fp32-FMA engine: window lists, FD, selection
+  //   otherwise  samples or windows too large for the lists of a CTA, the fp32-FMA engine, and a fixed workspace that the
+  //              keys of the tiled form do not fit: window lists, FD, selection
   const bool near = (long long)s.cap_in * a->hidden_row_stride * (long long)esz / 16 < 0xffffffffll;
   const bool in_ctas = near && windows_in_ctas(s);
   const bool streaming = in_ctas && (tc_fd || c.dtype == LIGHTKV_FP32) && fd_stream_supported(c.dtype, s.fd_side);
-  const bool tiled = in_ctas && tc_fd && !streaming;
+  const bool tiled = in_ctas && tc_fd && !streaming && a->workspace_bytes >= s.ws_tiled;
   auto launch_windows = [&](const LayerLaunch& l) { return streaming || tiled ? cudaSuccess : launch_window_build(l); };
   auto launch_fd = [&](const LayerLaunch& l) {
     return streaming ? launch_fd_stream(l) : tc_fd && near ? launch_fd_tc(l, !tiled) : launch_fd_simt(l);
@@ -361,6 +394,12 @@ int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* 
   if (launch_merge_rows(L) != cudaSuccess || mark(5) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   return LIGHTKV_OK;
 }
+
+}  // namespace lkv
+
+extern "C" {
+
+int lightkv_compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* a) { return compress_layer(p, a, false); }
 
 int lightkv_compact_kv(const lightkv_plan_t* p, const lightkv_kv_args_t* a) {
   if (!p || !a || a->struct_size != sizeof(lightkv_kv_args_t)) return LIGHTKV_ERR_INVALID_ARG;

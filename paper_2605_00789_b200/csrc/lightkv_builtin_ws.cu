@@ -40,11 +40,11 @@ extern "C" int lightkv_compress_layer_builtin_ws(const lightkv_plan_t* plan, con
   lightkv_stage_info_t info;
   const int rc = lightkv_plan_stage_info(plan, args->stage, &info);
   if (rc != LIGHTKV_OK) return rc;
-  if (info.workspace_bytes > size_t(LIGHTKV_BUILTIN_WS_BYTES)) return LIGHTKV_ERR_WORKSPACE;
+  if (lkv::least_workspace(plan, args->stage) > size_t(LIGHTKV_BUILTIN_WS_BYTES)) return LIGHTKV_ERR_WORKSPACE;
   void* ws = lkv::builtin_ws_for_current_device();
   if (!ws) return LIGHTKV_ERR_CUDA;
   lightkv_layer_args_t a = *args;              // the caller's workspace fields are ignored
   a.workspace = ws;
   a.workspace_bytes = size_t(LIGHTKV_BUILTIN_WS_BYTES);
-  return lightkv_compress_layer(plan, &a);
+  return lkv::compress_layer(plan, &a, true);
 }

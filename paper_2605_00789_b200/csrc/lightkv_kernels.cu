@@ -1021,7 +1021,7 @@ cudaError_t launch_map(const LayerLaunch& L, bool select) {
   m.n_q_heads = L.n_q_heads; m.xi_mode = L.xi_mode; m.cap_in = L.ws.cap_in; m.cap_out = L.ws.cap_out;
   m.cap_a = L.ws.cap_a; m.cap_b = L.ws.cap_b; m.n_grid = L.n_grid;
   m.n_vis = a->n_vis; m.pos = a->pos; m.xi_in = a->xi; m.xi_h = L.ws.xi_h; m.partner = L.ws.partner; m.place = L.ws.slot;
-  m.key = L.ws.a_key; m.win_tok = L.ws.win_tok; m.blocks = L.fd_blocks; m.max_cell = L.max_cell; m.n_windows = L.geo.n_windows;
+  m.key = L.ws.tile_key; m.win_tok = L.ws.win_tok; m.blocks = L.fd_blocks; m.max_cell = L.max_cell; m.n_windows = L.geo.n_windows;
   m.src_par = L.geo.src_par; m.keep = L.keep;
   m.n_vis_out = a->n_vis_out; m.pos_out = a->pos_out; m.dst = a->dst; m.weight = a->weight; m.grp_off = a->grp_off;
   m.grp_src = a->grp_src; m.xi_out = a->xi_out; m.status = a->status;

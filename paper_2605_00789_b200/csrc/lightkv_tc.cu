@@ -697,7 +697,7 @@ __device__ __forceinline__ void store_key(const FdTcArgs& a, int b, int ia, int 
   if (best_c >= 0)
     key = ((unsigned long long)orderable(best) << 32) | (unsigned)((a.lists ? b_first : 0) + ib * BLK + best_c);
   if (a.lists) atomicMin(a.ws.a_key + size_t(b) * a.ws.cap_a + a_first + ia * BLK + row, key);
-  else a.ws.a_key[(size_t(b) * a.blocks + ib) * a.cap_in + row_a[row]] = key;
+  else a.ws.tile_key[(size_t(b) * a.blocks + ib) * a.cap_in + row_a[row]] = key;
 }
 
 // CLUSTER = false is the plain launch (ks = 1) with the cluster code compiled out.

@@ -289,6 +289,22 @@ def test_builtin_workspace_entry_rejects_oversized_stages_on_the_host(L):
     assert re.search(r"#define LIGHTKV_BUILTIN_WS_BYTES \(8u << 20\)", header) and L.BUILTIN_WS_BYTES == 8 << 20
 
 
+@pytest.mark.parametrize("stage,xi,kw", [
+    (0, "XI_ATTN_FULL", dict(batch=8, n_q_heads=32, n_kv_heads=32, tiles=[(64, 64)], layers=[2], windows=[1], keep=[0.5])),
+    (1, "XI_ATTN_FULL", dict(batch=8, n_q_heads=8, n_kv_heads=8, tiles=[(128, 128)], layers=[2, 4], windows=[2, 2], keep=[0.5, 0.5])),
+    (0, "XI_UNIFORM", dict(batch=20, tiles=[(64, 64)], layers=[2], windows=[1], keep=[0.5])),
+])
+def test_builtin_workspace_takes_large_windows_whose_keys_do_not_fit(L, stage, xi, kw):
+    """The keys of the tiled FD kernel (one per token and block of destinations) are a matter of speed: stages whose list
+    form fits the built-in array are taken, in that form."""
+    p = _plan(L, hidden=512, head_dim=64, xi_mode=getattr(L, xi), **kw)
+    assert p.stage_info(stage).workspace_bytes > L.BUILTIN_WS_BYTES
+    a = L.lightkv._LayerArgs()
+    a.struct_size = C.sizeof(a)
+    a.stage = stage
+    assert L.library().lightkv_compress_layer_builtin_ws(p.handle, C.byref(a)) != -3
+
+
 def test_missing_library_fails_loudly(L, monkeypatch):
     from paper_2605_00789_b200 import lightkv
     monkeypatch.setattr(lightkv, "_LIB", None)

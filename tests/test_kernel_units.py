@@ -90,7 +90,7 @@ int main() {
     LayerLaunch L = {};
     L.batch = B; L.xi_mode = LIGHTKV_XI_UNIFORM; L.keep = 0.6; L.fd_blocks = blocks; L.max_cell = cell; L.n_grid = n;
     L.geo.n_windows = W;
-    L.ws.a_key = device(key); L.ws.win_tok = device(tok); L.ws.partner = device(ints); L.ws.slot = device(ints);
+    L.ws.tile_key = device(key); L.ws.win_tok = device(tok); L.ws.partner = device(ints); L.ws.slot = device(ints);
     L.ws.cap_in = L.ws.cap_out = L.ws.cap_a = L.ws.cap_b = n; L.ws.n_windows = W;
     L.a = &a;
     const cudaError_t launched = launch_map(L, true), ended = cudaDeviceSynchronize();

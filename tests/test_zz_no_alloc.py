@@ -73,3 +73,26 @@ def test_builtin_workspace_matches_caller_workspace_on_two_calls_in_a_row():
         _same(got, want, [int(n) for n in inp["n_vis"]])
     assert moved == [0, 0], f"free device memory moved across the calls: {moved}"
     plan.close()
+
+
+def test_builtin_workspace_takes_the_list_form_where_the_keys_do_not_fit():
+    # 20 samples of one window of 64 x 64 tokens: the keys of the tiled FD kernel take 10 MiB, the lists 4
+    import torch
+    import __graft_entry__ as entry
+    assert torch.cuda.is_available()
+    entry.build()
+    import paper_2605_00789_b200 as L
+
+    wl = S.Workload(name="big_windows", config_id=132, batch=20, tiles=((64, 64),), n_text=3, hidden=64, n_q_heads=2,
+                    n_kv_heads=2, head_dim=64, n_layers=4, layers=(2,), windows=(1,), keep=(0.6,))
+    plan = H.make_plan(wl, xi_mode="uniform")
+    assert plan.stage_info(0).workspace_bytes > L.BUILTIN_WS_BYTES
+    rng = np.random.default_rng(12)
+    full = np.arange(wl.n_vis, dtype=np.int32)
+    pos = [full, np.sort(rng.choice(full, 3001, replace=False)).astype(np.int32), full[:300], full[:0]] + [full] * 16
+    inp = H.prepare_stage(wl, 0, pos, repair=False, tensors=("hidden",))
+    got = H.gpu_stage(plan, wl, 0, inp, xi_mode="uniform", layer_fn=L.compress_layer_builtin_ws)
+    want = H.gpu_stage(plan, wl, 0, inp, xi_mode="uniform")
+    for key in INDEX_OUTPUTS + ("weight", "hidden_out"):
+        np.testing.assert_array_equal(got[key], want[key], err_msg=key)
+    plan.close()
