@@ -2,7 +2,7 @@
 """Benchmark of the LightKV compression hot path on B200 (one JSON line on stdout).
 
 A step = one pass of the whole hot path over one batch: for every stage of the workload's schedule,
-lightkv_compress_layer (window build, xi, FD + best partner, selection + merge map, hidden merge) and
+lightkv_compress_layer (windows, FD + best partner, xi, selection + merge map, hidden merge) and
 lightkv_compact_kv on that layer's K/V, chained through the surviving positions on the device.
 Inputs are seeded synthetic tensors (lightkv_synth), regenerated per compression layer and resident
 in HBM before the timed region.  `value` is vision tokens entering compression stages per second.
@@ -32,6 +32,35 @@ if ROOT not in sys.path:
 import lightkv_synth as S  # noqa: E402
 
 KERNELS = ("window_build", "xi", "fd_best_partner", "select_map", "merge_hidden", "kv_compact")
+
+
+def kernel_names(engine):
+    """What a stage of the benchmark's workloads launches: the FD kernels find their windows themselves, except on the
+    fp32-FMA engine, which has the windows listed by a kernel of its own first."""
+    return KERNELS if engine == "simt" else KERNELS[1:]
+
+
+def count_launches(step):
+    """Kernels `step` launches: the kernel nodes of a capture of it (the step holds nothing but the library's calls)."""
+    import ctypes
+    import torch
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(graph):
+        step()
+    rt = ctypes.CDLL(f"libcudart.so.{torch.version.cuda.split('.')[0]}")      # the runtime torch has loaded
+    raw, n = ctypes.c_void_p(graph.raw_cuda_graph()), ctypes.c_size_t(0)
+    if rt.cudaGraphGetNodes(raw, None, ctypes.byref(n)) != 0:
+        raise RuntimeError("cudaGraphGetNodes")
+    nodes = (ctypes.c_void_p * n.value)()
+    if rt.cudaGraphGetNodes(raw, nodes, ctypes.byref(n)) != 0:
+        raise RuntimeError("cudaGraphGetNodes")
+    kernels, kind = 0, ctypes.c_int(0)
+    for node in nodes:
+        if rt.cudaGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)) != 0:
+            raise RuntimeError("cudaGraphNodeGetType")
+        kernels += kind.value == 0                        # cudaGraphNodeTypeKernel
+    return kernels
 
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the committed ncu captures (profiles/),
 # of the stage-0 launch, keyed by (workload, kernel); null where no capture exists.
@@ -225,7 +254,7 @@ def run_step(L, plan, wl, stages, traces=None, kv_events=None, side=None, aux=No
     """The whole hot path once; stage i+1 reads positions and counts stage i left on the device.
     With `side`, the K/V compaction of stage i (HBM bound) runs on that second stream while stage i+1's
     compression (bound by the xi contraction) proceeds on the current one; the step ends with a join.
-    With `aux`, the library itself runs window build + FD beside the xi contraction (aux_stream)."""
+    With `aux`, the library itself runs FD beside the xi contraction (aux_stream)."""
     import torch
     pos, n_vis = stages[0]["dev"]["pos"], stages[0]["dev"]["n_vis"]
     for st, stg in enumerate(stages):
@@ -344,7 +373,7 @@ def main():
     ap.add_argument("--graph", type=int, default=1, choices=[0, 1],
                     help="1: replay the step from a CUDA graph captured once (timed region only)")
     ap.add_argument("--streams", type=int, default=2, choices=[1, 2],
-                    help="2: HBM-bound kernels (window build + FD, K/V compaction) on second streams beside the xi contraction")
+                    help="2: HBM-bound kernels (FD, K/V compaction) on second streams beside the xi contraction")
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
     args = ap.parse_args()
@@ -437,7 +466,7 @@ def main():
     for _ in range(args.warmup):
         run_step(L, plan, wl, stages, side=side, aux=aux)
 
-    # The step's launches (18 kernels on three streams) are captured once into a CUDA graph and replayed:
+    # The step's launches (five kernels a stage on three streams) are captured once into a CUDA graph and replayed:
     # the library's calls are plain stream work, so the caller may do that.  Plumbing only; if the capture is
     # refused the step is launched call by call and the JSON says so.
     step_graph = None
@@ -532,19 +561,21 @@ def main():
             print(f"bench: one-stream graph capture refused ({exc})", file=sys.stderr)
             torch.cuda.synchronize()
 
-    ktime = {k: 0.0 for k in KERNELS}       # ms per step, summed over stages
-    kstage = [{k: 0.0 for k in KERNELS} for _ in range(n_stages)]
+    names = kernel_names(args.engine)
+    ktime = {k: 0.0 for k in names}         # ms per step, summed over stages
+    kstage = [{k: 0.0 for k in names} for _ in range(n_stages)]
     for i in range(ksteps):
         for st in range(n_stages):
             e = traces[i][st]
             for j, name in enumerate(L.TRACE_NAMES):
-                kstage[st][name] += e[j].elapsed_time(e[j + 1]) / ksteps
+                if name in kstage[st]:
+                    kstage[st][name] += e[j].elapsed_time(e[j + 1]) / ksteps
             kstage[st]["kv_compact"] += e[-1].elapsed_time(kv_ev[i][st]) / ksteps
     for st in range(n_stages):
-        for k in KERNELS:
+        for k in names:
             ktime[k] += kstage[st][k]
     work_stage = algorithmic_work(wl, stages, args.xi_mode)
-    work = {k: sum(w[k] for w in work_stage) for k in KERNELS}
+    work = {k: sum(w[k] for w in work_stage) for k in names}
     peaks = measured_peaks()
 
     def rate(k, amount, ms):
@@ -557,13 +588,13 @@ def main():
         return amount / sec / 1e9, peaks["hbm_gbs"], "GB/s", "hbm"
 
     kernels = {}
-    for k in KERNELS:
+    for k in names:
         ach, peak, u, bound = rate(k, work[k], ktime[k])
         kernels[k] = {"ms_per_step": round(ktime[k], 4), "share": round(ktime[k] / sum(ktime.values()), 4),
                       "bound": bound, "achieved": round(ach, 2), "peak": peak, "unit": u, "frac": round(ach / peak, 4)}
     # roofline object: the kernel with the largest share, at its largest launch (stage 0), so that `achieved`
     # and `traffic` are both per launch
-    top = max(KERNELS, key=lambda k: ktime[k])
+    top = max(names, key=lambda k: ktime[k])
     ach, peak, u, bound = rate(top, work_stage[0][top], kstage[0][top])
     roofline = {"kernel": top, "launch": "stage 0", "bound": bound, "achieved": round(ach, 2), "peak": peak, "unit": u,
                 "frac": round(ach / peak, 4), "traffic": NCU_TRAFFIC_BYTES.get((wl.name, top)),
@@ -654,14 +685,13 @@ def main():
         except Exception as exc:      # noqa: BLE001
             cpu["c_oracle_one_thread"] = {"unavailable": str(exc)}
 
+    launches_per_step = count_launches(lambda: run_step(L, plan, wl, stages, side=side, aux=aux))
     if rank == 0:
-        # per stage: window build, xi, FD, selection, hidden merge, K/V compaction (+ the move kernel when in place)
-        launches_per_step = n_stages * (6 + (1 if args.kv_in_place else 0))
         line = {"metric": metric, "value": value, "unit": unit, "n_gpus": world, "steps": args.steps,
                 "warmup": args.warmup, "ms_per_step": ms_step, "higher_is_better": True, "scaling": "weak",
                 "vs_baseline": None, "dtype": "bf16", "data": "synthetic", "config": config,
                 "us_per_compression_layer": 1e3 * ms_step / n_stages,
-                "schedule": ("streams: window build + FD beside xi inside lightkv_compress_layer (aux_stream); "
+                "schedule": ("streams: FD beside xi inside lightkv_compress_layer (aux_stream); "
                              "lightkv_compact_kv of stage i behind the stage's map event, beside its hidden-state merge and lightkv_compress_layer of stage i+1"
                              if side is not None else "one stream"),
                 "cuda_graph": step_graph is not None,
