@@ -1,5 +1,6 @@
 // Host-side launch interface between the C ABI (lightkv_api.cu) and the kernel files.
 #pragma once
+#include <atomic>
 #include <mutex>
 
 #include "common.cuh"
@@ -46,24 +47,52 @@ struct LayerLaunch {
   cudaStream_t stream;
 };
 
-// cudaFuncSetAttribute(MaxDynamicSharedMemorySize) once per (kernel, device) instead of before every launch.
-struct SmemAttrEntry { const void* kernel; int dev; int bytes; };
+// How much dynamic shared memory every kernel has been allowed on every device, so that the attribute is set once and not
+// before every launch.  Looked up without a lock (a hash table per device whose entries only ever appear and grow).
+class SmemLimits {
+ public:
+  static constexpr int kDevices = 64, kSlots = 256;       // about 40 kernel instances a device
+  // `set(bytes)` raises the limit of `kernel` on the current device, which is `dev`
+  template <typename Set>
+  cudaError_t ensure(const void* kernel, int dev, int bytes, Set set) {
+    if (dev < 0 || dev >= kDevices) return set(bytes);
+    Slot* s = find(kernel, dev);
+    if (s && s->kernel.load(std::memory_order_acquire) == kernel && s->bytes.load(std::memory_order_acquire) >= bytes)
+      return cudaSuccess;
+    std::lock_guard<std::mutex> lock(mu_);
+    s = find(kernel, dev);
+    if (s && s->kernel.load(std::memory_order_relaxed) == kernel && s->bytes.load(std::memory_order_relaxed) >= bytes)
+      return cudaSuccess;                                 // another thread was here first
+    const cudaError_t rc = set(bytes);
+    if (rc == cudaSuccess && s) {                         // (a full table forgets: the attribute is set again)
+      s->bytes.store(bytes, std::memory_order_release);
+      s->kernel.store(kernel, std::memory_order_release);
+    }
+    return rc;
+  }
+
+ private:
+  struct Slot { std::atomic<const void*> kernel; std::atomic<int> bytes; };
+  // the kernel's slot or the first empty one on its way, nullptr: neither
+  Slot* find(const void* kernel, int dev) {
+    const uint32_t start = uint32_t((reinterpret_cast<uintptr_t>(kernel) >> 4) * 0x9e3779b97f4a7c15ull >> 32);
+    for (int i = 0; i < kSlots; ++i) {
+      Slot* s = &slot_[dev][(start + i) % kSlots];
+      const void* k = s->kernel.load(std::memory_order_acquire);
+      if (k == kernel || !k) return s;
+    }
+    return nullptr;
+  }
+  std::mutex mu_;
+  Slot slot_[kDevices][kSlots] = {};
+};
 inline cudaError_t ensure_dynamic_smem_ptr(const void* kernel, int bytes) {
-  static std::mutex mu;
-  static SmemAttrEntry table[64];
-  static int used = 0;
+  static SmemLimits limits;
   int dev = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return cudaErrorInvalidDevice;
-  std::lock_guard<std::mutex> lock(mu);
-  SmemAttrEntry* e = nullptr;
-  for (int i = 0; i < used; ++i)
-    if (table[i].kernel == kernel && table[i].dev == dev) { e = &table[i]; break; }
-  if (e && e->bytes >= bytes) return cudaSuccess;
-  const cudaError_t rc = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-  if (rc != cudaSuccess) return rc;
-  if (!e && used < 64) e = &table[used++];
-  if (e) { e->kernel = kernel; e->dev = dev; e->bytes = bytes; }
-  return cudaSuccess;
+  return limits.ensure(kernel, dev, bytes, [&](int n) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, n);
+  });
 }
 template <typename... P>
 inline cudaError_t ensure_dynamic_smem(void (*kernel)(P...), int bytes) {

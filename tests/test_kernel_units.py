@@ -46,6 +46,39 @@ int main() {
     assert out == ["0", "0"]
 
 
+def test_the_shared_memory_limit_is_set_once_per_kernel_and_device(tmp_path):
+    """Sixty kernels on eight devices, launched in turn with growing and shrinking sizes by two threads: a limit is only ever
+    set to raise it, and a set that failed is tried again."""
+    out = _run(tmp_path, r"""
+#include <stdio.h>
+#include <string.h>
+#include <atomic>
+#include <thread>
+#include "launch.h"
+static lkv::SmemLimits limits;
+int main() {
+  static char code[60 * 64];
+  static std::atomic<int> calls, limit[8][60];
+  auto launches = [&](int bytes) {
+    for (int dev = 0; dev < 8; ++dev)
+      for (int k = 0; k < 60; ++k) {
+        limits.ensure(code + 64 * k, dev, bytes, [&](int n) { ++calls; limit[dev][k] = n; return cudaSuccess; });
+        if (limit[dev][k] < bytes) calls += 1000000;
+      }
+  };
+  const int sizes[] = {1000, 1000, 500, 2000, 1000, 2000};             // two raises
+  for (int n : sizes) { std::thread other([&] { launches(n); }); launches(n); other.join(); }
+  int failed = 0;
+  for (int i = 0; i < 2; ++i)
+    failed += limits.ensure(code, 1, 9000, [](int) { return cudaErrorInvalidValue; }) == cudaErrorInvalidValue;
+  int far = 0;
+  for (int i = 0; i < 2; ++i) limits.ensure(code, 64, 10, [&](int) { ++far; return cudaSuccess; });   // beyond the table
+  printf("%d %d %d\n", calls.load(), failed, far);
+}
+""")
+    assert out == [str(2 * 8 * 60), "2", "2"]
+
+
 @pytest.mark.gpu
 def test_the_map_of_keys_that_were_never_written_is_a_partition(tmp_path):
     """What the map kernel makes of a workspace whose tiled FD kernel stored no key (its waits expired): the windows' tokens
