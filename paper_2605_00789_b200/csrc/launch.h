@@ -32,6 +32,21 @@ inline cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, si
   return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
+// SMs of the current device (looked up once per device).  The launches choose variants and splits by it; results do not
+// depend on it.
+inline int sm_count() {
+  constexpr int kB200 = 148, kDevices = 64;
+  static std::atomic<int> known[kDevices];
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevices) return kB200;
+  int n = known[dev].load(std::memory_order_relaxed);
+  if (n == 0) {
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = kB200;
+    known[dev].store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
+
 struct LayerLaunch {
   int batch, hidden, n_q_heads, n_kv_heads, head_dim;
   int dtype, xi_mode, divergence;

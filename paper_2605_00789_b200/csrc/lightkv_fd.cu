@@ -317,8 +317,9 @@ static cudaError_t launch_fd_stream_o(const LayerLaunch& L, const FdStreamArgs& 
   // few windows: clusters of 2, 4 or 8 CTAs split the hidden dimension further, while that fills no SM twice and leaves a
   // CTA 32 KB to read (fp32, bound by its FMAs: 8 KB) beside the two cluster barriers it costs
   const long long window_bytes = 2ll * L.fd_side * L.hidden * (long long)sizeof(T) * (sizeof(T) == 4 ? 4 : 1);
+  const int sms = sm_count();
   int ks = 1;
-  while (ks < 8 && (long long)L.geo.n_windows * L.batch * 2 * ks <= 148 && window_bytes >= 2 * ks * (32ll << 10)) ks *= 2;
+  while (ks < 8 && (long long)L.geo.n_windows * L.batch * 2 * ks <= sms && window_bytes >= 2 * ks * (32ll << 10)) ks *= 2;
   return launch_kernel(fd_stream_kernel<T, O, S, WARPS>, dim3(L.geo.n_windows * ks, L.batch), 32 * WARPS, smem, L.stream, ks, f);
 }
 
@@ -327,7 +328,7 @@ static cudaError_t launch_fd_stream_o(const LayerLaunch& L, const FdStreamArgs& 
 // window (its lists, the meeting of the warps) is paid by fewer threads.
 template <int O, int S>
 static cudaError_t launch_fd_stream_w(const LayerLaunch& L, const FdStreamArgs& f) {
-  const bool wide = L.hidden * (L.dtype == LIGHTKV_FP32 ? 4 : 2) > 1536 || (long long)L.geo.n_windows * L.batch <= 148;
+  const bool wide = L.hidden * (L.dtype == LIGHTKV_FP32 ? 4 : 2) > 1536 || (long long)L.geo.n_windows * L.batch <= sm_count();
   if (L.dtype == LIGHTKV_FP32) return wide ? launch_fd_stream_o<float, O, S, 8>(L, f) : launch_fd_stream_o<float, O, S, 2>(L, f);
   return wide ? launch_fd_stream_o<__nv_bfloat16, O, S, 8>(L, f) : launch_fd_stream_o<__nv_bfloat16, O, S, 2>(L, f);
 }

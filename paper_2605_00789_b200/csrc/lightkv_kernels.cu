@@ -318,6 +318,7 @@ struct XiSimtArgs {
   const int* seq_start;                            // first row of each sample in q, k, lse, lse_out (packed batches) or nullptr
   int vis_begin, n_text_after, bidirectional;
   int n_q_heads, n_kv_heads, dh;
+  unsigned int sms;                                // SMs of the device
   TextSet text;
 };
 
@@ -334,8 +335,8 @@ xi_simt_kernel(XiSimtArgs<T> a, Workspace ws) {
   // The queries with the most keys first.  Where every CTA is resident at once, two to an SM, the second half starts with
   // the fewest and hands its tiles to the warps in the other direction: the SMs, and the schedulers of an SM, have about
   // the same to do.
-  const bool second = gridDim.x <= 2 * 148 && blockIdx.x >= 148;
-  const int item = second ? gridDim.x - 1 - (blockIdx.x - 148) : blockIdx.x;
+  const bool second = gridDim.x <= 2 * a.sms && blockIdx.x >= a.sms;
+  const int item = second ? gridDim.x - 1 - (blockIdx.x - a.sms) : blockIdx.x;
   const int tiles = (ws.cap_in + XI_TQ - 1) / XI_TQ, heads = gridDim.x / tiles;           // (heads of all samples)
   const int b = item % heads / a.n_q_heads, h = item % heads % a.n_q_heads, t0 = (tiles - 1 - item / heads) * XI_TQ;
   const int n = a.n_vis ? min(a.n_vis[b], ws.cap_in) : ws.cap_in;
@@ -506,7 +507,8 @@ static cudaError_t launch_xi_simt_t(const LayerLaunch& L) {
   x.lse_out_bs = a->lse_out_batch_stride; x.lse_out_hs = a->lse_out_head_stride;
   x.n_vis = a->n_vis; x.seq_start = a->seq_start;
   x.vis_begin = a->vis_begin; x.n_text_after = a->n_text_after; x.bidirectional = a->bidirectional;
-  x.n_q_heads = L.n_q_heads; x.n_kv_heads = L.n_kv_heads; x.dh = dh; x.text = L.text;
+  x.n_q_heads = L.n_q_heads; x.n_kv_heads = L.n_kv_heads; x.dh = dh; x.sms = sm_count();
+  x.text = L.text;
   const cudaError_t e = ensure_dynamic_smem(xi_simt_kernel<T>, 108 * 1024);
   if (e != cudaSuccess) return e;
   return launch_kernel(xi_simt_kernel<T>, dim3(ctas), 32 * XI_WARPS, smem, L.stream, 1, x, L.ws);
@@ -1044,10 +1046,10 @@ cudaError_t launch_map(const LayerLaunch& L, bool select) {
   return select ? launch(map_kernel<false, 1, true>) : launch(map_kernel<false, 1, false>);
 }
 
-// Launches of at most this many rows do not fill the SMs' memory pipes by number: they get wider CTAs and more members of
+// Launches of at most four rows an SM do not fill the SMs' memory pipes by number: they get wider CTAs and more members of
 // a group in flight per thread: a group of ten tokens is three rounds of loads instead of five (one image of 576 tokens,
 // one layer: 39.6 -> 33.3 us a pass).
-constexpr int kFewRows = 4 * 148;
+static bool few_rows(long long rows) { return rows <= 4 * sm_count(); }
 
 // =====================================================================================================
 // Weighted merge of the hidden states (Eq. "message-passing", Steps 3-5): one CTA per output row.
@@ -1136,7 +1138,7 @@ cudaError_t launch_merge_rows(const LayerLaunch& L) {
   const lightkv_layer_args_t* a = L.a;
   const int rows = a->vis_begin + L.ws.cap_out + a->n_text_after;
   const dim3 grid(rows, L.batch);
-  const bool few = (long long)rows * L.batch <= kFewRows;
+  const bool few = few_rows((long long)rows * L.batch);
   auto run = [&](auto tag) -> cudaError_t {
     using T = decltype(tag);
     return launch_kernel(few ? merge_rows_kernel<T, 4> : merge_rows_kernel<T, 2>, grid, 256, 0, L.stream, 1,
@@ -1479,9 +1481,10 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
   const dim3 grid(a->vis_begin + K.cap_out + a->n_text_after, K.batch);
   const int units = 2 * K.n_kv_heads * ch_host;
   // two units per thread (both in flight); narrow caches (GQA) get narrow CTAs
-  const bool few = (long long)grid.x * grid.y <= kFewRows;
+  const bool few = few_rows((long long)grid.x * grid.y);
   const int threads = std::min(few ? 512 : 256, ((units + 1) / 2 + 31) / 32 * 32);
   const int gather = a->mode == LIGHTKV_KV_GATHER;
+  const int sms = sm_count();
   const bool in_place = a->k_src == a->k_dst;             // (the API checked that V and the addressing agree)
   auto run = [&](auto tag) -> cudaError_t {
     using T = decltype(tag);
@@ -1492,7 +1495,7 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
       const long long planes = 2ll * K.batch * K.n_kv_heads;
       int p = 1;
       while (ch_host % (2 * p) == 0 && ch_host / p >= 4 &&
-             (sm.bytes(ch_host / p) > 100 * 1024 || (planes * p < 2 * 148 && ch_host / p >= 8))) p *= 2;
+             (sm.bytes(ch_host / p) > 100 * 1024 || (planes * p < 2 * sms && ch_host / p >= 8))) p *= 2;
       const int ch = ch_host / p;
       if (sm.bytes(ch) <= 220 * 1024 && (long long)sm.rows_out * ch < 65536) {
         if ((e = ensure_dynamic_smem(kv_plane_kernel<T>, 220 * 1024)) != cudaSuccess) return e;
@@ -1510,7 +1513,7 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
     if (e != cudaSuccess || !in_place) return e;
     // planes: (sample, K / V, head), cut along head_dim while there are fewer of them than CTAs that fit
     int parts = 1;
-    while (parts < ch_host && K.batch * 2 * K.n_kv_heads * parts < 4 * 148 && ch_host % (2 * parts) == 0) parts *= 2;
+    while (parts < ch_host && K.batch * 2 * K.n_kv_heads * parts < 4 * sms && ch_host % (2 * parts) == 0) parts *= 2;
     const size_t smem = 2 * size_t(KVM_CHUNK_BYTES);
     if ((e = ensure_dynamic_smem(kv_move_kernel<T>, (int)smem)) != cudaSuccess) return e;
     return launch_kernel(kv_move_kernel<T>, dim3(K.batch * 2 * K.n_kv_heads * parts), KVM_THREADS, smem, K.stream, 1,

@@ -595,8 +595,6 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
 // A head of up to 64 (128) columns takes the kernel for 64 (128): the TMA loads fill the columns it lacks with zeros.
 bool tc_xi_supported(int head_dim) { return head_dim <= 128; }
 
-static int sm_count();
-
 cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first) {
   const lightkv_layer_args_t* a = L.a;
   const int rows = a->seq_rows > 0 ? a->seq_rows : a->vis_begin + L.ws.cap_in + a->n_text_after;
@@ -1005,19 +1003,6 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, FT_STAGES > 3 ? 1 : 2) fd_tc_
 }
 
 bool tc_fd_supported(int hidden) { return hidden % 8 == 0; }
-
-// SMs of the current device (cached per device ordinal).
-static int sm_count() {
-  static int cached[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-  if (!cached[dev]) {
-    int n = 0;
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) n = 148;
-    cached[dev] = n;
-  }
-  return cached[dev];
-}
 
 cudaError_t launch_fd_tc(const LayerLaunch& L, bool lists) {
   const lightkv_layer_args_t* a = L.a;
