@@ -420,8 +420,8 @@ def _sm_count():
 
 @pytest.mark.parametrize("head_dim", [64, 128])
 def test_lse_mode_persistent_ctas_walk_several_items(head_dim):
-    # 4 samples x 8 heads x 16 query tiles = 512 work items for at most 3 CTAs per SM: every CTA of the xi kernel
-    # takes a second item (its barriers and rings run on across items); 130 prompt rows span three key tiles
+    # 4 samples x 8 heads x 16 query tiles = 512 work items for 2 CTAs per SM: most CTAs of the xi kernel
+    # take a second item (its barriers and rings run on across items); 130 prompt rows span three key tiles
     wl = S.Workload(name="lsewalk", config_id=130, batch=4, tiles=((64, 32),), n_text=130, hidden=64, n_q_heads=8,
                     n_kv_heads=4, head_dim=head_dim, n_layers=16, layers=(3,), windows=(4,), keep=(0.5,))
     assert 16 * wl.n_q_heads * wl.batch > 3 * _sm_count()
@@ -467,7 +467,7 @@ def test_xi_items_taken_over_and_repeated(head_dim, text_ranges):
 
 
 def test_cfg2_lse_mode_full_size_sampled():
-    # the benchmark shape in ATTN_LSE mode (5888 work items walked by 3 CTAs per SM), bench.py's streams; the
+    # the benchmark shape in ATTN_LSE mode (5888 work items walked by 2 CTAs per SM), bench.py's streams; the
     # log-sum-exp input comes from plain torch ops, the oracle derives xi from Q and K alone
     stats = H.run_schedule(S.workload("cfg2"), xi_mode="lse", lse_source="torch", oracle_samples=[0, 5],
                            **_bench_streams())
@@ -476,10 +476,10 @@ def test_cfg2_lse_mode_full_size_sampled():
 
 @pytest.mark.parametrize("hidden,ragged", [(64, False), (72, True)])
 def test_fd_persistent_ctas_take_several_tiles(hidden, ragged):
-    # 160 samples x 36 windows of 16 tokens: three tiles of sixteen windows per sample (a tile holds at most 128 A
-    # nodes), 480 tiles for the 2 x SMs persistent CTAs of the tensor-core FD kernel, so most CTAs take a second
-    # tile (ring phases and the accumulator barrier run on); the ragged variant gives every sample its own subset
-    # of the grid under a plan built for subsets
+    # 160 samples x 36 windows of 16 tokens: 5760 CTAs of the streaming FD kernel, a window each, in many waves, with
+    # hidden sizes of one and two chunks a row; the ragged variant gives every sample its own subset of the grid under
+    # a plan built for subsets.  (CTAs of the tiled kernel that take several tiles: see
+    # test_fd_tiles_of_a_window_larger_than_the_plan_expects.)
     wl = S.Workload(name="fdmulti", config_id=131, batch=160, tiles=((24, 24),), n_text=4, hidden=hidden,
                     n_q_heads=2, n_kv_heads=1, head_dim=64, n_layers=16, layers=(3,), windows=(6,), keep=(0.5,))
     first = None
@@ -515,6 +515,21 @@ def test_fd_window_larger_than_the_plan_expects(grid, windows, seed):
     missing = int(rng.integers(4, 14))
     subset = np.sort(rng.choice(full, full.size - missing, replace=False)).astype(np.int32)
     H.run_schedule(wl, xi_mode="given", first_pos=[subset, full])
+
+
+@pytest.mark.parametrize("batch,hidden", [(2, 776), (30, 72), (45, 72)])
+def test_fd_tiles_of_a_window_larger_than_the_plan_expects(batch, hidden):
+    # the second stage's windows of up to 272 tokens are expected three quarters full (one tile of 128 x 128 nodes); here
+    # some are full (136 a side), so a CTA takes four tiles in a row: ring phases, accumulator barrier and lists run on.
+    # 8, 120 and 180 tiles: clusters, the deep ring, and neither
+    wl = S.Workload(name="tilewalk", config_id=137, batch=batch, tiles=((32, 34),), n_text=4, hidden=hidden, n_q_heads=2,
+                    n_kv_heads=1, head_dim=64, n_layers=16, layers=(3, 7), windows=(1, 2), keep=(0.75, 0.6))
+    rows, cols = np.divmod(np.arange(wl.n_vis, dtype=np.int32), 34)
+    window = (rows >= 16) * 2 + (cols >= 17)
+    three = np.nonzero(window != 2)[0].astype(np.int32)
+    one = np.concatenate([np.nonzero(window == 1)[0], np.nonzero(window != 1)[0][::5]])
+    pos = [three if b % 2 == 0 else np.sort(one).astype(np.int32) for b in range(batch)]
+    H.run_schedule(wl, xi_mode="uniform", stages=[1], ragged=True, first_pos=pos, oracle_samples=[0, 1, batch - 1])
 
 
 @pytest.mark.parametrize("grid,w", [((32, 32), 5), ((25, 41), 4), ((32, 64), 8), ((45, 46), 7), ((64, 64), 11),
@@ -713,6 +728,6 @@ def test_cfg4_gqa_video_full_schedule_sampled():
 
 
 def test_cfg4g_large_windows_uniform_xi():
-    # windows of 512, 1024 and 2048 tokens: FD tiles of 128 x 128 entries combined across B blocks (atomic
-    # minimum on the keys), the rank loops of the selection kernel over up to 1024 A entries
+    # windows of 512, 1024 and 2048 tokens: FD tiles of 128 x 128 nodes whose keys the map kernel combines across the
+    # blocks of destinations, and its selection among up to 1024 sources
     H.run_schedule(S.workload("cfg4g"), xi_mode="uniform", oracle_samples=[0])
