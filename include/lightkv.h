@@ -131,7 +131,8 @@ typedef struct {
   int32_t n_windows;               /* windows per sample */
   int32_t counts_exact;            /* 1: every sample holds exactly cap_in / cap_out tokens when
                                       it entered stage 0 with the full grid (host simulation)     */
-  int32_t uses_tensor_cores;       /* 1: the FD and xi contractions of this stage run on tcgen05  */
+  int32_t uses_tensor_cores;       /* 1: the FD and xi contractions of this stage run on tensor
+                                      cores                                                        */
   size_t  workspace_bytes;         /* DEVICE scratch lightkv_compress_layer needs                 */
   int32_t cap_a, cap_b;            /* upper bounds on the A / B nodes of one sample               */
   int32_t fd_tiles;                /* tiles (of nodes of one window) per sample the plan expects the FD
@@ -201,12 +202,15 @@ typedef struct {
                                       or NULL.  Event 0 is recorded on the stream before the first kernel,
                                       event i after kernel i: 1 window build, 2 xi, 3 FD + best partner,
                                       4 selection + merge map, 5 hidden-state merge (a kernel the mode skips
-                                      still gets its event).  For per-kernel timing. */
+                                      still gets its event; usually the FD kernel finds the windows itself and
+                                      nothing lies between events 0 and 1).  For per-kernel timing. */
   int32_t seq_rows;                /* rows every (sample, head) slice of q / k really holds (tensor-map
                                       bound of the TMA loads); 0 = vis_begin + cap_in + n_text_after */
   void*   aux_stream;              /* cudaStream_t or NULL.  When given (and xi comes from Q and K, and no
-                                      trace events are asked for), the window build and the FD kernel, which
-                                      stream the hidden states, are enqueued on this second stream while the
+                                      trace events are asked for), the FD kernel, which streams the hidden
+                                      states (and the window build, where one is launched: samples or windows
+                                      too long for the shared memory of a CTA, the fp32-FMA engine in bf16,
+                                      large windows in fp32), is enqueued on this second stream while the
                                       xi contraction runs on `stream`; the two are forked and joined with
                                       events inside the call, so the caller sees everything ordered on
                                       `stream` as before.  The stream must belong to the same device. */
@@ -248,7 +252,7 @@ typedef struct {
 
 #define LIGHTKV_TRACE_EVENTS 6
 
-/* Enqueue window build, xi, FD + best partner, selection + merge map and the weighted merge of the hidden states
+/* Enqueue windows, FD + best partner, xi, selection + merge map and the weighted merge of the hidden states
  * (Steps 1-5 of Sec. "LightKV"; Eq. "attention-factor", "similarity", "message-passing").  Nothing is allocated or
  * synchronised, and the workspace need not be cleared.  Errors: INVALID_ARG (NULL or misaligned buffers, strides below the row width, a prompt set
  * outside [0, vis_begin], aux_stream without its two events, lse_out outside ATTN_FULL, ...), WORKSPACE (too small
@@ -287,11 +291,12 @@ int lightkv_compress_layer_builtin_ws(const lightkv_plan_t* plan, const lightkv_
  * Out of place: the destinations do not overlap the sources.
  * In place: k_dst == k_src and v_dst == v_src with the same strides, page size and block table on both sides
  * (anything else that overlaps is INVALID_ARG or undefined).  The cache then shrinks inside its own rows or
- * pages, with no second copy of it: first every merged group is written over its surviving token's row (no
- * other group reads that row), then every output row moves forward to its slot -- a slot never lies behind its
- * source -- one (sample, K or V, head) plane per CTA, in ascending chunks that are gathered into shared memory
- * before any of their slots is written.  Rows behind the new end of a sample keep stale contents; pages that
- * became empty are the caller's to release. */
+ * pages, with no second copy of it.  Where the output rows of a (sample, K or V, head) plane fit into shared memory,
+ * perhaps cut by columns, one CTA gathers and merges them there before it stores any.  For longer samples every
+ * merged group is first written over its surviving token's row (no other group reads that row), then a second
+ * kernel moves every output row forward to its slot -- a slot never lies behind its source -- in ascending chunks
+ * that are gathered into shared memory before any of their slots is written.  Both forms leave the same bytes.  Rows
+ * behind the new end of a sample keep stale contents; pages that became empty are the caller's to release. */
 typedef struct {
   uint32_t struct_size;            /* sizeof(lightkv_kv_args_t) */
   int32_t  stage;

@@ -1,4 +1,4 @@
-// liblightkv kernels, part 3: FD + best partner for small windows (bf16), one pass over the hidden states.
+// liblightkv kernels, part 3: FD + best partner for small windows, one pass over the hidden states.
 #include <algorithm>
 
 #include "launch.h"
@@ -23,9 +23,11 @@ namespace lkv {
 // Since the CTA has its whole window, it also finds the window's tokens (from the positions; no list has to be built
 // before) and makes the selection of Steps 2 and 4; what is left for the map kernel is one prefix sum per sample.
 // A lane's pieces wait in shared memory (cp.async, a ring of S chunks per warp that only this lane writes and reads,
-// so no barrier): loads in flight then cost no registers.  Against the tcgen05 kernel with its gathered 128-row tiles:
-// 8 samples x 2880 tokens x 4096 in windows of 16: 59 -> 37 us between events (189 MB: 5.1 TB/s), windows of 18:
-// 41 -> 27, of 36: 39 -> 23; 32 x 576 x 5120 in windows of 36: 76 -> 45, of 72: 59 -> 29.
+// so no barrier): loads in flight then cost no registers.  Between events, search and selection included, against the
+// tcgen05 kernel with its gathered 128-row tiles alone (which had a window build of 11 to 17 us in front of it): 8 samples
+// x 2880 tokens x 4096 in windows of 16: 59 -> 42 us over the whole grid (189 MB: 4.5 TB/s), 49 where positions are given
+// and searched; windows of 18: 41 -> 35, of 36: 39 -> 27; 32 x 576 x 5120 in windows of 36: 76 -> 48, of 72: 59 -> 31.
+// The contraction alone took 37, 27, 23, 45 and 29 us; a CTA loads nothing while it searches and selects.
 // ======================================================================================================
 struct FdStreamArgs {
   const void* x;                       // first vision row of sample 0
@@ -347,7 +349,7 @@ cudaError_t launch_fd_stream(const LayerLaunch& L) {
   f.d = L.hidden; f.metric = L.divergence; f.keep = L.keep; f.g = L.geo; f.n_vis = a->n_vis; f.pos = a->pos;
   f.cap_in = L.ws.cap_in; f.max_cell = L.max_cell; f.partner = L.ws.partner; f.place = L.ws.slot;
   // chunks in flight per warp (S): as few as still leave enough CTAs on an SM; with more, fewer CTAs fit and the
-  // start and end of a window are less covered (S = 8, 6, 4 measured 39 / 33 / 25 us where 6, 4, 3 take 37 / 27 / 23)
+  // start and end of a window are less covered (contraction alone: S = 8, 6, 4 39 / 33 / 25 us, 6, 4, 3 37 / 27 / 23)
   switch ((L.fd_side + 7) / 8) {
     case 1: return launch_fd_stream_w<1, 6>(L, f);
     case 2: return launch_fd_stream_w<2, 4>(L, f);

@@ -785,8 +785,9 @@ cudaError_t launch_select_map(const LayerLaunch& L) {
 //   3  weights xi_i / sum over the group, the sum taken in member order (survivor first)
 // Bound by latency: one round trip to L2 for the loads, three cluster barriers, one round of stores.  A merged token
 // that would need a kernel-wide search for its group costs one remote read here, because the streaming FD kernel holds
-// whole windows.  (select_map_kernel, which starts from keys, takes six dependent rounds through L2: 9 us at 576 and
-// 20 us at 2880 tokens per sample against 5 and 7.)
+// whole windows.  Between events (2.7 us with nothing between them): one sample of 576 tokens 10.5 us, 8 x 720 12,
+// 8 x 2880 14 to 16; with the selection in front of it one window of 144 tokens 16, windows of 512 to 2048 20 to 25.
+// (select_map_kernel, which starts from keys, takes six dependent rounds through L2: 18 us for 8 x 720, 26 for 8 x 2880.)
 // =====================================================================================================
 struct MapArgs {
   int n_q_heads, xi_mode, cap_in, cap_out, cap_a, cap_b, n_grid;
