@@ -639,8 +639,8 @@ cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first) {
 //
 // A CTA (or a cluster of ks CTAs that split the hidden dimension, where there are few tiles) takes one tile of up to
 // 128 sources x 128 destinations of one window.  The rows of a tile are scattered over the sequence; the CTA finds them
-// from the positions (window_tokens) or, for samples too long for that, in the lists the window build left.  Eight warps gather them with 16-byte cp.async copies, eight threads per 128-byte row
-// segment, straight into the 128-byte-swizzled K-major layout tcgen05 reads, through a ring of stages of 32 KB (64 columns
+// from the positions (window_tokens) or, in the list form, in the lists the window build left.  Eight warps gather them
+// with 16-byte cp.async copies, eight threads per 128-byte row segment, straight into the 128-byte-swizzled K-major layout tcgen05 reads, through a ring of stages of 32 KB (64 columns
 // of both operands), and re-read their pieces to accumulate the squared norms.  A ninth warp issues
 // G += X_A X_B^T (128 x N x 64 per chunk, bf16 -> fp32 in TMEM).  The MMA always reads 128 A
 // rows: rows the tile does not have are never written and only feed accumulator rows nobody reads.  After the last chunk

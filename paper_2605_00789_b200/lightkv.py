@@ -264,7 +264,8 @@ def compress_layer(plan: Plan, stage: int, hidden, out: StageBuffers, **kw) -> N
 def compress_layer_builtin_ws(plan: Plan, stage: int, hidden, out: StageBuffers, **kw) -> None:
     """lightkv_compress_layer_builtin_ws: same call, but the stage's scratch is the fixed array inside
     the library (BUILTIN_WS_BYTES), so the workspace tensor of `out` is not used.  Meant for callers
-    that may not allocate device memory; stages needing more scratch than that are refused."""
+    that may not allocate device memory; stages whose tiled FD needs more scratch than that run in the
+    slower list form, what fits in neither is refused."""
     (_BINDING or _binding()).compress_layer_builtin_ws(plan, stage, hidden, out, **kw)
 
 
