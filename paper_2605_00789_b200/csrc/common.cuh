@@ -38,7 +38,7 @@ struct Workspace {
   // tiled FD kernel without window lists (these two lie over the arrays of the list form)
   unsigned long long* tile_key;  // [B, fd blocks, cap_in]  such keys by token and block of destinations, see fd_tc_kernel
   int* win_tok;    // [B, n_windows, max_cell + 1]  tiled FD kernel: the number of tokens of a window, then the tokens
-  float* xi_h;     // [B, H, cap_in]      per-head attention mass on the prompt (ATTN modes)
+  float* xi_h;     // [B, cap_in, H]      per-head attention mass on the prompt (ATTN modes): a token's heads in one line
   float* xi;       // [B, cap_in]
   int* partner;    // [B, cap_in]         token a source is merged into; negative: survives (-2: a source that was not
                    //                     selected, where the streaming FD kernel wrote it)
@@ -167,6 +167,8 @@ __device__ inline void st_stream16(void* p, const uint4& v) {
                :: "l"(p), "r"(v.x), "r"(v.y), "r"(v.z), "r"(v.w) : "memory");
 }
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // monotone map float -> uint32 (ascending floats give ascending integers)
 __device__ inline uint32_t orderable(float f) {
   uint32_t u = __float_as_uint(f);
@@ -188,10 +190,10 @@ __device__ __forceinline__ float pair_score(int metric, float g, float na, float
 // it may start once every CTA of the kernel before it has called grid_launch_dependents() or exited, and
 // grid_dependency_wait() returns when that kernel has completed and its writes are visible.  Every kernel waits
 // before it exits, so a kernel's completion implies that of all before it.  Most wait before they touch global memory
-// (grid_dependency_sync: a launch's latency then hides behind its predecessor).  Two use the order further: the window
-// build lets the next kernel start only after its own wait, so everything before the call is complete when that
-// kernel starts; and the xi kernel, which reads nothing the window build or FD write, waits only at its end, i.e. runs
-// beside them.  Launched without the attribute, the instructions do nothing.
+// (grid_dependency_sync: a launch's latency then hides behind its predecessor).  Two use the order further: the first
+// kernel of a call (window build or FD) lets the next start only after its own wait, so everything before the call is
+// complete when any later kernel of the call starts; and the xi kernels, which read nothing the window build, FD or the
+// map write, wait only at their end, i.e. run beside them.  Launched without the attribute, the instructions do nothing.
 __device__ __forceinline__ void grid_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dependency_sync() {

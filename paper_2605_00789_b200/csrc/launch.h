@@ -122,16 +122,21 @@ cudaError_t launch_fd_simt(const LayerLaunch& L);
 // and its place for launch_map
 bool fd_stream_supported(int dtype, int fd_side);
 cudaError_t launch_fd_stream(const LayerLaunch& L);
-// head sum of xi, merge map, weights from the partners (Steps 4, 5), with `select` from the keys of launch_fd_tc; at most
-// kMapMaxTokens per sample
+// merge map from the partners (Steps 4, 5), with `select` from the keys of launch_fd_tc, and the weights where xi is given or
+// uniform; at most kMapMaxTokens per sample
 constexpr int kMapMaxTokens = 16384;
 cudaError_t launch_map(const LayerLaunch& L, bool select);
-// xi per head (Eq. "attention-factor"), fp32 FMA path; handles ATTN_FULL and ATTN_LSE
-cudaError_t launch_xi_simt(const LayerLaunch& L);
+// xi per head (Eq. "attention-factor"), fp32 FMA path; handles ATTN_FULL and ATTN_LSE.  wait_first: the stream's last kernel
+// is not one of the same call that lets the next start behind its own wait (FD, or the map behind it)
+cudaError_t launch_xi_simt(const LayerLaunch& L, bool wait_first);
 // head sum of xi, ranking, merge map, weights (Steps 2-5)
 cudaError_t launch_select_map(const LayerLaunch& L);
-// weighted merge of the hidden states (Eq. "message-passing")
-cudaError_t launch_merge_rows(const LayerLaunch& L);
+// head sum of xi and weights behind launch_map and the xi kernel
+cudaError_t launch_weights(const LayerLaunch& L);
+// weighted merge of the hidden states (Eq. "message-passing"); `weights`: with the head sum of xi and the weights, for
+// the launches that are faster so
+bool merge_takes_weights(const LayerLaunch& L);
+cudaError_t launch_merge_rows(const LayerLaunch& L, bool weights);
 
 struct KvLaunch {
   int batch, n_kv_heads, head_dim, dtype, cap_in, cap_out;
@@ -145,7 +150,7 @@ bool tc_fd_supported(int hidden);
 bool tc_xi_supported(int head_dim);
 // lists: windows from launch_window_build, keys by source entry for launch_select_map; else by token for launch_map
 cudaError_t launch_fd_tc(const LayerLaunch& L, bool lists);
-// wait_first: the stream's last kernel is not the window build or FD of the same call
+// wait_first: as for launch_xi_simt
 cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first);
 
 // lightkv_compress_layer.  `least`: a workspace of least_workspace() bytes will do; where the tiled FD kernel's keys do not

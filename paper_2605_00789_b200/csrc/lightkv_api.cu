@@ -362,9 +362,15 @@ int compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* a, bool 
   auto launch_fd = [&](const LayerLaunch& l) {
     return streaming ? launch_fd_stream(l) : tc_fd && near ? launch_fd_tc(l, !tiled) : launch_fd_simt(l);
   };
+  // The map behind the FD kernels that hold whole windows needs no xi; the list form's does.
+  const bool early_map = streaming || tiled;
+  auto launch_groups = [&](const LayerLaunch& l) { return early_map ? launch_map(l, tiled) : cudaSuccess; };
+  auto launch_xi = [&](bool first) {
+    return !attn ? cudaSuccess : tc_xi ? launch_xi_tc(L, first) : launch_xi_simt(L, first);
+  };
   cudaStream_t aux = (a->aux_stream && attn && !ev) ? static_cast<cudaStream_t>(a->aux_stream) : nullptr;
   if (aux) {
-    // fork: window build + FD (HBM bound) on the second stream, xi (bound by the exponentials) on the first.
+    // fork: window build, FD (HBM bound) and the map on the second stream, xi (bound by the exponentials) on the first.
     // The events are the caller's; once the fork is recorded the join is enqueued whatever happens between.
     cudaEvent_t fork = static_cast<cudaEvent_t>(a->fork_event), join = static_cast<cudaEvent_t>(a->join_event);
     LayerLaunch La = L;
@@ -373,25 +379,33 @@ int compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* a, bool 
     bool ok = cudaStreamWaitEvent(aux, fork, 0) == cudaSuccess;
     ok = ok && launch_windows(La) == cudaSuccess;
     ok = ok && launch_fd(La) == cudaSuccess;
+    ok = ok && launch_groups(La) == cudaSuccess;
     const bool joined = cudaEventRecord(join, aux) == cudaSuccess;
-    ok = ok && (tc_xi ? launch_xi_tc(L, true) : launch_xi_simt(L)) == cudaSuccess;
+    ok = ok && launch_xi(true) == cudaSuccess;
     const bool waited = joined && cudaStreamWaitEvent(L.stream, join, 0) == cudaSuccess;
     if (!ok || !waited) return LIGHTKV_ERR_CUDA;
-  } else {
-    // FD in front of xi, which runs beside it and the window build (programmatic launch order, see
-    // grid_dependency_sync); for per-kernel timing the two keep the order of the trace events
-    auto launch_xi = [&](bool first) { return !attn ? cudaSuccess : tc_xi ? launch_xi_tc(L, first) : launch_xi_simt(L); };
+  } else if (ev) {
+    // per-kernel timing: one kernel after the other, in the order of the trace events
     if (mark(0) != cudaSuccess) return LIGHTKV_ERR_CUDA;
     if (launch_windows(L) != cudaSuccess || mark(1) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-    if (!ev && launch_fd(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-    if (launch_xi(ev != nullptr) != cudaSuccess || mark(2) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-    if (ev && (launch_fd(L) != cudaSuccess || mark(3) != cudaSuccess)) return LIGHTKV_ERR_CUDA;
+    if (launch_xi(true) != cudaSuccess || mark(2) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+    if (launch_fd(L) != cudaSuccess || mark(3) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+    if (launch_groups(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+  } else {
+    // FD and the map in front of xi, which runs beside them (programmatic launch order, see grid_dependency_sync)
+    if (launch_windows(L) != cudaSuccess || launch_fd(L) != cudaSuccess || launch_groups(L) != cudaSuccess ||
+        launch_xi(false) != cudaSuccess)
+      return LIGHTKV_ERR_CUDA;
   }
-  const cudaError_t mapped = streaming || tiled ? launch_map(L, tiled) : launch_select_map(L);
-  if (mapped != cudaSuccess || mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+  if (!early_map && launch_select_map(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+  // weights: by a kernel of their own where the merge does not take them along, and for a caller that waits for the map
+  // alone (to compact K/V beside the merge)
+  const bool late_weights = early_map && attn, with_merge = late_weights && !a->map_event && merge_takes_weights(L);
+  if (late_weights && !with_merge && launch_weights(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+  if (mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (a->map_event && cudaEventRecord(static_cast<cudaEvent_t>(a->map_event), L.stream) != cudaSuccess)
     return LIGHTKV_ERR_CUDA;
-  if (launch_merge_rows(L) != cudaSuccess || mark(5) != cudaSuccess) return LIGHTKV_ERR_CUDA;
+  if (launch_merge_rows(L, with_merge) != cudaSuccess || mark(5) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   return LIGHTKV_OK;
 }
 

@@ -1,6 +1,7 @@
 // liblightkv kernels, part 1: window build, fp32-FMA contractions (FD, xi), selection + merge map,
 // weighted merge of hidden states, K/V merge-compaction.  sm_100a.
 #include <algorithm>
+#include <type_traits>
 
 #include "launch.h"
 #include "tc_common.cuh"
@@ -319,13 +320,15 @@ struct XiSimtArgs {
   int vis_begin, n_text_after, bidirectional;
   int n_q_heads, n_kv_heads, dh;
   unsigned int sms;                                // SMs of the device
+  int wait_first;                                  // as in the tensor-core kernel
   TextSet text;
 };
 
 template <typename T>
 __global__ void __launch_bounds__(32 * XI_WARPS, 2)
 xi_simt_kernel(XiSimtArgs<T> a, Workspace ws) {
-  grid_dependency_sync();
+  grid_launch_dependents();
+  if (a.wait_first) grid_dependency_wait();              // else at the end: it reads nothing FD or the map write
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int dh = a.dh, ldq = xi_q_pitch(dh);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -340,7 +343,10 @@ xi_simt_kernel(XiSimtArgs<T> a, Workspace ws) {
   const int tiles = (ws.cap_in + XI_TQ - 1) / XI_TQ, heads = gridDim.x / tiles;           // (heads of all samples)
   const int b = item % heads / a.n_q_heads, h = item % heads % a.n_q_heads, t0 = (tiles - 1 - item / heads) * XI_TQ;
   const int n = a.n_vis ? min(a.n_vis[b], ws.cap_in) : ws.cap_in;
-  if (t0 >= n) return;
+  if (t0 >= n) {
+    grid_dependency_wait();
+    return;
+  }
   const int nq = min(XI_TQ, n - t0);
   const int hk = h / (a.n_q_heads / a.n_kv_heads);
   const int row0 = a.seq_start ? a.seq_start[b] : 0;
@@ -487,14 +493,15 @@ xi_simt_kernel(XiSimtArgs<T> a, Workspace ws) {
       all += s_all[k][r] * f;
       txt += s_txt[k][r] * f;
     }
-    ws.xi_h[(size_t(b) * a.n_q_heads + h) * ws.cap_in + t0 + r] = a.lse ? txt : txt / all;
+    ws.xi_h[(size_t(b) * ws.cap_in + t0 + r) * a.n_q_heads + h] = a.lse ? txt : txt / all;
     if (a.lse_out)
       a.lse_out[size_t(b) * a.lse_out_bs + size_t(h) * a.lse_out_hs + row0 + q_pos + r] = (m + log2f(all)) * 0.6931471805599453f;
   }
+  grid_dependency_wait();
 }
 
 template <typename T>
-static cudaError_t launch_xi_simt_t(const LayerLaunch& L) {
+static cudaError_t launch_xi_simt_t(const LayerLaunch& L, bool wait_first) {
   const lightkv_layer_args_t* a = L.a;
   const int dh = L.head_dim;
   const size_t smem = size_t(XI_WARPS * 2 * XI_TK * XI_LD + XI_TQ * xi_q_pitch(dh)) * sizeof(float);   // at most 105 KB: two CTAs per SM
@@ -508,14 +515,15 @@ static cudaError_t launch_xi_simt_t(const LayerLaunch& L) {
   x.n_vis = a->n_vis; x.seq_start = a->seq_start;
   x.vis_begin = a->vis_begin; x.n_text_after = a->n_text_after; x.bidirectional = a->bidirectional;
   x.n_q_heads = L.n_q_heads; x.n_kv_heads = L.n_kv_heads; x.dh = dh; x.sms = sm_count();
+  x.wait_first = wait_first ? 1 : 0;
   x.text = L.text;
   const cudaError_t e = ensure_dynamic_smem(xi_simt_kernel<T>, 108 * 1024);
   if (e != cudaSuccess) return e;
   return launch_kernel(xi_simt_kernel<T>, dim3(ctas), 32 * XI_WARPS, smem, L.stream, 1, x, L.ws);
 }
 
-cudaError_t launch_xi_simt(const LayerLaunch& L) {
-  return L.dtype == LIGHTKV_BF16 ? launch_xi_simt_t<__nv_bfloat16>(L) : launch_xi_simt_t<float>(L);
+cudaError_t launch_xi_simt(const LayerLaunch& L, bool wait_first) {
+  return L.dtype == LIGHTKV_BF16 ? launch_xi_simt_t<__nv_bfloat16>(L, wait_first) : launch_xi_simt_t<float>(L, wait_first);
 }
 
 // =====================================================================================================
@@ -663,7 +671,7 @@ __global__ void __launch_bounds__(1024) select_map_kernel(Workspace ws, SelectAr
     else {
       v = 0.f;
 #pragma unroll 8
-      for (int h = 0; h < a.n_q_heads; ++h) v += ws.xi_h[(size_t(b) * a.n_q_heads + h) * ws.cap_in + i];
+      for (int h = 0; h < a.n_q_heads; ++h) v += ws.xi_h[(size_t(b) * ws.cap_in + i) * a.n_q_heads + h];
     }
     xi[i] = v;
     if (a.xi_out) a.xi_out[size_t(b) * ws.cap_in + i] = v;
@@ -775,26 +783,35 @@ cudaError_t launch_select_map(const LayerLaunch& L) {
 // =====================================================================================================
 // Merge map behind the streaming FD kernel, which left every token's partner and its place (see Workspace), or, with
 // SELECT, behind the tiled one, which left the windows' tokens and keys: the CTAs of a sample then first take its windows
-// in turn and select.  One
+// in turn and select.  Groups, slots and positions need no xi: where xi comes from attention the kernel runs beside the xi
+// kernel and leaves the weights to those behind it (weights_kernel, merge_rows_kernel); given or uniform xi is at hand
+// (WEIGHTS).  One
 // cluster of 1-8 CTAs per sample, TPT consecutive tokens per thread, everything between the first loads and the last
 // stores in registers and (distributed) shared memory:
-//   1  xi = fixed-order sum over heads (or given / uniform); survivors and group sizes are counted in ONE pair of prefix
-//      sums: a survivor's slot, and the offset of its group (its members are 1 + place tokens)
-//   2  a merged token reads its partner's slot and offset from the CTA that owns it and stores its index and xi at its
-//      place in that CTA's member list (groups of one CTA's survivors are one contiguous range)
-//   3  weights xi_i / sum over the group, the sum taken in member order (survivor first)
-// Bound by latency: one round trip to L2 for the loads, three cluster barriers, one round of stores.  A merged token
-// that would need a kernel-wide search for its group costs one remote read here, because the streaming FD kernel holds
-// whole windows.  Between events (2.7 us with nothing between them): one sample of 576 tokens 10.5 us, 8 x 720 12,
-// 8 x 2880 14 to 16; with the selection in front of it one window of 144 tokens 16, windows of 512 to 2048 20 to 25.
-// (select_map_kernel, which starts from keys, takes six dependent rounds through L2: 18 us for 8 x 720, 26 for 8 x 2880.)
+//   1  survivors and group sizes are counted in ONE pair of prefix sums: a survivor's slot, and the offset of its group
+//      (its members are 1 + place tokens)
+//   2  a merged token reads its partner's slot and offset from the CTA that owns it (WEIGHTS: and puts its index and xi at
+//      its place in that CTA's member list; groups of one CTA's survivors are one contiguous range)
+//   3  WEIGHTS: xi_i / sum over the group, the sum taken in member order (survivor first)
+// Bound by latency: one round trip to L2 for the loads, three cluster barriers, one round of stores: 1.6 us from its wait to
+// its end for 576 tokens, 2 for 16 x 432, 4 to 8 for 2880 (5.6, 7 and 10.5 when it also summed xi, behind the xi kernel).  A
+// merged token that would need a kernel-wide search for its group costs one remote read here, because the streaming FD
+// kernel holds whole windows.
+// (select_map_kernel, which starts from keys, takes six dependent rounds through L2.)
 // =====================================================================================================
+// floor(n / d) for n, d < 65536 with m = ceil(2^32 / d): one multiply instead of a division
+__device__ inline int div_magic(int n, unsigned m) { return (int)__umulhi((unsigned)n, m); }
+
+// The weight of a member with `xi` in a group of `size` whose sum is `den`.
+__device__ __forceinline__ float member_weight(float xi, float den, int size) {
+  return den >= 1e-30f ? xi / den : 1.0f / (float)size;
+}
+
 struct MapArgs {
-  int n_q_heads, xi_mode, cap_in, cap_out, cap_a, cap_b, n_grid;
+  int xi_mode, cap_in, cap_out, cap_a, cap_b, n_grid;
+  const float* xi_in;
   const int* n_vis;
   const int* pos;
-  const float* xi_in;
-  const float* xi_h;
   int* partner;
   int* place;
   const unsigned long long* key;       // SELECT: [B, blocks, cap_in]
@@ -804,26 +821,26 @@ struct MapArgs {
   int* n_vis_out;
   int* pos_out;
   int* dst;
-  float* weight;
   int* grp_off;
   int* grp_src;
+  float* weight;
   float* xi_out;
   uint32_t* status;
 };
 
-template <bool CLUSTER, int TPT, bool SELECT>
+template <bool CLUSTER, int TPT, bool SELECT, bool WEIGHTS>
 __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapArgs a) {
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int nthr = blockDim.x, tid = threadIdx.x, lane = tid & 31, wp = tid >> 5;
   const int span = nthr * TPT;                              // tokens a CTA can own
   int* s_slot = reinterpret_cast<int*>(smem_raw);           // [span] slot of an owned survivor
-  int* s_at = s_slot + span;                                // [span] offset of its group inside this CTA's member list
-  int* m_tok = s_at + span;                                 // [cap_in] member list: token index
-  float* m_xi = reinterpret_cast<float*>(m_tok + a.cap_in); // [cap_in] ... and its xi
+  int* s_off = s_slot + span;                               // [span] offset of its group
+  int* m_tok = s_off + span;                                // WEIGHTS: [cap_in] member list: token index
+  float* m_xi = reinterpret_cast<float*>(m_tok + a.cap_in); // WEIGHTS: [cap_in] ... and its xi
+  __shared__ int base_off[8];                               // WEIGHTS: first member offset of every CTA
   __shared__ int warp_sums[2][33];
   __shared__ int cta_total[3];                              // survivors, members, sources of this CTA
-  __shared__ int base_off[8];                               // first member offset of every CTA
   const int cs = CLUSTER ? (int)tc::cluster_nctarank() : 1, rank = CLUSTER ? (int)tc::cluster_ctarank() : 0;
   auto sync_all = [&]() { if (CLUSTER) tc::cluster_sync(); else __syncthreads(); };
   const int b = blockIdx.x / cs;
@@ -864,8 +881,9 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
 #pragma unroll
   for (int j = 0; j < TPT; ++j) {
     const int i = i0 + j;
-    prt[j] = -1; plc[j] = 0; ps[j] = i; xi[j] = 0.f;
+    prt[j] = -1; plc[j] = 0; ps[j] = i; xi[j] = 1.0f;
     if (i < hi) {
+      if (WEIGHTS && a.xi_mode == LIGHTKV_XI_GIVEN) xi[j] = a.xi_in[row + i];
       prt[j] = __ldcg(a.partner + row + i);
       plc[j] = __ldcg(a.place + row + i);
       if (a.pos) {
@@ -873,18 +891,6 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
         bad = bad || ps[j] <= (i > 0 ? a.pos[row + i - 1] : -1) || ps[j] >= a.n_grid;
       } else {
         bad = bad || i >= a.n_grid;
-      }
-      if (a.xi_mode == LIGHTKV_XI_GIVEN) xi[j] = a.xi_in[row + i];
-      else if (a.xi_mode == LIGHTKV_XI_UNIFORM) xi[j] = 1.0f;
-      else {
-        const float* x = a.xi_h + size_t(b) * a.n_q_heads * a.cap_in + i;
-        for (int h0 = 0; h0 < a.n_q_heads; h0 += 16) {      // sixteen heads' loads in flight, added in head order
-          float v[16];
-#pragma unroll
-          for (int h = 0; h < 16; ++h) v[h] = h0 + h < a.n_q_heads ? x[size_t(h0 + h) * a.cap_in] : 0.f;
-#pragma unroll
-          for (int h = 0; h < 16; ++h) xi[j] += v[h];
-        }
       }
     }
   }
@@ -924,16 +930,26 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
   }
   sync_all();
   int before_s = 0, before_m = 0, survivors = 0, members = 0, sources = 0;
-  for (int j = 0; j < cs; ++j) {
-    auto total = [&](int k) {
-      return CLUSTER ? (int)tc::ld_cluster_u32(tc::map_to_cta(tc::smem_u32(&cta_total[k]), j)) : cta_total[k];
-    };
-    const int s = total(0), m = total(1);
-    if (tid == 0) base_off[j] = members;
-    if (j < rank) { before_s += s; before_m += m; }
-    survivors += s;
-    members += m;
-    sources += total(2);
+  if (CLUSTER) {
+    int total[8][3];                                        // all of the cluster's counts in flight
+#pragma unroll
+    for (int j = 0; j < 8; ++j)
+#pragma unroll
+      for (int k = 0; k < 3; ++k)
+        total[j][k] = j < cs ? (int)tc::ld_cluster_u32(tc::map_to_cta(tc::smem_u32(&cta_total[k]), j)) : 0;
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      if (j < rank) { before_s += total[j][0]; before_m += total[j][1]; }
+      if (WEIGHTS && tid == 0) base_off[j] = members;
+      survivors += total[j][0];
+      members += total[j][1];
+      sources += total[j][2];
+    }
+  } else {
+    if (WEIGHTS && tid == 0) base_off[0] = 0;
+    survivors = cta_total[0];
+    members = cta_total[1];
+    sources = cta_total[2];
   }
   // A sample whose A or B nodes do not fit the plan's capacities (a subset of the grid handed to a plan that was built
   // for full grids) keeps all of its tokens, and the status word says so.
@@ -956,9 +972,9 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
   for (int j = 0; j < TPT; ++j) {
     const int i = i0 + j;
     if (i < hi && prt[j] < 0) {
-      const int l = i - lo, at = off - before_m;
+      const int l = i - lo;
       s_slot[l] = slot;
-      s_at[l] = at;
+      s_off[l] = off;
       a.dst[row + i] = slot;
       if (slot < a.cap_out) {
         a.pos_out[size_t(b) * a.cap_out + slot] = ps[j];
@@ -967,8 +983,10 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
       } else if (slot == a.cap_out) {
         a.grp_off[size_t(b) * (a.cap_out + 1) + slot] = off;   // the groups that are kept end here
       }
-      m_tok[at] = i;
-      m_xi[at] = xi[j];
+      if (WEIGHTS) {
+        m_tok[off - before_m] = i;
+        m_xi[off - before_m] = xi[j];
+      }
       ++slot;
       off += 1 + plc[j];
     }
@@ -983,36 +1001,36 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
       int o, at;
       if (CLUSTER) {
         o = (int)tc::ld_cluster_u32(tc::map_to_cta(tc::smem_u32(&s_slot[l]), r));
-        at = (int)tc::ld_cluster_u32(tc::map_to_cta(tc::smem_u32(&s_at[l]), r));
+        at = (int)tc::ld_cluster_u32(tc::map_to_cta(tc::smem_u32(&s_off[l]), r));
       } else {
-        o = s_slot[l]; at = s_at[l];
+        o = s_slot[l]; at = s_off[l];
       }
       at += 1 + plc[j];
       a.dst[row + i] = o;
-      if (o < a.cap_out) a.grp_src[row + base_off[r] + at] = i;
-      if (CLUSTER) {
-        tc::st_cluster_u32(tc::map_to_cta(tc::smem_u32(&m_tok[at]), r), (uint32_t)i);
-        tc::st_cluster_u32(tc::map_to_cta(tc::smem_u32(&m_xi[at]), r), __float_as_uint(xi[j]));
-      } else {
-        m_tok[at] = i; m_xi[at] = xi[j];
+      if (o < a.cap_out) a.grp_src[row + at] = i;
+      if (WEIGHTS) {
+        at -= base_off[r];
+        if (CLUSTER) {
+          tc::st_cluster_u32(tc::map_to_cta(tc::smem_u32(&m_tok[at]), r), (uint32_t)i);
+          tc::st_cluster_u32(tc::map_to_cta(tc::smem_u32(&m_xi[at]), r), __float_as_uint(xi[j]));
+        } else {
+          m_tok[at] = i; m_xi[at] = xi[j];
+        }
       }
     }
-    if (i < hi && a.xi_out) a.xi_out[row + i] = xi[j];
+    if (WEIGHTS && i < hi && a.xi_out) a.xi_out[row + i] = xi[j];
   }
-  sync_all();
-  // ---- weights
+  if (CLUSTER || WEIGHTS) sync_all();                       // nobody reads or writes this CTA's shared memory any more
+  if (WEIGHTS) {
 #pragma unroll
-  for (int j = 0; j < TPT; ++j) {
-    const int i = i0 + j;
-    if (i < hi && prt[j] < 0 && s_slot[i - lo] < a.cap_out) {
-      const int at = s_at[i - lo], size = 1 + plc[j];
-      float den = 0.f;
-      for (int c = 0; c < size; ++c) den += m_xi[at + c];
-      if (den >= 1e-30f) {
-        for (int c = 0; c < size; ++c) a.weight[row + m_tok[at + c]] = m_xi[at + c] / den;
-      } else {
-        set_status(a.status, LIGHTKV_STATUS_ZERO_WEIGHT);
-        for (int c = 0; c < size; ++c) a.weight[row + m_tok[at + c]] = 1.0f / (float)size;
+    for (int j = 0; j < TPT; ++j) {
+      const int i = i0 + j;
+      if (i < hi && prt[j] < 0 && s_slot[i - lo] < a.cap_out) {
+        const int at = s_off[i - lo] - before_m, size = 1 + plc[j];
+        float den = 0.f;
+        for (int c = 0; c < size; ++c) den += m_xi[at + c];
+        for (int c = 0; c < size; ++c) a.weight[row + m_tok[at + c]] = member_weight(m_xi[at + c], den, size);
+        if (!(den >= 1e-30f)) set_status(a.status, LIGHTKV_STATUS_ZERO_WEIGHT);
       }
     }
   }
@@ -1020,14 +1038,17 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
 
 cudaError_t launch_map(const LayerLaunch& L, bool select) {
   const lightkv_layer_args_t* a = L.a;
+  // xi from attention is not there yet
+  const bool weights = L.xi_mode == LIGHTKV_XI_GIVEN || L.xi_mode == LIGHTKV_XI_UNIFORM;
   MapArgs m;
-  m.n_q_heads = L.n_q_heads; m.xi_mode = L.xi_mode; m.cap_in = L.ws.cap_in; m.cap_out = L.ws.cap_out;
+  m.xi_mode = L.xi_mode; m.xi_in = a->xi; m.weight = a->weight; m.xi_out = a->xi_out;
+  m.cap_in = L.ws.cap_in; m.cap_out = L.ws.cap_out;
   m.cap_a = L.ws.cap_a; m.cap_b = L.ws.cap_b; m.n_grid = L.n_grid;
-  m.n_vis = a->n_vis; m.pos = a->pos; m.xi_in = a->xi; m.xi_h = L.ws.xi_h; m.partner = L.ws.partner; m.place = L.ws.slot;
+  m.n_vis = a->n_vis; m.pos = a->pos; m.partner = L.ws.partner; m.place = L.ws.slot;
   m.key = L.ws.tile_key; m.win_tok = L.ws.win_tok; m.blocks = L.fd_blocks; m.max_cell = L.max_cell; m.n_windows = L.geo.n_windows;
   m.src_par = L.geo.src_par; m.keep = L.keep;
-  m.n_vis_out = a->n_vis_out; m.pos_out = a->pos_out; m.dst = a->dst; m.weight = a->weight; m.grp_off = a->grp_off;
-  m.grp_src = a->grp_src; m.xi_out = a->xi_out; m.status = a->status;
+  m.n_vis_out = a->n_vis_out; m.pos_out = a->pos_out; m.dst = a->dst; m.grp_off = a->grp_off;
+  m.grp_src = a->grp_src; m.status = a->status;
   // one cluster per sample: as many CTAs of up to 1024 threads as give every thread one token (two beyond 8192), and
   // with windows to select in, as many as there are windows (up to eight) of at least 256 threads
   const int n = L.ws.cap_in;
@@ -1035,51 +1056,229 @@ cudaError_t launch_map(const LayerLaunch& L, bool select) {
   while (cs < 8 && (cs * 1024 < n || (select && cs < L.geo.n_windows))) cs *= 2;
   const int tpt = n > 8192 ? 2 : 1;
   const int threads = std::max(select ? 256 : 32, std::min(1024, (((n + cs - 1) / cs + tpt - 1) / tpt + 31) / 32 * 32));
-  size_t smem = (size_t(2) * threads * tpt + size_t(2) * n) * 4;
+  size_t smem = (size_t(2) * threads * tpt + (weights ? size_t(2) * n : 0)) * 4;
   if (select) smem = std::max(smem, WindowLists::bytes(L.max_cell));
   auto launch = [&](auto kernel) -> cudaError_t {
     const cudaError_t e = ensure_dynamic_smem(kernel, (int)smem);
     if (e != cudaSuccess) return e;
     return launch_kernel(kernel, L.batch * cs, threads, smem, L.stream, cs, m);
   };
-  if (tpt == 2) return select ? launch(map_kernel<true, 2, true>) : launch(map_kernel<true, 2, false>);
-  if (cs > 1) return select ? launch(map_kernel<true, 1, true>) : launch(map_kernel<true, 1, false>);
-  return select ? launch(map_kernel<false, 1, true>) : launch(map_kernel<false, 1, false>);
+  auto form = [&](auto w) {
+    constexpr bool W = decltype(w)::value;
+    if (tpt == 2) return select ? launch(map_kernel<true, 2, true, W>) : launch(map_kernel<true, 2, false, W>);
+    if (cs > 1) return select ? launch(map_kernel<true, 1, true, W>) : launch(map_kernel<true, 1, false, W>);
+    return select ? launch(map_kernel<false, 1, true, W>) : launch(map_kernel<false, 1, false, W>);
+  };
+  return weights ? form(std::true_type()) : form(std::false_type());
 }
 
 // Launches of at most four rows an SM do not fill the SMs' memory pipes by number: they get wider CTAs and more members of
 // a group in flight per thread: a group of ten tokens is three rounds of loads instead of five (one image of 576 tokens,
 // one layer: 39.6 -> 33.3 us a pass).
 static bool few_rows(long long rows) { return rows <= 4 * sm_count(); }
+static bool few_rows(const LayerLaunch& L) {
+  return few_rows((long long)(L.a->vis_begin + L.ws.cap_out + L.a->n_text_after) * L.batch);
+}
+// The instructions a row's CTA spends on its weights are in nobody's way while a launch is short; a long one is bound by
+// memory only as long as little else is issued.  Whole passes, with the merge against by weights_kernel: 4 x 652 rows of 4096
+// 144.3 / 145.3 us, 16 x up to 624 rows of 2048 (23 MB) 138 / 144; 8 x 3008 rows of 4096 (100 MB) and its later stages 556 / 511.
+bool merge_takes_weights(const LayerLaunch& L) {
+  return (long long)(L.a->vis_begin + L.ws.cap_out + L.a->n_text_after) * L.batch * L.hidden * (L.dtype == LIGHTKV_BF16 ? 2 : 4) <= (24ll << 20);
+}
+
+// =====================================================================================================
+// xi of the tokens (fixed-order sum over the heads) and the weights of the groups (Eq. "message-passing"), behind
+// map_kernel, which knows the groups but runs beside the xi kernel: xi_i / sum over the group, the sum taken in member
+// order (survivor first).  A cluster of eight CTAs per sample: a warp sums the heads of eight tokens into
+// shared memory; then a thread per group reads its members' sums from the CTAs that hold them.  Bound by
+// the length of its chain of loads, shuffles and barriers: 4 to 6 us (32 tokens a warp, or a thread per token: 6 to 12).
+// =====================================================================================================
+struct WeightArgs {
+  int n_q_heads, cap_in, cap_out;
+  int chunk;                           // weights_kernel: tokens per CTA
+  unsigned magic_chunk;                // (see div_magic)
+  const float* xi_h;                   // [B, cap_in, H]
+  const int* n_vis;
+  const int* n_vis_out;
+  const int* grp_off;
+  const int* grp_src;
+  const int* dst;
+  float* weight;
+  float* xi_out;
+  uint32_t* status;
+};
+constexpr int kWeightCtas = 8;
+
+__global__ void __launch_bounds__(1024) weights_kernel(const __grid_constant__ WeightArgs a) {
+  grid_dependency_sync();
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  float* s_xi = reinterpret_cast<float*>(smem_raw);       // [chunk] xi of this CTA's tokens
+  const int rank = (int)tc::cluster_ctarank(), b = blockIdx.x / kWeightCtas, tid = threadIdx.x, nthr = blockDim.x;
+  const int warp = tid >> 5, lane = tid & 31, H = a.n_q_heads;
+  const size_t row = size_t(b) * a.cap_in;
+  // a thread's first group is looked up at once, before the counts are there (the lists have the room)
+  const int o0 = tid * kWeightCtas + rank;
+  const int* go = a.grp_off + size_t(b) * (a.cap_out + 1);
+  int g0 = 0, g1 = 0;
+  if (o0 < a.cap_out) { g0 = go[o0]; g1 = go[o0 + 1]; }
+  const int n = a.n_vis ? max(0, min(a.n_vis[b], a.cap_in)) : a.cap_in, n_out = a.n_vis_out[b];
+  const int lo = rank * a.chunk, hi = min(a.cap_in, lo + a.chunk);
+  const float* x = a.xi_h + row * H;
+  for (int i0 = lo + 8 * warp; i0 < hi; i0 += nthr >> 2) {
+    // eight tokens of a warp, the lanes over the heads (addresses are clamped, not loads left out: a load behind a branch
+    // waits for the one before); then lane l holds the sum of token l / 4
+    float p[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
+    const int last = a.cap_in - 1 - i0;
+    for (int h0 = lane; h0 - lane < H; h0 += 64) {
+      const float* xh = x + i0 * H + min(h0, H - 1);
+      const float* xg = x + i0 * H + min(h0 + 32, H - 1);
+      float v[8], w[8];
+#pragma unroll
+      for (int t = 0; t < 8; ++t) v[t] = xh[min(t, last) * H];
+      if (h0 - lane + 32 < H) {
+#pragma unroll
+        for (int t = 0; t < 8; ++t) w[t] = xg[min(t, last) * H];
+#pragma unroll
+        for (int t = 0; t < 8; ++t) p[t] += h0 + 32 < H ? w[t] : 0.f;
+      }
+#pragma unroll
+      for (int t = 0; t < 8; ++t) p[t] += h0 < H ? v[t] : 0.f;
+    }
+#pragma unroll
+    for (int o = 16; o >= 4; o >>= 1) {
+#pragma unroll
+      for (int t = 0; t < o / 4; ++t) {
+        const float give = lane & o ? p[t] : p[t + o / 4], keep = lane & o ? p[t + o / 4] : p[t];
+        p[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+      }
+    }
+    float v = p[0];
+    v += __shfl_xor_sync(0xffffffffu, v, 2);
+    v += __shfl_xor_sync(0xffffffffu, v, 1);
+    const int i = i0 + (lane >> 2);
+    if ((lane & 3) == 0 && i < hi) {
+      s_xi[i - lo] = v;
+      if (a.xi_out && i < n) a.xi_out[row + i] = v;
+    }
+  }
+  constexpr int AHEAD = 8;                                // members looked up at once
+  const int* gs = a.grp_src + row;
+  int tok[AHEAD];
+#pragma unroll
+  for (int k = 0; k < AHEAD; ++k) tok[k] = gs[min(max(g0 + k, 0), a.cap_in - 1)];
+  tc::cluster_sync();
+  const uint32_t base = tc::smem_u32(s_xi);
+  auto xi_of = [&](int i) {
+    const int r = div_magic(i, a.magic_chunk);
+    return tc::ld_cluster_f32(tc::map_to_cta(base + uint32_t(i - r * a.chunk) * 4, r));
+  };
+  for (int o = o0; o < n_out; o += kWeightCtas * nthr) {
+    if (o != o0) {
+      g0 = go[o];
+      g1 = go[o + 1];
+#pragma unroll
+      for (int k = 0; k < AHEAD; ++k) tok[k] = gs[min(g0 + k, a.cap_in - 1)];
+    }
+    const int size = g1 - g0;
+    float den = 0.f, first[AHEAD];
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k) first[k] = k < size ? xi_of(tok[k]) : 0.f;
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k) den += first[k];
+    for (int g = AHEAD; g < size; ++g) den += xi_of(gs[g0 + g]);
+#pragma unroll
+    for (int k = 0; k < AHEAD; ++k)
+      if (k < size) a.weight[row + tok[k]] = member_weight(first[k], den, size);
+    for (int g = AHEAD; g < size; ++g) {
+      const int i = gs[g0 + g];
+      a.weight[row + i] = member_weight(xi_of(i), den, size);
+    }
+    if (!(den >= 1e-30f)) set_status(a.status, LIGHTKV_STATUS_ZERO_WEIGHT);
+  }
+  tc::cluster_sync();                                     // nobody reads this CTA's shared memory any more
+}
+
+static WeightArgs weight_args(const LayerLaunch& L) {
+  const lightkv_layer_args_t* a = L.a;
+  const int chunk = (L.ws.cap_in + kWeightCtas - 1) / kWeightCtas;      // at most kMapMaxTokens / 8
+  return {L.n_q_heads, L.ws.cap_in, L.ws.cap_out, chunk, (unsigned)(((1ull << 32) + chunk - 1) / chunk), L.ws.xi_h, a->n_vis,
+          a->n_vis_out, a->grp_off, a->grp_src, a->dst, a->weight, a->xi_out, a->status};
+}
+
+cudaError_t launch_weights(const LayerLaunch& L) {
+  const WeightArgs w = weight_args(L);
+  const int threads = std::min(1024, std::max(4 * w.chunk, 128) / 32 * 32 + 32);       // warps for one round over the tokens
+  return launch_kernel(weights_kernel, L.batch * kWeightCtas, threads, size_t(4) * w.chunk, L.stream, kWeightCtas, w);
+}
+
+// xi of token i of sample b in every lane of the warp that asks; the lanes share the heads, two loads in flight
+__device__ __forceinline__ float warp_xi(const WeightArgs& a, int b, int i, int lane) {
+  const float* x = a.xi_h + (size_t(b) * a.cap_in + i) * a.n_q_heads;
+  float v = 0.f;
+#pragma unroll 1
+  for (int h = lane; h < a.n_q_heads; h += 64) v += x[h] + (h + 32 < a.n_q_heads ? x[h + 32] : 0.f);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// A sample cut at cap_out has tokens that belong to no group that is kept: their xi is still reported.
+__device__ __noinline__ void xi_of_cut_tokens(const WeightArgs& a, int b, int n, int n_out) {
+  if (!a.xi_out || a.grp_off[size_t(b) * (a.cap_out + 1) + n_out] >= n) return;
+  const int lane = threadIdx.x & 31;
+  for (int i = threadIdx.x >> 5; i < n; i += blockDim.x >> 5)
+    if (a.dst[size_t(b) * a.cap_in + i] >= a.cap_out) {
+      const float v = warp_xi(a, b, i, lane);
+      if (lane == 0) a.xi_out[size_t(b) * a.cap_in + i] = v;
+    }
+}
 
 // =====================================================================================================
 // Weighted merge of the hidden states (Eq. "message-passing", Steps 3-5): one CTA per output row.
 // Row o of the vision block is sum over its group of weight_i * x_i in fp32, rounded once to the
-// storage type; a group of one has weight exactly 1 and is therefore copied bit-exactly.  Text rows
+// storage type; a group of one has weight exactly 1 and is copied.  Text rows
 // before / after the vision block are copied.  Pure 16-byte streaming loads and stores.
+// WEIGHTS: the CTA computes its group's weights, too (a warp per member), while its first rows are on their way to L2: one
+// kernel less in a row of dependent ones.  See merge_takes_weights.
 // =====================================================================================================
-template <typename T, int MB>
-__global__ void __launch_bounds__(256)
-merge_rows_kernel(const T* __restrict__ src, int64_t src_bs, int64_t src_rs,
-                  T* __restrict__ out, int64_t out_bs, int64_t out_rs,
-                  int d, int vis_begin, int n_text_after, int cap_in, int cap_out,
-                  const int* __restrict__ n_vis, const int* __restrict__ n_vis_out,
-                  const int* __restrict__ grp_off, const int* __restrict__ grp_src,
-                  const float* __restrict__ weight, const int* __restrict__ seq_start,
-                  const int* __restrict__ seq_start_out) {
+template <typename T>
+struct MergeArgs {
+  const T* src; int64_t src_bs, src_rs;
+  T* out; int64_t out_bs, out_rs;
+  int d, vis_begin, n_text_after;
+  const int* seq_start;
+  const int* seq_start_out;
+  WeightArgs w;
+};
+
+template <typename T, int MB, bool WEIGHTS>
+__global__ void __launch_bounds__(256, MB > 2 ? 3 : 5) merge_rows_kernel(const __grid_constant__ MergeArgs<T> a) {
   grid_dependency_sync();
   constexpr int V = Vec<T>::n;
-  const int b = blockIdx.y, row = blockIdx.x;
-  const int n_in = n_vis ? min(n_vis[b], cap_in) : cap_in;
-  const int n_out = n_vis_out[b];
-  if (row >= vis_begin + n_out + n_text_after) return;
-  const T* sb = src + size_t(b) * src_bs + size_t(seq_start ? seq_start[b] : 0) * src_rs;
-  T* orow = out + size_t(b) * out_bs + size_t((seq_start_out ? seq_start_out[b] : 0) + row) * out_rs;
-  const int chunks = d / V;
-  if (row < vis_begin || row >= vis_begin + n_out) {
-    const T* srow = sb + size_t(row < vis_begin ? row : row - n_out + n_in) * src_rs;
-    for (int c0 = threadIdx.x; c0 < chunks; c0 += 2 * blockDim.x) {
-      const int c1 = c0 + blockDim.x;
+  constexpr int AHEAD = 64;                             // members whose weights stay on chip
+  __shared__ float s_xi[WEIGHTS ? AHEAD : 1], s_wt[WEIGHTS ? AHEAD : 1];
+  const int b = blockIdx.y, row = blockIdx.x, o = row - a.vis_begin;
+  const int cap_in = a.w.cap_in, cap_out = a.w.cap_out;
+  // (the row's group is looked up before it is known that the row has one: one round trip less)
+  const int* go = a.w.grp_off + size_t(b) * (cap_out + 1) + min(max(o, 0), cap_out - 1);
+  const int g0 = go[0], g1 = go[1];
+  const int n_in = a.w.n_vis ? min(a.w.n_vis[b], cap_in) : cap_in;
+  const int n_out = a.w.n_vis_out[b];
+  if (WEIGHTS && row == 0) xi_of_cut_tokens(a.w, b, n_in, n_out);
+  if (row >= a.vis_begin + n_out + a.n_text_after) return;
+  const T* sb = a.src + size_t(b) * a.src_bs + size_t(a.seq_start ? a.seq_start[b] : 0) * a.src_rs;
+  T* orow = a.out + size_t(b) * a.out_bs + size_t((a.seq_start_out ? a.seq_start_out[b] : 0) + row) * a.out_rs;
+  const int chunks = a.d / V, tid = threadIdx.x, nthr = blockDim.x;
+  const bool text = o < 0 || o >= n_out;
+  const int* gs = a.w.grp_src + size_t(b) * cap_in + g0;
+  float* wt = a.w.weight + size_t(b) * cap_in;
+  float* xo = a.w.xi_out ? a.w.xi_out + size_t(b) * cap_in : nullptr;
+  const int count = text ? 1 : g1 - g0;
+  if (count == 1) {                                     // copied
+    const int i = text ? 0 : gs[0];
+    const T* srow = sb + size_t(text ? (o < 0 ? row : row - n_out + n_in) : a.vis_begin + i) * a.src_rs;
+    for (int c0 = tid; c0 < chunks; c0 += 2 * nthr) {
+      const int c1 = c0 + nthr;
       const uint4 a0 = ld_stream16(srow + c0 * V);
       if (c1 < chunks) {
         const uint4 a1 = ld_stream16(srow + c1 * V);
@@ -1087,17 +1286,60 @@ merge_rows_kernel(const T* __restrict__ src, int64_t src_bs, int64_t src_rs,
       }
       st_stream16(orow + c0 * V, a0);
     }
+    if (WEIGHTS && !text && tid < 32) {
+      const float v = warp_xi(a.w, b, i, tid);
+      if (tid == 0) {
+        wt[i] = 1.0f;
+        if (xo) xo[i] = v;
+        if (!(v >= 1e-30f)) set_status(a.w.status, LIGHTKV_STATUS_ZERO_WEIGHT);
+      }
+    }
     return;
   }
-  const int o = row - vis_begin;
-  const int* go = grp_off + size_t(b) * (cap_out + 1);
-  const int g0 = go[o], count = go[o + 1] - g0;
-  const int* gs = grp_src + size_t(b) * cap_in;
-  const float* wt = weight + size_t(b) * cap_in;
-  const T* vis = sb + size_t(vis_begin) * src_rs;
+  const T* vis = sb + size_t(a.vis_begin) * a.src_rs;
+  if (WEIGHTS) {
+    // the rows are asked for while the weights are computed (prefetches hold no registers)
+    for (int g = 0; g < min(count, 8); ++g) {
+      const T* r = vis + size_t(gs[g]) * a.src_rs;
+      if (tid * V * 2 < a.d) prefetch_l2(r + tid * V * 2);
+    }
+    const int lane = tid & 31;
+    float den = 0.f;
+    for (int k0 = 0; k0 < count; k0 += AHEAD) {
+      const int m = min(AHEAD, count - k0);
+      for (int k = tid >> 5; k < m; k += nthr >> 5) {
+        const int i = gs[k0 + k];
+        const float v = warp_xi(a.w, b, i, lane);
+        if (lane == 0) {
+          s_xi[k] = v;
+          if (xo) xo[i] = v;
+          if (count > AHEAD) wt[i] = v;
+        }
+      }
+      __syncthreads();
+      for (int k = 0; k < m; ++k) den += s_xi[k];
+      if (count > AHEAD) __syncthreads();           // (s_xi is filled again, or read below)
+    }
+    if (count <= AHEAD) {
+      for (int k = tid; k < count; k += nthr) {
+        const float w = member_weight(s_xi[k], den, count);
+        s_wt[k] = w;
+        wt[gs[k]] = w;
+      }
+    } else {
+      for (int k = tid; k < count; k += nthr) {
+        const int i = gs[k];
+        const float w = member_weight(wt[i], den, count);
+        wt[i] = w;
+        if (k < AHEAD) s_wt[k] = w;
+      }
+    }
+    if (tid == 0 && !(den >= 1e-30f)) set_status(a.w.status, LIGHTKV_STATUS_ZERO_WEIGHT);
+    __syncthreads();
+  }
   // two 16-byte chunks per thread and MB members at a time: 2 MB loads in flight whatever the group's size
-  for (int c0 = threadIdx.x; c0 < chunks; c0 += 2 * blockDim.x) {
-    const int c1 = c0 + blockDim.x;
+  for (int c0 = tid; c0 < chunks; c0 += 2 * nthr) {
+    const int c1 = c0 + nthr;
     const bool two = c1 < chunks;
     float acc0[V], acc1[V];
 #pragma unroll
@@ -1108,9 +1350,9 @@ merge_rows_kernel(const T* __restrict__ src, int64_t src_bs, int64_t src_rs,
 #pragma unroll
       for (int u = 0; u < MB; ++u) {
         if (g + u < count) {
-          const int i = gs[g0 + g + u];
-          wv[u] = wt[i];
-          const T* r = vis + size_t(i) * src_rs;
+          const int i = gs[g + u];
+          if (!WEIGHTS) wv[u] = wt[i];
+          const T* r = vis + size_t(i) * a.src_rs;
           va[u] = ld_stream16(r + c0 * V);
           if (two) vb[u] = ld_stream16(r + c1 * V);
         }
@@ -1118,6 +1360,7 @@ merge_rows_kernel(const T* __restrict__ src, int64_t src_bs, int64_t src_rs,
 #pragma unroll
       for (int u = 0; u < MB; ++u) {
         if (g + u < count) {
+          if (WEIGHTS) wv[u] = g + u < AHEAD ? s_wt[g + u] : wt[gs[g + u]];
           float f[V];
           unpack16(va[u], f, T());
 #pragma unroll
@@ -1135,18 +1378,19 @@ merge_rows_kernel(const T* __restrict__ src, int64_t src_bs, int64_t src_rs,
   }
 }
 
-cudaError_t launch_merge_rows(const LayerLaunch& L) {
+cudaError_t launch_merge_rows(const LayerLaunch& L, bool weights) {
   const lightkv_layer_args_t* a = L.a;
   const int rows = a->vis_begin + L.ws.cap_out + a->n_text_after;
   const dim3 grid(rows, L.batch);
-  const bool few = few_rows((long long)rows * L.batch);
   auto run = [&](auto tag) -> cudaError_t {
     using T = decltype(tag);
-    return launch_kernel(few ? merge_rows_kernel<T, 4> : merge_rows_kernel<T, 2>, grid, 256, 0, L.stream, 1,
-        static_cast<const T*>(a->hidden), a->hidden_batch_stride, a->hidden_row_stride,
-        static_cast<T*>(a->hidden_out), a->hidden_out_batch_stride, a->hidden_out_row_stride,
-        L.hidden, a->vis_begin, a->n_text_after, L.ws.cap_in, L.ws.cap_out, a->n_vis, a->n_vis_out,
-        a->grp_off, a->grp_src, a->weight, a->seq_start, a->seq_start_out);
+    const MergeArgs<T> m = {static_cast<const T*>(a->hidden), a->hidden_batch_stride, a->hidden_row_stride,
+                            static_cast<T*>(a->hidden_out), a->hidden_out_batch_stride, a->hidden_out_row_stride,
+                            L.hidden, a->vis_begin, a->n_text_after, a->seq_start, a->seq_start_out, weight_args(L)};
+    if (few_rows(L)) return launch_kernel(weights ? merge_rows_kernel<T, 4, true> : merge_rows_kernel<T, 4, false>, grid, 256, 0, L.stream, 1, m);
+    // two chunks per thread: narrow rows get narrow CTAs, and more of them
+    const int pairs = (L.hidden / Vec<T>::n + 1) / 2, threads = std::max(64, std::min(256, (pairs + 31) / 32 * 32));
+    return launch_kernel(weights ? merge_rows_kernel<T, 2, true> : merge_rows_kernel<T, 2, false>, grid, threads, 0, L.stream, 1, m);
   };
   return L.dtype == LIGHTKV_BF16 ? run(__nv_bfloat16()) : run(float());
 }
@@ -1173,8 +1417,6 @@ struct KvAddr {
 };
 
 
-// floor(n / d) for n, d < 65536 with m = ceil(2^32 / d): one multiply instead of a division
-__device__ inline int div_magic(int n, unsigned m) { return (int)__umulhi((unsigned)n, m); }
 
 // THREADS per CTA, MB members of a group in flight
 template <typename T, int THREADS, int MB>

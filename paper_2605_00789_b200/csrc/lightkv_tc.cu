@@ -296,7 +296,7 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
       };
       bool asked = false;                                  // a request for another CTA's item is on its way
       auto ask = [&]() {
-        if (LSE || asked) return;
+        if (asked) return;
         mbar_expect_tx(clc_full, 16);
         clc_try_cancel(clc_slot, clc_full);
         asked = true;
@@ -325,22 +325,16 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
         }
         return true;
       };
-      const int n_items = a.n_qt * a.n_q_heads * a.batch;
       bool ok = true;
       Item it;
       for (int item = blockIdx.x; ok && item >= 0;) {
         if (decode(item, it)) ok = publish(item, it, 0) && feed(it, true);
-        if (LSE) {
-          // items of the LSE form are all alike: a fixed round-robin split balances them
-          item = item + int(gridDim.x) < n_items ? item + int(gridDim.x) : -1;
-        } else {
-          ask();
-          ok = mbar_wait(clc_full, n_clc & 1, abort_flag) && ok;   // the answer is awaited even when the item failed
-          ++n_clc;
-          asked = false;
-          item = clc_canceled_cta(clc_slot);
-          fence_proxy_async();                             // the slot has been read before the next answer is written
-        }
+        ask();
+        ok = mbar_wait(clc_full, n_clc & 1, abort_flag) && ok;   // the answer is awaited even when the item failed
+        ++n_clc;
+        asked = false;
+        item = clc_canceled_cta(clc_slot);
+        fence_proxy_async();                               // the slot has been read before the next answer is written
       }
       if (!LSE && ok) {
         // all items handed out: once the softmax warps are done with the last two, the list of this CTA is complete
@@ -573,7 +567,7 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
         if (lane == 0) mbar_arrive(pair_empty);             // the exchange buffers are free for the next item
       }
       if (r < nq && !*abort_flag) {
-        a.xi_h[(size_t(b) * a.n_q_heads + h) * a.cap_in + t0 + r] = LSE ? l_txt : l_txt / l_all;
+        a.xi_h[(size_t(b) * a.cap_in + t0 + r) * a.n_q_heads + h] = LSE ? l_txt : l_txt / l_all;
         if (!LSE && a.lse_out)
           a.lse_out[size_t(b) * a.lse_out_bs + size_t(h) * a.lse_out_hs + row0 + s_first + r] =
               fmaf(m_run, sc, log2f(l_all)) * 0.6931471805599453f;
@@ -618,9 +612,9 @@ cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first) {
   x.redo_next = L.ws.xi_redo; x.wait_first = wait_first ? 1 : 0;
   const long long n_items = (long long)x.n_qt * L.n_q_heads * L.batch;
   if (n_items > 0x7fffffffLL) return cudaErrorInvalidValue;
-  // One CTA per item, taken over by the resident ones; with the caller's log-sum-exp an item is one or two key tiles
-  // and as many CTAs as stay resident walk them round-robin.
-  const dim3 grid((unsigned)(x.lse ? std::min<long long>(n_items, XT_CTAS * sm_count()) : n_items));
+  // One CTA per item, taken over by the resident ones (with the caller's log-sum-exp, too, whose items are alike: FD and
+  // the map may hold some SMs for a while, and a fixed share of the items would wait for them)
+  const dim3 grid((unsigned)n_items);
   // Q tiles + K ring (LSE: two Q tiles, one K stage; otherwise one Q tile, XT_STAGES K stages) + control block + exchange
   const int halves = L.head_dim <= 64 ? 1 : 2;
   const size_t smem = size_t(halves) * (x.lse ? 2 * 16384 + XT_KEY_TILE * 128

@@ -637,6 +637,79 @@ def test_subset_given_to_a_full_grid_plan_raises_the_count_bit():
     plan.close()
 
 
+# ---- xi summed over the heads, and weights: with the merge of the rows, or in front of it -------------------------
+
+@pytest.mark.parametrize("heads", [1, 7, 33, 40, 70])
+@pytest.mark.parametrize("before_merge", [False, True])
+def test_weights_over_head_counts(heads, before_merge):
+    """A warp's lanes take the heads 32 at a time, in one and in two rounds.  With a map event the weights come from a
+    kernel of their own: clusters whose CTAs hold 8 to 41 tokens."""
+    import torch
+    wl = S.Workload(name="heads", config_id=133, batch=3, tiles=((13, 17), (9, 11)), n_text=9, hidden=72, n_q_heads=heads,
+                    n_kv_heads=1, head_dim=64, n_layers=8, layers=(2, 5), windows=(3, 2), keep=(0.6, 0.5))
+    H.run_schedule(wl, kv_stream=torch.cuda.Stream() if before_merge else None)
+
+
+@pytest.mark.parametrize("grid", [(11, 11), (13, 17), (32, 40)])
+@pytest.mark.parametrize("before_merge", [False, True])
+def test_weights_of_a_group_of_all_sources(grid, before_merge):
+    """Equal source rows all join one destination: groups of 61, 111 and 641 members, below and beyond what the kernels keep
+    on chip.  The weights are the reported xi over their sum (single precision: 1e-5 over up to 641 terms), and the merged
+    row is the weighted sum of the members' rows."""
+    import torch
+    import paper_2605_00789_b200 as L
+    wl = S.Workload(name="onegroup", config_id=134, batch=1, tiles=(grid,), n_text=5, hidden=1032, n_q_heads=6,
+                    n_kv_heads=2, head_dim=64, n_layers=4, layers=(2,), windows=(1,), keep=(0.5,))
+    n, na = grid[0] * grid[1], (grid[0] * grid[1] + 1) // 2
+    removed = n - int(np.ceil(0.5 * n))
+    plan = H.make_plan(wl)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(grid[0])
+    hidden_in = torch.randn((1, wl.n_text + n, wl.hidden), generator=gen, device="cuda")
+    hidden_in[:, wl.n_text::2] = hidden_in[:, wl.n_text:wl.n_text + 1].clone()
+    hidden_in = hidden_in.bfloat16()
+    q = torch.randn((1, 6, wl.n_text + n, 64), generator=gen, device="cuda").bfloat16()
+    k = torch.randn((1, 2, wl.n_text + n, 64), generator=gen, device="cuda").bfloat16()
+    kw = {}
+    if before_merge:
+        kw["map_event"] = torch.cuda.Event()
+        kw["map_event"].record()
+    out = L.StageBuffers(plan, 0, wl.n_text + plan.stage_info(0).cap_out, "cuda")
+    L.compress_layer(plan, 0, hidden_in, out, vis_begin=wl.n_text, q=q, k=k, **kw)
+    assert int(out.status) == 0 and int(out.n_vis_out) == n - removed and na - removed in (0, 1)
+    off, src = out.grp_off[0].cpu().numpy(), out.grp_src[0].cpu().numpy()
+    xi, weight = (t[0].cpu().numpy().astype(np.float64) for t in (out.xi_out, out.weight))
+    rows, merged = hidden_in[0].float().cpu().numpy(), out.hidden_out[0].float().cpu().numpy()
+    sizes = np.diff(off[:n - removed + 1])
+    assert (xi > 0).all() and sizes.max() == removed + 1 and sizes.sum() == n
+    for o in (int(sizes.argmax()), int(sizes.argmin())):
+        members = src[off[o]:off[o + 1]]
+        np.testing.assert_allclose(weight[members], xi[members] / xi[members].sum(), rtol=1e-5, atol=0)
+        want = weight[members] @ rows[wl.n_text + members]
+        np.testing.assert_allclose(merged[wl.n_text + o], want, rtol=2 ** -8, atol=1e-4)
+    plan.close()
+
+
+@pytest.mark.parametrize("before_merge", [False, True])
+def test_xi_of_tokens_cut_at_the_capacity_is_reported(before_merge):
+    """A subset under a full-grid plan keeps all of its tokens and is cut at cap_out: those behind the cut belong to no group,
+    and their xi is reported all the same -- the same as under a plan that has room for them."""
+    import torch
+    wl, first = _near_full_subset()
+    plan, roomy = H.make_plan(wl, batch=2), H.make_plan(wl, batch=2, ragged=True)
+    g0 = H.gpu_stage(plan, wl, 0, H.prepare_stage(wl, 0, first))
+    pos1 = [g0["pos_out"][b, :int(g0["n_vis_out"][b])] for b in range(2)]
+    inp1 = H.prepare_stage(wl, 1, pos1)
+    cut = H.gpu_stage(plan, wl, 1, inp1, kv_stream=torch.cuda.Stream() if before_merge else None)
+    whole = H.gpu_stage(roomy, wl, 1, inp1)
+    n = int(inp1["n_vis"][0])
+    assert int(cut["status"][0]) == 8 and int(cut["n_vis_out"][0]) < n
+    np.testing.assert_array_equal(cut["xi_out"][0, :n] > 0, True)
+    np.testing.assert_allclose(cut["xi_out"][0, :n], whole["xi_out"][0, :n], rtol=1e-6, atol=0)
+    plan.close()
+    roomy.close()
+
+
 # ---- seeded random geometries ---------------------------------------------------------------------
 
 def _random_workload(seed):
