@@ -799,8 +799,9 @@ cudaError_t launch_select_map(const LayerLaunch& L) {
 // kernel holds whole windows.
 // (select_map_kernel, which starts from keys, takes six dependent rounds through L2.)
 // =====================================================================================================
-// floor(n / d) for n, d < 65536 with m = ceil(2^32 / d): one multiply instead of a division
-__device__ inline int div_magic(int n, unsigned m) { return (int)__umulhi((unsigned)n, m); }
+// floor(n / d) for n, d < 65536 with m = ceil(2^32 / d): one multiply instead of a division.  For d = 1 that is one bit too
+// long and m arrives as 0.
+__device__ inline int div_magic(int n, unsigned m) { return m ? (int)__umulhi((unsigned)n, m) : n; }
 
 // The weight of a member with `xi` in a group of `size` whose sum is `den`.
 __device__ __forceinline__ float member_weight(float xi, float den, int size) {

@@ -804,3 +804,19 @@ def test_cfg4g_large_windows_uniform_xi():
     # windows of 512, 1024 and 2048 tokens: FD tiles of 128 x 128 nodes whose keys the map kernel combines across the
     # blocks of destinations, and its selection among up to 1024 sources
     H.run_schedule(S.workload("cfg4g"), xi_mode="uniform", oracle_samples=[0])
+
+
+@pytest.mark.parametrize("in_place", [False, True])
+def test_heads_of_one_piece(in_place):
+    # head_dim 8 in bf16: a head's row is a single 16-byte piece
+    wl = S.Workload(name="piece", config_id=142, batch=2, tiles=((9, 7),), n_text=3, hidden=64, n_q_heads=4,
+                    n_kv_heads=4, head_dim=8, n_layers=16, layers=(3,), windows=(2,), keep=(0.55,))
+    H.run_schedule(wl, xi_mode="given", kv_in_place=in_place)
+
+
+def test_weights_of_samples_with_a_token_per_cta():
+    # at most eight tokens a sample, weights by a kernel of their own (the caller waits for the map alone)
+    import torch
+    wl = S.Workload(name="few", config_id=143, batch=3, tiles=((2, 4),), n_text=9, hidden=64, n_q_heads=4,
+                    n_kv_heads=4, head_dim=64, n_layers=16, layers=(3,), windows=(1,), keep=(0.5,))
+    H.run_schedule(wl, kv_stream=torch.cuda.Stream())
