@@ -1409,11 +1409,13 @@ struct KvAddr {
   const int* table;       // nullptr = contiguous
   int page_size, max_blocks;
   const int* seq_start;   // first token of each sample (packed caches) or nullptr
+  unsigned magic_page;    // ceil(2^32 / page_size) where that divides every row of a table exactly, else 0
+  __device__ inline int page_of(int n) const { return magic_page ? (int)__umulhi((unsigned)n, magic_page) : n / page_size; }
   __device__ inline int64_t token(int b, int n) const {
     if (seq_start) n += seq_start[b];
     if (!table) return int64_t(b) * batch_stride + int64_t(n) * row_stride;
-    const int page = table[size_t(b) * max_blocks + n / page_size];
-    return int64_t(page) * page_stride + int64_t(n % page_size) * row_stride;
+    const int in_table = page_of(n), page = table[size_t(b) * max_blocks + in_table];
+    return int64_t(page) * page_stride + int64_t(n - in_table * page_size) * row_stride;
   }
 };
 
@@ -1532,30 +1534,33 @@ kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* _
 }
 
 // =====================================================================================================
-// In place, where a plane fits on chip: one CTA owns a plane -- one (sample, K or V, head, column part) --, gathers and
-// merges ALL of its output rows behind the first vision row into shared memory, synchronises, and stores them: no other
+// In place, where a plane fits on chip: one CTA owns a plane -- one (sample, K or V, head, column part) --, copies ALL of
+// its rows from the first vision row on into shared memory, synchronises, and stores the merged and moved rows: no other
 // CTA touches these bytes, so nothing is overwritten before it has been read, and one kernel does what the two below
-// need a pass over memory more for.  The group lists and the rows' offsets (a block-table lookup each) are staged once
-// per CTA, so that the gather is one round of loads, eight in flight per thread.  Columns are cut so that the launch has
-// two CTAs per SM, in parts of at least 64 bytes (32 where the rows would not fit otherwise).
-// 4 samples x 652 tokens, 8 KV heads x 128, pages of 16: 28 -> 18 us between events against merge + move; parts of 32
-// or 128 bytes 28 and 27 (with the first form of the gather; parts of 64: 22).  Members are taken two at a time over
-// four pieces: one piece after the other, the largest group of a warp was a chain of loads (22 us).
+// need a pass over memory more for.
+// Bound by latency: the rows' addresses need no group lists (only a block table's part of the sample), so rows and lists
+// are asked for at once (cp.async) and a plane is three round trips: counts and table, rows, stores.  In gather mode, where
+// only the survivors' rows are read, the lists are a round trip of their own.  Columns are cut so that the launch has
+// two CTAs per SM, in parts of at least 64 bytes (less where the rows would not fit otherwise).  A plane that leaves room
+// for a second CTA on the SM gets 512 threads, one that does not 1024.
+// us a call in a row of them, against gathering the merged rows into shared memory through the staged lists (which took
+// up to ten round trips for the largest groups): 4 samples x 652 tokens, 8 KV heads x 128, pages of 16 15.4 -> 8.9; up
+// to 16 x 624 x 8 x 64 packed 19.5 -> 12.4; 576 x 32 x 128 13.5 -> 8.2; 2304 x 8 x 128 24 -> 15; 5328 x 8 x 128 40 -> 18;
+// 8 x 3008 x 32 x 128 351 -> 207 (with 512 threads 289).  The two kernels below take 21.3, 22.8, 20.6, 24.5, 25 and 238.
+// 256 threads 12, 1024 13 in the first, where two CTAs of 512 fit.
 // =====================================================================================================
-constexpr int KVI_THREADS = 256, KVI_AHEAD = 4;
-
 struct KvPlaneSmem {
-  int rows_in, rows_out, n_in, n_out;          // capacities: moving rows in / out, vision tokens in / out
-  __host__ __device__ size_t addr() const { return 0; }
-  __host__ __device__ size_t mem() const { return size_t(rows_in) * 8; }
+  int rows_in, n_in, n_out, blocks;            // capacities: moving rows in, vision tokens in / out, pages of the moving rows
+  __host__ __device__ size_t mem() const { return 0; }
   __host__ __device__ size_t wgt() const { return mem() + size_t(n_in) * 4; }
   __host__ __device__ size_t off() const { return wgt() + size_t(n_in) * 4; }
-  __host__ __device__ size_t out() const { return (off() + size_t(n_out + 1) * 4 + 15) & ~size_t(15); }
-  __host__ __device__ size_t bytes(int pieces) const { return out() + size_t(rows_out) * pieces * 16; }
+  __host__ __device__ size_t blk() const { return off() + size_t(n_out + 1) * 4; }
+  __host__ __device__ size_t rows() const { return (blk() + size_t(blocks) * 4 + 15) & ~size_t(15); }
+  __host__ __device__ size_t bytes(int pieces) const { return rows() + size_t(rows_in) * pieces * 16; }
 };
 
-template <typename T>
-__global__ void __launch_bounds__(KVI_THREADS)
+template <typename T, int THREADS>
+__global__ void __launch_bounds__(THREADS)
 kv_plane_kernel(T* __restrict__ k_buf, T* __restrict__ v_buf, KvAddr ad, KvPlaneSmem sm, int n_kv_heads, int ch, int parts,
                 unsigned magic_ch, int vis_begin, int n_text_after, int gather, const int* __restrict__ n_vis,
                 const int* __restrict__ n_vis_out, const int* __restrict__ grp_off, const int* __restrict__ grp_src,
@@ -1563,88 +1568,83 @@ kv_plane_kernel(T* __restrict__ k_buf, T* __restrict__ v_buf, KvAddr ad, KvPlane
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int V = Vec<T>::n;
-  int64_t* addr = reinterpret_cast<int64_t*>(smem_raw + sm.addr());     // element offset of every row from the first vision row on
   int* mem = reinterpret_cast<int*>(smem_raw + sm.mem());               // group members, survivor first
-  float* wgt = reinterpret_cast<float*>(smem_raw + sm.wgt());           // their weights
+  float* wgt = reinterpret_cast<float*>(smem_raw + sm.wgt());           // weights of the tokens
   int* off = reinterpret_cast<int*>(smem_raw + sm.off());               // first member of every output row
-  uint4* rows = reinterpret_cast<uint4*>(smem_raw + sm.out());
+  int* blk = reinterpret_cast<int*>(smem_raw + sm.blk());               // pages of the moving rows
+  const uint4* rows = reinterpret_cast<const uint4*>(smem_raw + sm.rows());
+  const uint32_t s_rows = tc::smem_u32(rows);
   const int tid = threadIdx.x;
   int plane = blockIdx.x;
   const int part = plane % parts; plane /= parts;
   const int h = plane % n_kv_heads; plane /= n_kv_heads;
   const int kv = plane & 1, b = plane >> 1;
-  const int n_in = n_vis ? min(n_vis[b], sm.n_in) : sm.n_in;
-  const int n_out = n_vis_out[b];
-  if (n_out >= n_in) return;                               // nothing was merged away: every row is where it belongs
+  const int row0 = vis_begin + (ad.seq_start ? ad.seq_start[b] : 0), page0 = ad.table ? ad.page_of(row0) : 0;
+  const int n_out = n_vis_out[b], n_in = n_vis ? min(n_vis[b], sm.n_in) : sm.n_in;
+  if (ad.table)
+    for (int j = tid; j < sm.blocks; j += THREADS)
+      if (page0 + j < ad.max_blocks) tc::cp_async4(tc::smem_u32(blk + j), ad.table + size_t(b) * ad.max_blocks + page0 + j);
+  tc::cp_async_commit();
+  for (int o = tid; o <= sm.n_out; o += THREADS) tc::cp_async4(tc::smem_u32(off + o), grp_off + size_t(b) * (sm.n_out + 1) + o);
+  for (int k = tid; k < sm.n_in; k += THREADS) {       // (lists that a short sample does not fill are never read)
+    tc::cp_async4(tc::smem_u32(mem + k), grp_src + size_t(b) * sm.n_in + k);
+    if (!gather) tc::cp_async4(tc::smem_u32(wgt + k), weight + size_t(b) * sm.n_in + k);
+  }
+  tc::cp_async_commit();
   T* buf = (kv ? v_buf : k_buf) + int64_t(h) * ad.head_stride + part * ch * V;
-
-  for (int l = tid; l < n_in + n_text_after; l += KVI_THREADS) addr[l] = ad.token(b, vis_begin + l);
-  for (int o = tid; o <= n_out; o += KVI_THREADS) off[o] = grp_off[size_t(b) * (sm.n_out + 1) + o];
-  for (int k = tid; k < n_in; k += KVI_THREADS) {          // (a sample cut at its capacity has fewer: never read)
-    const int i = min(max(grp_src[size_t(b) * sm.n_in + k], 0), n_in - 1);
-    mem[k] = i;
-    if (!gather) wgt[k] = weight[size_t(b) * sm.n_in + i];
+  auto at = [&](int l) -> T* {                             // the plane's part of row l behind the first vision row
+    const int n = row0 + l;
+    if (!ad.table) return buf + int64_t(b) * ad.batch_stride + int64_t(n) * ad.row_stride;
+    const int page = ad.page_of(n);
+    return buf + int64_t(blk[page - page0]) * ad.page_stride + int64_t(n - page * ad.page_size) * ad.row_stride;
+  };
+  if (ad.table || gather) {
+    if (gather) tc::cp_async_wait<0>(); else tc::cp_async_wait<1>();
+    __syncthreads();
   }
-  __syncthreads();
-
-  const int total = (n_out + n_text_after) * ch;
-  for (int i0 = tid; i0 < total; i0 += KVI_AHEAD * KVI_THREADS) {
-    int first[KVI_AHEAD], count[KVI_AHEAD], col[KVI_AHEAD], most = 0;
-    float acc[KVI_AHEAD][V];
-#pragma unroll
-    for (int u = 0; u < KVI_AHEAD; ++u) {
-      const int idx = i0 + u * KVI_THREADS, r = div_magic(idx, magic_ch);
-      col[u] = (idx - r * ch) * V;
-      count[u] = 0;
-      if (idx < total) {
-        const bool group = r < n_out;
-        first[u] = group ? off[r] : -(n_in + r - n_out);     // a row behind the vision block is negative (or row 0)
-        count[u] = group && !gather ? off[r + 1] - first[u] : 1;
-        if (group && count[u] == 1) first[u] = -mem[first[u]];
-      }
-      most = max(most, count[u]);
-#pragma unroll
-      for (int j = 0; j < V; ++j) acc[u][j] = 0.f;
-    }
-    for (int g = 0; g < most; g += 2) {
-      uint4 v[KVI_AHEAD][2];
-#pragma unroll
-      for (int u = 0; u < KVI_AHEAD; ++u)
-#pragma unroll
-        for (int m = 0; m < 2; ++m)
-          if (g + m < count[u]) v[u][m] = ld_plane16(buf + addr[count[u] == 1 ? -first[u] : mem[first[u] + g + m]] + col[u]);
-#pragma unroll
-      for (int u = 0; u < KVI_AHEAD; ++u) {
-        if (count[u] == 1) {
-          if (g == 0) rows[i0 + u * KVI_THREADS] = v[u][0];
-        } else {
-#pragma unroll
-          for (int m = 0; m < 2; ++m)
-            if (g + m < count[u]) {
-              float f[V];
-              unpack16(v[u][m], f, T());
-              const float w = wgt[first[u] + g + m];
-#pragma unroll
-              for (int j = 0; j < V; ++j) acc[u][j] = fmaf(w, f[j], acc[u][j]);
-            }
-        }
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < KVI_AHEAD; ++u)
-      if (count[u] > 1) rows[i0 + u * KVI_THREADS] = pack16(acc[u], T());
+  auto member = [&](int k) { return (int)min((unsigned)mem[k], (unsigned)(n_in - 1)); };
+  if (n_out >= n_in) {                                     // nothing was merged away: every row is where it belongs
+    tc::cp_async_wait<0>();
+    return;
   }
-  __syncthreads();                                         // every source of the plane has been read
+  const int total = (n_out + n_text_after) * ch, staged = gather ? total : (n_in + n_text_after) * ch;
 #pragma unroll 4
-  for (int idx = tid; idx < total; idx += KVI_THREADS) {
+  for (int idx = tid; idx < staged; idx += THREADS) {
     const int r = div_magic(idx, magic_ch), c = idx - r * ch;
-    const uint4 v = rows[idx];
-    st_stream16(buf + addr[r] + c * V, v);
-    // a merged group also replaces its survivor's row where that lies behind the new end, as the two-phase form leaves it
-    if (r < n_out && !gather && off[r + 1] - off[r] > 1) {
-      const int s = mem[off[r]];
-      if (s >= n_out + n_text_after) st_stream16(buf + addr[s] + c * V, v);
+    const int l = !gather ? r : r < n_out ? member(off[r]) : r - n_out + n_in;
+    tc::cp_async16(s_rows + uint32_t(idx) * 16, at(l) + c * V, 16);
+  }
+  tc::cp_async_commit();
+  tc::cp_async_wait<0>();
+  __syncthreads();                                         // every source of the plane has been read
+#pragma unroll 2
+  for (int idx = tid; idx < total; idx += THREADS) {
+    const int r = div_magic(idx, magic_ch), c = idx - r * ch;
+    uint4 v;
+    if (gather || r >= n_out) {
+      v = rows[gather ? idx : idx + (n_in - n_out) * ch];
+    } else {
+      const int g0 = off[r], count = off[r + 1] - g0, first = member(g0);
+      v = rows[first * ch + c];
+      if (count > 1) {
+        float acc[V], f[V];
+        unpack16(v, f, T());
+        float w = wgt[first];
+#pragma unroll
+        for (int j = 0; j < V; ++j) acc[j] = fmaf(w, f[j], 0.f);
+        for (int g = 1; g < count; ++g) {
+          const int i = member(g0 + g);
+          unpack16(rows[i * ch + c], f, T());
+          w = wgt[i];
+#pragma unroll
+          for (int j = 0; j < V; ++j) acc[j] = fmaf(w, f[j], acc[j]);
+        }
+        v = pack16(acc, T());
+        // the merged group also replaces its survivor's row where that lies behind the new end, as the two-phase form leaves it
+        if (first >= n_out + n_text_after) st_stream16(at(first) + c * V, v);
+      }
     }
+    st_stream16(at(r) + c * V, v);
   }
 }
 
@@ -1715,10 +1715,13 @@ kv_move_kernel(T* __restrict__ k_buf, T* __restrict__ v_buf, KvAddr ad, int n_kv
 
 cudaError_t launch_kv_compact(const KvLaunch& K) {
   const lightkv_kv_args_t* a = K.a;
+  // n * ceil(2^32 / d) >> 32 is n / d while n * d < 2^32 (the multiplier is less than 1 / d too large); d = 1: 2^32 does not fit
+  const long long page = a->page_size;
+  const unsigned magic_page = page > 1 && page < 65536 && a->max_blocks * page * page < (1ll << 32) ? (unsigned)(((1ull << 32) + page - 1) / page) : 0;
   KvAddr sa{a->src_batch_stride, a->src_head_stride, a->src_row_stride, a->src_page_stride,
-            a->page_size > 0 ? a->src_block_table : nullptr, a->page_size, a->max_blocks, a->src_seq_start};
+            a->page_size > 0 ? a->src_block_table : nullptr, a->page_size, a->max_blocks, a->src_seq_start, magic_page};
   KvAddr da{a->dst_batch_stride, a->dst_head_stride, a->dst_row_stride, a->dst_page_stride,
-            a->page_size > 0 ? a->dst_block_table : nullptr, a->page_size, a->max_blocks, a->dst_seq_start};
+            a->page_size > 0 ? a->dst_block_table : nullptr, a->page_size, a->max_blocks, a->dst_seq_start, magic_page};
   const int ch_host = K.head_dim * (K.dtype == LIGHTKV_BF16 ? 2 : 4) / 16;
   if (2 * K.n_kv_heads * ch_host >= 65536) return cudaErrorInvalidValue;      // range of the unit decode
   const unsigned magic_ch = (unsigned)(((1ull << 32) + ch_host - 1) / ch_host);
@@ -1735,18 +1738,23 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
     cudaError_t e = cudaSuccess;
     if (in_place) {
       // planes: (sample, K / V, head, column part); see kv_plane_kernel for the cut
-      const KvPlaneSmem sm{K.cap_in + a->n_text_after, K.cap_out + a->n_text_after, K.cap_in, K.cap_out};
+      const int moving = K.cap_in + a->n_text_after;
+      const KvPlaneSmem sm{moving, K.cap_in, K.cap_out, a->page_size > 0 ? (moving + a->page_size - 1) / a->page_size + 1 : 0};
       const long long planes = 2ll * K.batch * K.n_kv_heads;
       int p = 1;
       while (ch_host % (2 * p) == 0 && ch_host / p >= 4 &&
-             (sm.bytes(ch_host / p) > 100 * 1024 || (planes * p < 2 * sms && ch_host / p >= 8))) p *= 2;
+             (sm.bytes(ch_host / p) > 220 * 1024 || (planes * p < 2 * sms && ch_host / p >= 8))) p *= 2;
       const int ch = ch_host / p;
-      if (sm.bytes(ch) <= 220 * 1024 && (long long)sm.rows_out * ch < 65536) {
-        if ((e = ensure_dynamic_smem(kv_plane_kernel<T>, 220 * 1024)) != cudaSuccess) return e;
-        return launch_kernel(kv_plane_kernel<T>, dim3((unsigned)(planes * p)), KVI_THREADS, sm.bytes(ch), K.stream, 1,
-            static_cast<T*>(a->k_dst), static_cast<T*>(a->v_dst), da, sm, K.n_kv_heads, ch, p,
-            (unsigned)(((1ull << 32) + ch - 1) / ch), a->vis_begin, a->n_text_after, gather, a->n_vis, a->n_vis_out,
-            a->grp_off, a->grp_src, a->weight);
+      if (sm.bytes(ch) <= 220 * 1024 && (long long)moving * ch < 65536) {
+        auto launch = [&](auto kernel, int threads) -> cudaError_t {
+          const cudaError_t rc = ensure_dynamic_smem(kernel, 220 * 1024);
+          if (rc != cudaSuccess) return rc;
+          return launch_kernel(kernel, dim3((unsigned)(planes * p)), threads, sm.bytes(ch), K.stream, 1,
+              static_cast<T*>(a->k_dst), static_cast<T*>(a->v_dst), da, sm, K.n_kv_heads, ch, p,
+              (unsigned)(((1ull << 32) + ch - 1) / ch), a->vis_begin, a->n_text_after, gather, a->n_vis, a->n_vis_out,
+              a->grp_off, a->grp_src, a->weight);
+        };
+        return sm.bytes(ch) <= 110 * 1024 ? launch(kv_plane_kernel<T, 512>, 512) : launch(kv_plane_kernel<T, 1024>, 1024);
       }
     }
     if (!(in_place && gather))                            // in place, gather mode has nothing to merge

@@ -820,3 +820,50 @@ def test_weights_of_samples_with_a_token_per_cta():
     wl = S.Workload(name="few", config_id=143, batch=3, tiles=((2, 4),), n_text=9, hidden=64, n_q_heads=4,
                     n_kv_heads=4, head_dim=64, n_layers=16, layers=(3,), windows=(1,), keep=(0.5,))
     H.run_schedule(wl, kv_stream=torch.cuda.Stream())
+@pytest.mark.parametrize("grid,n_kv,head_dim,page,vb,after", [
+    ((9, 7), 2, 8, 1, 0, 0),           # pages of one row (their index is divided, not multiplied)
+    ((24, 24), 2, 24, 7, 13, 5),       # rows of three pieces, the first page begins in front of the vision block
+    ((24, 24), 3, 128, 48, 47, 1),
+    ((48, 48), 2, 128, 16, 5, 40),     # one CTA per SM
+    ((24, 24), 2, 64, 70000, 3, 2),    # a page longer than the multiplier's range
+])
+@pytest.mark.parametrize("dtype,mode", [("bf16", "merge"), ("fp32", "merge"), ("bf16", "gather")])
+def test_in_place_pages_equal_contiguous_bit_for_bit(grid, n_kv, head_dim, page, vb, after, dtype, mode):
+    import torch
+    import paper_2605_00789_b200 as L
+    b, n = 2, grid[0] * grid[1]
+    plan = L.Plan(b, 64, n_kv, n_kv, head_dim, 8, [grid], [3], [2], [0.55], vb + after,
+                  dtype=L.BF16 if dtype == "bf16" else L.FP32, xi_mode=L.XI_GIVEN)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    gen = torch.Generator(device="cuda").manual_seed(7)
+    rows = vb + n + after
+    hidden = torch.randn((b, rows, 64), generator=gen, device="cuda").to(dt)
+    out = L.StageBuffers(plan, 0, vb + plan.stage_info(0).cap_out + after)
+    L.compress_layer(plan, 0, hidden, out, vis_begin=vb, n_text_after=after,
+                     xi=torch.rand((b, n), generator=gen, device="cuda") + 0.1)
+    m = L.KV_MERGE if mode == "merge" else L.KV_GATHER
+    k, v = (torch.randn((b, n_kv, rows, head_dim), generator=gen, device="cuda").to(dt) for _ in range(2))
+    kd, vd = torch.zeros_like(k), torch.zeros_like(v)
+    L.compact_kv(plan, 0, out, k, v, kd, vd, vis_begin=vb, n_text_after=after, mode=m)
+    blocks = -(-rows // page)
+    table = torch.randperm(b * blocks, generator=gen, device="cuda").view(b, blocks).int()
+
+    def pool(x):
+        full = torch.zeros((b, n_kv, blocks * page, head_dim), device="cuda", dtype=dt)
+        full[:, :, :rows] = x
+        p = torch.empty((b * blocks, n_kv, page, head_dim), device="cuda", dtype=dt)
+        p[table.reshape(-1).long()] = full.view(b, n_kv, blocks, page, head_dim).transpose(1, 2).reshape(p.shape)
+        return p
+
+    kp, vp = pool(k), pool(v)
+    L.compact_kv(plan, 0, out, kp, vp, kp, vp, vis_begin=vb, n_text_after=after, mode=m, page_size=page,
+                 src_block_table=table, dst_block_table=table)
+    L.compact_kv(plan, 0, out, k, v, k, v, vis_begin=vb, n_text_after=after, mode=m)
+    counts = out.n_vis_out.tolist()
+    for want, paged, flat in ((kd, kp, k), (vd, vp, v)):
+        got = paged[table.reshape(-1).long()].view(b, blocks, n_kv, page, head_dim).transpose(1, 2).reshape(b, n_kv, -1, head_dim)
+        for i in range(b):
+            end = vb + counts[i] + after
+            assert torch.equal(got[i, :, :end], want[i, :, :end])
+            assert torch.equal(flat[i, :, :end], want[i, :, :end])
+    plan.close()
