@@ -75,8 +75,12 @@ struct FdStreamSmem {
   }
 };
 
+// CTAs of eight warps an SM holds, by O (bf16).  Without the bound the compiler takes 156 registers for O = 5, one CTA per SM:
+// 128 CTAs in clusters of eight then take two turns (4 x 345 tokens x 4096 in windows of 72: 22.5 -> 16.0 us).
+__host__ __device__ constexpr int fd_min_ctas(int o) { return o <= 2 ? 4 : o == 5 ? 2 : 0; }
+
 template <typename T, int O, int S, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS) fd_stream_kernel(const __grid_constant__ FdStreamArgs a) {
+__global__ void __launch_bounds__(32 * WARPS, WARPS == 8 && sizeof(T) == 2 ? fd_min_ctas(O) : 0) fd_stream_kernel(const __grid_constant__ FdStreamArgs a) {
   grid_dependency_wait();
   grid_launch_dependents();                              // in this order: see grid_dependency_sync
   using M = FdStreamSmem<O, S, WARPS>;
@@ -349,10 +353,11 @@ cudaError_t launch_fd_stream(const LayerLaunch& L) {
   f.d = L.hidden; f.metric = L.divergence; f.keep = L.keep; f.g = L.geo; f.n_vis = a->n_vis; f.pos = a->pos;
   f.cap_in = L.ws.cap_in; f.max_cell = L.max_cell; f.partner = L.ws.partner; f.place = L.ws.slot;
   // chunks in flight per warp (S): as few as still leave enough CTAs on an SM; with more, fewer CTAs fit and the
-  // start and end of a window are less covered (contraction alone: S = 8, 6, 4 39 / 33 / 25 us, 6, 4, 3 37 / 27 / 23)
+  // start and end of a window are less covered (contraction alone: S = 8, 6, 4 39 / 33 / 25 us, 6, 4, 3 37 / 27 / 23; O = 2
+  // with S = 4 and three CTAs per SM 1 to 3 us more a pass of 8 x 2880 tokens than S = 3 and four)
   switch ((L.fd_side + 7) / 8) {
     case 1: return launch_fd_stream_w<1, 6>(L, f);
-    case 2: return launch_fd_stream_w<2, 4>(L, f);
+    case 2: return launch_fd_stream_w<2, 3>(L, f);
     case 3: return launch_fd_stream_w<3, 3>(L, f);
     case 4: return launch_fd_stream_w<4, 2>(L, f);
     default: return launch_fd_stream_w<5, 2>(L, f);
