@@ -867,3 +867,26 @@ def test_in_place_pages_equal_contiguous_bit_for_bit(grid, n_kv, head_dim, page,
             assert torch.equal(got[i, :, :end], want[i, :, :end])
             assert torch.equal(flat[i, :, :end], want[i, :, :end])
     plan.close()
+
+
+@pytest.mark.parametrize("grid,windows,batch", [((64, 64), 1, 1), ((48, 48), 2, 2), ((24, 24), 2, 1), ((256, 32), 4, 2)])
+def test_scores_near_the_ends_of_the_norms_range(grid, windows, batch):
+    # rows scaled by a power of two have the same cosines bit for bit; the tiled FD kernel compares them without a division
+    # where all norms of a tile are between 1e-15 and 1e15, with and without clusters, and pair by pair elsewhere
+    import torch
+    import paper_2605_00789_b200 as L
+    n = grid[0] * grid[1]
+    plan = L.Plan(batch, 256, 2, 2, 64, 8, [grid], [3], [windows], [0.6], 4, xi_mode=L.XI_UNIFORM)
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    rows = torch.randn((batch, 4 + n, 256), generator=gen, device="cuda").to(torch.bfloat16)
+    rows[:, 4 + 7] = 0
+    mixed = torch.ones((4 + n, 1), device="cuda")
+    mixed[4 + 13::57] = 2.0 ** -60
+    found = []
+    for scale in (1.0, 2.0 ** -60, 2.0 ** 52, mixed):
+        out = L.StageBuffers(plan, 0, 4 + plan.stage_info(0).cap_out)
+        L.compress_layer(plan, 0, (rows.float() * scale).to(torch.bfloat16), out, vis_begin=4)
+        found.append(out.dst.cpu())
+    for other in found[1:]:
+        assert torch.equal(found[0], other)
+    plan.close()
