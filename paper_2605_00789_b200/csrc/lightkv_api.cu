@@ -78,7 +78,8 @@ static void layout_workspace(const lightkv_plan_t& p, StagePlan& s) {
   o.a_partner = place(B * s.cap_a * 4);
   s.ws_list = end;
   end = forms;
-  o.tile_key = place(by_token ? B * s.fd_blocks * s.cap_in * 8 : 0);
+  // (at least a key per token and block: which calls fit a workspace of a given size does not depend on how keys are numbered)
+  o.tile_key = place(by_token ? B * s.fd_blocks * std::max(size_t(s.cap_in), s.n_windows * size_t((s.max_cell + 1) / 2)) * 8 : 0);
   o.win_tok = place(by_token ? B * s.n_windows * (size_t(s.max_cell) + 1) * 4 : 0);
   s.ws_tiled = end;
   s.ws_bytes = std::max(s.ws_list, s.ws_tiled);

@@ -76,11 +76,15 @@ struct FdStreamSmem {
 };
 
 // CTAs of eight warps an SM holds, by O (bf16).  Without the bound the compiler takes 156 registers for O = 5, one CTA per SM:
-// 128 CTAs in clusters of eight then take two turns (4 x 345 tokens x 4096 in windows of 72: 22.5 -> 16.0 us).
-__host__ __device__ constexpr int fd_min_ctas(int o) { return o <= 2 ? 4 : o == 5 ? 2 : 0; }
+// 128 CTAs in clusters of eight then take two turns (4 x 345 tokens x 4096 in windows of 72: 22.5 -> 16.0 us).  O = 3 takes 114
+// by itself, 112 with a bound for nine warps: with more the CTAs do not fit beside those of the kernel in front (one image,
+// one layer: 27.5 us a pass with up to 112, 30.0 with 120).
+__host__ __device__ constexpr int fd_min_ctas(int o) { return o <= 2 ? 4 : o == 4 ? 0 : 2; }
+__host__ __device__ constexpr int fd_max_threads(bool bf16, int o, int warps) { return 32 * (bf16 && o == 3 && warps == 8 ? 9 : warps); }
 
 template <typename T, int O, int S, int WARPS>
-__global__ void __launch_bounds__(32 * WARPS, WARPS == 8 && sizeof(T) == 2 ? fd_min_ctas(O) : 0) fd_stream_kernel(const __grid_constant__ FdStreamArgs a) {
+__global__ void __launch_bounds__(fd_max_threads(sizeof(T) == 2, O, WARPS), WARPS == 8 && sizeof(T) == 2 ? fd_min_ctas(O) : 0)
+fd_stream_kernel(const __grid_constant__ FdStreamArgs a) {
   grid_dependency_wait();
   grid_launch_dependents();                              // in this order: see grid_dependency_sync
   using M = FdStreamSmem<O, S, WARPS>;

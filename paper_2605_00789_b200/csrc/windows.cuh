@@ -94,9 +94,11 @@ struct WindowLists {
   int* best;             // [max_src] destination that attains the lowest score, -1: none
   int* count;            // [max_dst] sources merged into a destination
   int* tok;              // [max_cell] token index by local rank
+  unsigned short* part;  // [kParts][max_dst] the same by eighths of the sources (windows of more than 128 sources)
+  static constexpr int kParts = 8;
   static __host__ __device__ size_t bytes(int max_cell) {
     const size_t src = (max_cell + 1) / 2;
-    return (2 * ((src + 7) & ~size_t(3)) + 2 * src + max_cell) * 4;
+    return (2 * ((src + 7) & ~size_t(3)) + 2 * src + max_cell + (src > 128 ? kParts / 2 * src : 0)) * 4;
   }
   __device__ static WindowLists at(void* p, int max_cell) {     // p: 16-byte aligned
     const int src = (max_cell + 1) / 2;
@@ -106,6 +108,7 @@ struct WindowLists {
     w.best = w.into + ((src + 7) & ~3);
     w.count = w.best + src;
     w.tok = w.count + src;
+    w.part = reinterpret_cast<unsigned short*>(w.tok + max_cell);
     return w;
   }
 };
@@ -119,68 +122,96 @@ __host__ __device__ inline int key_partner(unsigned long long key, int nb) {
 
 // Selection: the `removed` sources with the lowest (score, index) are merged into their best destination.  Writes every
 // token's partner and place (see Workspace).  key / best / tok are complete in shared memory (synchronised) on entry; all
-// threads take part.  A source's rank among the sources of its destination is counted by its own thread in windows of up
-// to 128 sources; in larger ones a warp walks the sources in order, 32 at a time (match_any gives the rank within the 32, a
-// counter per destination the ones before).
+// threads take part, in whole warps.  Bound by the length of a thread's walk over the other sources, so as many lanes share
+// a source as there are threads for (18 of 256: 8).  A source's rank among the sources of its destination is counted the
+// same way in windows of up to 128 sources; in larger ones eight warps walk an eighth of the sources each, 32 at a time
+// (match_any gives the rank within the 32, a counter per destination and eighth the ones before): 1024 sources 8.0 us with
+// one warp for all of them, 2.2 with eight.
 __device__ __forceinline__ void select_window(const WindowLists& s, int nw, int removed, int par, int* __restrict__ partner,
                                               int* __restrict__ place) {
-  const int tid = threadIdx.x, nthr = blockDim.x;
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5;
   const int na = (nw + 1 - par) >> 1, nb = nw - na;      // sources: local ranks of parity `par`
   const bool ranked = removed > 0 && removed < na;
+  int share = 1;                                         // lanes per source
+  while (share < 32 && 2 * share * na <= nthr) share *= 2;
+  const int mine0 = tid / share, step = nthr / share, sub = tid & (share - 1);
   if (ranked) {
     if (tid < 4) s.key[na + tid] = 0xffffffffu;          // the last group of four keys
     __syncthreads();
-  }
-  for (int e = tid; e < na; e += nthr) {
-    bool sel = removed >= na;
-    if (ranked) {
+    for (int e0 = 0; e0 < na; e0 += step) {
+      const int e = min(e0 + mine0, na - 1);             // (whole warps stay together)
       const unsigned int mine = s.key[e];
       int rank = 0;
-      for (int k = 0; k < na; k += 4) {
+      for (int k = 4 * sub; k < na; k += 4 * share) {
         const uint4 v = *reinterpret_cast<const uint4*>(s.key + k);
         rank += (v.x < mine) + (v.y < mine) + (v.z < mine) + (v.w < mine);
         if (k < e) rank += (v.x == mine) + (k + 1 < e && v.y == mine) + (k + 2 < e && v.z == mine) + (k + 3 < e && v.w == mine);
       }
-      sel = rank < removed;
+      for (int o = share >> 1; o > 0; o >>= 1) rank += __shfl_xor_sync(0xffffffffu, rank, o);
+      if (sub == 0) s.into[e] = rank < removed ? s.best[e] : -1;
     }
-    s.into[e] = sel ? s.best[e] : -1;
+  } else {
+    for (int e = tid; e < na; e += nthr) s.into[e] = removed >= na ? s.best[e] : -1;
   }
-  for (int e = tid; e < nb; e += nthr) s.count[e] = 0;
-  __syncthreads();
   if (na <= 128) {
-    for (int e = tid; e < na; e += nthr) {
-      const int to = s.into[e], i = s.tok[2 * e + par];
+    for (int e = tid; e < nb; e += nthr) s.count[e] = 0;
+    __syncthreads();
+    for (int e0 = 0; e0 < na; e0 += step) {
+      const int e = min(e0 + mine0, na - 1), to = s.into[e];
       int q = 0;
-      if (to >= 0) {
-        for (int k = 0; k < e; k += 4) {
+      if (to >= 0)
+        for (int k = 4 * sub; k < e; k += 4 * share) {
           const int4 v = *reinterpret_cast<const int4*>(s.into + k);
           q += (v.x == to) + (k + 1 < e && v.y == to) + (k + 2 < e && v.z == to) + (k + 3 < e && v.w == to);
         }
-        atomicAdd(&s.count[to], 1);
-      }
-      partner[i] = to < 0 ? -2 : s.tok[2 * to + 1 - par];
-      place[i] = q;
-    }
-  } else if (tid < 32) {
-    for (int base = 0; base < na; base += 32) {
-      const int e = base + tid, to = e < na ? s.into[e] : -1;
-      const unsigned int peers = __match_any_sync(0xffffffffu, to);
-      const int before = to >= 0 ? s.count[to] : 0;
-      __syncwarp();
-      if (to >= 0 && tid == __ffs(peers) - 1) s.count[to] = before + __popc(peers);
-      __syncwarp();
-      if (e < na) {
+      for (int o = share >> 1; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
+      if (sub == 0 && e0 + mine0 < na) {
         const int i = s.tok[2 * e + par];
+        if (to >= 0) atomicAdd(&s.count[to], 1);
         partner[i] = to < 0 ? -2 : s.tok[2 * to + 1 - par];
-        place[i] = to < 0 ? 0 : before + __popc(peers & ((1u << tid) - 1u));
+        place[i] = q;
       }
+    }
+    __syncthreads();
+    for (int e = tid; e < nb; e += nthr) {
+      const int i = s.tok[2 * e + 1 - par];
+      partner[i] = -1;
+      place[i] = s.count[e];
+    }
+    return;
+  }
+  const int parts = min(WindowLists::kParts, nthr >> 5), len = ((na + parts - 1) / parts + 31) & ~31;
+  for (int k = tid; k < parts * nb; k += nthr) s.part[k] = 0;
+  __syncthreads();
+  if (warp < parts) {
+    unsigned short* count = s.part + warp * nb;
+    for (int base = warp * len; base < min(na, (warp + 1) * len); base += 32) {
+      const int e = base + lane, to = e < na ? s.into[e] : -1;
+      const unsigned int peers = __match_any_sync(0xffffffffu, to);
+      const int before = to >= 0 ? count[to] : 0;
+      __syncwarp();
+      if (to >= 0 && lane == __ffs(peers) - 1) count[to] = (unsigned short)(before + __popc(peers));
+      __syncwarp();
+      if (e < na) s.best[e] = before + __popc(peers & ((1u << lane) - 1u));    // (its destination is in `into` by now)
     }
   }
   __syncthreads();
   for (int e = tid; e < nb; e += nthr) {
+    int run = 0;
+    for (int k = 0; k < parts; ++k) {
+      const int c = s.part[k * nb + e];
+      s.part[k * nb + e] = (unsigned short)run;
+      run += c;
+    }
     const int i = s.tok[2 * e + 1 - par];
     partner[i] = -1;
-    place[i] = s.count[e];
+    place[i] = run;
+  }
+  __syncthreads();
+  for (int e = tid; e < na; e += nthr) {
+    const int i = s.tok[2 * e + par], to = s.into[e];
+    partner[i] = to < 0 ? -2 : s.tok[2 * to + 1 - par];
+    place[i] = to < 0 ? 0 : s.part[e / len * nb + to] + s.best[e];
   }
 }
 

@@ -890,3 +890,12 @@ def test_scores_near_the_ends_of_the_norms_range(grid, windows, batch):
     for other in found[1:]:
         assert torch.equal(found[0], other)
     plan.close()
+
+
+@pytest.mark.parametrize("grid", [(1, 255), (1, 257), (1, 259), (3, 401), (1, 2049)])
+@pytest.mark.parametrize("direction", ["a2b", "b2a"])
+def test_selection_over_eighths_of_the_sources(grid, direction):
+    # one window; up to 128 sources are walked by their own threads, more by eight warps in turns of 32
+    wl = S.Workload(name="eighths", config_id=144, batch=1, tiles=(grid,), n_text=3, hidden=64, n_q_heads=2,
+                    n_kv_heads=2, head_dim=64, n_layers=16, layers=(3,), windows=(1,), keep=(0.6,))
+    H.run_schedule(wl, xi_mode="given", direction=direction)
