@@ -123,9 +123,9 @@ cudaError_t launch_fd_simt(const LayerLaunch& L);
 bool fd_stream_supported(int dtype, int fd_side);
 cudaError_t launch_fd_stream(const LayerLaunch& L);
 // merge map from the partners (Steps 4, 5), with `select` from the keys of launch_fd_tc, and the weights where xi is given or
-// uniform; at most kMapMaxTokens per sample
+// uniform, or complete because the launch stands behind the xi kernel; at most kMapMaxTokens per sample
 constexpr int kMapMaxTokens = 16384;
-cudaError_t launch_map(const LayerLaunch& L, bool select);
+cudaError_t launch_map(const LayerLaunch& L, bool select, bool behind_xi = false);
 // xi per head (Eq. "attention-factor"), fp32 FMA path; handles ATTN_FULL and ATTN_LSE.  wait_first: the stream's last kernel
 // is not one of the same call that lets the next start behind its own wait (FD, or the map behind it)
 cudaError_t launch_xi_simt(const LayerLaunch& L, bool wait_first);

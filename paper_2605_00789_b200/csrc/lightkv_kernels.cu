@@ -811,6 +811,8 @@ __device__ __forceinline__ float member_weight(float xi, float den, int size) {
 struct MapArgs {
   int xi_mode, cap_in, cap_out, cap_a, cap_b, n_grid;
   const float* xi_in;
+  const float* xi_h;                   // WEIGHTS, xi from attention: [B, cap_in, H]
+  int n_q_heads;
   const int* n_vis;
   const int* pos;
   int* partner;
@@ -828,6 +830,21 @@ struct MapArgs {
   float* xi_out;
   uint32_t* status;
 };
+
+// xi of one token: the sum over its heads
+__device__ __forceinline__ float token_xi(const float* x, int heads) {
+  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+  int h = 0;
+  if ((heads & 3) == 0) {                                   // (rows of four floats are 16-byte aligned)
+#pragma unroll 8
+    for (; h < heads; h += 4) {
+      const float4 v = *reinterpret_cast<const float4*>(x + h);
+      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+    }
+  }
+  for (; h < heads; ++h) s.x += x[h];
+  return (s.x + s.y) + (s.z + s.w);
+}
 
 template <bool CLUSTER, int TPT, bool SELECT, bool WEIGHTS>
 __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapArgs a) {
@@ -894,6 +911,7 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
     prt[j] = -1; plc[j] = 0; ps[j] = i; xi[j] = 1.0f;
     if (i < hi) {
       if (WEIGHTS && a.xi_mode == LIGHTKV_XI_GIVEN) xi[j] = a.xi_in[row + i];
+      if (WEIGHTS && a.xi_h) xi[j] = token_xi(a.xi_h + (row + i) * a.n_q_heads, a.n_q_heads);
       prt[j] = __ldcg(a.partner + row + i);
       plc[j] = __ldcg(a.place + row + i);
       if (a.pos) {
@@ -1046,12 +1064,11 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
   }
 }
 
-cudaError_t launch_map(const LayerLaunch& L, bool select) {
+cudaError_t launch_map(const LayerLaunch& L, bool select, bool behind_xi) {
   const lightkv_layer_args_t* a = L.a;
-  // xi from attention is not there yet
-  const bool weights = L.xi_mode == LIGHTKV_XI_GIVEN || L.xi_mode == LIGHTKV_XI_UNIFORM;
+  const bool attn = L.xi_mode == LIGHTKV_XI_ATTN_FULL || L.xi_mode == LIGHTKV_XI_ATTN_LSE, weights = !attn || behind_xi;
   MapArgs m;
-  m.xi_mode = L.xi_mode; m.xi_in = a->xi; m.weight = a->weight; m.xi_out = a->xi_out;
+  m.xi_mode = L.xi_mode; m.xi_in = a->xi; m.xi_h = attn ? L.ws.xi_h : nullptr; m.n_q_heads = L.n_q_heads; m.weight = a->weight; m.xi_out = a->xi_out;
   m.cap_in = L.ws.cap_in; m.cap_out = L.ws.cap_out;
   m.cap_a = L.ws.cap_a; m.cap_b = L.ws.cap_b; m.n_grid = L.n_grid;
   m.n_vis = a->n_vis; m.pos = a->pos; m.partner = L.ws.partner; m.place = L.ws.slot;
