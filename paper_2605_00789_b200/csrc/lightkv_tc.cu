@@ -309,9 +309,11 @@ xi_tc_kernel(const __grid_constant__ CUtensorMap q_map, const __grid_constant__ 
         const int bc = a.seq_start ? 0 : it.b;
         if (q_use > 0 && !mbar_wait(&q_empty[qb], (q_use - 1) & 1, abort_flag)) return false;
         mbar_expect_tx(&q_full[qb], TILE_BYTES);
+        // Q is read once; what stays in L2 instead is read again: K here and by the compaction, the hidden states by the merge
+        // (us a pass with a given log-sum-exp: 8 x 2880 tokens 507 -> 500, 4 x 576 104.6 -> 102.2)
 #pragma unroll
         for (int hf = 0; hf < HALVES; ++hf)
-          tma_load_4d(q_s + qb * TILE_BYTES + hf * 16384, &q_map, &q_full[qb], hf * 64, it.row0 + a.vis_begin + it.t0, it.h, bc);
+          tma_load_4d_once(q_s + qb * TILE_BYTES + hf * 16384, &q_map, &q_full[qb], hf * 64, it.row0 + a.vis_begin + it.t0, it.h, bc);
         ++nq_loaded;
         const int hk = it.h / a.group;
         for (int kt = 0; kt < nkt; ++kt, ++kf) {
