@@ -1304,6 +1304,7 @@ __global__ void __launch_bounds__(256, MB > 2 ? 3 : 5) merge_rows_kernel(const _
   if (count == 1) {                                     // copied
     const int i = text ? 0 : gs[0];
     const T* srow = sb + size_t(text ? (o < 0 ? row : row - n_out + n_in) : a.vis_begin + i) * a.src_rs;
+    float w = WEIGHTS || text ? 1.0f : wt[i];
     for (int c0 = tid; c0 < chunks; c0 += 2 * nthr) {
       const int c1 = c0 + nthr;
       const uint4 a0 = ld_stream16(srow + c0 * V);
@@ -1313,13 +1314,22 @@ __global__ void __launch_bounds__(256, MB > 2 ? 3 : 5) merge_rows_kernel(const _
       }
       st_stream16(orow + c0 * V, a0);
     }
-    if (WEIGHTS && !text && tid < 32) {
+    if (text) return;
+    if (WEIGHTS && tid < 32) {
       const float v = warp_xi(a.w, b, i, tid);
+      w = member_weight(v, v, 1);
       if (tid == 0) {
-        wt[i] = 1.0f;
+        wt[i] = w;
         if (xo) xo[i] = v;
         if (!(v >= 1e-30f)) set_status(a.w.status, LIGHTKV_STATUS_ZERO_WEIGHT);
       }
+    }
+    // an infinite xi leaves no number as its weight, nor as the row
+    if (WEIGHTS ? __syncthreads_or(w != w) : w != w) {
+      float none[V];
+#pragma unroll
+      for (int j = 0; j < V; ++j) none[j] = __int_as_float(0x7fffffff);
+      for (int c = tid; c < chunks; c += nthr) st_stream16(orow + c * V, pack16(none, T()));
     }
     return;
   }

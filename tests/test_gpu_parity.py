@@ -690,6 +690,44 @@ def test_weights_of_a_group_of_all_sources(grid, before_merge):
     plan.close()
 
 
+@pytest.mark.parametrize("xi_mode", ["given", "lse"])
+@pytest.mark.parametrize("before_merge", [False, True])
+def test_an_infinite_score_leaves_no_number(xi_mode, before_merge):
+    """xi / sum is inf / inf for a token whose score is infinite, alone or in a group: its weight and its row are NaN, and no
+    other group's are.  (A log-sum-exp of -200 overflows the exponentials of its row.)"""
+    import torch
+    import paper_2605_00789_b200 as L
+    n, nt = 144, 5
+    plan = L.Plan(1, 264, 4, 4, 64, 4, [(12, 12)], [2], [3], [0.55], nt, xi_mode=L.XI_GIVEN if xi_mode == "given" else L.XI_ATTN_LSE)
+    gen = torch.Generator(device="cuda").manual_seed(11)
+    rows = torch.randn((1, nt + n, 264), generator=gen, device="cuda").bfloat16()
+    kw = {}
+    if xi_mode == "given":
+        kw["xi"] = 0.5 + torch.rand((1, n), generator=gen, device="cuda")
+        kw["xi"][:, ::7] = float("inf")
+    else:
+        kw["q"], kw["k"] = (torch.randn((1, 4, nt + n, 64), generator=gen, device="cuda").bfloat16() for _ in range(2))
+        kw["lse"] = torch.full((1, 4, nt + n), 3.0, device="cuda")
+        kw["lse"][:, :, nt::7] = -200.0
+    if before_merge:
+        kw["map_event"] = torch.cuda.Event()
+        kw["map_event"].record()
+    out = L.StageBuffers(plan, 0, nt + plan.stage_info(0).cap_out, "cuda")
+    L.compress_layer(plan, 0, rows, out, vis_begin=nt, **kw)
+    inf = ~torch.isfinite(out.xi_out[0])
+    assert torch.equal(inf.nonzero()[:, 0].cpu(), torch.arange(0, n, 7)) and bool((out.xi_out[0][inf] > 0).all())
+    assert torch.equal(torch.isnan(out.weight[0]), inf)
+    off, src = out.grp_off[0].cpu(), out.grp_src[0].cpu()
+    kinds = set()
+    for o in range(int(out.n_vis_out)):
+        members = src[off[o]:off[o + 1]].long()
+        bad = bool(inf.cpu()[members].any())
+        assert torch.isnan(out.hidden_out[0, nt + o]).all() if bad else torch.isfinite(out.hidden_out[0, nt + o]).all()
+        kinds.add((bad, len(members) > 1))
+    assert len(kinds) == 4
+    plan.close()
+
+
 @pytest.mark.parametrize("before_merge", [False, True])
 def test_xi_of_tokens_cut_at_the_capacity_is_reported(before_merge):
     """A subset under a full-grid plan keeps all of its tokens and is cut at cap_out: those behind the cut belong to no group,
@@ -820,6 +858,8 @@ def test_weights_of_samples_with_a_token_per_cta():
     wl = S.Workload(name="few", config_id=143, batch=3, tiles=((2, 4),), n_text=9, hidden=64, n_q_heads=4,
                     n_kv_heads=4, head_dim=64, n_layers=16, layers=(3,), windows=(1,), keep=(0.5,))
     H.run_schedule(wl, kv_stream=torch.cuda.Stream())
+
+
 @pytest.mark.parametrize("grid,n_kv,head_dim,page,vb,after", [
     ((9, 7), 2, 8, 1, 0, 0),           # pages of one row (their index is divided, not multiplied)
     ((24, 24), 2, 24, 7, 13, 5),       # rows of three pieces, the first page begins in front of the vision block
