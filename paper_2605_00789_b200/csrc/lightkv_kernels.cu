@@ -1278,8 +1278,10 @@ struct MergeArgs {
   WeightArgs w;
 };
 
+// Registers: with the weights the form for many rows spills at five CTAs per SM (4 x 652 rows of 4096, a pass: 103.9 us; with
+// four 100.7).
 template <typename T, int MB, bool WEIGHTS>
-__global__ void __launch_bounds__(256, MB > 2 ? 3 : 5) merge_rows_kernel(const __grid_constant__ MergeArgs<T> a) {
+__global__ void __launch_bounds__(256, MB > 2 ? 3 : WEIGHTS ? 4 : 5) merge_rows_kernel(const __grid_constant__ MergeArgs<T> a) {
   grid_dependency_sync();
   constexpr int V = Vec<T>::n;
   constexpr int AHEAD = 64;                             // members whose weights stay on chip
