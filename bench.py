@@ -65,10 +65,10 @@ def count_launches(step):
 # dram__bytes_read.sum + dram__bytes_write.sum per launch from the committed ncu captures (profiles/),
 # of the stage-0 launch, keyed by (workload, kernel); null where no capture exists.
 NCU_TRAFFIC_BYTES = {
-    ("cfg2", "xi"): 400.71e6,                # profiles/xi_tc_kernel_cfg2_stage0.txt
-    ("cfg2", "fd_best_partner"): 193.16e6,   # profiles/fd_stream_kernel_cfg2_stage0.txt
-    ("cfg2", "merge_hidden"): 262.91e6,      # profiles/merge_rows_kernel_cfg2_stage0.txt
-    ("cfg2", "kv_compact"): 562.67e6,        # profiles/kv_compact_kernel_cfg2_stage0.txt
+    ("cfg2", "xi"): 392.11e6,                # profiles/xi_tc_kernel_cfg2_stage0.txt
+    ("cfg2", "fd_best_partner"): 193.33e6,   # profiles/fd_stream_kernel_cfg2_stage0.txt
+    ("cfg2", "merge_hidden"): 263.62e6,      # profiles/merge_rows_kernel_cfg2_stage0.txt
+    ("cfg2", "kv_compact"): 563.52e6,        # profiles/kv_compact_kernel_cfg2_stage0.txt
 }
 
 
@@ -466,7 +466,7 @@ def main():
     for _ in range(args.warmup):
         run_step(L, plan, wl, stages, side=side, aux=aux)
 
-    # The step's launches (five kernels a stage on three streams) are captured once into a CUDA graph and replayed:
+    # The step's launches (six kernels a stage on three streams) are captured once into a CUDA graph and replayed:
     # the library's calls are plain stream work, so the caller may do that.  Plumbing only; if the capture is
     # refused the step is launched call by call and the JSON says so.
     step_graph = None
