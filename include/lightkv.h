@@ -185,7 +185,8 @@ typedef struct {
   const int32_t* pos;              /* DEVICE [B, cap_in] original flat grid positions, strictly
                                       ascending per sample; NULL = 0..n-1 (stage 0, full grid) */
 
-  int32_t* n_vis_out;              /* DEVICE [B] */
+  int32_t* n_vis_out;              /* DEVICE [B]; may be the array n_vis where n_text_after is 0 (the rows behind are found
+                                      by the count that came in; so is what lightkv_compact_kv has to move) */
   int32_t* pos_out;                /* DEVICE [B, cap_out] */
   /* the merge map of the stage */
   int32_t* dst;                    /* DEVICE [B, cap_in]   output slot of every input vision token */

@@ -126,6 +126,8 @@ cudaError_t launch_fd_stream(const LayerLaunch& L);
 // uniform, or complete because the launch stands behind the xi kernel; at most kMapMaxTokens per sample
 constexpr int kMapMaxTokens = 16384;
 cudaError_t launch_map(const LayerLaunch& L, bool select, bool behind_xi = false);
+// whether, with xi from attention, the map stands behind the xi kernel and not beside it
+bool map_behind_xi(const LayerLaunch& L);
 // xi per head (Eq. "attention-factor"), fp32 FMA path; handles ATTN_FULL and ATTN_LSE.  wait_first: the stream's last kernel
 // is not one of the same call that lets the next start behind its own wait (FD, or the map behind it)
 cudaError_t launch_xi_simt(const LayerLaunch& L, bool wait_first);

@@ -363,10 +363,8 @@ int compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* a, bool 
   auto launch_fd = [&](const LayerLaunch& l) {
     return streaming ? launch_fd_stream(l) : tc_fd && near ? launch_fd_tc(l, !tiled) : launch_fd_simt(l);
   };
-  // The map behind the FD kernels that hold whole windows needs no xi; the list form's does.  Where the caller waits for the
-  // map alone and the launch is short, one kernel behind xi makes map and weights: the map beside xi would save less than the
-  // second kernel costs (2 x 798 tokens x 32 heads, three stages with a given log-sum-exp: 162 us a pass against 169).
-  const bool in_map = streaming || tiled, late_map = in_map && attn && a->map_event && merge_takes_weights(L);
+  // The map behind the FD kernels that hold whole windows needs no xi; the list form's does.
+  const bool in_map = streaming || tiled, late_map = in_map && attn && map_behind_xi(L);
   const bool early_map = in_map && !late_map;
   auto launch_groups = [&](const LayerLaunch& l) { return early_map ? launch_map(l, tiled, false) : cudaSuccess; };
   auto launch_xi = [&](bool first) {
@@ -403,9 +401,8 @@ int compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* a, bool 
   }
   if (!in_map && launch_select_map(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (late_map && launch_map(L, tiled, true) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-  // weights: by a kernel of their own where the merge does not take them along, and for a caller that waits for the map
-  // alone (to compact K/V beside the merge)
-  const bool late_weights = early_map && attn, with_merge = late_weights && !a->map_event && merge_takes_weights(L);
+  // weights: by a kernel of their own where the merge does not take them along
+  const bool late_weights = early_map && attn, with_merge = late_weights && merge_takes_weights(L);
   if (late_weights && !with_merge && launch_weights(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (a->map_event && cudaEventRecord(static_cast<cudaEvent_t>(a->map_event), L.stream) != cudaSuccess)

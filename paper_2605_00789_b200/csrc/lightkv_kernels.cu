@@ -1112,6 +1112,13 @@ static bool few_rows(const LayerLaunch& L) {
 bool merge_takes_weights(const LayerLaunch& L) {
   return (long long)(L.a->vis_begin + L.ws.cap_out + L.a->n_text_after) * L.batch * L.hidden * (L.dtype == LIGHTKV_BF16 ? 2 : 4) <= (24ll << 20);
 }
+// The map behind xi, with the weights.  For a caller that waits for the map alone, where the launch is short: beside xi it would
+// save less than the second kernel costs (2 x 798 tokens x 32 heads, three stages with a given log-sum-exp: 162 us a pass
+// against 169).  And for one whose counts are replaced in place, whatever the launch: the xi kernel reads n_vis item by item,
+// and a map beside it would put the smaller counts there.
+bool map_behind_xi(const LayerLaunch& L) {
+  return L.a->n_vis == L.a->n_vis_out || (L.a->map_event && merge_takes_weights(L));
+}
 
 // =====================================================================================================
 // xi of the tokens (fixed-order sum over the heads) and the weights of the groups (Eq. "message-passing"), behind

@@ -748,6 +748,54 @@ def test_xi_of_tokens_cut_at_the_capacity_is_reported(before_merge):
     roomy.close()
 
 
+@pytest.mark.parametrize("xi_mode,dtype", [("attn", "bf16"), ("lse", "bf16"), ("attn", "fp32")])
+@pytest.mark.parametrize("streams", [1, 2])
+@pytest.mark.parametrize("hidden", [64, 2048])
+def test_counts_replaced_in_place(xi_mode, dtype, streams, hidden):
+    """One array for the counts that come in and those that go out gives what two arrays give, with more work items of xi than
+    CTAs and little else to do (hidden 64), and where the weights have a kernel of their own otherwise (2048: 28 MB)."""
+    import torch
+    import paper_2605_00789_b200 as L
+    b, grid, nt, h, dh = 12, (31, 37), 7, 12, 64
+    n = grid[0] * grid[1]
+    xm = L.XI_ATTN_FULL if xi_mode == "attn" else L.XI_ATTN_LSE
+    plan = L.Plan(b, hidden, h, 4, dh, 8, [grid], [3], [5], [0.5], nt, xi_mode=xm, ragged_input=True,
+                  dtype=L.BF16 if dtype == "bf16" else L.FP32)
+    dt = torch.bfloat16 if dtype == "bf16" else torch.float32
+    gen = torch.Generator(device="cuda").manual_seed(5)
+    rows = torch.randn((b, nt + n, hidden), generator=gen, device="cuda").to(dt)
+    q, k = (torch.randn((b, heads, nt + n, dh), generator=gen, device="cuda").to(dt) for heads in (h, 4))
+    pos = torch.full((b, n), -1, device="cuda", dtype=torch.int32)
+    counts = [n - 97 * (i % 5) for i in range(b)]
+    for i, m in enumerate(counts):
+        pos[i, :m] = torch.randperm(n, generator=gen, device="cuda")[:m].sort().values.int()
+    kw = dict(vis_begin=nt, q=q, k=k, pos=pos)
+    if xi_mode == "lse":
+        kw["lse"] = 3.0 + torch.rand((b, h, nt + n), generator=gen, device="cuda")
+    if streams == 2:
+        kw["aux_stream"] = torch.cuda.Stream()
+    found = []
+    for in_place in (False, True):
+        n_vis = torch.tensor(counts, device="cuda", dtype=torch.int32)
+        out = L.StageBuffers(plan, 0, nt + plan.stage_info(0).cap_out)
+        out.hidden_out.zero_()
+        out.workspace.fill_(255)                       # (a sum over heads that were not written is not a number)
+        if in_place:
+            out.n_vis_out = n_vis
+        L.compress_layer(plan, 0, rows, out, n_vis=n_vis, **kw)
+        found.append(out)
+    two, one = found
+    assert int(two.status) == int(one.status) == 0 and int(one.n_vis_out.max()) < min(counts)
+    for name in ("n_vis_out", "pos_out", "dst", "grp_off", "grp_src"):
+        assert torch.equal(getattr(two, name), getattr(one, name)), name
+    # (the heads of a token may be added in another order: 12 terms, each sum within 12 ulp; a row may then round to the
+    # neighbouring bf16 value, which is up to 2^-7 of it away)
+    torch.testing.assert_close(one.xi_out, two.xi_out, rtol=2e-6, atol=0)
+    torch.testing.assert_close(one.weight, two.weight, rtol=8e-6, atol=0)
+    torch.testing.assert_close(one.hidden_out.float(), two.hidden_out.float(), rtol=2 ** -7 if dtype == "bf16" else 1e-5, atol=1e-5)
+    plan.close()
+
+
 # ---- seeded random geometries ---------------------------------------------------------------------
 
 def _random_workload(seed):

@@ -79,6 +79,29 @@ int main() {
     assert out == [str(2 * 8 * 60), "2", "2"]
 
 
+def test_the_map_waits_for_xi_where_the_counts_are_replaced_in_place(tmp_path):
+    """The xi kernel reads the counts item by item, so a map that replaces them stands behind it, however long the launch;
+    one with counts of its own runs beside it unless the caller waits for the map of a short launch."""
+    entry.build()
+    out = _run(tmp_path, r"""
+#include <stdio.h>
+#include "launch.h"
+int main() {
+  int in[4], out[4], event;
+  for (int rows : {100, 100000})
+    for (bool waits : {false, true})
+      for (const int* counts : {(const int*)in, (const int*)out, (const int*)nullptr}) {
+        lightkv_layer_args_t a = {};
+        a.n_vis = counts; a.n_vis_out = out; a.map_event = waits ? &event : nullptr;
+        lkv::LayerLaunch L = {};
+        L.batch = 1; L.hidden = 4096; L.dtype = LIGHTKV_BF16; L.ws.cap_out = rows; L.a = &a;
+        printf("%d ", lkv::map_behind_xi(L));
+      }
+}
+""", "-L", os.path.dirname(CSRC), "-l:liblightkv.so", "-Xlinker", "-rpath=" + os.path.dirname(CSRC))
+    assert out == "0 1 0  1 1 1  0 1 0  0 1 0".split()
+
+
 @pytest.mark.gpu
 def test_the_map_of_keys_that_were_never_written_is_a_partition(tmp_path):
     """What the map kernel makes of a workspace whose tiled FD kernel stored no key (its waits expired): the windows' tokens
