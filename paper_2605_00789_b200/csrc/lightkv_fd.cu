@@ -75,15 +75,21 @@ struct FdStreamSmem {
   }
 };
 
-// CTAs of eight warps an SM holds, by O (bf16).  Without the bound the compiler takes 156 registers for O = 5, one CTA per SM:
-// 128 CTAs in clusters of eight then take two turns (4 x 345 tokens x 4096 in windows of 72: 22.5 -> 16.0 us).  O = 3 takes 114
-// by itself, 112 with a bound for nine warps: with more the CTAs do not fit beside those of the kernel in front (one image,
-// one layer: 27.5 us a pass with up to 112, 30.0 with 120).
-__host__ __device__ constexpr int fd_min_ctas(int o) { return o <= 2 ? 4 : o == 4 ? 0 : 2; }
+// CTAs an SM holds at least, which bounds the registers (0: as the compiler likes).  Eight warps, bf16: without the bound the
+// compiler takes 156 registers for O = 5, one CTA per SM: 128 CTAs in clusters of eight then take two turns (4 x 345 tokens x
+// 4096 in windows of 72: 22.5 -> 16.0 us).  O = 3 takes 94 by itself; it may have what nine warps leave, 112: with more the
+// CTAs do not fit beside those of the kernel in front (one image, one layer: 27.5 us a pass with up to 112, 30.0 with 120).
+// Two warps, where the SM is to hold as many CTAs as the shared memory of their rings allows: 24 samples x 547 tokens x 512 in
+// windows of 16 16.6 us with 78 registers, 14.9 with 64; 40 x 576 x 256 in windows of 25 14.6 us with 64 and spills, 13.1 with
+// 72; fp32, 24 x 576 x 384 in windows of 16 16.5 us with 80 and spills, 14.9 with 96.
+__host__ __device__ constexpr int fd_min_ctas(bool bf16, int o, int warps) {
+  if (warps == 8) return !bf16 || o == 4 ? 0 : o <= 2 ? 4 : 2;
+  return o == 1 ? (bf16 ? 16 : 10) : o == 2 && bf16 ? 14 : 0;
+}
 __host__ __device__ constexpr int fd_max_threads(bool bf16, int o, int warps) { return 32 * (bf16 && o == 3 && warps == 8 ? 9 : warps); }
 
 template <typename T, int O, int S, int WARPS>
-__global__ void __launch_bounds__(fd_max_threads(sizeof(T) == 2, O, WARPS), WARPS == 8 && sizeof(T) == 2 ? fd_min_ctas(O) : 0)
+__global__ void __launch_bounds__(fd_max_threads(sizeof(T) == 2, O, WARPS), fd_min_ctas(sizeof(T) == 2, O, WARPS))
 fd_stream_kernel(const __grid_constant__ FdStreamArgs a) {
   grid_dependency_wait();
   grid_launch_dependents();                              // in this order: see grid_dependency_sync
@@ -339,7 +345,9 @@ static cudaError_t launch_fd_stream_o(const LayerLaunch& L, const FdStreamArgs& 
 template <int O, int S>
 static cudaError_t launch_fd_stream_w(const LayerLaunch& L, const FdStreamArgs& f) {
   const bool wide = L.hidden * (L.dtype == LIGHTKV_FP32 ? 4 : 2) > 1536 || (long long)L.geo.n_windows * L.batch <= sm_count();
-  if (L.dtype == LIGHTKV_FP32) return wide ? launch_fd_stream_o<float, O, S, 8>(L, f) : launch_fd_stream_o<float, O, S, 2>(L, f);
+  // (fp32, two warps, O = 2: a fourth chunk in flight is worth more than a CTA; 24 x 576 x 384 in windows of 25 20.3 -> 18.9 us)
+  constexpr int NARROW32 = O == 2 ? 4 : S;
+  if (L.dtype == LIGHTKV_FP32) return wide ? launch_fd_stream_o<float, O, S, 8>(L, f) : launch_fd_stream_o<float, O, NARROW32, 2>(L, f);
   return wide ? launch_fd_stream_o<__nv_bfloat16, O, S, 8>(L, f) : launch_fd_stream_o<__nv_bfloat16, O, S, 2>(L, f);
 }
 

@@ -504,6 +504,15 @@ def test_fd_windows_around_groups_of_eight_nodes(grid, hidden):
     H.run_schedule(dataclasses.replace(wl, batch=1), xi_mode="uniform", direction="b2a", metric="l2")
 
 
+@pytest.mark.parametrize("dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("grid", [(3, 5), (4, 4), (3, 6), (4, 8), (3, 11), (6, 8), (8, 8), (8, 10)])
+def test_fd_narrow_rows_of_many_windows(grid, dtype):
+    # more windows than SMs and rows of at most 1.5 KB: CTAs of two warps, at the edges of every variant's 8 to 40 nodes a side
+    wl = S.Workload(name="fdnarrow", config_id=145, batch=151, tiles=(grid,), n_text=4, hidden=72, n_q_heads=2,
+                    n_kv_heads=1, head_dim=64, n_layers=16, layers=(3,), windows=(1,), keep=(0.6,))
+    H.run_schedule(wl, dtype=dtype, xi_mode="uniform", oracle_samples=[0, 75, 150])
+
+
 @pytest.mark.parametrize("grid,windows,seed", [((12, 20), (5, 3), 282), ((12, 32), (3, 2), 4)])
 def test_fd_window_larger_than_the_plan_expects(grid, windows, seed):
     # a near-full subset of the grid moves tokens between windows: one window of the second stage has a node more a
