@@ -107,6 +107,17 @@ __host__ __device__ inline int window_of(const Geometry& g, int pos) {
   return t * g.w * g.w + (r * g.w / g.rows[t]) * g.w + (c * g.w / g.cols[t]);
 }
 
+// floor(n / d) for n < 65536, 2 <= d < 65536 by one multiplication with m = ceil(2^32 / d): n * m / 2^32 is more than n / d by
+// less than n / 2^32 < 1 / d.  (For d = 1 the multiplier does not fit; the kernels have forms of their own for that.)
+inline unsigned int div_multiplier(int d) { return (unsigned int)(((1ull << 32) + d - 1) / d); }
+__host__ __device__ inline int div_magic(int n, unsigned int m) {
+#ifdef __CUDA_ARCH__
+  return (int)__umulhi((unsigned int)n, m);
+#else
+  return (int)((unsigned long long)(unsigned int)n * m >> 32);
+#endif
+}
+
 // ---- 16-byte vector access and element conversion -----------------------------------------------
 template <typename T> struct Vec;                      // elements per 16 bytes
 template <> struct Vec<__nv_bfloat16> { static constexpr int n = 8; };

@@ -799,10 +799,6 @@ cudaError_t launch_select_map(const LayerLaunch& L) {
 // kernel holds whole windows.
 // (select_map_kernel, which starts from keys, takes six dependent rounds through L2.)
 // =====================================================================================================
-// floor(n / d) for n, d < 65536 with m = ceil(2^32 / d): one multiply instead of a division.  For d = 1 that is one bit too
-// long and m arrives as 0.
-__device__ inline int div_magic(int n, unsigned m) { return m ? (int)__umulhi((unsigned)n, m) : n; }
-
 // The weight of a member with `xi` in a group of `size` whose sum is `den`.
 __device__ __forceinline__ float member_weight(float xi, float den, int size) {
   return den >= 1e-30f ? xi / den : 1.0f / (float)size;
@@ -1130,7 +1126,7 @@ bool map_behind_xi(const LayerLaunch& L) {
 struct WeightArgs {
   int n_q_heads, cap_in, cap_out;
   int chunk;                           // weights_kernel: tokens per CTA
-  unsigned magic_chunk;                // (see div_magic)
+  unsigned magic_chunk;                // div_multiplier(chunk)
   const float* xi_h;                   // [B, cap_in, H]
   const int* n_vis;
   const int* n_vis_out;
@@ -1234,8 +1230,8 @@ __global__ void __launch_bounds__(1024) weights_kernel(const __grid_constant__ W
 
 static WeightArgs weight_args(const LayerLaunch& L) {
   const lightkv_layer_args_t* a = L.a;
-  const int chunk = (L.ws.cap_in + kWeightCtas - 1) / kWeightCtas;      // at most kMapMaxTokens / 8
-  return {L.n_q_heads, L.ws.cap_in, L.ws.cap_out, chunk, (unsigned)(((1ull << 32) + chunk - 1) / chunk), L.ws.xi_h, a->n_vis,
+  const int chunk = std::max(2, (L.ws.cap_in + kWeightCtas - 1) / kWeightCtas);      // at most kMapMaxTokens / 8; 2: see div_magic
+  return {L.n_q_heads, L.ws.cap_in, L.ws.cap_out, chunk, div_multiplier(chunk), L.ws.xi_h, a->n_vis,
           a->n_vis_out, a->grp_off, a->grp_src, a->dst, a->weight, a->xi_out, a->status};
 }
 
@@ -1464,11 +1460,12 @@ struct KvAddr {
   }
 };
 
-
-
-// THREADS per CTA, MB members of a group in flight
-template <typename T, int THREADS, int MB>
-__global__ void __launch_bounds__(THREADS, THREADS > 256 ? 2 : (sizeof(T) == 2 ? 5 : 4))
+// THREADS per CTA, MB members of a group in flight.  ONE: heads of a single 16-byte piece, which there is no division for.  (A
+// division that also does for one piece, by a test or with twice the number and half the multiplier, costs more than the form:
+// 32 x 640 rows x 40 heads x 128 119.0 or 118.8 against 116.9 us, 8 x 3008 x 32 105.8 or 105.4 against 104.0; with the test the
+// kernel spills.)
+template <typename T, int THREADS, int MB, bool ONE>
+__global__ void __launch_bounds__(THREADS, (THREADS > 256 ? 2 : (sizeof(T) == 2 ? 5 : 4)) - ONE)
 kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* __restrict__ k_dst,
                   T* __restrict__ v_dst, KvAddr sa, KvAddr da, int n_kv_heads, int dh, int vis_begin,
                   int n_text_after, int cap_in, int cap_out, int gather, int merge_at_survivor, unsigned magic_ch,
@@ -1481,7 +1478,8 @@ kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* _
   const int n_in = n_vis ? min(n_vis[b], cap_in) : cap_in;
   const int n_out = n_vis_out[b];
   if (row >= vis_begin + n_out + n_text_after) return;
-  const int ch = dh / V, per_kv = n_kv_heads * ch, units = 2 * per_kv;
+  const int ch = ONE ? 1 : dh / V, per_kv = n_kv_heads * ch, units = 2 * per_kv;
+  auto head_of = [&](int piece) { return ONE ? piece : div_magic(piece, magic_ch); };
   int64_t d_tok = da.token(b, row);
   const bool text = row < vis_begin || row >= vis_begin + n_out;
   const int* gs = grp_src + size_t(b) * cap_in;
@@ -1507,7 +1505,7 @@ kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* _
       for (int q = 0; q < 4; ++q) {
         const int u = u0 + q * blockDim.x;
         if (u < units) {
-          const int kv = u >= per_kv ? 1 : 0, rem = u - kv * per_kv, h = div_magic(rem, magic_ch), c = rem - h * ch;
+          const int kv = u >= per_kv ? 1 : 0, rem = u - kv * per_kv, h = head_of(rem), c = rem - h * ch;
           v[q] = ld_stream16((kv ? v_src : k_src) + s_tok + int64_t(h) * sa.head_stride + c * V);
         }
       }
@@ -1515,7 +1513,7 @@ kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* _
       for (int q = 0; q < 4; ++q) {
         const int u = u0 + q * blockDim.x;
         if (u < units) {
-          const int kv = u >= per_kv ? 1 : 0, rem = u - kv * per_kv, h = div_magic(rem, magic_ch), c = rem - h * ch;
+          const int kv = u >= per_kv ? 1 : 0, rem = u - kv * per_kv, h = head_of(rem), c = rem - h * ch;
           st_stream16((kv ? v_dst : k_dst) + d_tok + int64_t(h) * da.head_stride + c * V, v[q]);
         }
       }
@@ -1538,9 +1536,9 @@ kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* _
   for (int base = 0; base < units; base += 2 * blockDim.x) {
     const int u0 = base + threadIdx.x, u1 = u0 + blockDim.x;
     const bool one = u0 < units, two = u1 < units;
-    const int kv0 = u0 >= per_kv ? 1 : 0, rem0 = u0 - kv0 * per_kv, h0 = div_magic(rem0, magic_ch), c0 = rem0 - h0 * ch;
+    const int kv0 = u0 >= per_kv ? 1 : 0, rem0 = u0 - kv0 * per_kv, h0 = head_of(rem0), c0 = rem0 - h0 * ch;
     const int ub = two ? u1 : u0;
-    const int kv1 = ub >= per_kv ? 1 : 0, rem1 = ub - kv1 * per_kv, h1 = div_magic(rem1, magic_ch), c1 = rem1 - h1 * ch;
+    const int kv1 = ub >= per_kv ? 1 : 0, rem1 = ub - kv1 * per_kv, h1 = head_of(rem1), c1 = rem1 - h1 * ch;
     const T* sp0 = (kv0 ? v_src : k_src) + int64_t(h0) * sa.head_stride + c0 * V;
     const T* sp1 = (kv1 ? v_src : k_src) + int64_t(h1) * sa.head_stride + c1 * V;
     float acc0[V], acc1[V];
@@ -1604,7 +1602,8 @@ struct KvPlaneSmem {
   __host__ __device__ size_t bytes(int pieces) const { return rows() + size_t(rows_in) * pieces * 16; }
 };
 
-template <typename T, int THREADS>
+// ONE: rows of a single piece, as above
+template <typename T, int THREADS, bool ONE>
 __global__ void __launch_bounds__(THREADS)
 kv_plane_kernel(T* __restrict__ k_buf, T* __restrict__ v_buf, KvAddr ad, KvPlaneSmem sm, int n_kv_heads, int ch, int parts,
                 unsigned magic_ch, int vis_begin, int n_text_after, int gather, const int* __restrict__ n_vis,
@@ -1655,7 +1654,7 @@ kv_plane_kernel(T* __restrict__ k_buf, T* __restrict__ v_buf, KvAddr ad, KvPlane
   const int total = (n_out + n_text_after) * ch, staged = gather ? total : (n_in + n_text_after) * ch;
 #pragma unroll 4
   for (int idx = tid; idx < staged; idx += THREADS) {
-    const int r = div_magic(idx, magic_ch), c = idx - r * ch;
+    const int r = ONE ? idx : div_magic(idx, magic_ch), c = ONE ? 0 : idx - r * ch;
     const int l = !gather ? r : r < n_out ? member(off[r]) : r - n_out + n_in;
     tc::cp_async16(s_rows + uint32_t(idx) * 16, at(l) + c * V, 16);
   }
@@ -1664,7 +1663,7 @@ kv_plane_kernel(T* __restrict__ k_buf, T* __restrict__ v_buf, KvAddr ad, KvPlane
   __syncthreads();                                         // every source of the plane has been read
 #pragma unroll 2
   for (int idx = tid; idx < total; idx += THREADS) {
-    const int r = div_magic(idx, magic_ch), c = idx - r * ch;
+    const int r = ONE ? idx : div_magic(idx, magic_ch), c = ONE ? 0 : idx - r * ch;
     uint4 v;
     if (gather || r >= n_out) {
       v = rows[gather ? idx : idx + (n_in - n_out) * ch];
@@ -1769,8 +1768,7 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
             a->page_size > 0 ? a->dst_block_table : nullptr, a->page_size, a->max_blocks, a->dst_seq_start, magic_page};
   const int ch_host = K.head_dim * (K.dtype == LIGHTKV_BF16 ? 2 : 4) / 16;
   if (2 * K.n_kv_heads * ch_host >= 65536) return cudaErrorInvalidValue;      // range of the unit decode
-  const unsigned magic_ch = (unsigned)(((1ull << 32) + ch_host - 1) / ch_host);
-  const dim3 grid(a->vis_begin + K.cap_out + a->n_text_after, K.batch);
+    const dim3 grid(a->vis_begin + K.cap_out + a->n_text_after, K.batch);
   const int units = 2 * K.n_kv_heads * ch_host;
   // two units per thread (both in flight); narrow caches (GQA) get narrow CTAs
   const bool few = few_rows((long long)grid.x * grid.y);
@@ -1796,17 +1794,28 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
           if (rc != cudaSuccess) return rc;
           return launch_kernel(kernel, dim3((unsigned)(planes * p)), threads, sm.bytes(ch), K.stream, 1,
               static_cast<T*>(a->k_dst), static_cast<T*>(a->v_dst), da, sm, K.n_kv_heads, ch, p,
-              (unsigned)(((1ull << 32) + ch - 1) / ch), a->vis_begin, a->n_text_after, gather, a->n_vis, a->n_vis_out,
+              div_multiplier(ch), a->vis_begin, a->n_text_after, gather, a->n_vis, a->n_vis_out,
               a->grp_off, a->grp_src, a->weight);
         };
-        return sm.bytes(ch) <= 110 * 1024 ? launch(kv_plane_kernel<T, 512>, 512) : launch(kv_plane_kernel<T, 1024>, 1024);
+        if constexpr (sizeof(T) == 2)                     // (fp32 heads have two pieces or more, and planes are not cut to one)
+          if (ch == 1) return sm.bytes(ch) <= 110 * 1024 ? launch(kv_plane_kernel<T, 512, true>, 512) : launch(kv_plane_kernel<T, 1024, true>, 1024);
+        return sm.bytes(ch) <= 110 * 1024 ? launch(kv_plane_kernel<T, 512, false>, 512) : launch(kv_plane_kernel<T, 1024, false>, 1024);
       }
     }
-    if (!(in_place && gather))                            // in place, gather mode has nothing to merge
-      e = launch_kernel(few ? kv_compact_kernel<T, 512, 4> : kv_compact_kernel<T, 256, 2>, grid, threads, 0, K.stream, 1,
-          static_cast<const T*>(a->k_src), static_cast<const T*>(a->v_src), static_cast<T*>(a->k_dst),
-          static_cast<T*>(a->v_dst), sa, da, K.n_kv_heads, K.head_dim, a->vis_begin, a->n_text_after, K.cap_in,
-          K.cap_out, gather, in_place ? 1 : 0, magic_ch, a->n_vis, a->n_vis_out, a->grp_off, a->grp_src, a->weight);
+    if (!(in_place && gather)) {                          // in place, gather mode has nothing to merge
+      auto launch = [&](auto kernel) -> cudaError_t {
+        return launch_kernel(kernel, grid, threads, 0, K.stream, 1,
+            static_cast<const T*>(a->k_src), static_cast<const T*>(a->v_src), static_cast<T*>(a->k_dst),
+            static_cast<T*>(a->v_dst), sa, da, K.n_kv_heads, K.head_dim, a->vis_begin, a->n_text_after, K.cap_in,
+            K.cap_out, gather, in_place ? 1 : 0, div_multiplier(ch_host), a->n_vis, a->n_vis_out, a->grp_off, a->grp_src, a->weight);
+      };
+      bool one = false;
+      if constexpr (sizeof(T) == 2) {
+        one = ch_host == 1;
+        if (one) e = few ? launch(kv_compact_kernel<T, 512, 4, true>) : launch(kv_compact_kernel<T, 256, 2, true>);
+      }
+      if (!one) e = few ? launch(kv_compact_kernel<T, 512, 4, false>) : launch(kv_compact_kernel<T, 256, 2, false>);
+    }
     if (e != cudaSuccess || !in_place) return e;
     // planes: (sample, K / V, head), cut along head_dim while there are fewer of them than CTAs that fit
     int parts = 1;

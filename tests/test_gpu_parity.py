@@ -909,6 +909,14 @@ def test_heads_of_one_piece(in_place):
     H.run_schedule(wl, xi_mode="given", kv_in_place=in_place)
 
 
+@pytest.mark.parametrize("batch,grid,in_place", [(40, (9, 7), False), (40, (9, 7), True), (1, (66, 70), True)])
+def test_heads_of_one_piece_over_variants(batch, grid, in_place):
+    # the form for many rows, and planes of one and of two CTAs per SM
+    wl = S.Workload(name="pieces", config_id=146, batch=batch, tiles=(grid,), n_text=3, hidden=64, n_q_heads=4,
+                    n_kv_heads=4, head_dim=8, n_layers=16, layers=(3,), windows=(6,), keep=(0.55,))
+    H.run_schedule(wl, xi_mode="given", kv_in_place=in_place, oracle_samples=sorted({0, batch - 1}))
+
+
 def test_weights_of_samples_with_a_token_per_cta():
     # at most eight tokens a sample, weights by a kernel of their own (the caller waits for the map alone)
     import torch

@@ -14,6 +14,11 @@ LIMITS = {
         "fd_stream_kernel<__nv_bfloat16, 2, 3, 2>": 72,        # fourteen
         "fd_stream_kernel<float, 2, 4, 2>": 96,                # ten
     },
+    "lightkv_kernels": {
+        "kv_compact_kernel<__nv_bfloat16, 256, 2, false>": 48,        # five CTAs of 256 threads
+        "kv_compact_kernel<__nv_bfloat16, 512, 4, false>": 64,        # two of 512
+        "kv_compact_kernel<float, 256, 2, false>": 64,                # four of 256
+    },
 }
 
 

@@ -46,6 +46,25 @@ int main() {
     assert out == ["0", "0"]
 
 
+def test_division_by_a_multiplier_is_exact(tmp_path):
+    """Every quotient of the range at small divisors, the numbers around every multiple at all of them."""
+    out = _run(tmp_path, r"""
+#include <stdio.h>
+#include "common.cuh"
+int main() {
+  int bad = 0;
+  for (int d = 2; d < 65536; ++d) {
+    const unsigned m = lkv::div_multiplier(d);
+    if (d <= 64) for (int n = 0; n < 65536; ++n) bad += lkv::div_magic(n, m) != n / d;
+    for (int k = d; k < 65536; k += d) bad += lkv::div_magic(k, m) != k / d || lkv::div_magic(k - 1, m) != (k - 1) / d;
+    bad += lkv::div_magic(65535, m) != 65535 / d;
+  }
+  printf("%d\n", bad);
+}
+""")
+    assert out == ["0"]
+
+
 def test_the_shared_memory_limit_is_set_once_per_kernel_and_device(tmp_path):
     """Sixty kernels on eight devices, launched in turn with growing and shrinking sizes by two threads: a limit is only ever
     set to raise it, and a set that failed is tried again."""
