@@ -526,12 +526,85 @@ cudaError_t launch_xi_simt(const LayerLaunch& L, bool wait_first) {
   return L.dtype == LIGHTKV_BF16 ? launch_xi_simt_t<__nv_bfloat16>(L, wait_first) : launch_xi_simt_t<float>(L, wait_first);
 }
 
+// ---- xi of a token, the sum over its heads.  They are added in one order everywhere, so that xi and the weights have the same
+// bits whichever kernels a call's size, workspace or map event select: head h counts to sum h % 32, in ascending order, and these
+// 32 meet as a warp's lanes do in a butterfly over 1, 2, 4, 8 and 16.
+
+// One token, in every lane; the lanes share the heads, two loads in flight.
+__device__ __forceinline__ float warp_xi(const float* x, int heads, int lane) {
+  float v = 0.f;
+#pragma unroll 1
+  for (int h = lane; h < heads; h += 64) {
+    const float v0 = x[h], v1 = h + 32 < heads ? x[h + 32] : 0.f;
+    v = (v + v0) + v1;
+  }
+#pragma unroll
+  for (int o = 1; o <= 16; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+// Of eight values a lane, summed over the eight lanes that differ in bits 0 to 2 (first over 1, then 2 and 4): lane l gets value
+// xi_value(l & 7).
+__host__ __device__ constexpr int xi_value(int l) { return (l & 1) << 2 | (l & 2) | (l & 4) >> 2; }
+__device__ __forceinline__ float sum_eight(float (&p)[8], int lane) {
+#pragma unroll
+  for (int o = 1, left = 4; o <= 4; o <<= 1, left >>= 1)
+#pragma unroll
+    for (int t = 0; t < left; ++t) {
+      const float give = lane & o ? p[t] : p[t + left], keep = lane & o ? p[t + left] : p[t];
+      p[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+    }
+  return p[0];
+}
+
+// One token by a thread: sixteen heads at a time, groups of four pair by pair.  (Little code and few registers: with all groups
+// unrolled, eight loads in flight or a warp's lanes over its tokens' heads a map takes 0.5 to 1.5 us more.)
+__device__ __forceinline__ float token_xi(const float* x, int heads) {
+  const bool quads = (heads & 3) == 0;                      // (rows of four floats are 16-byte aligned)
+  float sum = 0.f;
+#pragma unroll 1
+  for (int h = 0; h < min(heads, 32); h += 16) {
+    float4 s[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) s[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 1
+    for (int k = h; k < heads; k += 32) {
+      float4 v[4];
+      if (quads) {                                          // (clamped, not left out: a load behind a branch waits for the one before)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) v[m] = *reinterpret_cast<const float4*>(x + min(k + 4 * m, heads - 4));
+#pragma unroll
+        for (int m = 1; m < 4; ++m)
+          if (k + 4 * m >= heads) v[m] = make_float4(0.f, 0.f, 0.f, 0.f);
+      } else {
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int c = k + 4 * m, last = heads - 1;
+          v[m] = make_float4(x[min(c, last)], x[min(c + 1, last)], x[min(c + 2, last)], x[min(c + 3, last)]);
+        }
+#pragma unroll
+        for (int m = 0; m < 4; ++m) {
+          const int c = k + 4 * m;
+          v[m] = make_float4(c < heads ? v[m].x : 0.f, c + 1 < heads ? v[m].y : 0.f, c + 2 < heads ? v[m].z : 0.f, c + 3 < heads ? v[m].w : 0.f);
+        }
+      }
+#pragma unroll
+      for (int m = 0; m < 4; ++m) { s[m].x += v[m].x; s[m].y += v[m].y; s[m].z += v[m].z; s[m].w += v[m].w; }
+    }
+    float q[4];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) q[m] = (s[m].x + s[m].y) + (s[m].z + s[m].w);
+    sum += (q[0] + q[1]) + (q[2] + q[3]);
+  }
+  return sum;
+}
+
 // =====================================================================================================
 // Selection + merge map (Steps 2-5).  One cluster of 1-8 CTAs per sample (about a token per thread); every
 // CTA keeps a contiguous range of the sample's tokens through all phases, phases that read what other
 // threads wrote are separated by cluster barriers, prefix sums cross the cluster through distributed shared
 // memory.
-//   1  xi = fixed-order sum over heads (or given / uniform); every source token (local rank parity src_par): r =
+//   1  xi = sum over heads (token_xi; or given / uniform); every source token (local rank parity src_par): r =
 //      removal_count(n_w), selected iff it is among the r entries of its window with the smallest
 //      (FD, index) (rank by counting 32-bit keys; skipped when r = |A|); a selected token takes its best B
 //   2  survivors (all B, unselected A) get consecutive output slots in storage (= position) order: dst,
@@ -668,11 +741,7 @@ __global__ void __launch_bounds__(1024) select_map_kernel(Workspace ws, SelectAr
     float v;
     if (a.xi_mode == LIGHTKV_XI_GIVEN) v = a.xi_in[size_t(b) * ws.cap_in + i];
     else if (a.xi_mode == LIGHTKV_XI_UNIFORM) v = 1.0f;
-    else {
-      v = 0.f;
-#pragma unroll 8
-      for (int h = 0; h < a.n_q_heads; ++h) v += ws.xi_h[(size_t(b) * ws.cap_in + i) * a.n_q_heads + h];
-    }
+    else v = token_xi(ws.xi_h + (size_t(b) * ws.cap_in + i) * a.n_q_heads, a.n_q_heads);
     xi[i] = v;
     if (a.xi_out) a.xi_out[size_t(b) * ws.cap_in + i] = v;
     int p = -1;
@@ -826,21 +895,6 @@ struct MapArgs {
   float* xi_out;
   uint32_t* status;
 };
-
-// xi of one token: the sum over its heads
-__device__ __forceinline__ float token_xi(const float* x, int heads) {
-  float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
-  int h = 0;
-  if ((heads & 3) == 0) {                                   // (rows of four floats are 16-byte aligned)
-#pragma unroll 8
-    for (; h < heads; h += 4) {
-      const float4 v = *reinterpret_cast<const float4*>(x + h);
-      s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
-    }
-  }
-  for (; h < heads; ++h) s.x += x[h];
-  return (s.x + s.y) + (s.z + s.w);
-}
 
 template <bool CLUSTER, int TPT, bool SELECT, bool WEIGHTS>
 __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapArgs a) {
@@ -1117,7 +1171,7 @@ bool map_behind_xi(const LayerLaunch& L) {
 }
 
 // =====================================================================================================
-// xi of the tokens (fixed-order sum over the heads) and the weights of the groups (Eq. "message-passing"), behind
+// xi of the tokens (in the one order, see warp_xi) and the weights of the groups (Eq. "message-passing"), behind
 // map_kernel, which knows the groups but runs beside the xi kernel: xi_i / sum over the group, the sum taken in member
 // order (survivor first).  A cluster of eight CTAs per sample: a warp sums the heads of eight tokens into
 // shared memory; then a thread per group reads its members' sums from the CTAs that hold them.  Bound by
@@ -1156,7 +1210,7 @@ __global__ void __launch_bounds__(1024) weights_kernel(const __grid_constant__ W
   const float* x = a.xi_h + row * H;
   for (int i0 = lo + 8 * warp; i0 < hi; i0 += nthr >> 2) {
     // eight tokens of a warp, the lanes over the heads (addresses are clamped, not loads left out: a load behind a branch
-    // waits for the one before); then lane l holds the sum of token l / 4
+    // waits for the one before); then every lane holds the sum of a token
     float p[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     const int last = a.cap_in - 1 - i0;
     for (int h0 = lane; h0 - lane < H; h0 += 64) {
@@ -1169,24 +1223,17 @@ __global__ void __launch_bounds__(1024) weights_kernel(const __grid_constant__ W
 #pragma unroll
         for (int t = 0; t < 8; ++t) w[t] = xg[min(t, last) * H];
 #pragma unroll
-        for (int t = 0; t < 8; ++t) p[t] += h0 + 32 < H ? w[t] : 0.f;
-      }
+        for (int t = 0; t < 8; ++t) p[t] = (p[t] + v[t]) + (h0 + 32 < H ? w[t] : 0.f);
+      } else {
 #pragma unroll
-      for (int t = 0; t < 8; ++t) p[t] += h0 < H ? v[t] : 0.f;
-    }
-#pragma unroll
-    for (int o = 16; o >= 4; o >>= 1) {
-#pragma unroll
-      for (int t = 0; t < o / 4; ++t) {
-        const float give = lane & o ? p[t] : p[t + o / 4], keep = lane & o ? p[t + o / 4] : p[t];
-        p[t] = keep + __shfl_xor_sync(0xffffffffu, give, o);
+        for (int t = 0; t < 8; ++t) p[t] += h0 < H ? v[t] : 0.f;
       }
     }
-    float v = p[0];
-    v += __shfl_xor_sync(0xffffffffu, v, 2);
-    v += __shfl_xor_sync(0xffffffffu, v, 1);
-    const int i = i0 + (lane >> 2);
-    if ((lane & 3) == 0 && i < hi) {
+    float v = sum_eight(p, lane);
+    v += __shfl_xor_sync(0xffffffffu, v, 8);
+    v += __shfl_xor_sync(0xffffffffu, v, 16);
+    const int i = i0 + xi_value(lane & 7);
+    if (lane < 8 && i < hi) {
       s_xi[i - lo] = v;
       if (a.xi_out && i < n) a.xi_out[row + i] = v;
     }
@@ -1241,24 +1288,13 @@ cudaError_t launch_weights(const LayerLaunch& L) {
   return launch_kernel(weights_kernel, L.batch * kWeightCtas, threads, size_t(4) * w.chunk, L.stream, kWeightCtas, w);
 }
 
-// xi of token i of sample b in every lane of the warp that asks; the lanes share the heads, two loads in flight
-__device__ __forceinline__ float warp_xi(const WeightArgs& a, int b, int i, int lane) {
-  const float* x = a.xi_h + (size_t(b) * a.cap_in + i) * a.n_q_heads;
-  float v = 0.f;
-#pragma unroll 1
-  for (int h = lane; h < a.n_q_heads; h += 64) v += x[h] + (h + 32 < a.n_q_heads ? x[h + 32] : 0.f);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // A sample cut at cap_out has tokens that belong to no group that is kept: their xi is still reported.
 __device__ __noinline__ void xi_of_cut_tokens(const WeightArgs& a, int b, int n, int n_out) {
   if (!a.xi_out || a.grp_off[size_t(b) * (a.cap_out + 1) + n_out] >= n) return;
   const int lane = threadIdx.x & 31;
   for (int i = threadIdx.x >> 5; i < n; i += blockDim.x >> 5)
     if (a.dst[size_t(b) * a.cap_in + i] >= a.cap_out) {
-      const float v = warp_xi(a, b, i, lane);
+      const float v = warp_xi(a.xi_h + (size_t(b) * a.cap_in + i) * a.n_q_heads, a.n_q_heads, lane);
       if (lane == 0) a.xi_out[size_t(b) * a.cap_in + i] = v;
     }
 }
@@ -1305,6 +1341,7 @@ __global__ void __launch_bounds__(256, MB > 2 ? 3 : WEIGHTS ? 4 : 5) merge_rows_
   const int* gs = a.w.grp_src + size_t(b) * cap_in + g0;
   float* wt = a.w.weight + size_t(b) * cap_in;
   float* xo = a.w.xi_out ? a.w.xi_out + size_t(b) * cap_in : nullptr;
+  const float* xh = a.w.xi_h + size_t(b) * cap_in * a.w.n_q_heads;
   const int count = text ? 1 : g1 - g0;
   if (count == 1) {                                     // copied
     const int i = text ? 0 : gs[0];
@@ -1321,7 +1358,7 @@ __global__ void __launch_bounds__(256, MB > 2 ? 3 : WEIGHTS ? 4 : 5) merge_rows_
     }
     if (text) return;
     if (WEIGHTS && tid < 32) {
-      const float v = warp_xi(a.w, b, i, tid);
+      const float v = warp_xi(xh + size_t(i) * a.w.n_q_heads, a.w.n_q_heads, tid);
       w = member_weight(v, v, 1);
       if (tid == 0) {
         wt[i] = w;
@@ -1351,7 +1388,7 @@ __global__ void __launch_bounds__(256, MB > 2 ? 3 : WEIGHTS ? 4 : 5) merge_rows_
       const int m = min(AHEAD, count - k0);
       for (int k = tid >> 5; k < m; k += nthr >> 5) {
         const int i = gs[k0 + k];
-        const float v = warp_xi(a.w, b, i, lane);
+        const float v = warp_xi(xh + size_t(i) * a.w.n_q_heads, a.w.n_q_heads, lane);
         if (lane == 0) {
           s_xi[k] = v;
           if (xo) xo[i] = v;
