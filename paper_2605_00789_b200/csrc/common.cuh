@@ -36,8 +36,7 @@ struct Workspace {
   unsigned long long* a_key;  // [B, cap_a]  (orderable(lowest FD) << 32) | B entry index of the best partner;
                               //             all ones while no partner is known (set by the window build)
   // tiled FD kernel without window lists (these two lie over the arrays of the list form)
-  unsigned long long* tile_key;  // [B, n_windows, fd blocks, (max_cell + 1) / 2]  such keys by block of destinations and
-                   //                             source of the window, see fd_tc_kernel
+  unsigned long long* tile_key;  // [B, fd blocks, cap_in]  such keys by block of destinations and token, see fd_tc_kernel
   int* win_tok;    // [B, n_windows, max_cell + 1]  tiled FD kernel: the number of tokens of a window, then the tokens
   float* xi_h;     // [B, cap_in, H]      per-head attention mass on the prompt (ATTN modes): a token's heads in one line
   float* xi;       // [B, cap_in]

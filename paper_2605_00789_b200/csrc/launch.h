@@ -150,7 +150,7 @@ cudaError_t launch_kv_compact(const KvLaunch& K);
 // tcgen05 paths (lightkv_tc.cu).  `supported` queries are host-only.
 bool tc_fd_supported(int hidden);
 bool tc_xi_supported(int head_dim);
-// lists: windows from launch_window_build, keys by source entry for launch_select_map; else by window and source for launch_map
+// lists: windows from launch_window_build, keys by source entry for launch_select_map; else by token for launch_map
 cudaError_t launch_fd_tc(const LayerLaunch& L, bool lists);
 // wait_first: as for launch_xi_simt
 cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first);

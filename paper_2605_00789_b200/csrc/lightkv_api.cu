@@ -57,7 +57,7 @@ static void layout_workspace(const lightkv_plan_t& p, StagePlan& s) {
   const size_t B = p.cfg.batch, nW1 = s.n_windows + 1;
   const bool attn = p.cfg.xi_mode == LIGHTKV_XI_ATTN_FULL || p.cfg.xi_mode == LIGHTKV_XI_ATTN_LSE;
   const size_t xi_items = attn ? size_t((s.cap_in + 127) / 128) * p.cfg.n_q_heads * B : 0;
-  const bool by_token = s.use_tc && windows_in_ctas(s) && !fd_stream_supported(p.cfg.dtype, s.fd_side);
+  const bool tiled = s.use_tc && windows_in_ctas(s) && !fd_stream_supported(p.cfg.dtype, s.fd_side);
   WorkspaceOffsets& o = s.off;
   size_t end = 0;
   auto place = [&](size_t bytes) { const size_t at = end; end += align_up(bytes, 256); return at; };
@@ -78,9 +78,8 @@ static void layout_workspace(const lightkv_plan_t& p, StagePlan& s) {
   o.a_partner = place(B * s.cap_a * 4);
   s.ws_list = end;
   end = forms;
-  // (at least a key per token and block: which calls fit a workspace of a given size does not depend on how keys are numbered)
-  o.tile_key = place(by_token ? B * s.fd_blocks * std::max(size_t(s.cap_in), s.n_windows * size_t((s.max_cell + 1) / 2)) * 8 : 0);
-  o.win_tok = place(by_token ? B * s.n_windows * (size_t(s.max_cell) + 1) * 4 : 0);
+  o.tile_key = place(tiled ? B * s.fd_blocks * s.cap_in * 8 : 0);
+  o.win_tok = place(tiled ? B * s.n_windows * (size_t(s.max_cell) + 1) * 4 : 0);
   s.ws_tiled = end;
   s.ws_bytes = std::max(s.ws_list, s.ws_tiled);
 }

@@ -882,7 +882,7 @@ struct MapArgs {
   const int* pos;
   int* partner;
   int* place;
-  const unsigned long long* key;       // SELECT: [B, n_windows, blocks, (max_cell + 1) / 2]
+  const unsigned long long* key;       // SELECT: [B, blocks, cap_in]
   const int* win_tok;                  // SELECT: [B, n_windows, max_cell + 1]
   int blocks, max_cell, n_windows, src_par;
   double keep;
@@ -923,27 +923,25 @@ __global__ void __launch_bounds__(1024) map_kernel(const __grid_constant__ MapAr
   if (SELECT) {
     const WindowLists lists = WindowLists::at(smem_raw, a.max_cell);          // (before the arrays above are in use)
     for (int w = rank; w < a.n_windows; w += cs) {
-      // the counts, the tokens and the keys are asked for at once: what lies behind the window's last is not used
       const int* win_tok = a.win_tok + (size_t(b) * a.n_windows + w) * (a.max_cell + 1);
-      const int nw = win_tok[0], par = a.src_par, na = (nw + 1 - par) >> 1, nb = nw - na, src = (a.max_cell + 1) / 2;
-      for (int l = tid; l < a.max_cell; l += nthr) lists.tok[l] = win_tok[1 + l];
-      for (int e = tid; e < src; e += nthr) {
-        const unsigned long long* k = a.key + (size_t(b) * a.n_windows + w) * a.blocks * src + e;
+      const int nw = win_tok[0], par = a.src_par, na = (nw + 1 - par) >> 1, nb = nw - na;
+      for (int l = tid; l < nw; l += nthr) lists.tok[l] = win_tok[1 + l];
+      // (keys by window and source, asked for before the window's tokens and their number are there: no faster, and more keys
+      // than tokens where windows differ in size)
+      const int removed = nb > 0 ? removal_count(nw, a.keep, par) : 0, blocks = removed > 0 ? min(a.blocks, (nb + kFdTile - 1) / kFdTile) : 0;
+      for (int e = tid; e < na; e += nthr) {
+        const unsigned long long* k = a.key + size_t(b) * a.blocks * a.cap_in + win_tok[1 + 2 * e + par];
         unsigned long long key = ~0ull;
-        for (int ib = 0; ib < a.blocks; ib += 4) {
+        for (int ib = 0; ib < blocks; ib += 4) {
           unsigned long long v[4];
 #pragma unroll
-          for (int j = 0; j < 4; ++j) v[j] = ib + j < a.blocks ? k[size_t(ib + j) * src] : ~0ull;
+          for (int j = 0; j < 4; ++j) v[j] = ib + j < blocks ? k[size_t(ib + j) * a.cap_in] : ~0ull;
 #pragma unroll
-          for (int j = 0; j < 4; ++j)
-            if ((ib + j) * kFdTile < nb) key = min(key, v[j]);
+          for (int j = 0; j < 4; ++j) key = min(key, v[j]);
         }
-        if (e < na) {
-          lists.key[e] = (unsigned int)(key >> 32);
-          lists.best[e] = key_partner(key, nb);
-        }
+        lists.key[e] = (unsigned int)(key >> 32);
+        lists.best[e] = key_partner(key, nb);
       }
-      const int removed = nb > 0 ? removal_count(nw, a.keep, par) : 0;
       __syncthreads();
       select_window(lists, nw, removed, par, a.partner + row, a.place + row);
       __syncthreads();

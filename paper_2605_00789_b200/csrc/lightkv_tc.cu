@@ -684,14 +684,14 @@ struct FdTcSmem {
   }
 };
 
-// the best destination of source `row` of tile (ia, ib) of window w of sample b
-__device__ __forceinline__ void store_key(const FdTcArgs& a, int b, int w, int ia, int ib, int row, int a_first,
+// the best destination of source `row` of tile (ia, ib) of a window of sample b
+__device__ __forceinline__ void store_key(const FdTcArgs& a, int b, int ia, int ib, int row, const int* row_a, int a_first,
                                           int b_first, float best, int best_c) {
   unsigned long long key = ~0ull;
   if (best_c >= 0)
     key = ((unsigned long long)orderable(best) << 32) | (unsigned)((a.lists ? b_first : 0) + ib * BLK + best_c);
   if (a.lists) atomicMin(a.ws.a_key + size_t(b) * a.ws.cap_a + a_first + ia * BLK + row, key);
-  else a.ws.tile_key[((size_t(b) * a.g.n_windows + w) * a.blocks + ib) * ((a.max_cell + 1) / 2) + ia * BLK + row] = key;
+  else a.ws.tile_key[(size_t(b) * a.blocks + ib) * a.cap_in + row_a[row]] = key;
 }
 
 // CLUSTER = false is the plain launch (ks = 1) with the cluster code compiled out.
@@ -913,7 +913,7 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, FT_STAGES > 3 ? 1 : 2) fd_tc_
           named_barrier(1, FT_LOADERS);
           if (half == 0 && row < na && ok) {
             if (red_f[row] < best) { best = red_f[row]; best_c = red_c[row]; }   // ties stay with the lower column
-            store_key(a, b, w, ia, ib, row, a_first, b_first, best, best_c);
+            store_key(a, b, ia, ib, row, row_a, a_first, b_first, best, best_c);
           }
         } else {
           // ---- cluster: every CTA puts its partial G into shared memory (float [128][PITCH], over the drained ring), then CTA
@@ -998,7 +998,7 @@ __global__ void __launch_bounds__(FT_LOADERS + 32, FT_STAGES > 3 ? 1 : 2) fd_tc_
                 best = __shfl_sync(0xffffffffu, best, from);
                 best_c = __shfl_sync(0xffffffffu, best_c, from);
               }
-              if (lane == 0 && !*abort_flag) store_key(a, b, w, ia, ib, rr, a_first, b_first, best, best_c);
+              if (lane == 0 && !*abort_flag) store_key(a, b, ia, ib, rr, row_a, a_first, b_first, best, best_c);
             }
           }
           __syncwarp();

@@ -305,6 +305,37 @@ def test_builtin_workspace_takes_large_windows_whose_keys_do_not_fit(L, stage, x
     assert L.library().lightkv_compress_layer_builtin_ws(p.handle, C.byref(a)) != -3
 
 
+@pytest.mark.parametrize("tiles,windows,stage,blocks,cell", [
+    ([(64, 64)] + [(8, 8)] * 31, [1], 0, 16, 4096),            # one large window and many small ones
+    ([(32, 32)] * 8, [4, 2, 1], 2, 4, 1024),                   # a quarter of the tokens is left in the windows
+    ([(64, 64)] * 2, [1], 0, 16, 4096),                        # full windows of one size
+])
+def test_workspace_by_a_key_per_token_and_block_is_enough(L, tiles, windows, stage, blocks, cell):
+    """A caller that keeps a size of its own: sums per head, partners, places, repeat lists, the windows' tokens, and a key per
+    token and block of 128 destinations, each rounded up to 256 bytes."""
+    b, h = 2, 4
+    p = _plan(L, batch=b, n_q_heads=h, n_kv_heads=h, hidden=512, head_dim=64, tiles=tiles, n_layers=8,
+              layers=[2, 4, 6][:len(windows)], windows=windows, keep=[0.5] * len(windows))
+    info = p.stage_info(stage)
+    n = info.cap_in
+    up = lambda v: (v + 255) // 256 * 256
+    keys = b * blocks * n * 8
+    enough = up(b * h * n * 4) + 2 * up(b * n * 4) + up(-(-n // 128) * h * b * 4) + up(b * info.n_windows * (cell + 1) * 4) + up(keys)
+    assert info.workspace_bytes == enough
+    a = L.lightkv._LayerArgs()
+    a.struct_size = C.sizeof(a)
+    a.stage = stage
+    for f in ("hidden", "n_vis_out", "pos_out", "dst", "weight", "grp_off", "grp_src", "workspace", "pos"):
+        setattr(a, f, 0x1000)
+    a.hidden_out = 0x2000
+    a.hidden_row_stride = a.hidden_out_row_stride = 512
+    a.hidden_batch_stride = a.hidden_out_batch_stride = 512 * n
+    a.workspace_bytes = enough
+    assert L.library().lightkv_compress_layer(p.handle, C.byref(a)) == -1    # taken; q and k are missing
+    a.workspace_bytes = enough - 256
+    assert L.library().lightkv_compress_layer(p.handle, C.byref(a)) == -3
+
+
 def test_missing_library_fails_loudly(L, monkeypatch):
     from paper_2605_00789_b200 import lightkv
     monkeypatch.setattr(lightkv, "_LIB", None)
