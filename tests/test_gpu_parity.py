@@ -749,8 +749,8 @@ def test_xi_and_weights_have_the_same_bits_in_the_list_form(heads):
 @pytest.mark.parametrize("heads", [1, 7, 33, 40, 70])
 @pytest.mark.parametrize("before_merge", [False, True])
 def test_weights_over_head_counts(heads, before_merge):
-    """A warp's lanes take the heads 32 at a time, in one and in two rounds.  With a map event the weights come from a
-    kernel of their own: clusters whose CTAs hold 8 to 41 tokens."""
+    """The heads are taken 32 at a time, in one and in two rounds: by the merge's warps and, with a map event, by the threads of
+    a map behind xi.  (weights_kernel, that of long launches, gives the same bits as these, see above.)"""
     import torch
     wl = S.Workload(name="heads", config_id=133, batch=3, tiles=((13, 17), (9, 11)), n_text=9, hidden=72, n_q_heads=heads,
                     n_kv_heads=1, head_dim=64, n_layers=8, layers=(2, 5), windows=(3, 2), keep=(0.6, 0.5))
@@ -758,18 +758,17 @@ def test_weights_over_head_counts(heads, before_merge):
 
 
 @pytest.mark.parametrize("grid", [(11, 11), (13, 17), (32, 40)])
-@pytest.mark.parametrize("before_merge", [False, True])
-def test_weights_of_a_group_of_all_sources(grid, before_merge):
+@pytest.mark.parametrize("form", ["merge", "map", "kernel"])
+def test_weights_of_a_group_of_all_sources(grid, form):
     """Equal source rows all join one destination: groups of 61, 111 and 641 members, below and beyond what the kernels keep
     on chip.  The weights are the reported xi over their sum (single precision: 1e-5 over up to 641 terms), and the merged
     row is the weighted sum of the members' rows."""
     import torch
-    import paper_2605_00789_b200 as L
     wl = S.Workload(name="onegroup", config_id=134, batch=1, tiles=(grid,), n_text=5, hidden=1032, n_q_heads=6,
                     n_kv_heads=2, head_dim=64, n_layers=4, layers=(2,), windows=(1,), keep=(0.5,))
     n, na = grid[0] * grid[1], (grid[0] * grid[1] + 1) // 2
     removed = n - int(np.ceil(0.5 * n))
-    plan = H.make_plan(wl)
+    plan = H.make_plan(wl, max_text=20000)
     gen = torch.Generator(device="cuda")
     gen.manual_seed(grid[0])
     hidden_in = torch.randn((1, wl.n_text + n, wl.hidden), generator=gen, device="cuda")
@@ -777,12 +776,7 @@ def test_weights_of_a_group_of_all_sources(grid, before_merge):
     hidden_in = hidden_in.bfloat16()
     q = torch.randn((1, 6, wl.n_text + n, 64), generator=gen, device="cuda").bfloat16()
     k = torch.randn((1, 2, wl.n_text + n, 64), generator=gen, device="cuda").bfloat16()
-    kw = {}
-    if before_merge:
-        kw["map_event"] = torch.cuda.Event()
-        kw["map_event"].record()
-    out = L.StageBuffers(plan, 0, wl.n_text + plan.stage_info(0).cap_out, "cuda")
-    L.compress_layer(plan, 0, hidden_in, out, vis_begin=wl.n_text, q=q, k=k, **kw)
+    out = _layer_in_form(plan, form, hidden_in, wl.n_text, q=q, k=k)
     assert int(out.status) == 0 and int(out.n_vis_out) == n - removed and na - removed in (0, 1)
     off, src = out.grp_off[0].cpu().numpy(), out.grp_src[0].cpu().numpy()
     xi, weight = (t[0].cpu().numpy().astype(np.float64) for t in (out.xi_out, out.weight))
@@ -797,30 +791,27 @@ def test_weights_of_a_group_of_all_sources(grid, before_merge):
     plan.close()
 
 
-@pytest.mark.parametrize("xi_mode", ["given", "lse"])
-@pytest.mark.parametrize("before_merge", [False, True])
-def test_an_infinite_score_leaves_no_number(xi_mode, before_merge):
+@pytest.mark.parametrize("xi_mode,form", [("given", None), ("lse", "merge"), ("lse", "map"), ("lse", "kernel")])
+def test_an_infinite_score_leaves_no_number(xi_mode, form):
     """xi / sum is inf / inf for a token whose score is infinite, alone or in a group: its weight and its row are NaN, and no
     other group's are.  (A log-sum-exp of -200 overflows the exponentials of its row.)"""
     import torch
     import paper_2605_00789_b200 as L
     n, nt = 144, 5
-    plan = L.Plan(1, 264, 4, 4, 64, 4, [(12, 12)], [2], [3], [0.55], nt, xi_mode=L.XI_GIVEN if xi_mode == "given" else L.XI_ATTN_LSE)
+    plan = L.Plan(1, 264, 4, 4, 64, 4, [(12, 12)], [2], [3], [0.55], 60000, xi_mode=L.XI_GIVEN if xi_mode == "given" else L.XI_ATTN_LSE)
     gen = torch.Generator(device="cuda").manual_seed(11)
     rows = torch.randn((1, nt + n, 264), generator=gen, device="cuda").bfloat16()
     kw = {}
     if xi_mode == "given":
         kw["xi"] = 0.5 + torch.rand((1, n), generator=gen, device="cuda")
         kw["xi"][:, ::7] = float("inf")
+        out = L.StageBuffers(plan, 0, nt + plan.stage_info(0).cap_out, "cuda")
+        L.compress_layer(plan, 0, rows, out, vis_begin=nt, **kw)
     else:
         kw["q"], kw["k"] = (torch.randn((1, 4, nt + n, 64), generator=gen, device="cuda").bfloat16() for _ in range(2))
         kw["lse"] = torch.full((1, 4, nt + n), 3.0, device="cuda")
         kw["lse"][:, :, nt::7] = -200.0
-    if before_merge:
-        kw["map_event"] = torch.cuda.Event()
-        kw["map_event"].record()
-    out = L.StageBuffers(plan, 0, nt + plan.stage_info(0).cap_out, "cuda")
-    L.compress_layer(plan, 0, rows, out, vis_begin=nt, **kw)
+        out = _layer_in_form(plan, form, rows, nt, **kw)
     inf = ~torch.isfinite(out.xi_out[0])
     assert torch.equal(inf.nonzero()[:, 0].cpu(), torch.arange(0, n, 7)) and bool((out.xi_out[0][inf] > 0).all())
     assert torch.equal(torch.isnan(out.weight[0]), inf)
@@ -835,18 +826,31 @@ def test_an_infinite_score_leaves_no_number(xi_mode, before_merge):
     plan.close()
 
 
-@pytest.mark.parametrize("before_merge", [False, True])
-def test_xi_of_tokens_cut_at_the_capacity_is_reported(before_merge):
+@pytest.mark.parametrize("form", ["merge", "map", "kernel"])
+def test_xi_of_tokens_cut_at_the_capacity_is_reported(form):
     """A subset under a full-grid plan keeps all of its tokens and is cut at cap_out: those behind the cut belong to no group,
     and their xi is reported all the same -- the same as under a plan that has room for them."""
     import torch
+    import bench
     wl, first = _near_full_subset()
-    plan, roomy = H.make_plan(wl, batch=2), H.make_plan(wl, batch=2, ragged=True)
+    plan, roomy = H.make_plan(wl, batch=2, max_text=120000), H.make_plan(wl, batch=2, ragged=True)
     g0 = H.gpu_stage(plan, wl, 0, H.prepare_stage(wl, 0, first))
     pos1 = [g0["pos_out"][b, :int(g0["n_vis_out"][b])] for b in range(2)]
     inp1 = H.prepare_stage(wl, 1, pos1)
-    cut = H.gpu_stage(plan, wl, 1, inp1, kv_stream=torch.cuda.Stream() if before_merge else None)
     whole = H.gpu_stage(roomy, wl, 1, inp1)
+    after, launches = 0, []
+    if form == "kernel":                               # a long launch, by rows behind the vision block
+        after = (24 << 20) // (2 * wl.hidden * 2)
+        inp1["hidden"] = np.pad(inp1["hidden"], ((0, 0), (0, after - 1), (0, 0)))
+        del inp1["v"]
+
+    def layer(*args, **kw):
+        import paper_2605_00789_b200 as L
+        launches.append(bench.count_launches(lambda: L.compress_layer(*args, **kw)))
+        L.compress_layer(*args, **kw)
+
+    cut = H.gpu_stage(plan, wl, 1, inp1, n_text_after=after, kv_stream=torch.cuda.Stream() if form == "map" else None, layer_fn=layer)
+    assert launches == [5 if form == "kernel" else 4]
     n = int(inp1["n_vis"][0])
     assert int(cut["status"][0]) == 8 and int(cut["n_vis_out"][0]) < n
     np.testing.assert_array_equal(cut["xi_out"][0, :n] > 0, True)
@@ -1011,11 +1015,23 @@ def test_heads_of_one_piece_over_variants(batch, grid, in_place):
 
 
 def test_weights_of_samples_with_a_token_per_cta():
-    # at most eight tokens a sample, weights by a kernel of their own (the caller waits for the map alone)
+    # at most eight tokens a sample: the map behind xi (the caller waits for the map alone) against the oracle, and
+    # weights_kernel, whose clusters then have CTAs without a token, against it
     import torch
     wl = S.Workload(name="few", config_id=143, batch=3, tiles=((2, 4),), n_text=9, hidden=64, n_q_heads=4,
                     n_kv_heads=4, head_dim=64, n_layers=16, layers=(3,), windows=(1,), keep=(0.5,))
     H.run_schedule(wl, kv_stream=torch.cuda.Stream())
+    gen = torch.Generator(device="cuda").manual_seed(3)
+    for grid in ((1, 2), (2, 4), (3, 3), (2, 8), (1, 17)):
+        few = dataclasses.replace(wl, tiles=(grid,))
+        plan = H.make_plan(few, max_text=70000)
+        n = 9 + grid[0] * grid[1]
+        rows = torch.randn((3, n, 64), generator=gen, device="cuda").bfloat16()
+        q, k = (torch.randn((3, 4, n, 64), generator=gen, device="cuda").bfloat16() for _ in range(2))
+        short, long = (_layer_in_form(plan, form, rows, 9, q=q, k=k) for form in ("map", "kernel"))
+        for name in MAP_OUTPUTS:
+            assert torch.equal(getattr(short, name), getattr(long, name)), (grid, name)
+        plan.close()
 
 
 @pytest.mark.parametrize("grid,n_kv,head_dim,page,vb,after", [
