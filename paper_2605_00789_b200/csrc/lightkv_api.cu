@@ -400,8 +400,9 @@ int compress_layer(const lightkv_plan_t* p, const lightkv_layer_args_t* a, bool 
   }
   if (!in_map && launch_select_map(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (late_map && launch_map(L, tiled, true) != cudaSuccess) return LIGHTKV_ERR_CUDA;
-  // weights: by a kernel of their own where the merge does not take them along
-  const bool late_weights = early_map && attn, with_merge = late_weights && merge_takes_weights(L);
+  // weights: by a kernel of their own where the merge does not take them along, and for a caller that waits for the map alone
+  // (to compact K/V beside the merge)
+  const bool late_weights = early_map && attn, with_merge = late_weights && !a->map_event && merge_takes_weights(L);
   if (late_weights && !with_merge && launch_weights(L) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (mark(4) != cudaSuccess) return LIGHTKV_ERR_CUDA;
   if (a->map_event && cudaEventRecord(static_cast<cudaEvent_t>(a->map_event), L.stream) != cudaSuccess)

@@ -1155,17 +1155,27 @@ static bool few_rows(const LayerLaunch& L) {
   return few_rows((long long)(L.a->vis_begin + L.ws.cap_out + L.a->n_text_after) * L.batch);
 }
 // The instructions a row's CTA spends on its weights are in nobody's way while a launch is short; a long one is bound by
-// memory only as long as little else is issued.  Whole passes, with the merge against by weights_kernel: 4 x 652 rows of 4096
-// 144.3 / 145.3 us, 16 x up to 624 rows of 2048 (23 MB) 138 / 144; 8 x 3008 rows of 4096 (100 MB) and its later stages 556 / 511.
+// memory only as long as little else is issued.  us of compress_layer, a given log-sum-exp, with the merge / by weights_kernel:
+// 9.5 MB (2304 tokens x 4096) 28.7 / 31.8, 11 MB (4 x 576) 27.2 / 28.8, 17.5 MB (2 x 2048 x 3584) 39.9 / 42.7, 21 MB (16 x 576 x
+// 2048) 46.7 / 46.7, 22 MB (8 x 576 x 4096) 39.9 / 38.8, 27.5 MB (40 x 576 x 1024) 65.5 / 65.5, 30 MB (6 x 1152 x 4096) 53.9 / 51.4,
+// 44 MB (16 x 576 x 4096) 73.3 / 68.7, 59.5 MB (2 x 8192 x 3584) 128 / 119, 98 MB (8 x 2880 x 4096) 168 / 151; the same with xi from
+// all keys.  (Rows of 1 KB and a hundred samples, 40 MB: 112 / 115.)
 bool merge_takes_weights(const LayerLaunch& L) {
   return (long long)(L.a->vis_begin + L.ws.cap_out + L.a->n_text_after) * L.batch * L.hidden * (L.dtype == LIGHTKV_BF16 ? 2 : 4) <= (24ll << 20);
 }
-// The map behind xi, with the weights.  For a caller that waits for the map alone, where the launch is short: beside xi it would
-// save less than the second kernel costs (2 x 798 tokens x 32 heads, three stages with a given log-sum-exp: 162 us a pass
-// against 169).  And for one whose counts are replaced in place, whatever the launch: the xi kernel reads n_vis item by item,
-// and a map beside it would put the smaller counts there.
+// The map behind xi, with the weights.  For a caller that waits for the map alone, where it costs less than weights_kernel does
+// beside what the map beside xi saves: in short launches with few heads, whose sums are little work for a sample's CTAs, or few
+// tokens, fewer where the map has the longer xi from all keys to run beside.  us of compress_layer, map behind xi / beside it and
+// weights_kernel, samples x tokens x heads, given log-sum-exp: 1 x 576 x 32 19.6 / 20.2, 2 x 798 x 32 29.7 / 31.9, 2 x 1024 x 28 28.7
+// / 26.5, 4 x 576 x 32 29.8 / 28.8, 2 x 2048 x 28 47.6 / 42.5; 1 x 4096 x 8 22.4 / 26.5, 2 x 2048 x 16 27.1 / 28.4, 16 x 576 x 16 31.0 /
+// 31.9, 4 x 2304 x 16 33.3 / 32.8; all keys: 2 x 200 x 32 18.4 / 20.4, 1 x 288 x 32 19.2 / 21.6, 1 x 576 x 32 24.0 / 22.9, 2 x 400 x 32
+// 23.6 / 23.1, 2 x 798 x 32 39.0 / 33.7, 4 x 1152 x 32 67.5 / 62.4; 16 x 576 x 16 49.0 / 49.4, 4 x 2304 x 16 75.8 / 76.1.
+// And for one whose counts are replaced in place, whatever the launch: the xi kernel reads n_vis item by item, and a map beside it
+// would put the smaller counts there.
 bool map_behind_xi(const LayerLaunch& L) {
-  return L.a->n_vis == L.a->n_vis_out || (L.a->map_event && merge_takes_weights(L));
+  if (L.a->n_vis == L.a->n_vis_out) return true;
+  const long long few_tokens = L.xi_mode == LIGHTKV_XI_ATTN_LSE ? 2000 : 500;
+  return L.a->map_event && merge_takes_weights(L) && (L.n_q_heads <= 16 || (long long)L.batch * L.ws.cap_in <= few_tokens);
 }
 
 // =====================================================================================================

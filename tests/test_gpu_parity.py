@@ -650,16 +650,17 @@ def test_subset_given_to_a_full_grid_plan_raises_the_count_bit():
 
 def _layer_in_form(plan, form, rows, nt, **kw):
     """Stage 0 in one of the forms that make the weights: "merge" (with the merge of the rows), "map" (a map behind xi, for a
-    caller that waits for the map of a short launch) or "kernel" (weights_kernel: the launch is long, by rows behind the vision
-    block).  The launches of the call show that it was the form."""
+    caller that waits for the map of a short launch of few heads or tokens), "kernel" (weights_kernel: the launch is long, by
+    rows behind the vision block), "kernel and event" (the same where the caller waits for the map) or "event" (weights_kernel in
+    a short launch of many heads and tokens, for a caller that waits).  The launches of the call show that it was the form."""
     import torch
     import bench
     import paper_2605_00789_b200 as L
     after = 0
-    if form == "kernel":
+    if "kernel" in form:
         after = (24 << 20) // (rows.shape[0] * rows.shape[2] * rows.element_size())
         rows = torch.cat([rows, torch.zeros((rows.shape[0], after, rows.shape[2]), device="cuda", dtype=rows.dtype)], 1)
-    elif form == "map":
+    if form in ("map", "event", "kernel and event"):
         kw["map_event"] = torch.cuda.Event()
         kw["map_event"].record()
     out = L.StageBuffers(plan, 0, nt + plan.stage_info(0).cap_out + after)
@@ -667,7 +668,7 @@ def _layer_in_form(plan, form, rows, nt, **kw):
     call = lambda: L.compress_layer(plan, 0, rows, out, vis_begin=nt, n_text_after=after, **kw)
     call()
     torch.cuda.synchronize()
-    assert bench.count_launches(call) == (5 if form == "kernel" else 4)
+    assert bench.count_launches(call) == (4 if form in ("merge", "map") else 5)
     return out
 
 
@@ -698,7 +699,8 @@ def test_xi_and_weights_have_the_same_bits_in_every_form(heads, dtype, xi_mode):
     kw = dict(q=q, k=k, pos=pos, n_vis=torch.tensor(counts, device="cuda", dtype=torch.int32))
     if xi_mode == "lse":
         kw["lse"] = 3.0 + torch.rand((b, heads, nt + n), generator=gen, device="cuda")
-    found = {form: _layer_in_form(plan(b), form, rows, nt, **kw) for form in ("merge", "map", "kernel")}
+    waits = "event" if xi_mode == "attn" and heads > 16 else "map"      # 960 tokens
+    found = {form: _layer_in_form(plan(b), form, rows, nt, **kw) for form in ("merge", waits, "kernel", "kernel and event")}
     want = found["merge"]
     assert int(want.status) == 0 and bool((want.xi_out[0] > 0).all())
     for form, out in found.items():
@@ -750,7 +752,7 @@ def test_xi_and_weights_have_the_same_bits_in_the_list_form(heads):
 @pytest.mark.parametrize("before_merge", [False, True])
 def test_weights_over_head_counts(heads, before_merge):
     """The heads are taken 32 at a time, in one and in two rounds: by the merge's warps and, with a map event, by the threads of
-    a map behind xi.  (weights_kernel, that of long launches, gives the same bits as these, see above.)"""
+    a map behind xi or, beyond 16 heads, by weights_kernel.  (All give the same bits, see above.)"""
     import torch
     wl = S.Workload(name="heads", config_id=133, batch=3, tiles=((13, 17), (9, 11)), n_text=9, hidden=72, n_q_heads=heads,
                     n_kv_heads=1, head_dim=64, n_layers=8, layers=(2, 5), windows=(3, 2), keep=(0.6, 0.5))

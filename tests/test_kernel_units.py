@@ -99,26 +99,30 @@ int main() {
 
 
 def test_the_map_waits_for_xi_where_the_counts_are_replaced_in_place(tmp_path):
-    """The xi kernel reads the counts item by item, so a map that replaces them stands behind it, however long the launch;
-    one with counts of its own runs beside it unless the caller waits for the map of a short launch."""
+    """The xi kernel reads the counts item by item, so a map that replaces them stands behind it, however long the launch; one
+    with counts of its own runs beside it unless the caller waits for the map of a short launch of few heads or tokens."""
     entry.build()
     out = _run(tmp_path, r"""
 #include <stdio.h>
 #include "launch.h"
 int main() {
   int in[4], out[4], event;
-  for (int rows : {100, 100000})
-    for (bool waits : {false, true})
-      for (const int* counts : {(const int*)in, (const int*)out, (const int*)nullptr}) {
-        lightkv_layer_args_t a = {};
-        a.n_vis = counts; a.n_vis_out = out; a.map_event = waits ? &event : nullptr;
-        lkv::LayerLaunch L = {};
-        L.batch = 1; L.hidden = 4096; L.dtype = LIGHTKV_BF16; L.ws.cap_out = rows; L.a = &a;
-        printf("%d ", lkv::map_behind_xi(L));
-      }
+  const int sizes[][3] = {{16, 4000, 3000}, {16, 4000, 100000}, {17, 500, 300}, {17, 501, 300}, {17, 2000, 300}, {17, 2001, 300}};
+  for (int mode : {LIGHTKV_XI_ATTN_FULL, LIGHTKV_XI_ATTN_LSE})
+    for (const auto& size : sizes)
+      for (bool waits : {false, true})
+        for (const int* counts : {(const int*)in, (const int*)out, (const int*)nullptr}) {
+          lightkv_layer_args_t a = {};
+          a.n_vis = counts; a.n_vis_out = out; a.map_event = waits ? &event : nullptr;
+          lkv::LayerLaunch L = {};
+          L.batch = 1; L.hidden = 4096; L.dtype = LIGHTKV_BF16; L.xi_mode = mode; L.a = &a;
+          L.n_q_heads = size[0]; L.ws.cap_in = size[1]; L.ws.cap_out = size[2];
+          printf("%d ", lkv::map_behind_xi(L));
+        }
 }
 """, "-L", os.path.dirname(CSRC), "-l:liblightkv.so", "-Xlinker", "-rpath=" + os.path.dirname(CSRC))
-    assert out == "0 1 0  1 1 1  0 1 0  0 1 0".split()
+    behind, beside = "0 1 0  1 1 1", "0 1 0  0 1 0"
+    assert out == " ".join([behind, beside, behind, beside, beside, beside] + [behind, beside, behind, behind, behind, beside]).split()
 
 
 @pytest.mark.gpu
