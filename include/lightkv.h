@@ -211,7 +211,8 @@ typedef struct {
                                       trace events are asked for), the FD kernel, which streams the hidden
                                       states (and the window build, where one is launched: samples or windows
                                       too long for the shared memory of a CTA, the fp32-FMA engine in bf16,
-                                      large windows in fp32), is enqueued on this second stream while the
+                                      large windows in fp32), and the merge map, where it does not have to
+                                      wait for xi, are enqueued on this second stream while the
                                       xi contraction runs on `stream`; the two are forked and joined with
                                       events inside the call, so the caller sees everything ordered on
                                       `stream` as before.  The stream must belong to the same device. */
@@ -292,9 +293,9 @@ int lightkv_compress_layer_builtin_ws(const lightkv_plan_t* plan, const lightkv_
  * Out of place: the destinations do not overlap the sources.
  * In place: k_dst == k_src and v_dst == v_src with the same strides, page size and block table on both sides
  * (anything else that overlaps is INVALID_ARG or undefined).  The cache then shrinks inside its own rows or
- * pages, with no second copy of it.  Where the output rows of a (sample, K or V, head) plane fit into shared memory,
- * perhaps cut by columns, one CTA gathers and merges them there before it stores any.  For longer samples every
- * merged group is first written over its surviving token's row (no other group reads that row), then a second
+ * pages, with no second copy of it.  Where the rows of a (sample, K or V, head) plane from the vision block on fit into
+ * shared memory, perhaps cut by columns, one CTA copies all of them there before it stores the merged and moved rows.  For
+ * longer samples every merged group is first written over its surviving token's row (no other group reads that row), then a second
  * kernel moves every output row forward to its slot -- a slot never lies behind its source -- in ascending chunks
  * that are gathered into shared memory before any of their slots is written.  Both forms leave the same bytes.  Rows
  * behind the new end of a sample keep stale contents; pages that became empty are the caller's to release. */

@@ -1639,8 +1639,7 @@ kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* _
 // =====================================================================================================
 struct KvPlaneSmem {
   int rows_in, n_in, n_out, blocks;            // capacities: moving rows in, vision tokens in / out, pages of the moving rows
-  __host__ __device__ size_t mem() const { return 0; }
-  __host__ __device__ size_t wgt() const { return mem() + size_t(n_in) * 4; }
+  __host__ __device__ size_t wgt() const { return size_t(n_in) * 4; }                    // (the member list comes first)
   __host__ __device__ size_t off() const { return wgt() + size_t(n_in) * 4; }
   __host__ __device__ size_t blk() const { return off() + size_t(n_out + 1) * 4; }
   __host__ __device__ size_t rows() const { return (blk() + size_t(blocks) * 4 + 15) & ~size_t(15); }
@@ -1657,7 +1656,7 @@ kv_plane_kernel(T* __restrict__ k_buf, T* __restrict__ v_buf, KvAddr ad, KvPlane
   grid_dependency_sync();
   extern __shared__ __align__(16) unsigned char smem_raw[];
   constexpr int V = Vec<T>::n;
-  int* mem = reinterpret_cast<int*>(smem_raw + sm.mem());               // group members, survivor first
+  int* mem = reinterpret_cast<int*>(smem_raw);                          // group members, survivor first
   float* wgt = reinterpret_cast<float*>(smem_raw + sm.wgt());           // weights of the tokens
   int* off = reinterpret_cast<int*>(smem_raw + sm.off());               // first member of every output row
   int* blk = reinterpret_cast<int*>(smem_raw + sm.blk());               // pages of the moving rows
