@@ -647,8 +647,8 @@ cudaError_t launch_xi_tc(const LayerLaunch& L, bool wait_first) {
 // written, read by the norms and read by the MMA), not by HBM or the tensor pipe.  Tiles of 256 x 256 halve that, but the
 // four CTAs they then leave per SM's worth of work have to exchange partial products, and distributed shared memory gave
 // 10 bytes per nanosecond and SM (13 us per 128 rows of 256): 62, with the exchange vectorised 56 us, where tiles of 128
-// with a six-stage ring take 44 (two samples of 8192 tokens x 3584 in windows of 512; list-driven tiles that met in atomics
-// took 77; windows of 1024 and 2048: 76 -> 45 and 76 -> 43).  The launch has as many tiles as windows of the expected
+// with a six-stage ring take 44, and 35 with the scores compared by reciprocals (two samples of 8192 tokens x 3584 in windows of
+// 512; list-driven tiles that met in atomics took 77; windows of 1024 and 2048: 76 -> 45 and 76 -> 43 before the reciprocals).  The launch has as many tiles as windows of the expected
 // size need; a CTA goes on with the blocks of a window that has grown beyond that.
 // ======================================================================================================
 struct FdTcArgs {
