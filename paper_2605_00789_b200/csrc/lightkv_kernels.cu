@@ -1638,12 +1638,12 @@ kv_compact_kernel(const T* __restrict__ k_src, const T* __restrict__ v_src, T* _
 // 256 threads 12, 1024 13 in the first, where two CTAs of 512 fit.
 // =====================================================================================================
 struct KvPlaneSmem {
-  int rows_in, n_in, n_out, blocks;            // capacities: moving rows in, vision tokens in / out, pages of the moving rows
+  int staged, n_in, n_out, blocks;             // capacities: rows in shared memory, vision tokens in / out, pages of the moving rows
   __host__ __device__ size_t wgt() const { return size_t(n_in) * 4; }                    // (the member list comes first)
   __host__ __device__ size_t off() const { return wgt() + size_t(n_in) * 4; }
   __host__ __device__ size_t blk() const { return off() + size_t(n_out + 1) * 4; }
   __host__ __device__ size_t rows() const { return (blk() + size_t(blocks) * 4 + 15) & ~size_t(15); }
-  __host__ __device__ size_t bytes(int pieces) const { return rows() + size_t(rows_in) * pieces * 16; }
+  __host__ __device__ size_t bytes(int pieces) const { return rows() + size_t(staged) * pieces * 16; }
 };
 
 // ONE: rows of a single piece, as above
@@ -1812,7 +1812,7 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
             a->page_size > 0 ? a->dst_block_table : nullptr, a->page_size, a->max_blocks, a->dst_seq_start, magic_page};
   const int ch_host = K.head_dim * (K.dtype == LIGHTKV_BF16 ? 2 : 4) / 16;
   if (2 * K.n_kv_heads * ch_host >= 65536) return cudaErrorInvalidValue;      // range of the unit decode
-    const dim3 grid(a->vis_begin + K.cap_out + a->n_text_after, K.batch);
+  const dim3 grid(a->vis_begin + K.cap_out + a->n_text_after, K.batch);
   const int units = 2 * K.n_kv_heads * ch_host;
   // two units per thread (both in flight); narrow caches (GQA) get narrow CTAs
   const bool few = few_rows((long long)grid.x * grid.y);
@@ -1824,15 +1824,20 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
     using T = decltype(tag);
     cudaError_t e = cudaSuccess;
     if (in_place) {
-      // planes: (sample, K / V, head, column part); see kv_plane_kernel for the cut
-      const int moving = K.cap_in + a->n_text_after;
-      const KvPlaneSmem sm{moving, K.cap_in, K.cap_out, a->page_size > 0 ? (moving + a->page_size - 1) / a->page_size + 1 : 0};
+      // planes: (sample, K / V, head, column part); see kv_plane_kernel for the cut.  A gather stages the survivors' rows alone:
+      // with room for all, samples of 5120 tokens or more took kv_move_kernel and fewer CTAs shared an SM (us a call, 8 heads x
+      // 128, room for all / for these: 1 x 6400 tokens 14.4 / 9.4, 4 x 6400 57 / 35.6, 2 x 5776 24.9 / 16.6, 8 x 2304 22.4 / 15.7).
+      // Cut as if all rows were staged: wider parts leave fewer CTAs (1 x 5328 8.4 -> 10.8).
+      const int moving = K.cap_in + a->n_text_after, staged = gather ? K.cap_out + a->n_text_after : moving;
+      const KvPlaneSmem all{moving, K.cap_in, K.cap_out, a->page_size > 0 ? (moving + a->page_size - 1) / a->page_size + 1 : 0};
+      const KvPlaneSmem sm{staged, all.n_in, all.n_out, all.blocks};
       const long long planes = 2ll * K.batch * K.n_kv_heads;
       int p = 1;
       while (ch_host % (2 * p) == 0 && ch_host / p >= 4 &&
-             (sm.bytes(ch_host / p) > 220 * 1024 || (planes * p < 2 * sms && ch_host / p >= 8))) p *= 2;
+             (all.bytes(ch_host / p) > 220 * 1024 || (planes * p < 2 * sms && ch_host / p >= 8))) p *= 2;
       const int ch = ch_host / p;
-      if (sm.bytes(ch) <= 220 * 1024 && (long long)moving * ch < 65536) {
+      const bool two = all.bytes(ch) <= 110 * 1024 || (sm.bytes(ch) <= 110 * 1024 && planes * p > sms);   // CTAs share an SM
+      if (sm.bytes(ch) <= 220 * 1024 && (long long)staged * ch < 65536) {
         auto launch = [&](auto kernel, int threads) -> cudaError_t {
           const cudaError_t rc = ensure_dynamic_smem(kernel, 220 * 1024);
           if (rc != cudaSuccess) return rc;
@@ -1842,8 +1847,8 @@ cudaError_t launch_kv_compact(const KvLaunch& K) {
               a->grp_off, a->grp_src, a->weight);
         };
         if constexpr (sizeof(T) == 2)                     // (fp32 heads have two pieces or more, and planes are not cut to one)
-          if (ch == 1) return sm.bytes(ch) <= 110 * 1024 ? launch(kv_plane_kernel<T, 512, true>, 512) : launch(kv_plane_kernel<T, 1024, true>, 1024);
-        return sm.bytes(ch) <= 110 * 1024 ? launch(kv_plane_kernel<T, 512, false>, 512) : launch(kv_plane_kernel<T, 1024, false>, 1024);
+          if (ch == 1) return two ? launch(kv_plane_kernel<T, 512, true>, 512) : launch(kv_plane_kernel<T, 1024, true>, 1024);
+        return two ? launch(kv_plane_kernel<T, 512, false>, 512) : launch(kv_plane_kernel<T, 1024, false>, 1024);
       }
     }
     if (!(in_place && gather)) {                          // in place, gather mode has nothing to merge

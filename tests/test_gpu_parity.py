@@ -289,6 +289,7 @@ def test_in_place_kv_compaction_long_rows_and_text_behind():
     (3, 2, 24, (12, 14), 0),         # rows of three 16-byte pieces: not cut
     (2, 3, 96, (40, 41), 17),        # parts of 64 bytes (rows of twelve pieces)
     (1, 2, 128, (72, 74), 5),        # fits on chip in parts of 32 bytes only
+    (1, 2, 128, (80, 82), 5),        # gathered, the survivors' rows fit on chip; to be merged, all rows do not
     (1, 1, 128, (100, 96), 5),       # does not fit: merged at the survivors, then moved in chunks
 ])
 @pytest.mark.parametrize("kv_mode,paged", [("merge", 0), ("gather", 16)])
